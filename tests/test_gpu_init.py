@@ -100,3 +100,48 @@ def test_grad_init_matches_oracle(orc, gsct, n):
     if n > 1:
         np.testing.assert_allclose(g_sc[safe, 0], sc[safe, 0], rtol=1e-4, atol=1e-6)
     assert np.all(g_q[:, 0] == 1) and np.all(g_q[:, 1:] == 0)
+
+
+# detectors that no filter tile divides (16 outputs, 8 rows; the wide form above 2,700 columns),
+# volumes at the edges of the 16 x 16 blocks and of each voxels-per-thread choice, frames with a
+# component along z (the general back-projection)
+@pytest.mark.parametrize("nv,W,H,dims,tilt", [(1, 1, 1, (5, 4, 3), 0.0), (5, 17, 9, (17, 15, 23), 0.0),
+                                              (6, 97, 41, (33, 16, 47), 0.2),
+                                              (2, 2801, 6, (24, 20, 18), 0.1),
+                                              (70, 64, 48, (96, 80, 64), 0.0)])
+def test_fdk_ragged_and_tilted(orc, gsct, nv, W, H, dims, tilt):
+    """1e-4 of the peak as for images and volumes, plus the rounding of a detector position (about
+    2.5 x 2^-24 of the side) times the steepest slope, twice the peak per pixel."""
+    from oracle.init import fdk
+    B = gsct.binding
+    views = synth.cone_views(nv, W, H)
+    if tilt:
+        for v in views:
+            n = v["det_center"] - v["src"]
+            n = n / np.linalg.norm(n) + np.array([0, 0, tilt])
+            n /= np.linalg.norm(n)
+            pitch = np.linalg.norm(v["v"])
+            u = np.cross([0, 0, 1], n)
+            u /= np.linalg.norm(u)
+            w = np.cross(n, u)
+            v["src"], v["det_center"] = -4 * n, 2 * n
+            v["u"] = pitch * (np.cos(0.3) * u + np.sin(0.3) * w)
+            v["v"] = pitch * (np.cos(0.3) * w - np.sin(0.3) * u)
+    rng = np.random.default_rng(W)
+    proj = (1 + rng.random((nv, H, W))).astype(np.float32)
+    grid = synth.cube_grid(8)
+    grid["dims"] = dims
+    # the whole detector and some voxels outside it
+    half = 2.2 * min(W, H) / max(W, H)
+    grid["voxel"] = [half / d for d in dims]
+    grid["origin"] = [-half / 2] * 3
+    want = fdk(proj.astype(np.float64), orc.views64(views), grid)
+    d_proj, d_views = torch.from_numpy(proj).cuda(), gsct.views_to_device(views, "cuda")
+    ws = torch.full((B.lib().gs_fdk_workspace_size(nv, W, H),), 255, dtype=torch.uint8, device="cuda")
+    vol = torch.full(dims[::-1], float("nan"), device="cuda")
+    B.check(B.lib().gs_fdk(B.ptr(d_proj), B.ptr(d_views), nv, W, H,
+                           ctypes.byref(B.grid_struct(grid)), B.ptr(vol), B.ptr(ws), ws.numel(),
+                           _s()), "gs_fdk")
+    assert np.abs(want).max() > 0
+    tol = 1e-4 + 2.0 ** -21 * max(W, H)
+    assert np.abs(vol.cpu().numpy() - want).max() <= tol * np.abs(want).max()
