@@ -15,7 +15,9 @@
 //            activations applied in the same pass.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "gs_internal.cuh"
 #include "gs_tma.cuh"
@@ -25,7 +27,8 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ float sgnf(float x) { return (x > 0.f) - (x < 0.f); }
+// two set-on-compare instructions and a subtraction (no integer conversion)
+__device__ __forceinline__ float sgnf(float x) { return (x > 0.f ? 1.f : 0.f) - (x < 0.f ? 1.f : 0.f); }
 
 template <typename T>
 __device__ __forceinline__ void block_add(T v, T* target) {
@@ -84,31 +87,80 @@ __global__ void __launch_bounds__(kThreads)
 // ------------------------------------------------------------------------------------------
 // TV 3D
 // ------------------------------------------------------------------------------------------
+// Bound by HBM: the volume in and the gradient out (8 bytes per voxel).  A thread owns VW
+// consecutive voxels of a row (a 16-byte vector where rows are 16-byte aligned, nx a multiple
+// of 4) and walks zc planes: its own column's planes stay in registers, the rows above and below
+// are neighbours' vectors in L1, x neighbours come by shuffle, and each difference along z gives
+// its sign to both planes.  Threads are laid over the flattened (x, y) plane, so no lane idles
+// at a row's end.  256^3: 96 -> 34 us (one block per row and six scalar loads per voxel before).
+template <int VW>
 __global__ void __launch_bounds__(kThreads)
-    k_tv3d(const float* __restrict__ v, int nx, int ny, int nz, float scale,
+    k_tv3d(const float* __restrict__ v, int nx, int ny, int nz, int zc, float scale,
            float* __restrict__ loss, float* __restrict__ grad, int accumulate) {
-  // blocks stride over the (y, z) rows, threads over x: one 32-bit index division per row
-  // (the entry point keeps ny nz below 2^31)
-  const uint32_t rows = (uint32_t)ny * (uint32_t)nz;
-  const int64_t sy = nx, sz = (int64_t)nx * ny;
+  const int nxv = nx / VW;
+  const int64_t sy = nx, sz = (int64_t)nx * ny, cols = (int64_t)nxv * ny;
+  const int64_t pt = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const bool live = pt < cols;
+  const int64_t p = live ? pt : cols - 1;
+  const int y = cols >> 32 ? (int)(p / nxv) : (int)((uint32_t)p / (uint32_t)nxv);
+  const int x = (int)(p - (int64_t)y * nxv) * VW;
+  const int lane = threadIdx.x & 31;
+  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  const bool xl = x > 0, xr = x + VW < nx, yl = y > 0, yr = y + 1 < ny;
+  using V = typename std::conditional<VW == 4, float4, float>::type;
+  auto load = [&](int64_t i, float (&f)[VW]) {
+    const V q = __ldg(reinterpret_cast<const V*>(v + i));
+    memcpy(f, &q, sizeof(V));
+  };
+  int64_t i = (int64_t)z0 * sz + (int64_t)y * sy + x;
   float s = 0.f;
-  for (uint32_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const int z = (int)(row / (uint32_t)ny), y = (int)(row - (uint32_t)z * (uint32_t)ny);
-    const int64_t r0 = row * nx;
-    for (int x = threadIdx.x; x < nx; x += kThreads) {
-      const int64_t i = r0 + x;
-      const float c = v[i];
-      float g = 0.f;
-      if (x + 1 < nx) { const float d = v[i + 1] - c; s += fabsf(d); g -= sgnf(d); }
-      if (x > 0) g += sgnf(c - v[i - 1]);
-      if (y + 1 < ny) { const float d = v[i + sy] - c; s += fabsf(d); g -= sgnf(d); }
-      if (y > 0) g += sgnf(c - v[i - sy]);
-      if (z + 1 < nz) { const float d = v[i + sz] - c; s += fabsf(d); g -= sgnf(d); }
-      if (z > 0) g += sgnf(c - v[i - sz]);
-      if (grad) grad[i] = (accumulate ? grad[i] : 0.f) + scale * g;
-    }
+  float c[VW], gz[VW];  // the current plane, and the sign of its difference to the one below
+  load(i, c);
+#pragma unroll
+  for (int k = 0; k < VW; ++k) gz[k] = 0.f;
+  if (z0 > 0) {
+    float m[VW];
+    load(i - sz, m);
+#pragma unroll
+    for (int k = 0; k < VW; ++k) gz[k] = sgnf(c[k] - m[k]);
   }
-  if (loss) block_add(s * scale, loss);
+  for (int z = z0; z < z1; ++z, i += sz) {
+    float n[VW], ym[VW], yp[VW], g[VW];
+    const bool zr = z + 1 < nz;
+#pragma unroll
+    for (int k = 0; k < VW; ++k) n[k] = ym[k] = yp[k] = c[k];  // no neighbour: no difference
+    if (zr) load(i + sz, n);
+    if (yl) load(i - sy, ym);
+    if (yr) load(i + sy, yp);
+    float xm = __shfl_up_sync(0xffffffffu, c[VW - 1], 1), xp = __shfl_down_sync(0xffffffffu, c[0], 1);
+    if (lane == 0 && xl) xm = __ldg(v + i - 1);
+    if (lane == 31 && xr) xp = __ldg(v + i + VW);
+    if (!xl) xm = c[0];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) {
+      const float dx = k + 1 < VW ? c[k + 1 < VW ? k + 1 : k] - c[k] : xr ? xp - c[k] : 0.f;
+      const float dy = yr ? yp[k] - c[k] : 0.f, dz = zr ? n[k] - c[k] : 0.f;
+      const float bx = sgnf(c[k] - (k > 0 ? c[k > 0 ? k - 1 : 0] : xm));
+      const float fz = sgnf(dz);
+      s += fabsf(dx) + fabsf(dy) + fabsf(dz);
+      g[k] = (bx - sgnf(dx)) + (sgnf(c[k] - ym[k]) - sgnf(dy)) + (gz[k] - fz);
+      gz[k] = fz;
+    }
+    if (grad && live) {
+      float o[VW];
+#pragma unroll
+      for (int k = 0; k < VW; ++k) o[k] = 0.f;
+      if (accumulate) memcpy(o, grad + i, sizeof(V));
+#pragma unroll
+      for (int k = 0; k < VW; ++k) o[k] += scale * g[k];
+      V q;
+      memcpy(&q, o, sizeof(V));
+      *reinterpret_cast<V*>(grad + i) = q;
+    }
+#pragma unroll
+    for (int k = 0; k < VW; ++k) c[k] = n[k];
+  }
+  if (loss) block_add(live ? s * scale : 0.f, loss);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1297,9 +1349,19 @@ int gs_tv3d_loss(const float* d_vol, int nx, int ny, int nz, float weight, float
   const int64_t total = (int64_t)nx * ny * nz;
   const int64_t rows = (int64_t)ny * nz;
   if (rows >= ((int64_t)1 << 31)) return GS_ERR_ARG;
-  const int blocks = (int)std::min<int64_t>(rows, 8 * (int64_t)num_sms());
-  return launch("tv3d_loss", k_tv3d, dim3(blocks), dim3(kThreads), 0,
-                (cudaStream_t)stream, d_vol, nx, ny, nz, weight / (float)total, d_loss, d_grad,
+  // 16-byte vectors where every row starts aligned
+  const bool vec = nx % 4 == 0 && al16(d_vol) && al16(d_grad);
+  const int64_t cols = rows / nz * (vec ? nx / 4 : nx);  // threads of one plane
+  const int64_t bx = (cols + kThreads - 1) / kThreads;
+  if (bx > ((int64_t)1 << 31) - 1) return GS_ERR_ARG;
+  // planes per thread: 16 (one extra plane read per 16), fewer while the grid would hold less
+  // than eight CTAs per SM
+  const int64_t want = std::max<int64_t>(1, 8 * (int64_t)num_sms() / bx);
+  int zc = (int)std::max<int64_t>(1, std::min<int64_t>(16, nz / want));
+  zc = std::max(zc, (nz + 65534) / 65535);
+  const dim3 grid((unsigned)bx, (unsigned)((nz + zc - 1) / zc));
+  return launch("tv3d_loss", vec ? k_tv3d<4> : k_tv3d<1>, grid, dim3(kThreads), 0,
+                (cudaStream_t)stream, d_vol, nx, ny, nz, zc, weight / (float)total, d_loss, d_grad,
                 accumulate);
 }
 

@@ -82,6 +82,23 @@ def test_tv3d(B):
     np.testing.assert_allclose(g, gw, rtol=1e-5, atol=1e-9)
 
 
+# rows of whole 16-byte vectors and others, planes smaller and larger than one CTA, row ends inside
+# a warp, one to many planes per thread, single rows and planes
+@pytest.mark.parametrize("shape", [(1, 1, 1), (1, 1, 4), (3, 1, 8), (1, 5, 3), (40, 9, 36),
+                                   (35, 130, 12), (70, 33, 127), (129, 64, 128)])
+@pytest.mark.parametrize("acc", [0, 1])
+def test_tv3d_shapes(B, shape, acc):
+    """Each gradient entry is a small whole number times one scale: one rounding (two when added
+    to what is there); the value is a sum of non-negative terms."""
+    rng = np.random.default_rng(sum(shape))
+    v = _x32(np.round(rng.random(shape) * 64) / 64)  # ties: sign(0) = 0
+    g0 = _x32(rng.standard_normal(shape) * 0.3 / v.size) if acc else None
+    val, g = _run_loss(B, "tv", v, None, weight=0.3, accumulate_into=g0)
+    want, gw = OL.value_and_grad(lambda a: 0.3 * OL.tv3d(a), v)
+    assert abs(val - want) <= 1e-5 * abs(want) + 1e-12
+    np.testing.assert_allclose(g, gw + (g0 if acc else 0), rtol=1e-6, atol=1e-6 * 0.3 / v.size)
+
+
 # (3, 37, 53) and (1, 5, 7) take the register-staged kernels (width not a multiple of 4, or
 # smaller than one box); the others the TMA-staged ones, (2, 45, 52) and (1, 70, 100) with
 # ragged tiles, (2, 512, 512) at the reconstruction step's detector size
