@@ -46,6 +46,59 @@ def test_brick_loss_matches_oracle(gsct):
     assert float((got - g).abs().max()) <= 2e-3 * scale, float((got - g).abs().max() / scale)
 
 
+# boxes inside the region, clipped by it and covering it; thin and rotated Gaussians
+@pytest.mark.parametrize("log_scale,spread,rot", [(-3.0, 0.0, 0.5), (0.0, 0.7, 1.0), (2.0, 0.2, 0.5),
+                                                  (3.0, 0.0, 0.0)])
+def test_brick_loss_boxes(gsct, log_scale, spread, rot):
+    """The rendering within 1e-3 of its peak (the quadratic form's FP32 terms reach about 2e3,
+    6 x 2^-24 of them is 7e-4 of the exponent) but for pairs at the cut (q within 0.01 of 9),
+    and the gradient as in the test above."""
+    B = gsct.binding
+    rng = np.random.default_rng(5)
+    nb = 3
+    raw = rng.standard_normal((nb, 32, 11)).astype(np.float32)
+    raw[..., 0:3] *= 2.0  # tanh towards the cell's corners
+    raw[..., 3:6] = log_scale + spread * raw[..., 3:6]
+    raw[..., 6:10] *= rot
+    tgt = rng.random((nb, 4096)).astype(np.float32)
+    y = torch.zeros((nb, 384), device="cuda")
+    y[:, :352] = torch.from_numpy(raw.reshape(nb, 352)).cuda()
+    loss, dy = torch.zeros(1, device="cuda"), torch.zeros((nb, 384), device="cuda")
+    out = torch.full((nb, 4096), float("nan"), device="cuda")
+    B.check(B.lib().gs_brick_loss(B.ptr(y), 384, B.ptr(torch.from_numpy(tgt).cuda()), nb,
+                                  B.ptr(loss), B.ptr(dy), 384, B.ptr(out),
+                                  torch.cuda.current_stream().cuda_stream), "brick_loss")
+    torch.cuda.synchronize()
+    rr = torch.from_numpy(raw.reshape(nb, 352).astype(np.float64)).requires_grad_(True)
+    c, s, q, rho = (x.detach() for x in OM.decode(rr.reshape(nb, 32, 11)))
+    ax = torch.arange(16, dtype=torch.float64) + 0.5
+    zz, yy, xx = torch.meshgrid(ax, ax, ax, indexing="ij")
+    d = torch.stack([xx, yy, zz], -1).reshape(1, 1, -1, 3) - c[:, :, None, :]
+    u = torch.einsum("ngva,ngab->ngvb", d, OM.quat_rot(q)) / s[:, :, None, :]
+    qf = (u * u).sum(-1)
+    edge = torch.where((qf - 9).abs() < 0.01, rho[:, :, None] * np.exp(-4.49), 0 * qf).sum(1)
+    want = torch.where(qf < 9, rho[:, :, None] * torch.exp(-0.5 * qf), 0 * qf).sum(1)
+    err = (out.cpu().double() - want).abs()
+    assert bool((err <= 1e-3 * want.max() + edge).all()), float(err.max())
+    (g,) = torch.autograd.grad(OM.brick_l1(rr, torch.from_numpy(tgt.astype(np.float64))), rr)
+    got = dy[:, :352].cpu().double()
+    assert float((got - g).abs().max()) <= 2e-3 * float(g.abs().max())
+
+
+# one row and column, parts of a 32-column group, rows that eight CTAs share unevenly
+@pytest.mark.parametrize("rows,cols", [(1, 1), (7, 33), (1000, 96), (4099, 384)])
+def test_colsum(gsct, rows, cols):
+    """At most rows / 256 additions per thread, then 5 + 3 levels: each rounds to 2^-24 of the sum
+    of magnitudes."""
+    B = gsct.binding
+    x = torch.from_numpy(np.random.default_rng(rows).standard_normal((rows, cols)).astype(np.float32))
+    out = torch.full((cols,), float("nan"), device="cuda")
+    B.check(B.lib().gs_colsum(B.ptr(x.cuda()), rows, cols, B.ptr(out),
+                              torch.cuda.current_stream().cuda_stream), "colsum")
+    tol = (rows / 256 + 9 + 8) * 2.0 ** -24 * x.double().abs().sum(0) + 1e-30
+    assert bool(((out.cpu().double() - x.double().sum(0)).abs() <= tol).all())
+
+
 def _mlp_ref(m):
     Ws = [w.detach().cpu().double() for w in m.W]
     bs = [b.detach().cpu().double() for b in m.b]
