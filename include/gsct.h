@@ -701,7 +701,7 @@ int gs_colsum(const float* d_g, int rows, int cols, float* d_out, void* stream);
 
 size_t gs_mlp_param_count(void);
 size_t gs_mlp_weight_count(void);
-/* Scratch bytes for batches of M bricks (activations, transposes, output gradients). */
+/* Scratch bytes for batches of M bricks (activations and output gradients). */
 size_t gs_mlp_workspace_size(int M);
 
 /* d_w16 = bf16(weights of d_params). */

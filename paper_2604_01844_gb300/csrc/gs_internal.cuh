@@ -117,6 +117,14 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
            float weight, float l1_weight, float* d_loss, float* d_grad, int accumulate,
            void* d_ws, size_t ws_bytes, void* stream);
 
+// gs_gemm_bf16 with either operand's storage and a ReLU mask (a bf16 array laid out like C whose
+// entries > 0 let the output pass).  GEMM_TN: A [M][K], B [N][K]; GEMM_BMN: A [M][K], B [K][N];
+// GEMM_MN: A [K][M], B [K][N].  The sizes are gs_gemm_bf16's (checked there).
+enum GemmForm { GEMM_TN, GEMM_BMN, GEMM_MN };
+int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm form,
+              const float* d_bias, int relu, const void* d_mask, float* d_c32, void* d_c16,
+              int ldc, int* d_err, cudaStream_t s);
+
 }  // namespace gs
 
 // ------------------------------------------------------------------------------------------

@@ -1,16 +1,17 @@
 // BF16 tensor-core GEMM for sm_103a (tcgen05 + TMEM + TMA), the dense layers of the per-brick
 // MLP initializer, and its helper kernels.
 //
-// gemm_tn:  C[M, N] = A[M, K] . B[N, K]^T (+ bias[N]) (ReLU), A and B bf16 row-major with K
-// contiguous ("K-major"), FP32 accumulation in tensor memory, outputs FP32 and/or BF16.
-// One CTA computes a 128 x BN tile with 128 threads, BN = 256 when N is a multiple of 256 and
-// the grid still covers the SMs (A is then streamed once for both halves), else 128:
-//   warp 0 / lane 0  TMA producer: 64-wide K slices of A and B (128-byte swizzle) into a
-//                    4-stage shared-memory ring guarded by mbarriers (full / empty);
+// gemm:  C[M, N] = A[M, K] . B[N, K]^T (+ bias[N]) (ReLU or a ReLU mask), A and B bf16, FP32
+// accumulation in tensor memory, outputs FP32 and/or BF16.  Each operand is stored either with K
+// contiguous ("K-major", rows of A or B) or with M or N contiguous ("MN-major", rows of K): the
+// backward's weight gradient g^T a and input gradient g W read g, a and W where the forward
+// left them, without transposed copies.  One CTA computes a 128 x BN tile with 128 threads:
+//   warp 0 / lane 0  TMA producer: 64-wide K slices of A and B (128-byte swizzle) into a ring of
+//                    shared-memory stages guarded by mbarriers (full / empty);
 //   warp 1 / lane 0  MMA issuer: 4 x tcgen05.mma (128 x BN x 16, kind::f16) per slice into a
 //                    BN-column TMEM accumulator; tcgen05.commit frees the slice;
-//   all 4 warps      epilogue: tcgen05.ld of their 32 TMEM lanes (rows), bias, ReLU, and each
-//                    lane's 32 consecutive outputs stored as 16-byte vectors (per element
+//   all 4 warps      epilogue: tcgen05.ld of their 32 TMEM lanes (rows), bias, ReLU or mask, and
+//                    each lane's 32 consecutive outputs stored as 16-byte vectors (per element
 //                    when the row stride is not a multiple of 8).
 // Every mbarrier wait is bounded; on timeout the kernel records GS_ERR_TIMEOUT in a status word,
 // stops issuing work, still releases its tensor memory, and returns.
@@ -18,6 +19,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -27,39 +29,55 @@
 namespace gs {
 namespace {
 
-constexpr int kBM = 128, kBN = 128, kBK = 64;  // kBN: the narrower tile (N % 128 == 0)
-constexpr int kStages = 4;
+constexpr int kBM = 128, kBN = 128, kBK = 64;  // kBN: every N is a multiple of it
 constexpr int kGemmThreads = 128;
 constexpr uint32_t kTileBytes = kBM * kBK * 2;  // 16 KiB per 128-row operand slice
-// Tile N = BN (128, or 256 when N allows): A slice 128 x 64, B slice BN x 64 per stage.
+// One 64 (MN) x 64 (K) box of an MN-major operand; boxes of a slice follow each other.
+constexpr uint32_t kBoxBytes = 64 * kBK * 2;
+// Tile N = BN: A slice 128 x 64, B slice BN x 64 per stage.  As many stages as fit one CTA per
+// SM (the ring hides the L2 latency of a slice; with four stages a 64-slice K loop on an idle
+// chip waits for it).
 template <int BN>
 struct GemmTile {
   static constexpr uint32_t kBBytes = BN * kBK * 2;
   static constexpr uint32_t kStageBytes = kTileBytes + kBBytes;
+  static constexpr int kStages = BN == 256 ? 4 : BN == 128 ? 6 : 8;
   static constexpr uint32_t kSmemBytes = kStages * kStageBytes + 1024 + 256;
-  // instruction descriptor of kind::f16: D f32, A/B bf16, both K-major, M = 128, N = BN
+  // instruction descriptor of kind::f16: D f32, A/B bf16, M = 128, N = BN; bits 15 and 16 set
+  // for an MN-major A or B
   static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                      ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
 };
-// shared-memory matrix descriptor: K-major tile of 128-byte rows with the 128-byte swizzle,
-// 8-row groups 1024 bytes apart
+// Shared-memory matrix descriptor of a slice with the 128-byte swizzle.  K-major: 128-byte rows
+// of K, 8-row groups 1024 bytes apart (the leading offset is unused).  MN-major: 128-byte rows of
+// MN, groups of 8 K rows 1024 bytes apart (stride offset), 64-wide MN boxes kBoxBytes apart
+// (leading offset).
+template <bool MN>
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);          // start address
-  d |= (uint64_t)1u << 16;                           // leading byte offset (unused when swizzled)
-  d |= (uint64_t)(1024u >> 4) << 32;                 // stride byte offset
-  d |= (uint64_t)1u << 46;                           // descriptor version
-  d |= (uint64_t)2u << 61;                           // 128-byte swizzle
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);                      // start address
+  d |= (uint64_t)(MN ? kBoxBytes >> 4 : 1u) << 16;              // leading byte offset
+  d |= (uint64_t)(1024u >> 4) << 32;                            // stride byte offset
+  d |= (uint64_t)1u << 46;                                      // descriptor version
+  d |= (uint64_t)2u << 61;                                      // 128-byte swizzle
   return d;
 }
 
-template <int BN>
+struct GemmOut {
+  const float* bias;
+  const __nv_bfloat16* mask;  // outputs whose entry is not > 0 become 0 (same ldc)
+  float* C32;
+  __nv_bfloat16* C16;
+  int ldc, relu, vec;
+};
+
+template <int BN, bool AMN, bool BMN>
 __global__ void __launch_bounds__(kGemmThreads)
-    k_gemm_tn(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              int M, int N, int K, const float* __restrict__ bias, int relu,
-              float* __restrict__ C32, __nv_bfloat16* __restrict__ C16, int ldc, int vec_out,
-              int* __restrict__ err) {
+    k_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+           int M, int N, int K, const GemmOut O, int* __restrict__ err) {
   using TT = GemmTile<BN>;
+  constexpr int kStages = TT::kStages;
+  static_assert(!BMN || BN % 64 == 0, "MN-major boxes are 64 wide");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
@@ -70,6 +88,10 @@ __global__ void __launch_bounds__(kGemmThreads)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
   const int ktiles = K / kBK;
+  const float* __restrict__ bias = O.bias;
+  float* __restrict__ C32 = O.C32;
+  __nv_bfloat16* __restrict__ C16 = O.C16;
+  const int ldc = O.ldc, relu = O.relu, vec_out = O.vec;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -102,8 +124,19 @@ __global__ void __launch_bounds__(kGemmThreads)
       }
       if (abort_flag) break;
       mbar_expect_tx(&full[s], TT::kStageBytes);
-      tma_load_2d(&tmA, &full[s], sA + s * kTileBytes, kt * kBK, m0);
-      tma_load_2d(&tmB, &full[s], sB + s * TT::kBBytes, kt * kBK, n0);
+      uint8_t *a = sA + s * kTileBytes, *bs = sB + s * TT::kBBytes;
+      if constexpr (AMN) {
+        for (int i = 0; i < kBM / 64; ++i)
+          tma_load_2d(&tmA, &full[s], a + i * kBoxBytes, m0 + 64 * i, kt * kBK);
+      } else {
+        tma_load_2d(&tmA, &full[s], a, kt * kBK, m0);
+      }
+      if constexpr (BMN) {
+        for (int i = 0; i < BN / 64; ++i)
+          tma_load_2d(&tmB, &full[s], bs + i * kBoxBytes, n0 + 64 * i, kt * kBK);
+      } else {
+        tma_load_2d(&tmB, &full[s], bs, kt * kBK, n0);
+      }
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
@@ -117,12 +150,14 @@ __global__ void __launch_bounds__(kGemmThreads)
       const uint32_t a0 = smem_u32(sA + s * kTileBytes), b0 = smem_u32(sB + s * TT::kBBytes);
 #pragma unroll
       for (int kk = 0; kk < kBK / 16; ++kk) {
-        const uint64_t ad = smem_desc(a0 + kk * 32), bd = smem_desc(b0 + kk * 32);
+        // 16 K: 32 bytes along a K-major row, two 8-row groups of an MN-major box
+        const uint64_t ad = smem_desc<AMN>(a0 + kk * (AMN ? 2048 : 32));
+        const uint64_t bd = smem_desc<BMN>(b0 + kk * (BMN ? 2048 : 32));
         const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
             " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(TT::kIdesc), "r"(acc));
+            "l"(ad), "l"(bd), "r"(TT::kIdesc | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u)), "r"(acc));
       }
       asm volatile(
           "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -172,6 +207,20 @@ __global__ void __launch_bounds__(kGemmThreads)
           if (bias) x += __ldg(bias + col0 + j);
           v[j] = relu ? fmaxf(x, 0.f) : x;
         }
+        if (O.mask) {
+          const uint4* q = reinterpret_cast<const uint4*>(O.mask + (size_t)row * ldc + col0);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint4 u = __ldg(q + j);
+            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[k]));
+              if (!(f.x > 0.f)) v[8 * j + 2 * k] = 0.f;
+              if (!(f.y > 0.f)) v[8 * j + 2 * k + 1] = 0.f;
+            }
+          }
+        }
         if (C32) {
           float4* o = reinterpret_cast<float4*>(C32 + (size_t)row * ldc + col0);
 #pragma unroll
@@ -199,6 +248,7 @@ __global__ void __launch_bounds__(kGemmThreads)
           if (col < N) {
             if (bias) v += bias[col];
             if (relu) v = fmaxf(v, 0.f);
+            if (O.mask && !(__bfloat162float(O.mask[(size_t)row * ldc + col]) > 0.f)) v = 0.f;
             if (C32) C32[(size_t)row * ldc + col] = v;
             if (C16) C16[(size_t)row * ldc + col] = __float2bfloat16_rn(v);
           }
@@ -216,7 +266,7 @@ __global__ void __launch_bounds__(kGemmThreads)
 // ------------------------------------------------------------------------------------------
 // tensor maps
 // ------------------------------------------------------------------------------------------
-// rows x cols bf16 row-major (cols contiguous), box kBK x box_rows with the 128-byte swizzle
+// rows x cols bf16 row-major (cols contiguous), box 64 x box_rows with the 128-byte swizzle
 int make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return GS_ERR_CUDA;
@@ -310,7 +360,62 @@ __global__ void __cluster_dims__(1, kColsumCtas, 1) __launch_bounds__(1024)
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+template <int BN, bool AMN, bool BMN>
+int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int K,
+                const GemmOut& o, int* err, cudaStream_t s) {
+  using TT = GemmTile<BN>;
+  int dev = 0;
+  GS_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return GS_ERR_ARG;
+  static std::atomic<bool> attr_set[64] = {};
+  if (!attr_set[dev]) {
+    GS_CUDA(cudaFuncSetAttribute(k_gemm<BN, AMN, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)TT::kSmemBytes));
+    attr_set[dev] = true;
+  }
+  return launch("gemm_bf16", k_gemm<BN, AMN, BMN>, dim3(N / BN, M / kBM), dim3(kGemmThreads),
+                TT::kSmemBytes, s, ma, mb, M, N, K, o, err);
+}
+
 }  // namespace
+
+int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm form,
+              const float* d_bias, int relu, const void* d_mask, float* d_c32, void* d_c16,
+              int ldc, int* d_err, cudaStream_t s) {
+  if (((uintptr_t)d_a & 15u) || ((uintptr_t)d_b & 15u)) return GS_ERR_ARG;
+  // 128 x 256 tiles when N allows (A read once per pair of 128-column tiles) and the grid
+  // still covers the SMs; narrower ones while the grid is under half of them (every tile shape
+  // adds the same products in the same order).  A training batch of 1024 bricks, whose layers
+  // make 16 to 64 tiles of 128 columns: forward and backward of the four layers 235 -> 145 us
+  // with the transposed copies gone.  MN-major operands come in 64-wide boxes, which
+  // also keeps their TMA coordinates 16-byte aligned.
+  const int rows = M / kBM, sms = num_sms();
+  int bn = N % 256 == 0 && (int64_t)(N / 256) * rows >= sms ? 256 : 128;
+  if (bn == 128 && 2 * (int64_t)(N / 128) * rows < sms) bn = 64;
+  if (bn == 64 && form == GEMM_TN && 2 * (int64_t)(N / 64) * rows < sms) bn = 32;
+  GemmOut o{d_bias, (const __nv_bfloat16*)d_mask, d_c32, (__nv_bfloat16*)d_c16, ldc, relu, 0};
+  o.vec = ldc % 8 == 0 && ((uintptr_t)d_c32 & 15u) == 0 && ((uintptr_t)d_c16 & 15u) == 0 &&
+          ((uintptr_t)d_mask & 15u) == 0;
+  CUtensorMap ma, mb;
+  GS_TRY(form == GEMM_MN ? make_map(&ma, d_a, K, M, kBK) : make_map(&ma, d_a, M, K, kBM));
+  GS_TRY(form == GEMM_TN ? make_map(&mb, d_b, N, K, bn) : make_map(&mb, d_b, K, N, kBK));
+  switch (form) {
+    case GEMM_TN:
+      if (bn == 256) return launch_gemm<256, false, false>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 128) return launch_gemm<128, false, false>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 64) return launch_gemm<64, false, false>(ma, mb, M, N, K, o, d_err, s);
+      return launch_gemm<32, false, false>(ma, mb, M, N, K, o, d_err, s);
+    case GEMM_BMN:
+      if (bn == 256) return launch_gemm<256, false, true>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 128) return launch_gemm<128, false, true>(ma, mb, M, N, K, o, d_err, s);
+      return launch_gemm<64, false, true>(ma, mb, M, N, K, o, d_err, s);
+    default:
+      if (bn == 256) return launch_gemm<256, true, true>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 128) return launch_gemm<128, true, true>(ma, mb, M, N, K, o, d_err, s);
+      return launch_gemm<64, true, true>(ma, mb, M, N, K, o, d_err, s);
+  }
+}
+
 }  // namespace gs
 
 using namespace gs;
@@ -322,37 +427,8 @@ int gs_gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, const fl
   if (!d_a || !d_b || !d_err || (!d_c32 && !d_c16)) return GS_ERR_ARG;
   if (M < 1 || N < 1 || K < kBK || K % kBK != 0 || M % kBM != 0 || N % kBN != 0 || ldc < N)
     return GS_ERR_ARG;
-  if (((uintptr_t)d_a & 15u) || ((uintptr_t)d_b & 15u)) return GS_ERR_ARG;
-  // 128 x 256 tiles when N allows (A read once per pair of 128-column tiles) and the grid
-  // still covers the SMs, else 128 x 128
-  const int bn = (N % 256 == 0 && (int64_t)(N / 256) * (M / kBM) >= num_sms()) ? 256 : kBN;
-  const int vec = (ldc % 8 == 0 && ((uintptr_t)d_c32 & 15u) == 0 && ((uintptr_t)d_c16 & 15u) == 0)
-                      ? 1 : 0;
-  CUtensorMap ma, mb;
-  GS_TRY(make_map(&ma, d_a, M, K, kBM));
-  GS_TRY(make_map(&mb, d_b, N, K, bn));
-  int dev = 0;
-  GS_CUDA(cudaGetDevice(&dev));
-  static bool attr_set[2][64] = {};
-  const int which = bn == 256 ? 1 : 0;
-  if (dev < 0 || dev >= 64) return GS_ERR_ARG;
-  if (!attr_set[which][dev]) {
-    if (bn == 256)
-      GS_CUDA(cudaFuncSetAttribute(k_gemm_tn<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)GemmTile<256>::kSmemBytes));
-    else
-      GS_CUDA(cudaFuncSetAttribute(k_gemm_tn<kBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)GemmTile<kBN>::kSmemBytes));
-    attr_set[which][dev] = true;
-  }
-  dim3 grid(N / bn, M / kBM);
-  if (bn == 256)
-    return launch("gemm_bf16", k_gemm_tn<256>, grid, dim3(kGemmThreads),
-                  GemmTile<256>::kSmemBytes, (cudaStream_t)stream, ma, mb, M, N, K, d_bias, relu,
-                  d_c32, (__nv_bfloat16*)d_c16, ldc, vec, d_err);
-  return launch("gemm_bf16", k_gemm_tn<kBN>, grid, dim3(kGemmThreads), GemmTile<kBN>::kSmemBytes,
-                (cudaStream_t)stream, ma, mb, M, N, K, d_bias, relu, d_c32,
-                (__nv_bfloat16*)d_c16, ldc, vec, d_err);
+  return gemm_bf16(d_a, d_b, M, N, K, GEMM_TN, d_bias, relu, nullptr, d_c32, d_c16, ldc, d_err,
+                   (cudaStream_t)stream);
 }
 
 int gs_f32_to_bf16(const float* d_x, void* d_y, int64_t n, void* stream) {

@@ -1,8 +1,8 @@
 // The per-brick MLP initializer as one network behind the C ABI: forward, backward, a whole
 // training step and inference over a flat parameter layout (gsct.h).  Every step is one of the
-// library's kernels (the tcgen05 GEMM, transposes, the ReLU mask, column sums, the fused
-// brick render + L1, Adam), issued here in the order of the network's layers; this file only
-// plans the workspace and sequences the launches on the caller's stream.
+// library's kernels (the tcgen05 GEMM, column sums, the fused brick render + L1, Adam), issued
+// here in the order of the network's layers; this file only plans the workspace and sequences
+// the launches on the caller's stream.
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -34,11 +34,8 @@ struct NetLayout {
   float* y = nullptr;                             // raw outputs, M x 384
   float* dy = nullptr;                            // dL/dy of the training step, M x 384
   uint16_t* g16_out = nullptr;                    // bf16(dL/dy), M x 384
-  uint16_t* gT[kLayers] = {};                     // (dL/d layer output)^T, out x M bf16
-  uint16_t* aT[kLayers] = {};                     // (layer input)^T, in x M bf16
-  uint16_t* WT[kLayers] = {};                     // W^T, in x out bf16 (layers 1..3)
-  float* gp[kLayers] = {};                        // dL/d layer input, M x in (layers 1..3)
-  uint16_t* g16[kLayers] = {};                    // its bf16 after the ReLU mask
+  float* gp[kLayers] = {};                        // dL/d layer input after the ReLU mask,
+  uint16_t* g16[kLayers] = {};                    // M x in, and its bf16 (layers 1..3)
   size_t bytes = 0;
 };
 
@@ -50,10 +47,7 @@ NetLayout carve_net(void* ws, int M) {
   L.dy = c.take<float>((size_t)M * kOutPad);
   L.g16_out = c.take<uint16_t>((size_t)M * kOutPad);
   for (int li = 0; li < kLayers; ++li) {
-    L.gT[li] = c.take<uint16_t>((size_t)layer_out(li) * M);
-    L.aT[li] = c.take<uint16_t>((size_t)layer_in(li) * M);
     if (li > 0) {
-      L.WT[li] = c.take<uint16_t>((size_t)layer_in(li) * layer_out(li));
       L.gp[li] = c.take<float>((size_t)M * layer_in(li));
       L.g16[li] = c.take<uint16_t>((size_t)M * layer_in(li));
     }
@@ -89,27 +83,25 @@ int forward(const float* params, const void* w16, const void* x16, int M, float*
 }
 
 // Backward from dL/dy through the four layers into grad (parameter layout): bias gradients
-// are column sums, weight gradients the TN GEMM of the transposed output gradient and layer
-// input (K = M), input gradients g W followed by the previous layer's ReLU mask.
+// are column sums, weight gradients g^T a (K = M) and input gradients g W with the previous
+// layer's ReLU mask in the epilogue.  The GEMM reads g, a and W as they are stored (MN-major
+// operands), so nothing is transposed in memory.
 int backward(const void* w16, const void* x16, int M, const float* dy, float* grad,
              const NetLayout& L, int* err, void* stream) {
   const void* acts[kLayers] = {x16, L.h[0], L.h[1], L.h[2]};
   const float* g32 = dy;
   const uint16_t* g16 = L.g16_out;
+  cudaStream_t s = (cudaStream_t)stream;
   GS_TRY(gs_f32_to_bf16(dy, L.g16_out, (int64_t)M * kOutPad, stream));
   int width = kOutPad;
   for (int li = kLayers - 1; li >= 0; --li) {
     const int k_in = layer_in(li);
     GS_TRY(gs_colsum(g32, M, width, grad + bias_offset(li), stream));
-    GS_TRY(gs_transpose_bf16(g16, M, width, L.gT[li], stream));
-    GS_TRY(gs_transpose_bf16(acts[li], M, k_in, L.aT[li], stream));
-    GS_TRY(gs_gemm_bf16(L.gT[li], L.aT[li], width, k_in, M, nullptr, 0,
-                        grad + weight_offset(li), nullptr, k_in, err, stream));
+    GS_TRY(gemm_bf16(g16, acts[li], width, k_in, M, GEMM_MN, nullptr, 0, nullptr,
+                     grad + weight_offset(li), nullptr, k_in, err, s));
     if (li == 0) break;
-    GS_TRY(gs_transpose_bf16(w16_of(w16, li), width, k_in, L.WT[li], stream));
-    GS_TRY(gs_gemm_bf16(g16, L.WT[li], M, k_in, width, nullptr, 0, L.gp[li], nullptr, k_in,
-                        err, stream));
-    GS_TRY(gs_relu_mask_bf16(L.gp[li], L.h[li - 1], (int64_t)M * k_in, L.g16[li], stream));
+    GS_TRY(gemm_bf16(g16, w16_of(w16, li), M, k_in, width, GEMM_BMN, nullptr, 0, L.h[li - 1],
+                     L.gp[li], L.g16[li], k_in, err, s));
     g32 = L.gp[li];
     g16 = L.g16[li];
     width = k_in;

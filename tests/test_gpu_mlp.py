@@ -248,6 +248,26 @@ def test_exported_train_step_equals_primitive_sequence(gsct):
     assert abs(float(la) - float(lb)) <= 1e-6 * abs(float(lb))
 
 
+def test_train_step_large_batch_equals_primitive_sequence(gsct):
+    """A batch whose GEMMs fill the SMs (128 x 256 tiles in every operand form) against the
+    primitive calls, which transpose their operands in memory: the same products in the same
+    order, so the gradients are equal bit for bit."""
+    from paper_2604_01844_gb300.mlp import BrickMLP
+
+    B = gsct.binding
+    M = 19456
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x16 = torch.rand(M, 4096, device="cuda", generator=g).to(torch.bfloat16)
+    t = 0.4 * torch.rand(M, 4096, device="cuda", generator=g)
+    a, b = BrickMLP(seed=5), BrickMLP(seed=5)
+    la, lb = torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda")
+    a.train_step(x16, t, la, lr=1e-3)
+    _primitive_train_step(B, b, x16, t, lb, 1e-3, M)
+    torch.cuda.synchronize()
+    assert int(a.err.item()) == 0 and int(b.err.item()) == 0
+    assert torch.equal(a.flat_grad, b.flat_grad)
+
+
 def test_infer_equals_forward_and_decode(gsct):
     from paper_2604_01844_gb300.mlp import BrickMLP
 
