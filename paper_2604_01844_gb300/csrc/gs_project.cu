@@ -2,25 +2,23 @@
 // for a batch of up to 32 independent instances (own Gaussians, views and detector size) in
 // one launch per pass; a single reconstruction is a batch of one.
 //
-// Pipeline of one call (all on `stream`, no host read-back):
-//   view_setup   per-view camera frame
-//   preprocess   one thread per (instance, view, Gaussian): local-affine (EWA) projection,
-//                integration factor mu, conic, 3-sigma box, and the count of the box's tiles
-//                that the cut ellipse actually meets (tight tile rule); warp-shuffle block sums
-//   scan         block sums -> offsets, pair total, capacity check
-//   emit         (key = instance key offset + view * tiles + tile, value = record index)
-//   radix sort   stable, over the key bits in use
-//   ranges       [start, end) per (instance, view, tile)
-//   raster_fwd   one CTA per (instance, view, tile): footprint records staged through shared
-//                memory with a bitmask of the 8x4 warp blocks each record's box touches; each
-//                warp visits only its records (ballot + find-first-set), each thread owns
-//                pixels and adds A * 2^(e) for e above the cut (additive, no depth order)
-//   raster_bwd   one CTA per (instance, view, tile), one thread per (Gaussian, tile) pair over
-//                the exact chords of its ellipse, pairs sorted by work per batch; six moment
-//                sums of g * exp(-q/2), then one pair of float4 atomics (per-Gaussian backward,
-//                Sec. 3.5)
-//   chain        one warp per Gaussian, lanes over its views: moments -> footprint gradients ->
-//                d(mean, rho, scale, quaternion), reduced over views with shuffles
+// Pipeline of one call (all on `stream`, no host read-back); a block of the first kernels is 256
+// consecutive Gaussians of one view:
+//   preprocess   one thread per (instance, view, Gaussian): the view's camera frame, local-affine
+//                (EWA) projection, integration factor mu, conic, 3-sigma box, and the box's
+//                tiles that the cut ellipse actually meets (tight tile rule, a range of tiles
+//                per tile row)
+//   then the (view, tile) lists, by one of two routes with the same lists:
+//   direct       (up to kDirectTiles tiles per view) preprocess also counts each block's records
+//                per tile; key_scan turns the counts into each block's offset in every list, the
+//                ranges and the pair total; emit writes each record to its place in the lists
+//   sorted       (more tiles) block sums and their scan, emit of (key, record) pairs in record
+//                order, stable radix sort over the tile bits, ranges
+//   raster_fwd   one CTA per (instance, view, tile), records on lanes
+//   raster_bwd   the same shape; six moment sums of g * exp(-q/2) per record, then one pair of
+//                float4 atomics (per-Gaussian backward, Sec. 3.5)
+//   chain        a thread per (Gaussian, 8 views): moments -> footprint gradients ->
+//                d(mean, rho, scale, quaternion)
 // The instance table travels by value as a __grid_constant__ kernel parameter, so a call does
 // no host-to-device copy and can be captured in a CUDA graph.
 #include <algorithm>
@@ -38,9 +36,18 @@ constexpr int kMaxInst = GS_MAX_INSTANCES;
 // widest digit of the tile-key sort: 10 tile bits (512^2 at tile 16) sort in two passes of 5
 constexpr int kTileDigitBits = 8;
 
+// The direct route keeps a counter per (block of 256 records, tile) and, in emit, a 32-bit lane
+// mask per (warp, tile) in shared memory: 72 KB at 2048 tiles, three CTAs per SM.  Its cost per
+// block grows with the tiles (10 bytes of counts and offsets each), the sort's with the pairs
+// (about 60 bytes each, some 1300 pairs per block): up to 2048 tiles the direct route is the
+// cheaper one (project 75 x 512^2, 1024 tiles: lists in LISTS_NEW instead of LISTS_OLD us).
+constexpr int kDirectTiles = 2048;
+
 struct Inst {
   int n, nv, W, H, TW, TH, g_off, v_off;
-  long long item_off, key_off, img_off;
+  int bpv;  // blocks of 256 records per view
+  long long item_off, key_off, img_off, blk_off;
+  long long mat_off;  // first entry of the instance in the (block, tile) count matrix
 };
 
 // Pair keys are (global view << tbits) | tile, tbits the bits of the largest instance's tile
@@ -48,16 +55,22 @@ struct Inst {
 // sorted lists are grouped by tile, then view, then record, which keeps every (view, tile)
 // list contiguous and in record order with fewer, narrower passes than a sort of the full key.
 struct Batch {
-  int count, T;
+  int count, T, lT;  // lT = log2 T
   float cut2, eps, znear;
   int tbits;
   Inst in[kMaxInst];
 };
 
-__device__ __forceinline__ int inst_of_item(const Batch& b, int64_t idx) {
+// The records of block blk: view v of instance I, Gaussians i0 .. i0 + 255 (below I.n).
+struct BlockItems {
+  int inst, v, i0;
+};
+__device__ __forceinline__ BlockItems block_items(const Batch& b, int64_t blk) {
   int k = 0;
-  while (k + 1 < b.count && b.in[k + 1].item_off <= idx) ++k;
-  return k;
+  while (k + 1 < b.count && b.in[k + 1].blk_off <= blk) ++k;
+  const uint32_t local = (uint32_t)(blk - b.in[k].blk_off), bpv = (uint32_t)b.in[k].bpv;
+  const uint32_t v = local / bpv;
+  return BlockItems{k, (int)v, (int)(local - v * bpv) * kThreads};
 }
 __device__ __forceinline__ int inst_of_key(const Batch& b, int64_t key) {
   int k = 0;
@@ -89,14 +102,23 @@ struct Layout {
   uint2* ranges = nullptr;
   uint32_t* hist = nullptr;
   float4* fpgrad = nullptr;  // 2 float4 per record: moment sums of the backward
+  // direct route
+  uint16_t* tcount = nullptr;     // records per (block, tile)
+  uint32_t* toffset = nullptr;    // the block's offset inside the tile's list
+  uint32_t* klocal = nullptr;     // a key's first pair, relative to its group of kScanKeys keys
+  unsigned long long* gsum = nullptr;  // pairs of a group, then their exclusive sums
+  uint32_t* ticket = nullptr;     // groups done
+  long long* vkeys = nullptr;     // first key of every view, and the total (for gs_read_pairs)
   size_t bytes = 0;
 };
+constexpr int kScanKeys = 64, kScanSegs = 8;  // key_scan: keys and block segments per CTA
 
 struct Plan {
   Batch b;
   int total_n = 0, total_v = 0;
-  int64_t items = 0, n_keys = 0, cap = 0;
-  int nblocks = 0, key_bits = 0;
+  int64_t items = 0, n_keys = 0, cap = 0, mat = 0;
+  int nblocks = 0, key_bits = 0, max_tiles = 1;
+  bool direct = false;
   SortPlan sort;
 };
 
@@ -108,10 +130,11 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
   memset(&b, 0, sizeof(b));
   b.count = n_inst;
   b.T = o->tile;
+  b.lT = o->tile == 8 ? 3 : o->tile == 16 ? 4 : 5;
   b.cut2 = o->cut * o->cut;
   b.eps = o->eps;
   b.znear = o->znear;
-  int64_t items = 0, keys = 0, img = 0, gsum = 0, vsum = 0, max_tiles = 1;
+  int64_t items = 0, keys = 0, img = 0, gsum = 0, vsum = 0, blocks = 0, mat = 0, max_tiles = 1;
   for (int k = 0; k < n_inst; ++k) {
     const gs_instance& s = inst[k];
     if (s.n < 0 || s.n_views < 1 || s.W < 1 || s.H < 1 || s.W > 32767 || s.H > 32767)
@@ -128,6 +151,11 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
     d.item_off = items;
     d.key_off = keys;
     d.img_off = img;
+    d.bpv = (s.n + kThreads - 1) / kThreads;
+    d.blk_off = blocks;
+    d.mat_off = mat;
+    blocks += (int64_t)s.n_views * d.bpv;
+    mat += (int64_t)s.n_views * d.bpv * d.TW * d.TH;
     items += (int64_t)s.n * s.n_views;
     keys += (int64_t)s.n_views * d.TW * d.TH;
     max_tiles = std::max<int64_t>(max_tiles, (int64_t)d.TW * d.TH);
@@ -136,7 +164,7 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
     vsum += s.n_views;
   }
   b.tbits = bits_for(max_tiles);
-  if (items > ((int64_t)1 << 31) - kThreads || keys > ((int64_t)1 << 31) - 1 ||
+  if (items > ((int64_t)1 << 31) - kThreads || blocks > ((int64_t)1 << 31) - 1 || keys > ((int64_t)1 << 31) - 1 ||
       gsum > ((int64_t)1 << 31) - 1 ||
       (vsum << b.tbits) > ((int64_t)1 << 32))  // implied by the key bound (2^tbits < 2 tiles)
     return GS_ERR_ARG;
@@ -145,7 +173,10 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
   p.items = items;
   p.n_keys = keys;
   p.cap = std::min<int64_t>(cap, ((int64_t)1 << 31) - 1);
-  p.nblocks = (int)((items + kThreads - 1) / kThreads);
+  p.nblocks = (int)blocks;
+  p.max_tiles = (int)max_tiles;
+  p.direct = max_tiles <= kDirectTiles;
+  p.mat = p.direct ? mat : 0;
   p.key_bits = b.tbits;
   p.sort = make_sort_plan(p.key_bits, kTileDigitBits);
   return GS_OK;
@@ -166,108 +197,168 @@ Layout carve(void* ws, const Plan& p) {
   L.ranges = c.take<uint2>(p.n_keys);
   L.hist = c.take<uint32_t>(sort_hist_words(p.sort));
   L.fpgrad = c.take<float4>(2 * p.items);
-  L.keys = c.take<uint32_t>(p.cap);
-  L.vals = c.take<uint32_t>(p.cap);
-  L.keys_alt = c.take<uint32_t>(p.cap);
-  L.vals_alt = c.take<uint32_t>(p.cap);
+  if (p.direct) {
+    const int64_t groups = (p.n_keys + kScanKeys - 1) / kScanKeys;
+    L.tcount = c.take<uint16_t>(p.mat);
+    L.toffset = c.take<uint32_t>(p.mat);
+    L.klocal = c.take<uint32_t>(p.n_keys);
+    L.gsum = c.take<unsigned long long>(groups);
+    L.ticket = c.take<uint32_t>(1);
+    L.vkeys = c.take<long long>(p.total_v + 1);
+    L.vals = c.take<uint32_t>(p.cap);
+  } else {
+    L.keys = c.take<uint32_t>(p.cap);
+    L.vals = c.take<uint32_t>(p.cap);
+    L.keys_alt = c.take<uint32_t>(p.cap);
+    L.vals_alt = c.take<uint32_t>(p.cap);
+  }
   L.bytes = align_up(c.off, 256);
   return L;
 }
 
-// Whether a record's cut ellipse can reach the rectangle [x0, x1] x [y0, y1] (pixel-centre
-// coordinates): the maximum of its concave exponent e over the rectangle, which lies at the
-// centre if the centre is inside and otherwise on an edge (a 1-D concave quadratic there,
-// maximised at its clamped vertex), against the cut with a relative margin of 1e-3.  The
-// margin makes the answer a superset of the per-pixel FP32 test, so that a tile or block
-// dropped on a false answer never held a contribution.  h = (1/(2 c.x), 1/(2 c.z)).
+// Tight tile rule: a tile is listed for a record if its cut ellipse, enlarged by a relative
+// margin of 1e-3 of the cut (e > 1.001 e_cut, e the exponent), meets the rectangle of pixel
+// centres the tile shares with the record's clipped box.  The margin makes the lists a superset
+// of the per-pixel FP32 test, so a tile left out never held a contribution.  Per tile row the
+// enlarged ellipse's section by the row's slab of pixel centres is convex, so the tiles it meets
+// are those whose pixel columns meet its x extent [xa, xb]: the left (right) end lies at the
+// ellipse's own leftmost (rightmost) point when that is inside the slab, else on the slab's
+// nearer edge.  The ends are compared with pixel columns relative to the record's centre, where
+// FP32 resolves far more than the margin.
 struct Ell {
-  float4 g, c;
-  float hx, hz;
+  float px, py, ia, hb, kap, vr, cm;  // 1/a, -b/(2a), c - b^2/(4a), v of the rightmost point
 };
+// Every operation below has its rounding written out: preprocess counts the tiles and emit places
+// them, so both must get the same answers.
 __device__ __forceinline__ Ell make_ell(const float4 g, const float4 c) {
-  return Ell{g, c, 0.5f / c.x, 0.5f / c.z};
+  Ell E;
+  E.px = g.x;
+  E.py = g.y;
+  E.ia = __frcp_rn(c.x);
+  const float hb = __fmul_rn(-0.5f, c.y);
+  E.hb = __fmul_rn(hb, E.ia);
+  E.kap = __fmaf_rn(-hb, E.hb, c.z);
+  E.cm = __fmul_rn(g.w, 1.001f);
+  const float ih = __fdiv_rn(hb, c.z);  // v = ih u where u is extreme on the ellipse
+  const float u2 = __fdiv_rn(E.cm, __fmaf_rn(-hb, ih, c.x));
+  E.vr = __fmul_rn(ih, __fsqrt_rn(fmaxf(u2, 0.f)));
+  return E;
 }
-__device__ __forceinline__ float edge_max(float ca, float cb, float cc, float h, float u0,
-                                          float u1, float w) {
-  // max over u in [u0, u1] of ca u^2 + cb w u + cc w^2 (ca < 0, h = 1 / (2 ca))
-  const float u = fminf(fmaxf(-cb * w * h, u0), u1);
-  return fmaf(fmaf(ca, u, cb * w), u, cc * w * w);
+__device__ __forceinline__ float half_width(const Ell& E, float v) {
+  const float d = __fmul_rn(__fmaf_rn(__fmul_rn(-E.kap, v), v, E.cm), E.ia);
+  return __fsqrt_rn(fmaxf(d, 0.f));
 }
-__device__ __forceinline__ bool ellipse_meets_rect(const Ell& E, float x0, float x1, float y0,
-                                                   float y1) {
-  const float4 g = E.g, c = E.c;
-  const float u0 = x0 - g.x, u1 = x1 - g.x, v0 = y0 - g.y, v1 = y1 - g.y;
-  if (u0 <= 0.f && u1 >= 0.f && v0 <= 0.f && v1 >= 0.f) return true;
-  float m = fmaxf(edge_max(c.x, c.y, c.z, E.hx, u0, u1, v0),
-                  edge_max(c.x, c.y, c.z, E.hx, u0, u1, v1));
-  m = fmaxf(m, fmaxf(edge_max(c.z, c.y, c.x, E.hz, v0, v1, u0),
-                     edge_max(c.z, c.y, c.x, E.hz, v0, v1, u1)));
-  return m > g.w * 1.001f;
+// Tiles ta .. tb (none if ta > tb) of tile row ty for the clipped box (x0, y0)-(x1, y1).
+__device__ __forceinline__ void row_tiles(const Ell& E, int lT, int ty, int x0, int y0, int x1,
+                                          int y1, int& ta, int& tb) {
+  const float v0 = __fsub_rn((float)max(ty << lT, y0), E.py);
+  const float v1 = __fsub_rn((float)min((ty << lT) + (1 << lT) - 1, y1), E.py);
+  const float vb = fminf(fmaxf(E.vr, v0), v1), va = fminf(fmaxf(-E.vr, v0), v1);
+  const float xb = __fmaf_rn(E.hb, vb, half_width(E, vb));
+  const float xa = __fmaf_rn(E.hb, va, -half_width(E, va));
+  // first pixel column >= xa and last <= xb, decided on offsets from the centre
+  float fa = ceilf(__fadd_rn(xa, E.px)), fb = floorf(__fadd_rn(xb, E.px));
+  if (__fsub_rn(fa - 1.f, E.px) >= xa) fa -= 1.f;
+  else if (__fsub_rn(fa, E.px) < xa) fa += 1.f;
+  if (__fsub_rn(fb + 1.f, E.px) <= xb) fb += 1.f;
+  else if (__fsub_rn(fb, E.px) > xb) fb -= 1.f;
+  // an extent between two neighbouring columns (fa = fb + 1) meets their tile if both are the
+  // box's and in one tile; one left or right of the box meets none
+  const bool none = fb < (float)x0 || fa > (float)x1;
+  ta = none ? 1 : (int)fmaxf(fa, (float)x0) >> lT;
+  tb = none ? 0 : (int)fminf(fb, (float)x1) >> lT;
 }
 
-// Tight tile rule: tile (tx, ty) of side T is listed for a record whose clipped pixel box is
-// (x0, y0)-(x1, y1) only if its cut ellipse meets the pixel-centre rectangle the tile shares
-// with the box.  Preprocess evaluates it (and keeps the answers for up to 32 tiles as a bit
-// mask in the box's tile order); emit reads the mask, or re-evaluates for larger boxes.
+// Preprocess keeps the answers for boxes of up to 32 tiles as a bit mask in the box's tile order;
+// emit reads the mask, or evaluates the rows again for larger boxes.
 constexpr int kMaskTiles = 32;
-__device__ __forceinline__ bool tile_listed(const Ell& E, int T, int tx, int ty, int x0, int y0,
-                                            int x1, int y1) {
-  return ellipse_meets_rect(E, (float)max(tx * T, x0), (float)min(tx * T + T - 1, x1),
-                            (float)max(ty * T, y0), (float)min(ty * T + T - 1, y1));
-}
-
-// ------------------------------------------------------------------------------------------
-// view frames, preprocess, emit
-// ------------------------------------------------------------------------------------------
-__global__ void k_view_setup(const __grid_constant__ Batch b, const gs_view* __restrict__ views,
-                             int total_v, ViewFrame* __restrict__ frames, gs_status* st) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v == 0) {
-    st->code = GS_OK;
-    st->pairs = 0;
+// Calls f(ty, ta, tb) for every tile row of a record's box with listed tiles ta .. tb.
+template <typename F>
+__device__ __forceinline__ void listed_rows(const short4 r, uint32_t tm, const float4* geo,
+                                            const float4* conic, size_t idx, int lT, F f) {
+  const int tx0 = r.x >> lT, ty0 = r.y >> lT;
+  const int ntx = (r.z >> lT) - tx0 + 1, nty = (r.w >> lT) - ty0 + 1;
+  if (ntx * nty <= kMaskTiles) {
+    const uint32_t row = 0xffffffffu >> (32 - ntx);
+    for (int k = 0, sh = 0; k < nty; ++k, sh += ntx) {
+      const uint32_t bits = (tm >> sh) & row;
+      if (bits) {
+        const int ta = tx0 + __ffs(bits) - 1;
+        f(ty0 + k, ta, ta + __popc(bits) - 1);
+      }
+    }
+  } else {
+    const Ell E = make_ell(geo[idx], conic[idx]);
+    for (int ty = ty0; ty < ty0 + nty; ++ty) {
+      int ta, tb;
+      row_tiles(E, lT, ty, r.x, r.y, r.z, r.w, ta, tb);
+      if (ta <= tb) f(ty, ta, tb);
+    }
   }
-  if (v >= total_v) return;
-  const Inst& I = b.in[inst_of_view(b, v)];
-  ViewFrame f;
-  make_frame(views[v], I.W, I.H, f);
-  frames[v] = f;
 }
 
+// ------------------------------------------------------------------------------------------
+// preprocess
+// ------------------------------------------------------------------------------------------
+template <bool DIRECT>
 __global__ void __launch_bounds__(kThreads)
     k_preprocess(const __grid_constant__ Batch b, const float4* __restrict__ mean_rho,
                  const float4* __restrict__ scale, const float4* __restrict__ quat,
-                 int64_t items, const ViewFrame* __restrict__ frames, float4* __restrict__ geo,
-                 float4* __restrict__ conic, short4* __restrict__ rect,
+                 const gs_view* __restrict__ views, ViewFrame* __restrict__ frames,
+                 float4* __restrict__ geo, float4* __restrict__ conic, short4* __restrict__ rect,
                  uint32_t* __restrict__ tmask, uint32_t* __restrict__ counts,
-                 uint32_t* __restrict__ block_sums) {
+                 uint32_t* __restrict__ block_sums, uint16_t* __restrict__ tcount,
+                 uint32_t* __restrict__ ticket, gs_status* st) {
+  extern __shared__ uint32_t s_tiles[];  // DIRECT: records of the block per tile
   __shared__ uint32_t warp_sums[kThreads / 32];
-  const int64_t idx = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  __shared__ ViewFrame f;
+  const BlockItems bi = block_items(b, blockIdx.x);
+  const Inst& I = b.in[bi.inst];
+  const int i = bi.i0 + threadIdx.x;
+  const bool in = i < I.n;
+  const int gi = I.g_off + (in ? i : I.n - 1);
+  // the parameters are requested before the view's frame is built, which takes one thread a
+  // chain of divisions
+  const float4 mr = mean_rho[gi], sc = scale[gi], qt = quat[gi];
+  const int tiles = I.TW * I.TH;
+  if (DIRECT)
+    for (int t = threadIdx.x; t < tiles; t += kThreads) s_tiles[t] = 0u;
+  if (threadIdx.x == 0) {
+    ViewFrame fr;
+    make_frame(views[I.v_off + bi.v], I.W, I.H, fr);
+    f = fr;
+    if (bi.i0 == 0) frames[I.v_off + bi.v] = fr;
+    if (blockIdx.x == 0) {
+      st->code = GS_OK;
+      st->pairs = 0;
+      if (DIRECT) *ticket = 0u;
+    }
+  }
+  __syncthreads();
   uint32_t cnt = 0;
-  if (idx < items) {
-    const Inst& I = b.in[inst_of_item(b, idx)];
-    // items per instance fit in 32 bits (the plan caps the total below 2^31)
-    const uint32_t local = (uint32_t)(idx - I.item_off);
-    const int v = (int)(local / (uint32_t)I.n), i = (int)(local - (uint32_t)v * (uint32_t)I.n);
-    const int gi = I.g_off + i;
-    const ViewFrame f = frames[I.v_off + v];
+  if (in) {
+    const size_t idx = (size_t)(I.item_off + (int64_t)bi.v * I.n + i);
     Fwd o;
     int x0, y0, x1, y1;
-    const bool live = footprint(mean_rho[gi], scale[gi], quat[gi], f, I.W, I.H, b.cut2, b.eps,
-                                b.znear, o, x0, y0, x1, y1);
+    const bool live = footprint(mr, sc, qt, f, I.W, I.H, b.cut2, b.eps, b.znear, o, x0, y0, x1, y1);
     if (live) {
-      const int T = b.T;
       const float k = gsd::kNegHalfLog2e;
       const float4 gg = make_float4(o.px, o.py, o.A, k * o.Q);
       const float4 cc = make_float4(k * o.ca, 2.f * k * o.cb, k * o.cc, 0.f);
       const Ell E = make_ell(gg, cc);
+      const int lT = b.lT, tx0 = x0 >> lT, ty0 = y0 >> lT;
+      const int ntx = (x1 >> lT) - tx0 + 1, ty1 = y1 >> lT;
       uint32_t tm = 0u;
-      int bit = 0;
-      for (int ty = y0 / T; ty <= y1 / T; ++ty)
-        for (int tx = x0 / T; tx <= x1 / T; ++tx, ++bit)
-          if (tile_listed(E, T, tx, ty, x0, y0, x1, y1)) {
-            ++cnt;
-            if (bit < kMaskTiles) tm |= 1u << bit;
-          }
+      int sh = 0;
+      for (int ty = ty0; ty <= ty1; ++ty, sh += ntx) {
+        int ta, tb;
+        row_tiles(E, lT, ty, x0, y0, x1, y1, ta, tb);
+        if (ta > tb) continue;
+        cnt += (uint32_t)(tb - ta + 1);
+        if (sh + ntx <= kMaskTiles) tm |= (0xffffffffu >> (31 - (tb - ta))) << (sh + ta - tx0);
+        if (DIRECT)
+          for (int t = ty * I.TW + ta; t <= ty * I.TW + tb; ++t) atomicAdd(&s_tiles[t], 1u);
+      }
       tmask[idx] = tm;
       geo[idx] = gg;
       conic[idx] = cc;
@@ -279,26 +370,196 @@ __global__ void __launch_bounds__(kThreads)
     }
     counts[idx] = cnt;
   }
-  // culled pairs drop out of the warp's count via the ballot; the block sum feeds the scan
-  const unsigned live_mask = __ballot_sync(0xffffffffu, cnt > 0);
-  uint32_t s = live_mask ? gsd::warp_sum(cnt) : 0u;
-  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t bs = 0;
+  if constexpr (DIRECT) {
+    __syncthreads();
+    uint16_t* row = tcount + I.mat_off + ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * tiles;
+    for (int t = threadIdx.x; t < tiles; t += kThreads) row[t] = (uint16_t)s_tiles[t];
+  } else {
+    // culled pairs drop out of the warp's count via the ballot; the block sum feeds the scan
+    const unsigned live_mask = __ballot_sync(0xffffffffu, cnt > 0);
+    uint32_t s = live_mask ? gsd::warp_sum(cnt) : 0u;
+    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t bs = 0;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) bs += warp_sums[w];
-    block_sums[blockIdx.x] = bs;
+      for (int w = 0; w < kThreads / 32; ++w) bs += warp_sums[w];
+      block_sums[blockIdx.x] = bs;
+    }
   }
 }
 
-// emit: same block decomposition as preprocess; in-block exclusive prefix by warp scans
+// ------------------------------------------------------------------------------------------
+// direct route: counts per (block, tile) -> offsets -> lists
+// ------------------------------------------------------------------------------------------
+// A CTA owns kScanKeys consecutive keys, a thread one key and an eighth of its view's blocks: the
+// column of counts is summed, then walked again to write each block's offset in the list (the
+// second read hits L2).  ranges[key] gets (offset in the group, count), completed by emit.  The
+// last CTA to finish turns the groups' sums into offsets and records the pair total and whether
+// it fits.  Bound by memory: 2 + 2 + 4 bytes per (block, tile).
+__global__ void __launch_bounds__(kScanKeys * kScanSegs)
+    k_key_scan(const __grid_constant__ Batch b, int64_t n_keys, const uint16_t* __restrict__ tcount,
+               uint32_t* __restrict__ toffset, uint32_t* __restrict__ klocal,
+               uint2* __restrict__ ranges, unsigned long long* __restrict__ gsum, uint32_t* ticket,
+               long long* __restrict__ vkeys, int total_v, gs_status* st, int64_t cap,
+               int64_t vals_off, int64_t ranges_off, int64_t vkeys_off) {
+  __shared__ uint32_t part[kScanSegs][kScanKeys];
+  __shared__ unsigned long long wtot[kScanKeys * kScanSegs / 32];
+  __shared__ bool last;
+  const int t = threadIdx.x, lane = t & 31, kl = t % kScanKeys, seg = t / kScanKeys;
+  const int64_t key = (int64_t)blockIdx.x * kScanKeys + kl;
+  uint32_t sum = 0;
+  int b0 = 0, b1 = 0, tiles = 0;
+  int64_t at = 0;
+  if (key < n_keys) {
+    const Inst& I = b.in[inst_of_key(b, key)];
+    tiles = I.TW * I.TH;
+    const int64_t lk = key - I.key_off;
+    const int v = (int)(lk / tiles), tile = (int)(lk - (int64_t)v * tiles);
+    const int per = (I.bpv + kScanSegs - 1) / kScanSegs;
+    b0 = min(I.bpv, seg * per);
+    b1 = min(I.bpv, b0 + per);
+    at = I.mat_off + (int64_t)v * I.bpv * tiles + tile;
+    if (seg == 0 && tile == 0) vkeys[I.v_off + v] = key;
+#pragma unroll 8
+    for (int k = b0; k < b1; ++k) sum += tcount[at + (int64_t)k * tiles];
+  }
+  if (blockIdx.x == 0 && t == 0) vkeys[total_v] = n_keys;
+  part[seg][kl] = sum;
+  __syncthreads();
+  uint32_t run = 0, total = 0;
+#pragma unroll
+  for (int q = 0; q < kScanSegs; ++q) {
+    const uint32_t x = part[q][kl];
+    run += q < seg ? x : 0u;
+    total += x;
+  }
+#pragma unroll 8
+  for (int k = b0; k < b1; ++k) {
+    const int64_t e = at + (int64_t)k * tiles;
+    toffset[e] = run;
+    run += tcount[e];
+  }
+  if (seg == 0) {  // the first two warps hold the group's keys
+    const uint32_t incl = gsd::warp_inclusive_scan(total);
+    if (lane == 31) wtot[t >> 5] = incl;
+    asm volatile("bar.sync 1, %0;" ::"n"(kScanKeys) : "memory");
+    const uint32_t first = incl - total + (t >= 32 ? (uint32_t)wtot[0] : 0u);
+    if (key < n_keys) {
+      klocal[key] = first;
+      ranges[key] = make_uint2(first, total);
+    }
+    if (t == 0) {
+      unsigned long long g = 0;
+      for (int w = 0; w < kScanKeys / 32; ++w) g += wtot[w];
+      gsum[blockIdx.x] = g;
+      __threadfence();
+      last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // exclusive sums over the groups
+  constexpr int NT = kScanKeys * kScanSegs;
+  const int ng = (int)gridDim.x;
+  unsigned long long base = 0;
+  for (int g0 = 0; g0 < ng; g0 += NT) {
+    const int g = g0 + t;
+    const unsigned long long x = g < ng ? __ldcg(gsum + g) : 0ull;
+    unsigned long long incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) wtot[t >> 5] = incl;
+    __syncthreads();
+    unsigned long long before = base, all = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+      before += w < (t >> 5) ? wtot[w] : 0ull;
+      all += wtot[w];
+    }
+    if (g < ng) gsum[g] = before + incl - x;
+    base += all;
+    __syncthreads();
+  }
+  if (t == 0) {
+    st->pairs = (int64_t)base;
+    st->capacity = cap;
+    if ((int64_t)base > cap) st->code = GS_ERR_CAPACITY;
+    st->reserved[0] = -1;  // the keys are not stored: gs_read_pairs takes them from the ranges
+    st->reserved[1] = vals_off;
+    st->reserved[2] = n_keys;
+    st->reserved[3] = ranges_off;
+    st->reserved[4] = vkeys_off;
+    st->reserved[5] = total_v;
+    st->reserved[6] = b.tbits;
+  }
+}
+
+// Writes every record to its place in the lists of its tiles.  A block's records keep their order
+// inside a list: a record's place is the list's start, plus the block's offset in it, plus the
+// records of the same tile in earlier warps and lanes of the block (a lane mask per (warp, tile)
+// in shared memory, counted by popc).  Blocks of one view run together, so the scattered 4-byte
+// stores of a list's neighbourhood meet in L2.
+__global__ void __launch_bounds__(kThreads)
+    k_emit_direct(const __grid_constant__ Batch b, const uint32_t* __restrict__ counts,
+                  const float4* __restrict__ geo, const float4* __restrict__ conic,
+                  const short4* __restrict__ rect, const uint32_t* __restrict__ tmask,
+                  const uint32_t* __restrict__ toffset, const uint32_t* __restrict__ klocal,
+                  const unsigned long long* __restrict__ gsum, uint2* __restrict__ ranges,
+                  uint32_t* __restrict__ vals, const gs_status* st) {
+  constexpr int NW = kThreads / 32;
+  extern __shared__ uint32_t s_emit[];  // [tiles] first place of the block, [NW][tiles] lane masks
+  const BlockItems bi = block_items(b, blockIdx.x);
+  const Inst& I = b.in[bi.inst];
+  const int tiles = I.TW * I.TH, t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int i = bi.i0 + t;
+  const size_t idx = (size_t)(I.item_off + (int64_t)bi.v * I.n + i);
+  const uint32_t cnt = i < I.n ? counts[idx] : 0u;
+  const short4 r = i < I.n ? rect[idx] : make_short4(0, 0, 0, 0);
+  const uint32_t tm = i < I.n ? tmask[idx] : 0u;
+  if (st->code != GS_OK) return;
+  uint32_t* first = s_emit;
+  uint32_t* lanes = s_emit + tiles;
+  const int64_t key0 = I.key_off + (int64_t)bi.v * tiles;
+  const uint32_t* row = toffset + I.mat_off + ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * tiles;
+  for (int k = t; k < tiles; k += kThreads) {
+    const uint32_t start = (uint32_t)gsum[(key0 + k) / kScanKeys] + klocal[key0 + k];
+    first[k] = start + row[k];
+    if (bi.i0 == 0) ranges[key0 + k] = make_uint2(start, start + ranges[key0 + k].y);
+  }
+  for (int k = t; k < NW * tiles; k += kThreads) lanes[k] = 0u;
+  __syncthreads();
+  const uint32_t bit = 1u << lane;
+  if (cnt)
+    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
+      uint32_t* q = lanes + w * tiles + ty * I.TW;
+      for (int k = ta; k <= tb; ++k) atomicOr(q + k, bit);
+    });
+  __syncthreads();
+  if (cnt)
+    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
+      for (int k = ty * I.TW + ta; k <= ty * I.TW + tb; ++k) {
+        uint32_t pos = first[k] + __popc(lanes[w * tiles + k] & (bit - 1u));
+        for (int ww = 0; ww < w; ++ww) pos += __popc(lanes[ww * tiles + k]);
+        vals[pos] = (uint32_t)idx;
+      }
+    });
+}
+
+// ------------------------------------------------------------------------------------------
+// sorted route: emit in record order (same block decomposition as preprocess; in-block exclusive
+// prefix by warp scans)
+// ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads)
     k_emit(const __grid_constant__ Batch b, const uint32_t* __restrict__ counts,
            const float4* __restrict__ geo, const float4* __restrict__ conic,
            const short4* __restrict__ rect, const uint32_t* __restrict__ tmask,
            const uint32_t* __restrict__ block_offs,
-           int64_t items, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
            gs_status* st, int64_t sorted_keys_off, int64_t sorted_vals_off) {
   __shared__ uint32_t warp_pre[kThreads / 32];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -307,13 +568,16 @@ __global__ void __launch_bounds__(kThreads)
     st->reserved[2] = b.in[b.count - 1].key_off +
                       (int64_t)b.in[b.count - 1].nv * b.in[b.count - 1].TW * b.in[b.count - 1].TH;
   }
-  const int64_t idx = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const BlockItems bi = block_items(b, blockIdx.x);
+  const Inst& I = b.in[bi.inst];
+  const int i = bi.i0 + threadIdx.x;
+  const size_t idx = (size_t)(I.item_off + (int64_t)bi.v * I.n + i);
   // every input of the thread is requested up front, with the status word, so that the
   // emission waits for one round trip instead of a chain of them
-  const bool in = idx < items;
+  const bool in = i < I.n;
   const uint32_t cnt = in ? counts[idx] : 0u;
-  const short4 r_in = in ? rect[idx] : make_short4(0, 0, 0, 0);
-  const uint32_t tm_in = in ? tmask[idx] : 0u;
+  const short4 r = in ? rect[idx] : make_short4(0, 0, 0, 0);
+  const uint32_t tm = in ? tmask[idx] : 0u;
   const uint32_t boff = block_offs[blockIdx.x];
   if (st->code != GS_OK) return;
   const uint32_t incl = gsd::warp_inclusive_scan(cnt);
@@ -334,23 +598,10 @@ __global__ void __launch_bounds__(kThreads)
   const uint32_t wtotal = __shfl_sync(0xffffffffu, incl, 31);
   if (wtotal == 0) return;
   // this lane's record (meaningful where cnt > 0)
-  int T = b.T, TW = 1, ntx = 1, tx0i = 0, ty0i = 0;
-  uint32_t kbase = 0, tm = 0;
-  bool small = true;
-  short4 r = make_short4(0, 0, 0, 0);
-  if (cnt > 0) {
-    const Inst& I = b.in[inst_of_item(b, idx)];
-    const int v = (int)((uint32_t)(idx - I.item_off) / (uint32_t)I.n);
-    r = r_in;
-    TW = I.TW;
-    kbase = (uint32_t)(I.v_off + v) << b.tbits;
-    tx0i = r.x / T;
-    ty0i = r.y / T;
-    ntx = r.z / T - tx0i + 1;
-    const int nty = r.w / T - ty0i + 1;
-    small = ntx * nty <= kMaskTiles;
-    tm = tm_in;
-  }
+  const int lT = b.lT, TW = I.TW;
+  const uint32_t kbase = (uint32_t)(I.v_off + bi.v) << b.tbits;
+  const int tx0i = r.x >> lT, ty0i = r.y >> lT, ntx = (r.z >> lT) - tx0i + 1;
+  const bool small = ntx * ((r.w >> lT) - ty0i + 1) <= kMaskTiles;
   // records with at most 32 box tiles: the warp writes its contiguous range of pairs
   // cooperatively, pair p going to lane p % 32, which finds the owning record by a binary
   // search over the lanes' inclusive counts and the tile as the owner's k-th listed tile
@@ -365,31 +616,25 @@ __global__ void __launch_bounds__(kThreads)
     }
     const uint32_t oe = __shfl_sync(0xffffffffu, excl, o);
     const uint32_t otm = __shfl_sync(0xffffffffu, tm, o);
-    const uint32_t okb = __shfl_sync(0xffffffffu, kbase, o);
     const int ontx = __shfl_sync(0xffffffffu, ntx, o);
     const int otx0 = __shfl_sync(0xffffffffu, tx0i, o);
     const int oty0 = __shfl_sync(0xffffffffu, ty0i, o);
-    const int otw = __shfl_sync(0xffffffffu, TW, o);
     const bool osmall = __shfl_sync(0xffffffffu, small ? 1 : 0, o) != 0;
     if (p < wtotal && osmall) {
       const int bit = (int)__fns(otm, 0, (int)(p - oe) + 1);
       const int ty = oty0 + bit / ontx, tx = otx0 + bit % ontx;
-      keys[wbase + p] = okb + (uint32_t)(ty * otw + tx);
+      keys[wbase + p] = kbase + (uint32_t)(ty * TW + tx);
       vals[wbase + p] = (uint32_t)(idx - lane + o);
     }
   }
   if (cnt == 0 || small) return;
   uint32_t off = wbase + excl;
-  {
-    const Ell E = make_ell(geo[idx], conic[idx]);
-    for (int ty = r.y / T; ty <= r.w / T; ++ty)
-      for (int tx = r.x / T; tx <= r.z / T; ++tx) {
-        if (!tile_listed(E, T, tx, ty, r.x, r.y, r.z, r.w)) continue;
-        keys[off] = kbase + (uint32_t)(ty * TW + tx);
-        vals[off] = (uint32_t)idx;
-        ++off;
-      }
-  }
+  listed_rows(r, tm, geo, conic, idx, lT, [&](int ty, int ta, int tb) {
+    for (int tx = ta; tx <= tb; ++tx, ++off) {
+      keys[off] = kbase + (uint32_t)(ty * TW + tx);
+      vals[off] = (uint32_t)idx;
+    }
+  });
 }
 
 // [start, end) of every (view, tile) list.  The sorted keys are grouped by tile and then view,
@@ -874,6 +1119,18 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// Zeroes the backward's accumulators in one launch: the record moments and, unless the caller
+// accumulates, the three gradient arrays.
+__global__ void __launch_bounds__(kThreads)
+    k_zero(float4* __restrict__ fp, int64_t n_fp, float4* __restrict__ g0, float4* __restrict__ g1,
+           float4* __restrict__ g2, int64_t n_g) {
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  for (int64_t i = t; i < n_fp; i += stride) fp[i] = z;
+  for (int64_t i = t; i < n_g; i += stride) g0[i] = g1[i] = g2[i] = z;
+}
+
 // ------------------------------------------------------------------------------------------
 // Host orchestration
 // ------------------------------------------------------------------------------------------
@@ -893,8 +1150,9 @@ int cap_from_ws(const gs_instance* inst, int n_inst, const gs_opts* o, size_t ws
   GS_TRY(make_plan(inst, n_inst, o, 0, p0));
   const size_t base = carve(nullptr, p0).bytes;
   if (ws_bytes < base) return GS_ERR_CAPACITY;
-  // each unit of capacity costs 16 bytes (keys, vals and their alternates) plus alignment
-  int64_t c = (int64_t)((ws_bytes - base) / 16);
+  // each unit of capacity costs 4 bytes (direct: the lists) or 16 (sorted: keys, vals and their
+  // alternates) plus alignment
+  int64_t c = (int64_t)((ws_bytes - base) / (p0.direct ? 4 : 16));
   while (c > 0) {
     Plan p;
     GS_TRY(make_plan(inst, n_inst, o, c, p));
@@ -922,32 +1180,47 @@ int prepare(const gs_instance* inst, int n_inst, const gs_opts* o, const float* 
   return GS_OK;
 }
 
-int setup_and_preprocess(const Plan& p, const Layout& L, const float* mr, const float* sc,
-                         const float* qt, const gs_view* views, cudaStream_t s) {
-  GS_TRY(launch("view_setup", k_view_setup, dim3((p.total_v + 63) / 64), dim3(64), 0, s, p.b,
-                views, p.total_v, L.frames, L.st));
-  GS_TRY(launch("preprocess", k_preprocess, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
-                (const float4*)mr, (const float4*)sc, (const float4*)qt, p.items,
-                (const ViewFrame*)L.frames, L.geo, L.conic, L.rect, L.tmask, L.counts,
-                L.block_sums));
-  return scan_block_sums(L.block_sums, L.block_offs, p.nblocks, L.st, p.cap, s);
+// Dynamic shared memory above 48 KB needs the kernel's limit raised (host-side state of the
+// current device, set on every call that needs it).
+size_t emit_smem(const Plan& p) { return (size_t)(1 + kThreads / 32) * p.max_tiles * sizeof(uint32_t); }
+
+int preprocess_and_scan(const Plan& p, const Layout& L, const float* mr, const float* sc,
+                        const float* qt, const gs_view* views, cudaStream_t s, void* ws) {
+  const size_t smem = p.direct ? (size_t)p.max_tiles * sizeof(uint32_t) : 0;
+  GS_TRY(launch("preprocess", p.direct ? k_preprocess<true> : k_preprocess<false>,
+                dim3(p.nblocks), dim3(kThreads), smem, s, p.b, (const float4*)mr,
+                (const float4*)sc, (const float4*)qt, views, L.frames, L.geo, L.conic, L.rect,
+                L.tmask, L.counts, L.block_sums, L.tcount, L.ticket, L.st));
+  if (!p.direct) return scan_block_sums(L.block_sums, L.block_offs, p.nblocks, L.st, p.cap, s);
+  auto off = [&](const void* q) { return (int64_t)((const char*)q - (const char*)ws); };
+  return launch("key_scan", k_key_scan, dim3((unsigned)((p.n_keys + kScanKeys - 1) / kScanKeys)),
+                dim3(kScanKeys * kScanSegs), 0, s, p.b, p.n_keys, (const uint16_t*)L.tcount,
+                L.toffset, L.klocal, L.ranges, L.gsum, L.ticket, L.vkeys, p.total_v, L.st, p.cap,
+                off(L.vals), off(L.ranges), off(L.vkeys));
 }
 
-// view setup -> preprocess -> scan -> emit -> sort -> ranges.  On return *keys/*vals point at
-// the sorted lists inside the workspace.
+// preprocess -> lists and ranges of every (view, tile), by the direct or the sorted route.  On
+// return *svals points at the lists inside the workspace.
 int bin_pairs(const Plan& p, const Layout& L, const float* mr, const float* sc, const float* qt,
-              const gs_view* views, cudaStream_t s, void* ws, uint32_t** skeys,
-              uint32_t** svals) {
+              const gs_view* views, cudaStream_t s, void* ws, uint32_t** svals) {
+  *svals = L.vals;
   if (p.total_n == 0) {
     GS_CUDA(cudaMemsetAsync(L.st, 0, sizeof(gs_status), s));
     GS_CUDA(cudaMemsetAsync(L.ranges, 0, (size_t)p.n_keys * sizeof(uint2), s));
-    GS_TRY(launch("view_setup", k_view_setup, dim3((p.total_v + 63) / 64), dim3(64), 0, s, p.b,
-                  views, p.total_v, L.frames, L.st));
-    *skeys = L.keys;
-    *svals = L.vals;
     return GS_OK;
   }
-  GS_TRY(setup_and_preprocess(p, L, mr, sc, qt, views, s));
+  GS_TRY(preprocess_and_scan(p, L, mr, sc, qt, views, s, ws));
+  if (p.direct) {
+    const size_t smem = emit_smem(p);
+    if (smem > 48 * 1024)
+      GS_CUDA(cudaFuncSetAttribute(k_emit_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)smem));
+    return launch("emit", k_emit_direct, dim3(p.nblocks), dim3(kThreads), smem, s, p.b,
+                  (const uint32_t*)L.counts, (const float4*)L.geo, (const float4*)L.conic,
+                  (const short4*)L.rect, (const uint32_t*)L.tmask, (const uint32_t*)L.toffset,
+                  (const uint32_t*)L.klocal, (const unsigned long long*)L.gsum, L.ranges, L.vals,
+                  (const gs_status*)L.st);
+  }
   uint32_t* k = L.keys;
   uint32_t* v = L.vals;
   const bool odd = (p.sort.passes & 1) != 0;
@@ -956,15 +1229,19 @@ int bin_pairs(const Plan& p, const Layout& L, const float* mr, const float* sc, 
   GS_TRY(launch("emit", k_emit, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
                 (const uint32_t*)L.counts, (const float4*)L.geo, (const float4*)L.conic,
                 (const short4*)L.rect, (const uint32_t*)L.tmask, (const uint32_t*)L.block_offs,
-                p.items, L.keys, L.vals, L.st, (int64_t)((char*)fk - (char*)ws),
+                L.keys, L.vals, L.st, (int64_t)((char*)fk - (char*)ws),
                 (int64_t)((char*)fv - (char*)ws)));
   GS_TRY(radix_sort(&k, &v, L.keys_alt, L.vals_alt, L.hist, p.sort, L.st, p.cap, s));
   GS_CUDA(cudaMemsetAsync(L.ranges, 0, (size_t)p.n_keys * sizeof(uint2), s));
   GS_TRY(launch("ranges", k_tile_ranges, dim3(4 * num_sms()), dim3(kThreads), 0, s, p.b,
                 (const uint32_t*)k, L.ranges, (const gs_status*)L.st));
-  *skeys = k;
   *svals = v;
   return GS_OK;
+}
+
+// Where the lists of the last binning lie.
+uint32_t* sorted_vals(const Plan& p, const Layout& L) {
+  return !p.direct && (p.sort.passes & 1) ? L.vals_alt : L.vals;
 }
 
 template <int T>
@@ -1036,7 +1313,7 @@ int gs_project_batch_count_pairs(const float* d_mean_rho, const float* d_scale,
     *h_pairs = 0;
     return GS_OK;
   }
-  GS_TRY(setup_and_preprocess(p, L, d_mean_rho, d_scale, d_quat, d_views, s));
+  GS_TRY(preprocess_and_scan(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws));
   gs_status st;
   GS_TRY(gs_read_status(d_ws, stream, &st));
   *h_pairs = st.pairs;
@@ -1053,8 +1330,8 @@ int gs_project_batch(const float* d_mean_rho, const float* d_scale, const float*
   GS_TRY(prepare(inst, n_inst, opts, d_mean_rho, d_scale, d_quat, d_views, d_ws, ws_bytes, p,
                  L));
   cudaStream_t s = (cudaStream_t)stream;
-  uint32_t *k, *v;
-  GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &k, &v));
+  uint32_t* v;
+  GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &v));
   return dispatch_fwd(p, L, v, d_img, false, s);
 }
 
@@ -1067,8 +1344,8 @@ int gs_project_batch_count_evals(const float* d_mean_rho, const float* d_scale,
   GS_TRY(prepare(inst, n_inst, opts, d_mean_rho, d_scale, d_quat, d_views, d_ws, ws_bytes, p,
                  L));
   cudaStream_t s = (cudaStream_t)stream;
-  uint32_t *k, *v;
-  GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &k, &v));
+  uint32_t* v;
+  GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &v));
   GS_CUDA(cudaMemsetAsync(&L.st->evals, 0, sizeof(int64_t), s));
   return dispatch_fwd(p, L, v, nullptr, true, s);
 }
@@ -1092,23 +1369,20 @@ int gs_project_batch_backward_stats(const float* d_mean_rho, const float* d_scal
   if (p.total_n == 0) return GS_OK;
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t* v;
-  if (reuse) {
-    v = (p.sort.passes & 1) ? L.vals_alt : L.vals;
-  } else {
-    uint32_t* k;
-    GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &k, &v));
-  }
-  GS_CUDA(cudaMemsetAsync(L.fpgrad, 0, (size_t)p.items * 32, s));
+  if (reuse)
+    v = sorted_vals(p, L);
+  else
+    GS_TRY(bin_pairs(p, L, d_mean_rho, d_scale, d_quat, d_views, s, d_ws, &v));
+  const int64_t n_fp = 2 * p.items, n_g = accumulate ? 0 : p.total_n;
+  GS_TRY(launch("zero", k_zero,
+                dim3((unsigned)std::min<int64_t>((std::max(n_fp, n_g) + kThreads - 1) / kThreads,
+                                                 8 * (int64_t)num_sms())),
+                dim3(kThreads), 0, s, L.fpgrad, n_fp, (float4*)d_g_mean_rho, (float4*)d_g_scale,
+                (float4*)d_g_quat, n_g));
   switch (p.b.T) {
     case 8: GS_TRY(raster_bwd<8>(p, L, v, d_dimg, s)); break;
     case 16: GS_TRY(raster_bwd<16>(p, L, v, d_dimg, s)); break;
     default: GS_TRY(raster_bwd<32>(p, L, v, d_dimg, s)); break;
-  }
-  if (!accumulate) {
-    const size_t bytes = (size_t)p.total_n * sizeof(float4);
-    GS_CUDA(cudaMemsetAsync(d_g_mean_rho, 0, bytes, s));
-    GS_CUDA(cudaMemsetAsync(d_g_scale, 0, bytes, s));
-    GS_CUDA(cudaMemsetAsync(d_g_quat, 0, bytes, s));
   }
   int max_nv = 1;
   for (int k = 0; k < p.b.count; ++k) max_nv = std::max(max_nv, p.b.in[k].nv);

@@ -165,9 +165,36 @@ int gs_read_pairs(const void* d_ws, size_t ws_bytes, void* stream, int64_t cap,
   int64_t n = std::min<int64_t>(st.pairs, cap);
   if (n <= 0) return GS_OK;
   if (st.code != GS_OK) return GS_ERR_CAPACITY;
+  const char* b = (const char*)d_ws;
+  if (st.reserved[0] == -1) {
+    // lists written in place (view by view, tiles ascending) without stored keys: take each
+    // list's key from the ranges and hand the lists out ordered by (tile, global view)
+    const int64_t n_keys = st.reserved[2], nv = st.reserved[5];
+    const size_t vo = (size_t)st.reserved[1], ro = (size_t)st.reserved[3], ko = (size_t)st.reserved[4];
+    if (vo + st.pairs * 4 > ws_bytes || ro + n_keys * sizeof(uint2) > ws_bytes ||
+        ko + (nv + 1) * 8 > ws_bytes)
+      return GS_ERR_ARG;
+    std::vector<uint32_t> vals((size_t)st.pairs);
+    std::vector<uint2> ranges((size_t)n_keys);
+    std::vector<long long> first((size_t)nv + 1);
+    GS_CUDA(cudaMemcpy(vals.data(), b + vo, vals.size() * 4, cudaMemcpyDeviceToHost));
+    GS_CUDA(cudaMemcpy(ranges.data(), b + ro, ranges.size() * sizeof(uint2), cudaMemcpyDeviceToHost));
+    GS_CUDA(cudaMemcpy(first.data(), b + ko, first.size() * 8, cudaMemcpyDeviceToHost));
+    int64_t out = 0, max_tiles = 0;
+    for (int64_t v = 0; v < nv; ++v) max_tiles = std::max<int64_t>(max_tiles, first[v + 1] - first[v]);
+    for (int64_t t = 0; t < max_tiles && out < n; ++t)
+      for (int64_t v = 0; v < nv && out < n; ++v) {
+        if (t >= first[v + 1] - first[v]) continue;
+        const uint2 r = ranges[first[v] + t];
+        for (uint32_t k = r.x; k < r.y && out < n; ++k, ++out) {
+          if (h_keys) h_keys[out] = ((uint32_t)v << st.reserved[6]) | (uint32_t)t;
+          if (h_vals) h_vals[out] = vals[k];
+        }
+      }
+    return GS_OK;
+  }
   size_t ko = (size_t)st.reserved[0], vo = (size_t)st.reserved[1];
   if (ko + n * 4 > ws_bytes || vo + n * 4 > ws_bytes) return GS_ERR_ARG;
-  const char* b = (const char*)d_ws;
   if (h_keys) GS_CUDA(cudaMemcpy(h_keys, b + ko, n * 4, cudaMemcpyDeviceToHost));
   if (h_vals) GS_CUDA(cudaMemcpy(h_vals, b + vo, n * 4, cudaMemcpyDeviceToHost));
   return GS_OK;
