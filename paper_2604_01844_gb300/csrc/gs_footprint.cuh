@@ -148,16 +148,18 @@ __device__ __forceinline__ bool footprint(const float4 mr, const float4 sc, cons
   return true;
 }
 
-// footprint moments -> parameter gradients (reverse mode through `footprint`)
+// footprint moments -> parameter gradients (reverse mode through `footprint`), added to gp, grho,
+// gs and gR.  The gradient of the rotation matrix is left as such: it is linear, so a Gaussian's
+// views add up before one step to the quaternion.
 __device__ __forceinline__ void chain_one(const Fwd& o, const ViewFrame& f, const float4 m0,
                                           const float4 m1, float gp[3], float& grho,
-                                          float gs[3], float gq[4]) {
+                                          float gs[3], float gR[3][3]) {
   const float S0 = m0.x, Sx = m0.y, Sy = m0.z, Sxx = m0.w, Sxy = m1.x, Syy = m1.y;
   // image = A exp(-q/2), q = ca dx^2 + 2 cb dx dy + cc dy^2, dx = x - px
   const float dA = S0;
   const float dca = -0.5f * o.A * Sxx, dcb = -o.A * Sxy, dcc = -0.5f * o.A * Syy;
   const float dpx = o.A * (o.ca * Sx + o.cb * Sy), dpy = o.A * (o.cb * Sx + o.cc * Sy);
-  grho = dA * o.mu;
+  grho += dA * o.mu;
   const float dmu = dA * o.rho;
   // conic = P^-1 (full-matrix gradients): G_P = -C G_C C
   const float gc01 = 0.5f * dcb;
@@ -171,9 +173,9 @@ __device__ __forceinline__ void chain_one(const Fwd& o, const ViewFrame& f, cons
   float gh00 = gP00 * ipu * ipu, gh01 = gP01 * ipu * ipv, gh11 = gP11 * ipv * ipv;
   // mu = sqrt(2 pi) |det J| s0 s1 s2 / sqrt(det Sigma^)
   const float g = dmu * o.mu;
-  gs[0] = g / o.s[0];
-  gs[1] = g / o.s[1];
-  gs[2] = g / o.s[2];
+  gs[0] += g / o.s[0];
+  gs[1] += g / o.s[1];
+  gs[2] += g / o.s[2];
   const float gdet = -0.5f * g / o.det2w;
   gh00 += gdet * o.h11;
   gh11 += gdet * o.h00;
@@ -186,7 +188,7 @@ __device__ __forceinline__ void chain_one(const Fwd& o, const ViewFrame& f, cons
     gK[1][k] = 2.f * (gh01 * o.K[0][k] + gh11 * o.K[1][k]);
   }
   // K = T2 R diag(s)
-  float gT2[2][3], gR[3][3];
+  float gT2[2][3];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -198,7 +200,7 @@ __device__ __forceinline__ void chain_one(const Fwd& o, const ViewFrame& f, cons
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const float gRS = o.T2[0][b] * gK[0][k] + o.T2[1][b] * gK[1][k];
-      gR[b][k] = gRS * o.s[k];
+      gR[b][k] += gRS * o.s[k];
       gs[k] += gRS * o.R[b][k];
     }
   // camera frame position gradient
@@ -231,12 +233,7 @@ __device__ __forceinline__ void chain_one(const Fwd& o, const ViewFrame& f, cons
     gx[1] = dpy * ipv;
   }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) gp[c] = f.M[0][c] * gx[0] + f.M[1][c] * gx[1] + f.M[2][c] * gx[2];
-  float dq[4];
-  gsd::rot_to_quat_grad(o.qn[0], o.qn[1], o.qn[2], o.qn[3], gR, dq);
-  gsd::quat_normalize_grad(o.qn, o.inv_norm, dq);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) gq[k] = dq[k];
+  for (int c = 0; c < 3; ++c) gp[c] += f.M[0][c] * gx[0] + f.M[1][c] * gx[1] + f.M[2][c] * gx[2];
 }
 
 }  // namespace gs

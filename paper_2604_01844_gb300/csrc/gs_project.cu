@@ -37,15 +37,16 @@ constexpr int kMaxInst = GS_MAX_INSTANCES;
 constexpr int kTileDigitBits = 8;
 
 // The direct route keeps a counter per (block of 256 records, tile) and, in emit, a 32-bit lane
-// mask per (warp, tile) in shared memory: 72 KB at 2048 tiles, three CTAs per SM.  Its cost per
+// mask per (warp, tile) in shared memory: 88 KB at 2048 tiles, two CTAs per SM.  Its cost per
 // block grows with the tiles (10 bytes of counts and offsets each), the sort's with the pairs
 // (about 60 bytes each, some 1300 pairs per block): up to 2048 tiles the direct route is the
-// cheaper one (project 75 x 512^2, 1024 tiles: lists in LISTS_NEW instead of LISTS_OLD us).
+// cheaper one (project 75 x 512^2, 1024 tiles: lists from the counts in 172 instead of 390 us).
 constexpr int kDirectTiles = 2048;
 
 struct Inst {
   int n, nv, W, H, TW, TH, g_off, v_off;
   int bpv;  // blocks of 256 records per view
+  int tp;   // tiles per view rounded up to 8: row pitch of the (block, tile) matrices
   long long item_off, key_off, img_off, blk_off;
   long long mat_off;  // first entry of the instance in the (block, tile) count matrix
 };
@@ -117,7 +118,7 @@ struct Plan {
   Batch b;
   int total_n = 0, total_v = 0;
   int64_t items = 0, n_keys = 0, cap = 0, mat = 0;
-  int nblocks = 0, key_bits = 0, max_tiles = 1;
+  int nblocks = 0, key_bits = 0, max_tp = 8;
   bool direct = false;
   SortPlan sort;
 };
@@ -152,10 +153,11 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
     d.key_off = keys;
     d.img_off = img;
     d.bpv = (s.n + kThreads - 1) / kThreads;
+    d.tp = (d.TW * d.TH + 7) / 8 * 8;
     d.blk_off = blocks;
     d.mat_off = mat;
     blocks += (int64_t)s.n_views * d.bpv;
-    mat += (int64_t)s.n_views * d.bpv * d.TW * d.TH;
+    mat += (int64_t)s.n_views * d.bpv * d.tp;
     items += (int64_t)s.n * s.n_views;
     keys += (int64_t)s.n_views * d.TW * d.TH;
     max_tiles = std::max<int64_t>(max_tiles, (int64_t)d.TW * d.TH);
@@ -174,7 +176,7 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
   p.n_keys = keys;
   p.cap = std::min<int64_t>(cap, ((int64_t)1 << 31) - 1);
   p.nblocks = (int)blocks;
-  p.max_tiles = (int)max_tiles;
+  p.max_tp = (int)((max_tiles + 7) / 8 * 8);
   p.direct = max_tiles <= kDirectTiles;
   p.mat = p.direct ? mat : 0;
   p.key_bits = b.tbits;
@@ -223,30 +225,44 @@ Layout carve(void* ws, const Plan& p) {
 // enlarged ellipse's section by the row's slab of pixel centres is convex, so the tiles it meets
 // are those whose pixel columns meet its x extent [xa, xb]: the left (right) end lies at the
 // ellipse's own leftmost (rightmost) point when that is inside the slab, else on the slab's
-// nearer edge.  The ends are compared with pixel columns relative to the record's centre, where
-// FP32 resolves far more than the margin.
+// nearer edge.  The ends become pixel columns through the centre's integer and fractional parts,
+// where FP32 resolves far more than the margin.
 struct Ell {
-  float px, py, ia, hb, kap, vr, cm;  // 1/a, -b/(2a), c - b^2/(4a), v of the rightmost point
+  float py, fx, ia, hb, kap, vr, cm;  // 1/a, -b/(2a), c - b^2/(4a), v of the rightmost point
+  int ix;                             // centre column px = ix + fx
 };
-// Every operation below has its rounding written out: preprocess counts the tiles and emit places
-// them, so both must get the same answers.
+// Every operation below is one fixed instruction: preprocess counts the tiles and emit places
+// them, so both must get the same answers.  The approximate reciprocals and roots are within two
+// ulp, far inside the margin.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ Ell make_ell(const float4 g, const float4 c) {
   Ell E;
-  E.px = g.x;
+  const float fl = floorf(g.x);  // |px| stays far below 2^24 where a box meets the detector
+  E.ix = (int)fl;
+  E.fx = __fsub_rn(g.x, fl);
   E.py = g.y;
-  E.ia = __frcp_rn(c.x);
+  E.ia = rcp_approx(c.x);
   const float hb = __fmul_rn(-0.5f, c.y);
   E.hb = __fmul_rn(hb, E.ia);
   E.kap = __fmaf_rn(-hb, E.hb, c.z);
   E.cm = __fmul_rn(g.w, 1.001f);
-  const float ih = __fdiv_rn(hb, c.z);  // v = ih u where u is extreme on the ellipse
-  const float u2 = __fdiv_rn(E.cm, __fmaf_rn(-hb, ih, c.x));
-  E.vr = __fmul_rn(ih, __fsqrt_rn(fmaxf(u2, 0.f)));
+  const float ih = __fmul_rn(hb, rcp_approx(c.z));  // v = ih u where u is extreme on the ellipse
+  const float u2 = __fmul_rn(E.cm, rcp_approx(__fmaf_rn(-hb, ih, c.x)));
+  E.vr = __fmul_rn(ih, sqrt_approx(fmaxf(u2, 0.f)));
   return E;
 }
 __device__ __forceinline__ float half_width(const Ell& E, float v) {
   const float d = __fmul_rn(__fmaf_rn(__fmul_rn(-E.kap, v), v, E.cm), E.ia);
-  return __fsqrt_rn(fmaxf(d, 0.f));
+  return sqrt_approx(fmaxf(d, 0.f));
 }
 // Tiles ta .. tb (none if ta > tb) of tile row ty for the clipped box (x0, y0)-(x1, y1).
 __device__ __forceinline__ void row_tiles(const Ell& E, int lT, int ty, int x0, int y0, int x1,
@@ -256,17 +272,13 @@ __device__ __forceinline__ void row_tiles(const Ell& E, int lT, int ty, int x0, 
   const float vb = fminf(fmaxf(E.vr, v0), v1), va = fminf(fmaxf(-E.vr, v0), v1);
   const float xb = __fmaf_rn(E.hb, vb, half_width(E, vb));
   const float xa = __fmaf_rn(E.hb, va, -half_width(E, va));
-  // first pixel column >= xa and last <= xb, decided on offsets from the centre
-  float fa = ceilf(__fadd_rn(xa, E.px)), fb = floorf(__fadd_rn(xb, E.px));
-  if (__fsub_rn(fa - 1.f, E.px) >= xa) fa -= 1.f;
-  else if (__fsub_rn(fa, E.px) < xa) fa += 1.f;
-  if (__fsub_rn(fb + 1.f, E.px) <= xb) fb += 1.f;
-  else if (__fsub_rn(fb, E.px) > xb) fb -= 1.f;
+  // first pixel column >= xa and last <= xb, from the centre's integer and fractional column
+  const int fa = E.ix + (int)ceilf(__fadd_rn(xa, E.fx)), fb = E.ix + (int)floorf(__fadd_rn(xb, E.fx));
   // an extent between two neighbouring columns (fa = fb + 1) meets their tile if both are the
   // box's and in one tile; one left or right of the box meets none
-  const bool none = fb < (float)x0 || fa > (float)x1;
-  ta = none ? 1 : (int)fmaxf(fa, (float)x0) >> lT;
-  tb = none ? 0 : (int)fminf(fb, (float)x1) >> lT;
+  const bool none = fb < x0 || fa > x1;
+  ta = none ? 1 : max(fa, x0) >> lT;
+  tb = none ? 0 : min(fb, x1) >> lT;
 }
 
 // Preprocess keeps the answers for boxes of up to 32 tiles as a bit mask in the box's tile order;
@@ -309,7 +321,7 @@ __global__ void __launch_bounds__(kThreads)
                  uint32_t* __restrict__ tmask, uint32_t* __restrict__ counts,
                  uint32_t* __restrict__ block_sums, uint16_t* __restrict__ tcount,
                  uint32_t* __restrict__ ticket, gs_status* st) {
-  extern __shared__ uint32_t s_tiles[];  // DIRECT: records of the block per tile
+  extern __shared__ __align__(16) uint32_t s_tiles[];  // DIRECT: records of the block per tile
   __shared__ uint32_t warp_sums[kThreads / 32];
   __shared__ ViewFrame f;
   const BlockItems bi = block_items(b, blockIdx.x);
@@ -320,9 +332,9 @@ __global__ void __launch_bounds__(kThreads)
   // the parameters are requested before the view's frame is built, which takes one thread a
   // chain of divisions
   const float4 mr = mean_rho[gi], sc = scale[gi], qt = quat[gi];
-  const int tiles = I.TW * I.TH;
   if (DIRECT)
-    for (int t = threadIdx.x; t < tiles; t += kThreads) s_tiles[t] = 0u;
+    for (int t = threadIdx.x; t < I.tp / 4; t += kThreads)
+      reinterpret_cast<uint4*>(s_tiles)[t] = make_uint4(0u, 0u, 0u, 0u);
   if (threadIdx.x == 0) {
     ViewFrame fr;
     make_frame(views[I.v_off + bi.v], I.W, I.H, fr);
@@ -372,8 +384,14 @@ __global__ void __launch_bounds__(kThreads)
   }
   if constexpr (DIRECT) {
     __syncthreads();
-    uint16_t* row = tcount + I.mat_off + ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * tiles;
-    for (int t = threadIdx.x; t < tiles; t += kThreads) row[t] = (uint16_t)s_tiles[t];
+    // the row in 16-byte vectors (entries past the last tile are zero)
+    uint4* row = reinterpret_cast<uint4*>(tcount + I.mat_off +
+                                          ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * I.tp);
+    for (int t = threadIdx.x; t < I.tp / 8; t += kThreads) {
+      const uint4 x = reinterpret_cast<const uint4*>(s_tiles)[2 * t];
+      const uint4 y = reinterpret_cast<const uint4*>(s_tiles)[2 * t + 1];
+      row[t] = make_uint4(x.x | x.y << 16, x.z | x.w << 16, y.x | y.y << 16, y.z | y.w << 16);
+    }
   } else {
     // culled pairs drop out of the warp's count via the ballot; the block sum feeds the scan
     const unsigned live_mask = __ballot_sync(0xffffffffu, cnt > 0);
@@ -409,20 +427,21 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
   const int t = threadIdx.x, lane = t & 31, kl = t % kScanKeys, seg = t / kScanKeys;
   const int64_t key = (int64_t)blockIdx.x * kScanKeys + kl;
   uint32_t sum = 0;
-  int b0 = 0, b1 = 0, tiles = 0;
+  int b0 = 0, b1 = 0, tp = 0;
   int64_t at = 0;
   if (key < n_keys) {
     const Inst& I = b.in[inst_of_key(b, key)];
-    tiles = I.TW * I.TH;
+    const int tiles = I.TW * I.TH;
     const int64_t lk = key - I.key_off;
+    tp = I.tp;
     const int v = (int)(lk / tiles), tile = (int)(lk - (int64_t)v * tiles);
     const int per = (I.bpv + kScanSegs - 1) / kScanSegs;
     b0 = min(I.bpv, seg * per);
     b1 = min(I.bpv, b0 + per);
-    at = I.mat_off + (int64_t)v * I.bpv * tiles + tile;
+    at = I.mat_off + (int64_t)v * I.bpv * tp + tile;
     if (seg == 0 && tile == 0) vkeys[I.v_off + v] = key;
 #pragma unroll 8
-    for (int k = b0; k < b1; ++k) sum += tcount[at + (int64_t)k * tiles];
+    for (int k = b0; k < b1; ++k) sum += tcount[at + (int64_t)k * tp];
   }
   if (blockIdx.x == 0 && t == 0) vkeys[total_v] = n_keys;
   part[seg][kl] = sum;
@@ -436,7 +455,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
   }
 #pragma unroll 8
   for (int k = b0; k < b1; ++k) {
-    const int64_t e = at + (int64_t)k * tiles;
+    const int64_t e = at + (int64_t)k * tp;
     toffset[e] = run;
     run += tcount[e];
   }
@@ -502,7 +521,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
 // Writes every record to its place in the lists of its tiles.  A block's records keep their order
 // inside a list: a record's place is the list's start, plus the block's offset in it, plus the
 // records of the same tile in earlier warps and lanes of the block (a lane mask per (warp, tile)
-// in shared memory, counted by popc).  Blocks of one view run together, so the scattered 4-byte
+// in shared memory; its set bits give the counts).  Blocks of one view run together, so the scattered 4-byte
 // stores of a list's neighbourhood meet in L2.
 __global__ void __launch_bounds__(kThreads)
     k_emit_direct(const __grid_constant__ Batch b, const uint32_t* __restrict__ counts,
@@ -512,7 +531,8 @@ __global__ void __launch_bounds__(kThreads)
                   const unsigned long long* __restrict__ gsum, uint2* __restrict__ ranges,
                   uint32_t* __restrict__ vals, const gs_status* st) {
   constexpr int NW = kThreads / 32;
-  extern __shared__ uint32_t s_emit[];  // [tiles] first place of the block, [NW][tiles] lane masks
+  extern __shared__ __align__(16) uint32_t s_emit[];
+  static_assert(NW == 8, "eight bytes of warp counts per tile");
   const BlockItems bi = block_items(b, blockIdx.x);
   const Inst& I = b.in[bi.inst];
   const int tiles = I.TW * I.TH, t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -522,31 +542,48 @@ __global__ void __launch_bounds__(kThreads)
   const short4 r = i < I.n ? rect[idx] : make_short4(0, 0, 0, 0);
   const uint32_t tm = i < I.n ? tmask[idx] : 0u;
   if (st->code != GS_OK) return;
-  uint32_t* first = s_emit;
-  uint32_t* lanes = s_emit + tiles;
+  // [NW][tp] lane masks, [tp] first place of the block in the tile's list, [tp] eight bytes: records
+  // of the tile in the warps before each
+  const int tp = I.tp;
+  uint32_t* lanes = s_emit;
+  uint32_t* first = lanes + NW * tp;
+  uint2* before = reinterpret_cast<uint2*>(first + tp);
+  for (int k = t; k < NW * tp / 4; k += kThreads)
+    reinterpret_cast<uint4*>(lanes)[k] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  const uint32_t bit = 1u << lane;
+  uint32_t* mine = lanes + w * tp;
+  if (cnt)
+    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
+      uint32_t* q = mine + ty * I.TW;
+      for (int k = ta; k <= tb; ++k) atomicOr(q + k, bit);
+    });
   const int64_t key0 = I.key_off + (int64_t)bi.v * tiles;
-  const uint32_t* row = toffset + I.mat_off + ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * tiles;
+  const uint32_t* row = toffset + I.mat_off + ((int64_t)bi.v * I.bpv + bi.i0 / kThreads) * tp;
+  __syncthreads();
   for (int k = t; k < tiles; k += kThreads) {
     const uint32_t start = (uint32_t)gsum[(key0 + k) / kScanKeys] + klocal[key0 + k];
     first[k] = start + row[k];
     if (bi.i0 == 0) ranges[key0 + k] = make_uint2(start, start + ranges[key0 + k].y);
+    uint32_t run = 0, lo = 0, hi = 0;  // at most 7 x 32 before the last warp: a byte
+#pragma unroll
+    for (int ww = 0; ww < 4; ++ww) {
+      lo |= run << (8 * ww);
+      run += __popc(lanes[ww * tp + k]);
+    }
+#pragma unroll
+    for (int ww = 0; ww < 4; ++ww) {
+      hi |= run << (8 * ww);
+      run += __popc(lanes[(ww + 4) * tp + k]);
+    }
+    before[k] = make_uint2(lo, hi);
   }
-  for (int k = t; k < NW * tiles; k += kThreads) lanes[k] = 0u;
   __syncthreads();
-  const uint32_t bit = 1u << lane;
+  const uint8_t* pre = reinterpret_cast<const uint8_t*>(before) + w;
   if (cnt)
     listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
-      uint32_t* q = lanes + w * tiles + ty * I.TW;
-      for (int k = ta; k <= tb; ++k) atomicOr(q + k, bit);
-    });
-  __syncthreads();
-  if (cnt)
-    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
-      for (int k = ty * I.TW + ta; k <= ty * I.TW + tb; ++k) {
-        uint32_t pos = first[k] + __popc(lanes[w * tiles + k] & (bit - 1u));
-        for (int ww = 0; ww < w; ++ww) pos += __popc(lanes[ww * tiles + k]);
-        vals[pos] = (uint32_t)idx;
-      }
+      for (int k = ty * I.TW + ta; k <= ty * I.TW + tb; ++k)
+        vals[first[k] + pre[8 * k] + __popc(mine[k] & (bit - 1u))] = (uint32_t)idx;
     });
 }
 
@@ -921,7 +958,7 @@ __global__ void __launch_bounds__(BwdBlocks<T>::NT, T == 32 ? 3 : 1024 / BwdBloc
                  const float4* __restrict__ conic, const short4* __restrict__ rect,
                  const float* __restrict__ dimg, float4* __restrict__ fpgrad,
                  const gs_status* st) {
-  using S = BwdBlocks<T>;
+  using S = BwdBlocks<T>;  // blockIdx.y: the part of the list this CTA takes
   constexpr int BW = S::BW;
   __shared__ __align__(16) float s_g[T][T];
   constexpr int SB = 2 * S::NT;  // records staged per batch (more costs occupancy here)
@@ -932,8 +969,13 @@ __global__ void __launch_bounds__(BwdBlocks<T>::NT, T == 32 ? 3 : 1024 / BwdBloc
   __shared__ float s_acc[6][SB];
   __shared__ uint16_t s_list[S::NW][SB];
   const int64_t key = blockIdx.x;
-  const uint2 r = ranges[key];  // requested together with the status word, not after it
+  uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
+  if (gridDim.y > 1) {  // an equal part, in whole warps of records
+    const uint32_t part = ((r.y - r.x + gridDim.y - 1) / gridDim.y + 31u) & ~31u;
+    r.x = min(r.y, r.x + blockIdx.y * part);
+    r.y = min(r.y, r.x + part);
+  }
   if (r.x == r.y) return;
   const Inst& I = b.in[inst_of_key(b, key)];
   const int64_t lk = key - I.key_off;
@@ -1051,18 +1093,22 @@ __global__ void __launch_bounds__(BwdBlocks<T>::NT, T == 32 ? 3 : 1024 / BwdBloc
 }
 
 // ------------------------------------------------------------------------------------------
-// chain: a thread per (Gaussian, chunk of kChainViews views), consecutive threads on
+// chain: a thread per (Gaussian, chunk of up to kChainViews views), consecutive threads on
 // consecutive Gaussians of one chunk, so that the moment loads of a warp are one contiguous
 // run and the view frame is the same for all its lanes; each thread chains its views'
-// moments to the Gaussian's parameters and adds its sums with float4 atomics (the gradients
-// are zeroed first unless accumulating)
+// moments to the Gaussian's parameters (the rotation's gradient stays a matrix until the last
+// view), requests the next view's moments one view ahead, and adds its sums with float4
+// atomics (the gradients are zeroed first unless accumulating).  Bound by FP32 issue.
+// 75 x 512^2, 50k Gaussians: 107 -> 89 us; a third CTA per SM costs spills (112), one leaves
+// latency open (137).  Small calls take fewer views per thread (one at 2000 Gaussians x 8 views,
+// 17 -> 8 us): the chunks then fill the SMs.
 // ------------------------------------------------------------------------------------------
 constexpr int kChainViews = 8;
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
     k_project_chain(const __grid_constant__ Batch b, const float4* __restrict__ mean_rho,
                     const float4* __restrict__ scale, const float4* __restrict__ quat,
-                    int total_n, int vchunks, const ViewFrame* __restrict__ frames,
+                    int total_n, int vchunks, int cv, const ViewFrame* __restrict__ frames,
                     const float4* __restrict__ fpgrad, float4* __restrict__ g_mr,
                     float4* __restrict__ g_sc, float4* __restrict__ g_q,
                     const uint32_t* __restrict__ counts, float* __restrict__ stat,
@@ -1072,28 +1118,37 @@ __global__ void __launch_bounds__(kThreads)
   const int gi = (int)(tid % total_n), ch = (int)(tid / total_n);
   const Inst& I = b.in[inst_of_gaussian(b, gi)];
   const int il = gi - I.g_off;
-  const int v0 = ch * kChainViews, v1 = min(v0 + kChainViews, I.nv);
+  const int v0 = ch * cv, v1 = min(v0 + cv, I.nv);
   if (v0 >= v1) return;
   const float4 mr = mean_rho[gi], sc = scale[gi], qt = quat[gi];
-  float acc[11];
-#pragma unroll
-  for (int k = 0; k < 11; ++k) acc[k] = 0.f;
+  float gp[3] = {0.f, 0.f, 0.f}, grho = 0.f, gsc[3] = {0.f, 0.f, 0.f};
+  float gR[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+  bool any = false;
+  float qn[4] = {0.f, 0.f, 0.f, 0.f}, inv_norm = 0.f;
   // adaptive density control statistics: NDC detector-position gradient norms and the
   // number of views with a listed tile
   float st_acc = 0.f;
   int vis_acc = 0;
-  for (int v = v0; v < v1; ++v) {
-    const size_t rec = (size_t)(I.item_off + (int64_t)v * I.n + il);
+  size_t rec = (size_t)(I.item_off + (int64_t)v0 * I.n + il);
+  float4 n0 = fpgrad[2 * rec], n1 = fpgrad[2 * rec + 1];  // the next view's moments, one ahead
+  for (int v = v0; v < v1; ++v, rec += I.n) {
     if (stat && counts[rec] > 0u) ++vis_acc;
-    const float4 m0 = fpgrad[2 * rec], m1 = fpgrad[2 * rec + 1];
+    const float4 m0 = n0, m1 = n1;
+    if (v + 1 < v1) {
+      n0 = fpgrad[2 * (rec + I.n)];
+      n1 = fpgrad[2 * (rec + I.n) + 1];
+    }
     if (m0.x == 0.f && m0.y == 0.f && m0.z == 0.f && m0.w == 0.f && m1.x == 0.f && m1.y == 0.f)
       continue;
     const ViewFrame f = frames[I.v_off + v];
     Fwd o;
     int x0, y0, x1, y1;
     if (!footprint(mr, sc, qt, f, I.W, I.H, b.cut2, b.eps, b.znear, o, x0, y0, x1, y1)) continue;
-    float gp[3], grho, gs3[3], gq[4];
-    chain_one(o, f, m0, m1, gp, grho, gs3, gq);
+    chain_one(o, f, m0, m1, gp, grho, gsc, gR);
+    any = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) qn[k] = o.qn[k];
+    inv_norm = o.inv_norm;
     if (stat) {
       // dI/dpx = A e (ca dx + cb dy) summed against dL/dI: the moments' first-order terms
       const float dpx = o.A * (o.ca * m0.y + o.cb * m0.z);
@@ -1101,17 +1156,14 @@ __global__ void __launch_bounds__(kThreads)
       const float nx = 0.5f * (float)I.W * dpx, ny = 0.5f * (float)I.H * dpy;
       st_acc += sqrtf(nx * nx + ny * ny);
     }
-    acc[0] += gp[0]; acc[1] += gp[1]; acc[2] += gp[2]; acc[3] += grho;
-    acc[4] += gs3[0]; acc[5] += gs3[1]; acc[6] += gs3[2];
-    acc[7] += gq[0]; acc[8] += gq[1]; acc[9] += gq[2]; acc[10] += gq[3];
   }
-  bool any = false;
-#pragma unroll
-  for (int k = 0; k < 11; ++k) any |= acc[k] != 0.f;
   if (any) {
-    atomicAdd(&g_mr[gi], make_float4(acc[0], acc[1], acc[2], acc[3]));
-    atomicAdd(&g_sc[gi], make_float4(acc[4], acc[5], acc[6], 0.f));
-    atomicAdd(&g_q[gi], make_float4(acc[7], acc[8], acc[9], acc[10]));
+    float gq[4];
+    gsd::rot_to_quat_grad(qn[0], qn[1], qn[2], qn[3], gR, gq);
+    gsd::quat_normalize_grad(qn, inv_norm, gq);
+    atomicAdd(&g_mr[gi], make_float4(gp[0], gp[1], gp[2], grho));
+    atomicAdd(&g_sc[gi], make_float4(gsc[0], gsc[1], gsc[2], 0.f));
+    atomicAdd(&g_q[gi], make_float4(gq[0], gq[1], gq[2], gq[3]));
   }
   if (stat) {
     if (st_acc != 0.f) atomicAdd(&stat[gi], st_acc);
@@ -1182,11 +1234,11 @@ int prepare(const gs_instance* inst, int n_inst, const gs_opts* o, const float* 
 
 // Dynamic shared memory above 48 KB needs the kernel's limit raised (host-side state of the
 // current device, set on every call that needs it).
-size_t emit_smem(const Plan& p) { return (size_t)(1 + kThreads / 32) * p.max_tiles * sizeof(uint32_t); }
+size_t emit_smem(const Plan& p) { return (size_t)(3 + kThreads / 32) * p.max_tp * sizeof(uint32_t); }
 
 int preprocess_and_scan(const Plan& p, const Layout& L, const float* mr, const float* sc,
                         const float* qt, const gs_view* views, cudaStream_t s, void* ws) {
-  const size_t smem = p.direct ? (size_t)p.max_tiles * sizeof(uint32_t) : 0;
+  const size_t smem = p.direct ? (size_t)p.max_tp * sizeof(uint32_t) : 0;
   GS_TRY(launch("preprocess", p.direct ? k_preprocess<true> : k_preprocess<false>,
                 dim3(p.nblocks), dim3(kThreads), smem, s, p.b, (const float4*)mr,
                 (const float4*)sc, (const float4*)qt, views, L.frames, L.geo, L.conic, L.rect,
@@ -1260,7 +1312,11 @@ int raster_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* img,
 template <int T>
 int raster_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float* dimg,
                cudaStream_t s) {
-  return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys),
+  // few tiles: their lists are split over up to 8 CTAs (the records' sums meet in atomics anyway),
+  // while the grid holds less than four CTAs per SM.  8 views of 64^2, 2000 Gaussians (128 tiles):
+  // 19 -> 11 us
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(8, 4 * (int64_t)num_sms() / p.n_keys));
+  return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys, parts),
                 dim3(BwdBlocks<T>::NT), 0, s,
                 p.b, (const uint2*)L.ranges, vals, (const float4*)L.geo, (const float4*)L.conic,
                 (const short4*)L.rect, dimg, L.fpgrad, (const gs_status*)L.st);
@@ -1386,12 +1442,15 @@ int gs_project_batch_backward_stats(const float* d_mean_rho, const float* d_scal
   }
   int max_nv = 1;
   for (int k = 0; k < p.b.count; ++k) max_nv = std::max(max_nv, p.b.in[k].nv);
-  const int vchunks = (max_nv + kChainViews - 1) / kChainViews;
+  int cv = kChainViews;  // halved while the chunks make less than two CTAs per SM
+  while (cv > 1 && (int64_t)p.total_n * ((max_nv + cv - 1) / cv) < 2 * (int64_t)num_sms() * kThreads)
+    cv /= 2;
+  const int vchunks = (max_nv + cv - 1) / cv;
   const int64_t threads = (int64_t)p.total_n * vchunks;
   const int blocks = (int)((threads + kThreads - 1) / kThreads);
   return launch("project_chain", k_project_chain, dim3(blocks), dim3(kThreads), 0, s, p.b,
                 (const float4*)d_mean_rho, (const float4*)d_scale, (const float4*)d_quat,
-                p.total_n, vchunks, (const ViewFrame*)L.frames, (const float4*)L.fpgrad,
+                p.total_n, vchunks, cv, (const ViewFrame*)L.frames, (const float4*)L.fpgrad,
                 (float4*)d_g_mean_rho, (float4*)d_g_scale, (float4*)d_g_quat,
                 (const uint32_t*)L.counts, d_grad_stat, (int*)d_vis);
 }

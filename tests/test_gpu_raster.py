@@ -308,3 +308,33 @@ def test_view_chunking_matches_single_call(gsct, monkeypatch):
         assert torch.allclose(a, b, rtol=1e-4, atol=1e-6 * float(a.abs().max()))
     assert many.count_evals(*d) == one.count_evals(*d)
     assert many.status().code == 0
+
+
+# both routes to the (view, tile) lists at their border (2048 tiles per view: 32 x 64 tiles of 8
+# pixels direct, one more tile column sorted), blocks of 256 records that end inside a view,
+# boxes of more than 32 tiles, and views without a record
+@pytest.mark.parametrize("W,H", [(256, 512), (264, 512), (250, 507)])
+@pytest.mark.parametrize("n,median", [(1, 0.2), (256, 0.02), (257, 0.05), (1500, 0.01)])
+def test_lists_of_both_routes(orc, gsct, W, H, n, median):
+    """Lists against the oracle's outside its guard band: the same pairs, every key's pairs in
+    record order, keys grouped by (tile, view)."""
+    tile = 8
+    mr, sc, qt, views = _case(n, n, 3, W, H, median=median)
+    views["src"][1, 2], views["det_center"][1, 2] = 40.0, 40.0  # this view sees nothing
+    P, V = orc.params64(mr, sc, qt), orc.views64(views)
+    keys_o, vals_o, _ = orc.keys(P, V, W, H, tile)
+    amb = (orc.pair_flags(P, V, W, H, REL_BAND, px_band(W, H), tile=tile) & 21) != 0
+    proj = gsct.Projector(views, W, H, tile=tile)
+    proj.forward(*to_dev(mr, sc, qt))
+    keys_g, recs_g = proj.read_pairs()
+    TWH, nv = ((W + 7) // 8) * ((H + 7) // 8), len(views)
+    tb = (TWH - 1).bit_length()
+    kd, rd = keys_g.astype(np.int64), recs_g.astype(np.int64)
+    v_g, t_g = kd >> tb, kd & ((1 << tb) - 1)
+    assert np.array_equal(rd // n, v_g) and not np.any(v_g == 1)
+    assert np.all(np.diff((t_g * nv + v_g) * n + rd % n) > 0)
+    ko, vo = keys_o.astype(np.int64), vals_o.astype(np.int64)
+    ko, vo = ko[~amb[ko // TWH, vo]], vo[~amb[ko // TWH, vo]]
+    keep = ~amb[v_g, rd % n]
+    want = np.sort((ko % TWH * nv + ko // TWH) * n + vo)
+    assert np.array_equal(want, ((t_g * nv + v_g) * n + rd % n)[keep])
