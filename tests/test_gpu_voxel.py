@@ -239,3 +239,29 @@ def test_brick_autotuner_picks_a_valid_side(gsct):
     best, times = tune_brick(synth.cube_grid(128), *to_dev(mr, sc, qt))
     assert best in (16, 32, 64) and set(times) == {16, 32, 64}
     assert all(t > 0 for t in times.values())
+
+
+# empty bricks inside and at the ragged ends of a region, rows that are and are not whole 16-byte
+# vectors, an output that is not 16-byte aligned; regions of one to many bricks per axis
+@pytest.mark.parametrize("lo,dim", [((0, 0, 0), (64, 48, 33)), ((5, 3, 2), (37, 50, 61)),
+                                    ((1, 0, 7), (64, 1, 17)), ((0, 0, 0), (1, 1, 1))])
+@pytest.mark.parametrize("brick", [16, 32, 64])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_empty_bricks_are_zeroed(orc, gsct, lo, dim, brick, shift):
+    """Gaussians in one corner only: voxels no Gaussian reaches are exactly 0, the others within
+    the volume tolerance of the oracle."""
+    import torch
+
+    mr, sc, qt = synth.gaussians(3, 60, radius=0.1, scale_median=0.03)
+    mr[:, :3] -= 0.75
+    grid = synth.cube_grid(72)
+    n = dim[0] * dim[1] * dim[2]
+    out = torch.full((n + shift,), float("nan"), device="cuda")[shift:].view(dim[2], dim[1], dim[0])
+    vox = gsct.Voxelizer(grid, lo, dim, brick=brick)
+    vox.forward(*to_dev(mr, sc, qt), out=out)
+    P = orc.params64(mr, sc, qt)
+    want, _ = orc.voxelize(P, grid, lo, dim)
+    allow = orc.voxelize_ambiguity(P, grid, lo, dim, REL_BAND, IDX_BAND)
+    got = out.cpu().numpy().astype(np.float64)
+    assert (np.abs(got - want) <= IMG_TOL * np.abs(want).max() + allow).all()
+    assert np.all(got[(want == 0) & (allow == 0)] == 0)
