@@ -19,6 +19,7 @@ namespace {
 
 __global__ void k_scan_block_sums(const uint32_t* __restrict__ sums, uint32_t* __restrict__ offs,
                                   int nb, gs_status* st, int64_t cap) {
+  gsd::pdl_begin();
   __shared__ unsigned long long warp_tot[32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int per = (nb + blockDim.x - 1) / blockDim.x;
@@ -75,6 +76,7 @@ template <bool LANE>
 __global__ void __launch_bounds__(kSortThreads)
     k_radix_hist(const uint32_t* __restrict__ keys, const gs_status* st, int shift, int dbits,
                  uint32_t* __restrict__ hist, int G) {
+  gsd::pdl_begin();
   extern __shared__ uint32_t sh_hist[];
   if (st->code != GS_OK) return;
   constexpr int NW = kSortThreads / 32;
@@ -137,6 +139,7 @@ __global__ void __launch_bounds__(kSortThreads)
 // One block per digit: exclusive scan over the G blocks' counts of that digit; totals[d].
 __global__ void k_radix_digit_scan(uint32_t* __restrict__ hist, uint32_t* __restrict__ totals,
                                    const gs_status* st, int G) {
+  gsd::pdl_begin();
   __shared__ uint32_t warp_tot[32];
   if (st->code != GS_OK) return;
   const int d = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -169,6 +172,7 @@ __global__ void __launch_bounds__(kSortThreads)
                     uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, const gs_status* st,
                     int shift, int dbits, const uint32_t* __restrict__ hist,
                     const uint32_t* __restrict__ totals, int G) {
+  gsd::pdl_begin();
   extern __shared__ uint32_t sh[];
   if (st->code != GS_OK) return;
   const int D = 1 << dbits;
@@ -286,6 +290,7 @@ __global__ void __launch_bounds__(kSortThreads)
 
 __global__ void k_ranges(const uint32_t* __restrict__ keys, uint2* __restrict__ ranges,
                          const gs_status* st) {
+  gsd::pdl_begin();
   if (st->code != GS_OK) return;
   const int64_t n = st->pairs;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -333,7 +338,7 @@ size_t sort_hist_words(const SortPlan& p) {
 int scan_block_sums(const uint32_t* block_sums, uint32_t* block_offsets, int nblocks,
                     gs_status* st, int64_t cap, cudaStream_t s) {
   if (nblocks < 0) return GS_ERR_ARG;
-  return launch("scan_block_sums", k_scan_block_sums, dim3(1), dim3(1024), 0, s, block_sums,
+  return launch_after("scan_block_sums", k_scan_block_sums, dim3(1), dim3(1024), 0, s, block_sums,
                 block_offsets, nblocks, st, cap);
 }
 
@@ -355,18 +360,18 @@ int radix_sort(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt, uint32_t* v
     const int D = 1 << db;
     uint32_t* totals = hist + (size_t)D * G;
     if (db <= kLaneHistMaxBits)
-      GS_TRY(launch("radix_hist", k_radix_hist<true>, dim3(G), dim3(kSortThreads),
+      GS_TRY(launch_after("radix_hist", k_radix_hist<true>, dim3(G), dim3(kSortThreads),
                     (size_t)(kSortThreads / 32) * D * 32 * sizeof(uint32_t), s,
                     (const uint32_t*)*keys, (const gs_status*)st, sh, db, hist, G));
     else
-      GS_TRY(launch("radix_hist", k_radix_hist<false>, dim3(G), dim3(kSortThreads),
+      GS_TRY(launch_after("radix_hist", k_radix_hist<false>, dim3(G), dim3(kSortThreads),
                     D * sizeof(uint32_t), s, (const uint32_t*)*keys, (const gs_status*)st, sh, db,
                     hist, G));
     const int scan_threads = (G + 31) / 32 * 32;
-    GS_TRY(launch("radix_digit_scan", k_radix_digit_scan, dim3(D), dim3(scan_threads), 0, s,
+    GS_TRY(launch_after("radix_digit_scan", k_radix_digit_scan, dim3(D), dim3(scan_threads), 0, s,
                   hist, totals, (const gs_status*)st, G));
     const size_t smem = scatter_smem_bytes(db);
-    GS_TRY(launch("radix_scatter", k_radix_scatter, dim3(G), dim3(kSortThreads), smem, s,
+    GS_TRY(launch_after("radix_scatter", k_radix_scatter, dim3(G), dim3(kSortThreads), smem, s,
                   (const uint32_t*)*keys, (const uint32_t*)*vals, keys_alt, vals_alt,
                   (const gs_status*)st, sh, db, (const uint32_t*)hist, (const uint32_t*)totals,
                   G));
@@ -376,13 +381,10 @@ int radix_sort(uint32_t** keys, uint32_t** vals, uint32_t* keys_alt, uint32_t* v
   return GS_OK;
 }
 
-int build_ranges(const uint32_t* keys, uint2* ranges, int64_t n_keys, gs_status* st, int64_t cap,
-                 cudaStream_t s) {
-  (void)cap;
-  GS_CUDA(cudaMemsetAsync(ranges, 0, (size_t)n_keys * sizeof(uint2), s));
+int build_ranges(const uint32_t* keys, uint2* ranges, gs_status* st, cudaStream_t s) {
   const int grid = 4 * num_sms();
-  return launch("ranges", k_ranges, dim3(grid), dim3(256), 0, s, keys, ranges,
-                (const gs_status*)st);
+  return launch_after("ranges", k_ranges, dim3(grid), dim3(256), 0, s, keys, ranges,
+                      (const gs_status*)st);
 }
 
 }  // namespace gs

@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(kThreads)
   q[i] = pq;
 }
 
-__global__ void k_step_incr(int* step) { *step += 1; }
+__global__ void k_step_incr(int* step) { gsd::pdl_begin(); *step += 1; }
 
 // dst += src over n floats (float4 body, scalar tail)
 __global__ void __launch_bounds__(kThreads)
@@ -1557,7 +1557,7 @@ int gs_adam_step(float* d_raw_mean_rho, float* d_raw_scale, float* d_raw_quat, f
                 (float4*)d_v, (const float4*)d_g_mean_rho, (const float4*)d_g_scale,
                 (const float4*)d_g_quat, (float4*)d_mean_rho, (float4*)d_scale, (float4*)d_quat,
                 n, (const int*)d_step, *opts));
-  return launch("step_incr", k_step_incr, dim3(1), dim3(1), 0, s, d_step);
+  return launch_after("step_incr", k_step_incr, dim3(1), dim3(1), 0, s, d_step);
 }
 
 int gs_activate(const float* d_raw_mean_rho, const float* d_raw_scale, const float* d_raw_quat,

@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(kGemmThreads)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base_sh;
+  gsd::pdl_begin();  // the barriers and the tensor memory are set up beside the previous kernel
 
   if (warp == 0 && lane == 0) {
     // producer
@@ -325,6 +326,7 @@ __global__ void k_relu_mask_bf16(float* __restrict__ g, const __nv_bfloat16* __r
 constexpr int kColsumCtas = 8;
 __global__ void __cluster_dims__(1, kColsumCtas, 1) __launch_bounds__(1024)
     k_colsum(const float* __restrict__ g, int rows, int cols, float* __restrict__ out) {
+  gsd::pdl_begin();
   __shared__ float part[32][33];
   __shared__ float cta_sum[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -362,7 +364,7 @@ __global__ void __cluster_dims__(1, kColsumCtas, 1) __launch_bounds__(1024)
 
 template <int BN, bool AMN, bool BMN>
 int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int K,
-                const GemmOut& o, int* err, cudaStream_t s) {
+                const GemmOut& o, int* err, bool after, cudaStream_t s) {
   using TT = GemmTile<BN>;
   int dev = 0;
   GS_CUDA(cudaGetDevice(&dev));
@@ -373,15 +375,18 @@ int launch_gemm(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int 
                                  (int)TT::kSmemBytes));
     attr_set[dev] = true;
   }
-  return launch("gemm_bf16", k_gemm<BN, AMN, BMN>, dim3(N / BN, M / kBM), dim3(kGemmThreads),
-                TT::kSmemBytes, s, ma, mb, M, N, K, o, err);
+  const dim3 grid(N / BN, M / kBM), block(kGemmThreads);
+  return after ? launch_after("gemm_bf16", k_gemm<BN, AMN, BMN>, grid, block, TT::kSmemBytes, s,
+                              ma, mb, M, N, K, o, err)
+               : launch("gemm_bf16", k_gemm<BN, AMN, BMN>, grid, block, TT::kSmemBytes, s, ma, mb,
+                        M, N, K, o, err);
 }
 
 }  // namespace
 
 int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm form,
               const float* d_bias, int relu, const void* d_mask, float* d_c32, void* d_c16,
-              int ldc, int* d_err, cudaStream_t s) {
+              int ldc, int* d_err, bool after, cudaStream_t s) {
   if (((uintptr_t)d_a & 15u) || ((uintptr_t)d_b & 15u)) return GS_ERR_ARG;
   // 128 x 256 tiles when N allows (A read once per pair of 128-column tiles) and the grid
   // still covers the SMs; narrower ones while the grid is under half of them (every tile shape
@@ -401,19 +406,26 @@ int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm fo
   GS_TRY(form == GEMM_TN ? make_map(&mb, d_b, N, K, bn) : make_map(&mb, d_b, K, N, kBK));
   switch (form) {
     case GEMM_TN:
-      if (bn == 256) return launch_gemm<256, false, false>(ma, mb, M, N, K, o, d_err, s);
-      if (bn == 128) return launch_gemm<128, false, false>(ma, mb, M, N, K, o, d_err, s);
-      if (bn == 64) return launch_gemm<64, false, false>(ma, mb, M, N, K, o, d_err, s);
-      return launch_gemm<32, false, false>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 256) return launch_gemm<256, false, false>(ma, mb, M, N, K, o, d_err, after, s);
+      if (bn == 128) return launch_gemm<128, false, false>(ma, mb, M, N, K, o, d_err, after, s);
+      if (bn == 64) return launch_gemm<64, false, false>(ma, mb, M, N, K, o, d_err, after, s);
+      return launch_gemm<32, false, false>(ma, mb, M, N, K, o, d_err, after, s);
     case GEMM_BMN:
-      if (bn == 256) return launch_gemm<256, false, true>(ma, mb, M, N, K, o, d_err, s);
-      if (bn == 128) return launch_gemm<128, false, true>(ma, mb, M, N, K, o, d_err, s);
-      return launch_gemm<64, false, true>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 256) return launch_gemm<256, false, true>(ma, mb, M, N, K, o, d_err, after, s);
+      if (bn == 128) return launch_gemm<128, false, true>(ma, mb, M, N, K, o, d_err, after, s);
+      return launch_gemm<64, false, true>(ma, mb, M, N, K, o, d_err, after, s);
     default:
-      if (bn == 256) return launch_gemm<256, true, true>(ma, mb, M, N, K, o, d_err, s);
-      if (bn == 128) return launch_gemm<128, true, true>(ma, mb, M, N, K, o, d_err, s);
-      return launch_gemm<64, true, true>(ma, mb, M, N, K, o, d_err, s);
+      if (bn == 256) return launch_gemm<256, true, true>(ma, mb, M, N, K, o, d_err, after, s);
+      if (bn == 128) return launch_gemm<128, true, true>(ma, mb, M, N, K, o, d_err, after, s);
+      return launch_gemm<64, true, true>(ma, mb, M, N, K, o, d_err, after, s);
   }
+}
+
+int colsum(const float* d_g, int rows, int cols, float* d_out, bool after, cudaStream_t s) {
+  if (!d_g || !d_out || rows < 0 || cols < 1) return GS_ERR_ARG;
+  const dim3 grid((cols + 31) / 32, kColsumCtas), block(1024);
+  return after ? launch_after("colsum", k_colsum, grid, block, 0, s, d_g, rows, cols, d_out)
+               : launch("colsum", k_colsum, grid, block, 0, s, d_g, rows, cols, d_out);
 }
 
 }  // namespace gs
@@ -428,7 +440,7 @@ int gs_gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, const fl
   if (M < 1 || N < 1 || K < kBK || K % kBK != 0 || M % kBM != 0 || N % kBN != 0 || ldc < N)
     return GS_ERR_ARG;
   return gemm_bf16(d_a, d_b, M, N, K, GEMM_TN, d_bias, relu, nullptr, d_c32, d_c16, ldc, d_err,
-                   (cudaStream_t)stream);
+                   false, (cudaStream_t)stream);
 }
 
 int gs_f32_to_bf16(const float* d_x, void* d_y, int64_t n, void* stream) {
@@ -455,9 +467,7 @@ int gs_relu_mask_bf16(float* d_g, const void* d_act, int64_t n, void* d_out, voi
 }
 
 int gs_colsum(const float* d_g, int rows, int cols, float* d_out, void* stream) {
-  if (!d_g || !d_out || rows < 0 || cols < 1) return GS_ERR_ARG;
-  return launch("colsum", k_colsum, dim3((cols + 31) / 32, kColsumCtas), dim3(1024), 0,
-                (cudaStream_t)stream, d_g, rows, cols, d_out);
+  return colsum(d_g, rows, cols, d_out, false, (cudaStream_t)stream);
 }
 
 }  // extern "C"

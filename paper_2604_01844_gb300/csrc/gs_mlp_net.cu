@@ -73,13 +73,14 @@ const uint16_t* w16_of(const void* w16, int li) {
 int forward(const float* params, const void* w16, const void* x16, int M, float* y,
             const NetLayout& L, int* err, void* stream) {
   const void* a = x16;
+  cudaStream_t s = (cudaStream_t)stream;
   for (int li = 0; li < 3; ++li) {
-    GS_TRY(gs_gemm_bf16(a, w16_of(w16, li), M, kHid, layer_in(li), params + bias_offset(li), 1,
-                        nullptr, L.h[li], kHid, err, stream));
+    GS_TRY(gemm_bf16(a, w16_of(w16, li), M, kHid, layer_in(li), GEMM_TN, params + bias_offset(li),
+                     1, nullptr, nullptr, L.h[li], kHid, err, li > 0, s));
     a = L.h[li];
   }
-  return gs_gemm_bf16(a, w16_of(w16, 3), M, kOutPad, kHid, params + bias_offset(3), 0, y,
-                      nullptr, kOutPad, err, stream);
+  return gemm_bf16(a, w16_of(w16, 3), M, kOutPad, kHid, GEMM_TN, params + bias_offset(3), 0,
+                   nullptr, y, nullptr, kOutPad, err, true, s);
 }
 
 // Backward from dL/dy through the four layers into grad (parameter layout): bias gradients
@@ -96,12 +97,12 @@ int backward(const void* w16, const void* x16, int M, const float* dy, float* gr
   int width = kOutPad;
   for (int li = kLayers - 1; li >= 0; --li) {
     const int k_in = layer_in(li);
-    GS_TRY(gs_colsum(g32, M, width, grad + bias_offset(li), stream));
+    GS_TRY(colsum(g32, M, width, grad + bias_offset(li), true, s));
     GS_TRY(gemm_bf16(g16, acts[li], width, k_in, M, GEMM_MN, nullptr, 0, nullptr,
-                     grad + weight_offset(li), nullptr, k_in, err, s));
+                     grad + weight_offset(li), nullptr, k_in, err, true, s));
     if (li == 0) break;
     GS_TRY(gemm_bf16(g16, w16_of(w16, li), M, k_in, width, GEMM_BMN, nullptr, 0, L.h[li - 1],
-                     L.gp[li], L.g16[li], k_in, err, s));
+                     L.gp[li], L.g16[li], k_in, err, true, s));
     g32 = L.gp[li];
     g16 = L.g16[li];
     width = k_in;

@@ -421,6 +421,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
                uint2* __restrict__ ranges, unsigned long long* __restrict__ gsum, uint32_t* ticket,
                long long* __restrict__ vkeys, int total_v, gs_status* st, int64_t cap,
                int64_t vals_off, int64_t ranges_off, int64_t vkeys_off) {
+  gsd::pdl_begin();
   __shared__ uint32_t part[kScanSegs][kScanKeys];
   __shared__ unsigned long long wtot[kScanKeys * kScanSegs / 32];
   __shared__ bool last;
@@ -1113,6 +1114,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                     float4* __restrict__ g_sc, float4* __restrict__ g_q,
                     const uint32_t* __restrict__ counts, float* __restrict__ stat,
                     int* __restrict__ vis) {
+  gsd::pdl_begin();
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (tid >= (int64_t)total_n * vchunks) return;
   const int gi = (int)(tid % total_n), ch = (int)(tid / total_n);
@@ -1245,7 +1247,7 @@ int preprocess_and_scan(const Plan& p, const Layout& L, const float* mr, const f
                 L.tmask, L.counts, L.block_sums, L.tcount, L.ticket, L.st));
   if (!p.direct) return scan_block_sums(L.block_sums, L.block_offs, p.nblocks, L.st, p.cap, s);
   auto off = [&](const void* q) { return (int64_t)((const char*)q - (const char*)ws); };
-  return launch("key_scan", k_key_scan, dim3((unsigned)((p.n_keys + kScanKeys - 1) / kScanKeys)),
+  return launch_after("key_scan", k_key_scan, dim3((unsigned)((p.n_keys + kScanKeys - 1) / kScanKeys)),
                 dim3(kScanKeys * kScanSegs), 0, s, p.b, p.n_keys, (const uint16_t*)L.tcount,
                 L.toffset, L.klocal, L.ranges, L.gsum, L.ticket, L.vkeys, p.total_v, L.st, p.cap,
                 off(L.vals), off(L.ranges), off(L.vkeys));
@@ -1448,7 +1450,7 @@ int gs_project_batch_backward_stats(const float* d_mean_rho, const float* d_scal
   const int vchunks = (max_nv + cv - 1) / cv;
   const int64_t threads = (int64_t)p.total_n * vchunks;
   const int blocks = (int)((threads + kThreads - 1) / kThreads);
-  return launch("project_chain", k_project_chain, dim3(blocks), dim3(kThreads), 0, s, p.b,
+  return launch_after("project_chain", k_project_chain, dim3(blocks), dim3(kThreads), 0, s, p.b,
                 (const float4*)d_mean_rho, (const float4*)d_scale, (const float4*)d_quat,
                 p.total_n, vchunks, cv, (const ViewFrame*)L.frames, (const float4*)L.fpgrad,
                 (float4*)d_g_mean_rho, (float4*)d_g_scale, (float4*)d_g_quat,

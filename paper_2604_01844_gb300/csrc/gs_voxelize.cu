@@ -235,13 +235,16 @@ __global__ void __launch_bounds__(kThreads)
                gs_status* st,
                float4* __restrict__ geo, float4* __restrict__ cov0, float4* __restrict__ cov1,
                short4* __restrict__ lo_out, short4* __restrict__ hi_out,
-               uint32_t* __restrict__ counts, uint32_t* __restrict__ block_sums) {
+               uint32_t* __restrict__ counts, uint32_t* __restrict__ block_sums,
+               uint2* __restrict__ ranges, int64_t n_keys) {
   __shared__ uint32_t warp_sums[kThreads / 32];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->code = GS_OK;
     st->pairs = 0;
   }
   const int i = blockIdx.x * kThreads + threadIdx.x;
+  // every brick starts empty
+  for (int64_t k = i; k < n_keys; k += (int64_t)gridDim.x * kThreads) ranges[k] = make_uint2(0u, 0u);
   uint32_t cnt = 0;
   if (i < n) {
     const VGrid& g = bt.in[inst_of_gaussian(bt, i)].g;
@@ -307,6 +310,7 @@ __global__ void __launch_bounds__(kThreads)
                const uint32_t* __restrict__ block_offs, int n, int64_t n_keys,
                uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, gs_status* st,
                int64_t sorted_keys_off, int64_t sorted_vals_off) {
+  gsd::pdl_begin();
   __shared__ uint32_t warp_pre[kThreads / 32];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->reserved[0] = sorted_keys_off;
@@ -777,6 +781,7 @@ __global__ void __launch_bounds__(kThreads)
                 const float4* __restrict__ quat, int n, const float4* __restrict__ vgrad,
                 float4* __restrict__ g_mr, float4* __restrict__ g_sc, float4* __restrict__ g_q,
                 int accumulate) {
+  gsd::pdl_begin();
   const int i = blockIdx.x * kThreads + threadIdx.x;
   if (i >= n) return;
   const float4 a = vgrad[3 * i], b = vgrad[3 * i + 1], c = vgrad[3 * i + 2];
@@ -870,7 +875,7 @@ int prep_and_scan(const Plan& p, const Layout& L, const float* mr, const float* 
                   const float* qt, cudaStream_t s) {
   GS_TRY(launch("vox_prep", k_vox_prep, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
                 (const float4*)mr, (const float4*)sc, (const float4*)qt, p.n, L.st, L.geo,
-                L.cov0, L.cov1, L.lo, L.hi, L.counts, L.block_sums));
+                L.cov0, L.cov1, L.lo, L.hi, L.counts, L.block_sums, L.ranges, p.n_keys));
   return scan_block_sums(L.block_sums, L.block_offs, p.nblocks, L.st, p.cap, s);
 }
 
@@ -888,14 +893,14 @@ int bin_bricks(const Plan& p, const Layout& L, const float* mr, const float* sc,
   const bool odd = (p.sort.passes & 1) != 0;
   uint32_t* fk = odd ? L.keys_alt : L.keys;
   uint32_t* fv = odd ? L.vals_alt : L.vals;
-  GS_TRY(launch("vox_emit", k_vox_emit, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
+  GS_TRY(launch_after("vox_emit", k_vox_emit, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
                 (const uint32_t*)L.counts, (const short4*)L.lo, (const short4*)L.hi,
                 (const uint32_t*)L.block_offs, p.n, p.n_keys, L.keys, L.vals, L.st,
                 (int64_t)((char*)fk - (char*)ws), (int64_t)((char*)fv - (char*)ws)));
   uint32_t* k = L.keys;
   uint32_t* v = L.vals;
   GS_TRY(radix_sort(&k, &v, L.keys_alt, L.vals_alt, L.hist, p.sort, L.st, p.cap, s));
-  GS_TRY(build_ranges(k, L.ranges, p.n_keys, L.st, p.cap, s));
+  GS_TRY(build_ranges(k, L.ranges, L.st, s));
   *skeys = k;
   *svals = v;
   return GS_OK;
@@ -1011,7 +1016,7 @@ int gs_voxelize_batch_backward(const float* d_mean_rho, const float* d_scale,
                 (const uint2*)L.ranges, (const uint32_t*)v, (const float4*)L.geo,
                 (const float4*)L.cov0, (const float4*)L.cov1, (const short4*)L.lo,
                 (const short4*)L.hi, p.b, d_dvol, L.vgrad, (const gs_status*)L.st));
-  return launch("vox_chain", k_vox_chain, dim3(p.nblocks), dim3(kThreads), 0, s,
+  return launch_after("vox_chain", k_vox_chain, dim3(p.nblocks), dim3(kThreads), 0, s,
                 (const float4*)d_mean_rho, (const float4*)d_scale, (const float4*)d_quat, p.n,
                 (const float4*)L.vgrad, (float4*)d_g_mean_rho, (float4*)d_g_scale,
                 (float4*)d_g_quat, accumulate);
