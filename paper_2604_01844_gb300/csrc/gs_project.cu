@@ -792,27 +792,39 @@ struct BlockShape {
 template <int T>
 using BwdBlocks = BlockShape<T, (T >= 16 ? 16 : 8)>;
 
-// Raster forward (and the in-cut evaluation counter) with records on lanes, one warp per
-// 4 x BW block of the (view, tile).  Per batch of staged records each warp lists the records
-// whose cut ellipse reaches its block (the block masks of the backward) and takes them one per
-// lane; every lane walks the block's pixels in the same unrolled order (pixel pairs in packed
-// FP32x2 arithmetic, the exponent and the cut exactly as the backward computes them) and adds
-// A 2^e to its own accumulator of each pixel.  The accumulators live through all batches; at
-// the end one butterfly reduce-scatter over the warp's lanes sums them per pixel, lane l
-// keeping pixels 2l and 2l + 1.  A pixel's sum is thus taken in a fixed order: per lane in
-// list order, then over the lanes.
+// Raster forward (and the in-cut evaluation counter) with records on lanes, LPB lanes per
+// 4 x BW block of the (view, tile), 32 / LPB vertically adjacent blocks per warp.  Per batch of
+// staged records each warp lists the records whose cut ellipse reaches each of its blocks (the
+// block masks of the backward); the LPB lanes of a block take its records one per lane, and every
+// lane walks the block's pixels in the same unrolled order (pixel pairs in packed FP32x2
+// arithmetic, the exponent and the cut exactly as the backward computes them) and adds A 2^e to
+// its own accumulator of each pixel.  The accumulators live through all batches; at the end one
+// butterfly reduce-scatter over the block's lanes sums them per pixel, lane l keeping NPR / LPB
+// consecutive pairs.  A pixel's sum is thus taken in a fixed order: per lane in list order, then
+// over the lanes.
+// Bound by issue and latency (64 accumulators leave 16 warps per SM).  Fewer lanes per block make
+// the reduction cheaper per pixel (with 32 lanes it is 12 % of the instructions at 75 x 512^2) and
+// the tile's CTA smaller, so that more CTAs load and walk independently on an SM; but a warp
+// walks as long as the longest of its blocks' lists.  75 x 1024^2, tile 32: 32 lanes 6.48 ms (one
+// CTA of 16 warps per SM, idle while it loads), 16 lanes 5.14, 8 lanes 4.49, 4 lanes 4.70, with
+// 4 records staged per thread and batch (3: 4.58, 6: 4.82; the rest of the SM's memory caches the
+// gathers).  30 x 512^2, tile 8: 32 lanes 0.57, 16 lanes 0.48 ms.  Tiles of 16 keep 32 lanes: 16
+// would take 1.00 -> 0.88 ms at 75 x 512^2, but in another order of the sums, and the L1 term of
+// a reconstruction step turns last-bit differences into flipped signs of its gradient.
 template <int T>
 struct FwdBlocks {
   static constexpr int BW = T >= 16 ? 16 : 8;  // block width; 4 rows
   static constexpr int LBW = BW == 16 ? 4 : 3;
   static constexpr int NBX = T / BW, NBY = T / 4, NB = NBX * NBY;
-  static constexpr int NW = NB;  // one block per warp
+  static constexpr int LPB = T == 32 ? 8 : T == 16 ? 32 : 16;  // lanes per block
+  static constexpr int BPW = 32 / LPB;             // blocks per warp, one above the other
+  static constexpr int NW = NB / BPW;
   static constexpr int NT = 32 * NW;
-  static constexpr int SB = (T == 32 ? 2 : 4) * NT;  // records staged per batch
+  static constexpr int SB = (T == 8 ? 8 : 4) * NT;  // records staged per batch
 };
 
 template <int T, bool COUNT>
-__global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlocks<T>::NT)
+__global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
     k_raster_fwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
                  const uint32_t* __restrict__ vals, const float4* __restrict__ geo,
                  const float4* __restrict__ conic, const short4* __restrict__ rect,
@@ -822,7 +834,7 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlock
   __shared__ float4 s_geo[S::SB];
   __shared__ float4 s_con[S::SB];
   __shared__ uint32_t s_mask[S::SB];
-  __shared__ uint16_t s_list[S::NW][S::SB];
+  __shared__ uint16_t s_list[S::NB][S::SB];
   __shared__ unsigned long long s_cnt;
   const int64_t key = blockIdx.x;
   const uint2 r = ranges[key];  // requested together with the status word, not after it
@@ -833,7 +845,11 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlock
   const int W = I.W, H = I.H;
   const int tx0 = (tile % I.TW) * T, ty0 = (tile / I.TW) * T;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int bxl = (w % S::NBX) * BW, byl = (w / S::NBX) * 4;  // the warp's block in the tile
+  constexpr int LPB = S::LPB, BPW = S::BPW;
+  const int part = lane / LPB, lp = lane % LPB;
+  // the warp's blocks bit0 (half 0) and bit0 + NBX (half 1, the block below)
+  const int bit0 = (w / S::NBX) * BPW * S::NBX + w % S::NBX;
+  const int bxl = (w % S::NBX) * BW, byl = ((w / S::NBX) * BPW + part) * 4;
   const float fx0 = (float)(tx0 + bxl), fy0 = (float)(ty0 + byl);
   const unsigned lt = gsd::lanemask_lt();
   constexpr int NPR = 4 * HP;  // float2 accumulators per lane: pair ry * HP + p
@@ -845,27 +861,48 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlock
   for (uint32_t base = r.x; base < r.y; base += S::SB) {
     const int m = (int)min((uint32_t)S::SB, r.y - base);
     __syncthreads();
-    for (int q = t; q < m; q += S::NT) {
-      const uint32_t rec = vals[base + q];
-      const float4 g = geo[rec], c = conic[rec];
-      s_geo[q] = g;
-      s_con[q] = c;
-      s_mask[q] = block_mask<T, BW, S::LBW, S::NBX, S::NBY>(g, c, rect[rec], tx0, ty0);
+    // two records per thread at a time, so that their gathers overlap
+    for (int q = t; q < m; q += 2 * S::NT) {
+      const bool two = q + S::NT < m;
+      const uint32_t rec0 = vals[base + q], rec1 = two ? vals[base + q + S::NT] : rec0;
+      const float4 g0 = geo[rec0], c0 = conic[rec0], g1 = geo[rec1], c1 = conic[rec1];
+      const short4 b0 = rect[rec0], b1 = rect[rec1];
+      s_geo[q] = g0;
+      s_con[q] = c0;
+      s_mask[q] = block_mask<T, BW, S::LBW, S::NBX, S::NBY>(g0, c0, b0, tx0, ty0);
+      if (two) {
+        s_geo[q + S::NT] = g1;
+        s_con[q + S::NT] = c1;
+        s_mask[q + S::NT] = block_mask<T, BW, S::LBW, S::NBX, S::NBY>(g1, c1, b1, tx0, ty0);
+      }
     }
     __syncthreads();
-    int cnt = 0;
+    int cnts[BPW];
+#pragma unroll
+    for (int k = 0; k < BPW; ++k) cnts[k] = 0;
     for (int j0 = 0; j0 < m; j0 += 32) {
       const int jl = j0 + lane;
-      const bool hit = jl < m && ((s_mask[jl] >> w) & 1u);
-      const unsigned bits = __ballot_sync(0xffffffffu, hit);
-      if (hit) s_list[w][cnt + __popc(bits & lt)] = (uint16_t)jl;
-      cnt += __popc(bits);
+      const uint32_t mk = jl < m ? s_mask[jl] >> bit0 : 0u;
+#pragma unroll
+      for (int k = 0; k < BPW; ++k) {
+        const bool hit = (mk >> (k * S::NBX)) & 1u;
+        const unsigned bits = __ballot_sync(0xffffffffu, hit);
+        if (hit) s_list[BPW * w + k][cnts[k] + __popc(bits & lt)] = (uint16_t)jl;
+        cnts[k] += __popc(bits);
+      }
     }
     __syncwarp();
-    for (int c0 = 0; c0 < cnt; c0 += 32) {
-      const int li = c0 + lane;
+    const uint16_t* list = s_list[BPW * w + part];
+    int cnt = 0, most = 0;
+#pragma unroll
+    for (int k = 0; k < BPW; ++k) {
+      cnt = part == k ? cnts[k] : cnt;
+      most = max(most, cnts[k]);
+    }
+    for (int c0 = 0; c0 < most; c0 += LPB) {
+      const int li = c0 + lp;
       const bool active = li < cnt;
-      const int j = active ? s_list[w][li] : 0;
+      const int j = active ? list[li] : 0;
       const float4 g = s_geo[j];
       const float4 c = s_con[j];
       const float cut = active ? g.w : 1.f;  // e <= 0 < 1: an idle lane never passes
@@ -905,36 +942,32 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlock
     __syncthreads();
     if (t == 0 && s_cnt) atomicAdd((unsigned long long*)&st->evals, s_cnt);
   } else {
-    // butterfly reduce-scatter of the warp's 4 x BW pixel sums: at each stage a lane keeps the
+    // butterfly reduce-scatter of the half's 4 x BW pixel sums: at each stage a lane keeps the
     // half of its pairs on its side of the partner bit and adds the partner's copy of that half;
-    // after log2(NPR) stages lane l holds the sum of pair l % NPR over its group of NPR lanes
+    // after four stages lane l holds the sums of pairs l NPR / 16 and up
+    constexpr int KEEP = NPR / LPB;
 #pragma unroll
-    for (int half = NPR / 2; half >= 1; half >>= 1) {
-      const bool up = (lane & half) != 0;
+    for (int bit = LPB / 2, n = NPR / 2; bit >= 1; bit >>= 1, n >>= 1) {
+      const bool up = (lane & bit) != 0;
 #pragma unroll
-      for (int i = 0; i < half; ++i) {
-        const float2 mine = up ? acc[i + half] : acc[i];
-        const float2 send = up ? acc[i] : acc[i + half];
+      for (int i = 0; i < n; ++i) {
+        const float2 mine = up ? acc[i + n] : acc[i];
+        const float2 send = up ? acc[i] : acc[i + n];
         float2 recv;
-        recv.x = __shfl_xor_sync(0xffffffffu, send.x, half);
-        recv.y = __shfl_xor_sync(0xffffffffu, send.y, half);
+        recv.x = __shfl_xor_sync(0xffffffffu, send.x, bit);
+        recv.y = __shfl_xor_sync(0xffffffffu, send.y, bit);
         acc[i] = __fadd2_rn(mine, recv);
       }
     }
-    // fewer pairs than lanes (BW = 8): the groups' sums are added across the remaining bits
-#pragma unroll
-    for (int k = NPR; k < 32; k <<= 1) {
-      const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, acc[0].x, k),
-                                   __shfl_xor_sync(0xffffffffu, acc[0].y, k));
-      acc[0] = __fadd2_rn(acc[0], o);
-    }
-    const int pi = lane % NPR;  // pair index: row pi / HP, columns 2 (pi % HP) + {0, 1}
-    if (lane >= NPR) return;
+    const int pi = lp * KEEP;  // first pair: row pi / HP, columns 2 (pi % HP) and up
     const int y = ty0 + byl + pi / HP, x = tx0 + bxl + 2 * (pi % HP);
     if (y >= H) return;
     float* row = img + I.img_off + ((int64_t)v * H + y) * W;
-    if (x < W) row[x] = acc[0].x;
-    if (x + 1 < W) row[x + 1] = acc[0].y;
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {
+      if (x + 2 * k < W) row[x + 2 * k] = acc[k].x;
+      if (x + 2 * k + 1 < W) row[x + 2 * k + 1] = acc[k].y;
+    }
   }
 }
 
@@ -953,7 +986,7 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, T == 32 ? 1 : 512 / FwdBlock
 // record's moments (two float4 atomics).
 // ------------------------------------------------------------------------------------------
 template <int T>
-__global__ void __launch_bounds__(BwdBlocks<T>::NT, T == 32 ? 3 : 1024 / BwdBlocks<T>::NT)
+__global__ void __launch_bounds__(BwdBlocks<T>::NT, 1024 / BwdBlocks<T>::NT)
     k_raster_bwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
                  const uint32_t* __restrict__ vals, const float4* __restrict__ geo,
                  const float4* __restrict__ conic, const short4* __restrict__ rect,
