@@ -92,8 +92,9 @@ __device__ __forceinline__ int inst_of_gaussian(const Batch& b, int g) {
 struct Layout {
   gs_status* st = nullptr;
   ViewFrame* frames = nullptr;
-  float4* geo = nullptr;    // (px, py, A, e_cut): e_cut = -1/2 log2(e) * Q
-  float4* conic = nullptr;  // -1/2 log2(e) * (a, 2b, c, 0): exponent = a'dx^2 + b'dx dy + c'dy^2
+  // two float4 per record, one 32-byte sector: (px, py, A, e_cut), e_cut = -1/2 log2(e) * Q, and
+  // -1/2 log2(e) * (a, 2b, c, 0): exponent = a'dx^2 + b'dx dy + c'dy^2
+  float4* rec = nullptr;
   short4* rect = nullptr;   // clipped inclusive pixel box (x0, y0, x1, y1); x0 > x1 if culled
   uint32_t* tmask = nullptr;  // tight tile rule answers for the box's first 32 tiles
   uint32_t* counts = nullptr;
@@ -189,8 +190,7 @@ Layout carve(void* ws, const Plan& p) {
   Layout L;
   L.st = c.take<gs_status>(1);
   L.frames = c.take<ViewFrame>(p.total_v);
-  L.geo = c.take<float4>(p.items);
-  L.conic = c.take<float4>(p.items);
+  L.rec = c.take<float4>(2 * p.items);
   L.rect = c.take<short4>(p.items);
   L.tmask = c.take<uint32_t>(p.items);
   L.counts = c.take<uint32_t>(p.items);
@@ -286,8 +286,8 @@ __device__ __forceinline__ void row_tiles(const Ell& E, int lT, int ty, int x0, 
 constexpr int kMaskTiles = 32;
 // Calls f(ty, ta, tb) for every tile row of a record's box with listed tiles ta .. tb.
 template <typename F>
-__device__ __forceinline__ void listed_rows(const short4 r, uint32_t tm, const float4* geo,
-                                            const float4* conic, size_t idx, int lT, F f) {
+__device__ __forceinline__ void listed_rows(const short4 r, uint32_t tm, const float4* rec,
+                                            size_t idx, int lT, F f) {
   const int tx0 = r.x >> lT, ty0 = r.y >> lT;
   const int ntx = (r.z >> lT) - tx0 + 1, nty = (r.w >> lT) - ty0 + 1;
   if (ntx * nty <= kMaskTiles) {
@@ -300,7 +300,7 @@ __device__ __forceinline__ void listed_rows(const short4 r, uint32_t tm, const f
       }
     }
   } else {
-    const Ell E = make_ell(geo[idx], conic[idx]);
+    const Ell E = make_ell(rec[2 * idx], rec[2 * idx + 1]);
     for (int ty = ty0; ty < ty0 + nty; ++ty) {
       int ta, tb;
       row_tiles(E, lT, ty, r.x, r.y, r.z, r.w, ta, tb);
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kThreads)
     k_preprocess(const __grid_constant__ Batch b, const float4* __restrict__ mean_rho,
                  const float4* __restrict__ scale, const float4* __restrict__ quat,
                  const gs_view* __restrict__ views, ViewFrame* __restrict__ frames,
-                 float4* __restrict__ geo, float4* __restrict__ conic, short4* __restrict__ rect,
+                 float4* __restrict__ rec, short4* __restrict__ rect,
                  uint32_t* __restrict__ tmask, uint32_t* __restrict__ counts,
                  uint32_t* __restrict__ block_sums, uint16_t* __restrict__ tcount,
                  uint32_t* __restrict__ ticket, gs_status* st) {
@@ -372,12 +372,11 @@ __global__ void __launch_bounds__(kThreads)
           for (int t = ty * I.TW + ta; t <= ty * I.TW + tb; ++t) atomicAdd(&s_tiles[t], 1u);
       }
       tmask[idx] = tm;
-      geo[idx] = gg;
-      conic[idx] = cc;
+      rec[2 * idx] = gg;
+      rec[2 * idx + 1] = cc;
       rect[idx] = make_short4((short)x0, (short)y0, (short)x1, (short)y1);
     } else {
-      geo[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
-      conic[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
+      rec[2 * idx] = rec[2 * idx + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
       rect[idx] = make_short4(1, 1, 0, 0);
     }
     counts[idx] = cnt;
@@ -526,7 +525,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
 // stores of a list's neighbourhood meet in L2.
 __global__ void __launch_bounds__(kThreads)
     k_emit_direct(const __grid_constant__ Batch b, const uint32_t* __restrict__ counts,
-                  const float4* __restrict__ geo, const float4* __restrict__ conic,
+                  const float4* __restrict__ rec,
                   const short4* __restrict__ rect, const uint32_t* __restrict__ tmask,
                   const uint32_t* __restrict__ toffset, const uint32_t* __restrict__ klocal,
                   const unsigned long long* __restrict__ gsum, uint2* __restrict__ ranges,
@@ -555,7 +554,7 @@ __global__ void __launch_bounds__(kThreads)
   const uint32_t bit = 1u << lane;
   uint32_t* mine = lanes + w * tp;
   if (cnt)
-    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
+    listed_rows(r, tm, rec, idx, b.lT, [&](int ty, int ta, int tb) {
       uint32_t* q = mine + ty * I.TW;
       for (int k = ta; k <= tb; ++k) atomicOr(q + k, bit);
     });
@@ -582,7 +581,7 @@ __global__ void __launch_bounds__(kThreads)
   __syncthreads();
   const uint8_t* pre = reinterpret_cast<const uint8_t*>(before) + w;
   if (cnt)
-    listed_rows(r, tm, geo, conic, idx, b.lT, [&](int ty, int ta, int tb) {
+    listed_rows(r, tm, rec, idx, b.lT, [&](int ty, int ta, int tb) {
       for (int k = ty * I.TW + ta; k <= ty * I.TW + tb; ++k)
         vals[first[k] + pre[8 * k] + __popc(mine[k] & (bit - 1u))] = (uint32_t)idx;
     });
@@ -594,7 +593,7 @@ __global__ void __launch_bounds__(kThreads)
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads)
     k_emit(const __grid_constant__ Batch b, const uint32_t* __restrict__ counts,
-           const float4* __restrict__ geo, const float4* __restrict__ conic,
+           const float4* __restrict__ rec,
            const short4* __restrict__ rect, const uint32_t* __restrict__ tmask,
            const uint32_t* __restrict__ block_offs,
            uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
@@ -667,7 +666,7 @@ __global__ void __launch_bounds__(kThreads)
   }
   if (cnt == 0 || small) return;
   uint32_t off = wbase + excl;
-  listed_rows(r, tm, geo, conic, idx, lT, [&](int ty, int ta, int tb) {
+  listed_rows(r, tm, rec, idx, lT, [&](int ty, int ta, int tb) {
     for (int tx = ta; tx <= tb; ++tx, ++off) {
       keys[off] = kbase + (uint32_t)(ty * TW + tx);
       vals[off] = (uint32_t)idx;
@@ -736,21 +735,23 @@ __device__ __forceinline__ float row_c(const float4 c, float dy) { return (c.z *
 struct SlabExt {
   float dyt, dxt;  // the ellipse's top point relative to its centre (bottom = -top)
 };
+// (Approximate reciprocals and roots, within two ulp: far inside the 1/100 pixel.)
 __device__ __forceinline__ SlabExt make_slab(const float4 c, float cm) {
-  const float kz = c.z - c.y * c.y * (0.25f / c.x);  // < 0
-  const float dyt = sqrtf(fmaxf(cm / kz, 0.f));
-  return SlabExt{dyt, -c.y * dyt * (0.5f / c.x)};
+  const float ia = rcp_approx(c.x);
+  const float kz = fmaf(-0.25f * c.y * c.y, ia, c.z);  // < 0
+  const float dyt = sqrt_approx(fmaxf(cm * rcp_approx(kz), 0.f));
+  return SlabExt{dyt, -0.5f * c.y * dyt * ia};
 }
 __device__ __forceinline__ void slab_rows(const float4 g, const float4 c, float cm,
                                           const SlabExt& X, float x0, float x1, int ty0, int T,
                                           int& ylo, int& yhi) {
   const float u0 = x0 - g.x, u1 = x1 - g.x;
-  const float inv2c = 0.5f / c.z;  // < 0
+  const float inv2c = 0.5f * rcp_approx(c.z);  // < 0
   const float xu = fminf(fmaxf(X.dxt, u0), u1), xl = fminf(fmaxf(-X.dxt, u0), u1);
   const float Du = fmaxf(fmaf(c.y * xu, c.y * xu, -4.f * c.z * fmaf(c.x * xu, xu, -cm)), 0.f);
   const float Dl = fmaxf(fmaf(c.y * xl, c.y * xl, -4.f * c.z * fmaf(c.x * xl, xl, -cm)), 0.f);
-  const float ymax = (-c.y * xu - sqrtf(Du)) * inv2c;
-  const float ymin = (-c.y * xl + sqrtf(Dl)) * inv2c;
+  const float ymax = (-c.y * xu - sqrt_approx(Du)) * inv2c;
+  const float ymin = (-c.y * xl + sqrt_approx(Dl)) * inv2c;
   ylo = max(0, (int)ceilf(g.y + ymin - 0.01f) - ty0);
   yhi = min(T - 1, (int)floorf(g.y + ymax + 0.01f) - ty0);
 }
@@ -811,6 +812,9 @@ using BwdBlocks = BlockShape<T, (T >= 16 ? 16 : 8)>;
 // gathers).  30 x 512^2, tile 8: 32 lanes 0.57, 16 lanes 0.48 ms.  Tiles of 16 keep 32 lanes: 16
 // would take 1.00 -> 0.88 ms at 75 x 512^2, but in another order of the sums, and the L1 term of
 // a reconstruction step turns last-bit differences into flipped signs of its gradient.
+// Staging (two dependent gathers per record and its block mask) is about 30 % of the kernel:
+// records as one 32-byte sector, two gathers in flight per thread and approximate roots in the
+// mask took tile 16 from 1.00 to 0.93 ms and tile 32 from 4.49 to 4.34.
 template <int T>
 struct FwdBlocks {
   static constexpr int BW = T >= 16 ? 16 : 8;  // block width; 4 rows
@@ -826,8 +830,8 @@ struct FwdBlocks {
 template <int T, bool COUNT>
 __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
     k_raster_fwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
-                 const uint32_t* __restrict__ vals, const float4* __restrict__ geo,
-                 const float4* __restrict__ conic, const short4* __restrict__ rect,
+                 const uint32_t* __restrict__ vals, const float4* __restrict__ recs,
+                 const short4* __restrict__ rect,
                  float* __restrict__ img, gs_status* st) {
   using S = FwdBlocks<T>;
   constexpr int BW = S::BW, HP = BW / 2;  // pixel pairs per row
@@ -865,7 +869,8 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
     for (int q = t; q < m; q += 2 * S::NT) {
       const bool two = q + S::NT < m;
       const uint32_t rec0 = vals[base + q], rec1 = two ? vals[base + q + S::NT] : rec0;
-      const float4 g0 = geo[rec0], c0 = conic[rec0], g1 = geo[rec1], c1 = conic[rec1];
+      const float4 g0 = recs[2 * (size_t)rec0], c0 = recs[2 * (size_t)rec0 + 1];
+      const float4 g1 = recs[2 * (size_t)rec1], c1 = recs[2 * (size_t)rec1 + 1];
       const short4 b0 = rect[rec0], b1 = rect[rec1];
       s_geo[q] = g0;
       s_con[q] = c0;
@@ -988,8 +993,8 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 template <int T>
 __global__ void __launch_bounds__(BwdBlocks<T>::NT, 1024 / BwdBlocks<T>::NT)
     k_raster_bwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
-                 const uint32_t* __restrict__ vals, const float4* __restrict__ geo,
-                 const float4* __restrict__ conic, const short4* __restrict__ rect,
+                 const uint32_t* __restrict__ vals, const float4* __restrict__ recs,
+                 const short4* __restrict__ rect,
                  const float* __restrict__ dimg, float4* __restrict__ fpgrad,
                  const gs_status* st) {
   using S = BwdBlocks<T>;  // blockIdx.y: the part of the list this CTA takes
@@ -1028,7 +1033,7 @@ __global__ void __launch_bounds__(BwdBlocks<T>::NT, 1024 / BwdBlocks<T>::NT)
     __syncthreads();
     for (int q = t; q < m; q += S::NT) {
       const uint32_t rec = vals[base + q];
-      const float4 g = geo[rec], c = conic[rec];
+      const float4 g = recs[2 * (size_t)rec], c = recs[2 * (size_t)rec + 1];
       const short4 bx = rect[rec];
       s_rec[q] = rec;
       s_geo[q] = g;
@@ -1276,7 +1281,7 @@ int preprocess_and_scan(const Plan& p, const Layout& L, const float* mr, const f
   const size_t smem = p.direct ? (size_t)p.max_tp * sizeof(uint32_t) : 0;
   GS_TRY(launch("preprocess", p.direct ? k_preprocess<true> : k_preprocess<false>,
                 dim3(p.nblocks), dim3(kThreads), smem, s, p.b, (const float4*)mr,
-                (const float4*)sc, (const float4*)qt, views, L.frames, L.geo, L.conic, L.rect,
+                (const float4*)sc, (const float4*)qt, views, L.frames, L.rec, L.rect,
                 L.tmask, L.counts, L.block_sums, L.tcount, L.ticket, L.st));
   if (!p.direct) return scan_block_sums(L.block_sums, L.block_offs, p.nblocks, L.st, p.cap, s);
   auto off = [&](const void* q) { return (int64_t)((const char*)q - (const char*)ws); };
@@ -1303,7 +1308,7 @@ int bin_pairs(const Plan& p, const Layout& L, const float* mr, const float* sc, 
       GS_CUDA(cudaFuncSetAttribute(k_emit_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)smem));
     return launch("emit", k_emit_direct, dim3(p.nblocks), dim3(kThreads), smem, s, p.b,
-                  (const uint32_t*)L.counts, (const float4*)L.geo, (const float4*)L.conic,
+                  (const uint32_t*)L.counts, (const float4*)L.rec,
                   (const short4*)L.rect, (const uint32_t*)L.tmask, (const uint32_t*)L.toffset,
                   (const uint32_t*)L.klocal, (const unsigned long long*)L.gsum, L.ranges, L.vals,
                   (const gs_status*)L.st);
@@ -1314,7 +1319,7 @@ int bin_pairs(const Plan& p, const Layout& L, const float* mr, const float* sc, 
   uint32_t* fk = odd ? L.keys_alt : L.keys;
   uint32_t* fv = odd ? L.vals_alt : L.vals;
   GS_TRY(launch("emit", k_emit, dim3(p.nblocks), dim3(kThreads), 0, s, p.b,
-                (const uint32_t*)L.counts, (const float4*)L.geo, (const float4*)L.conic,
+                (const uint32_t*)L.counts, (const float4*)L.rec,
                 (const short4*)L.rect, (const uint32_t*)L.tmask, (const uint32_t*)L.block_offs,
                 L.keys, L.vals, L.st, (int64_t)((char*)fk - (char*)ws),
                 (int64_t)((char*)fv - (char*)ws)));
@@ -1337,10 +1342,10 @@ int raster_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* img,
   dim3 grid((unsigned)p.n_keys), block(FwdBlocks<T>::NT);
   if (count)
     return launch("raster_count", k_raster_fwd<T, true>, grid, block, 0, s, p.b,
-                  (const uint2*)L.ranges, vals, (const float4*)L.geo, (const float4*)L.conic,
+                  (const uint2*)L.ranges, vals, (const float4*)L.rec,
                   (const short4*)L.rect, img, L.st);
   return launch("raster_fwd", k_raster_fwd<T, false>, grid, block, 0, s, p.b,
-                (const uint2*)L.ranges, vals, (const float4*)L.geo, (const float4*)L.conic,
+                (const uint2*)L.ranges, vals, (const float4*)L.rec,
                 (const short4*)L.rect, img, L.st);
 }
 
@@ -1353,7 +1358,7 @@ int raster_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float
   const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(8, 4 * (int64_t)num_sms() / p.n_keys));
   return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys, parts),
                 dim3(BwdBlocks<T>::NT), 0, s,
-                p.b, (const uint2*)L.ranges, vals, (const float4*)L.geo, (const float4*)L.conic,
+                p.b, (const uint2*)L.ranges, vals, (const float4*)L.rec,
                 (const short4*)L.rect, dimg, L.fpgrad, (const gs_status*)L.st);
 }
 
