@@ -395,14 +395,15 @@ __device__ __forceinline__ float rect_max_e2(const VisitCoef& v, float u0, float
 }
 
 // Visit code of a staged record for warp patch w of the sub-brick whose first voxel is
-// (sx, sy, sz): kNoVisit, or the first and last z pair the cut can reach, p0 | p1 << 4.  A patch
+// (sx, sy, sz), in its layers k_lo .. k_lo + depth - 1: kNoVisit, or the first and last z pair of
+// them the cut can reach, p0 | p1 << 4.  A patch
 // is visited when the record's index box meets its columns and the cut ellipsoid reaches one
 // of its columns.
 __device__ __forceinline__ uint8_t visit_code(const VGrid& g, const float4 G, const VisitCoef& vc,
                                               const short4 a, const short4 b, int sx, int sy,
-                                              int sz, int w, float inv_hz) {
+                                              int sz, int k_lo, int depth, int w, float inv_hz) {
   const int x0 = sx + (w & 1) * 8, y0 = sy + (w >> 1) * 4;
-  if (b.z < sz || a.z > sz + kS - 1 || b.x < x0 || a.x > x0 + 7 || b.y < y0 || a.y > y0 + 3)
+  if (b.z < sz + k_lo || a.z > sz + k_lo + depth - 1 || b.x < x0 || a.x > x0 + 7 || b.y < y0 || a.y > y0 + 3)
     return kNoVisit;
   // column-centre offsets of the patch's rectangle, as the walking lanes compute them
   const float u0 = g.o[0] + ((float)x0 + 0.5f) * g.h[0] - G.x;
@@ -417,22 +418,22 @@ __device__ __forceinline__ uint8_t visit_code(const VGrid& g, const float4 G, co
   const float h = hh * rsqrtf(hh);
   const float cmin = fminf(vc.az * u0, vc.az * u1) + fminf(vc.bz * v0, vc.bz * v1);
   const float cmax = fmaxf(vc.az * u0, vc.az * u1) + fmaxf(vc.bz * v0, vc.bz * v1);
-  const int kmax = min(kS - 1, g.lo[2] + g.dim[2] - 1 - sz);
-  const int k0 = max(0, (int)ceilf((cmin - h - dz0) * inv_hz - 0.02f));
+  const int kmax = min(k_lo + depth - 1, g.lo[2] + g.dim[2] - 1 - sz);
+  const int k0 = max(k_lo, (int)ceilf((cmin - h - dz0) * inv_hz - 0.02f));
   const int k1 = min(kmax, (int)floorf((cmax + h - dz0) * inv_hz + 0.02f));
-  return k0 <= k1 ? (uint8_t)((k0 >> 1) | ((k1 >> 1) << 4)) : kNoVisit;
+  return k0 <= k1 ? (uint8_t)(((k0 - k_lo) >> 1) | (((k1 - k_lo) >> 1) << 4)) : kNoVisit;
 }
 
 // Codes of all (record, patch) items of m staged records, eight threads per record.
 __device__ __forceinline__ void visit_codes(const VGrid& g, const float4* s_geo,
                                             const VisitCoef* s_vc, const short4* s_lo,
                                             const short4* s_hi, int m, int sx, int sy, int sz,
-                                            uint8_t* s_zr) {
+                                            int k_lo, int depth, uint8_t* s_zr) {
   const float inv_hz = 1.f / g.h[2];
   for (int t = threadIdx.x; t < m * kWarps; t += kThreads) {
     const int j = t >> 3, w = t & 7;
-    s_zr[w * kThreads + j] = visit_code(g, s_geo[j], s_vc[j], s_lo[j], s_hi[j], sx, sy, sz, w,
-                                        inv_hz);
+    s_zr[w * kThreads + j] = visit_code(g, s_geo[j], s_vc[j], s_lo[j], s_hi[j], sx, sy, sz,
+                                        k_lo, depth, w, inv_hz);
   }
 }
 
@@ -459,11 +460,11 @@ __device__ __forceinline__ void sub_origin(const VInst& I, uint32_t brick, int B
 // Writes zeros over an empty sub-brick: most of a volume around an object.  16-byte stores, four
 // lanes per 16-voxel row, where the rows are aligned and whole.
 __device__ __forceinline__ void zero_brick(const VGrid& g, float* __restrict__ vol, int sx, int sy,
-                                           int sz) {
+                                           int sz, int depth) {
   const int x = sx - g.lo[0], y0 = sy - g.lo[1], z0 = sz - g.lo[2];
   const size_t sxy = (size_t)g.dim[0] * g.dim[1];
   float* base = vol + (size_t)z0 * sxy + (size_t)y0 * g.dim[0] + x;
-  const int ny = min(kS, g.dim[1] - y0), nz = min(kS, g.dim[2] - z0), nx = min(kS, g.dim[0] - x);
+  const int ny = min(kS, g.dim[1] - y0), nz = min(depth, g.dim[2] - z0), nx = min(kS, g.dim[0] - x);
   if (nx == kS && (g.dim[0] & 3) == 0 && ((uintptr_t)base & 15u) == 0) {
     const int c = (threadIdx.x & 3) * 4, y = (threadIdx.x >> 2) & (kS - 1);
     if (y < ny)
@@ -476,7 +477,10 @@ __device__ __forceinline__ void zero_brick(const VGrid& g, float* __restrict__ v
   }
 }
 
-template <bool COUNT>
+// NP: z pairs per column and CTA, all eight of a sub-brick or two of them (a quarter).  Few
+// sub-bricks leave SMs idle and hold long lists; quartered, their warps walk in parallel and visit
+// only the records that reach their layers.  Every voxel's sum stays what it is.
+template <bool COUNT, int NP>
 __global__ void __launch_bounds__(kThreads, 4)
     k_vox_fwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
               const float4* __restrict__ geo, const float4* __restrict__ cov0,
@@ -491,9 +495,12 @@ __global__ void __launch_bounds__(kThreads, 4)
   __shared__ VisitCoef s_vc[kThreads];
   __shared__ uint8_t s_zr[kWarps * kThreads];
   __shared__ unsigned long long s_cnt;
-  // one CTA per (brick, sub-brick)
-  const int key = (int)(blockIdx.x >> (3 * bt.lsub));
-  const int sb = (int)(blockIdx.x & ((1u << (3 * bt.lsub)) - 1u));
+  // one CTA per (brick, sub-brick, run of NP z pairs)
+  constexpr uint32_t PARTS = kS / 2 / NP;
+  const uint32_t cta = blockIdx.x / PARTS;
+  const int k_lo = (int)(blockIdx.x % PARTS) * 2 * NP;  // first layer in the sub-brick
+  const int key = (int)(cta >> (3 * bt.lsub));
+  const int sb = (int)(cta & ((1u << (3 * bt.lsub)) - 1u));
   const uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
   const VInst& I = bt.in[inst_of_key(bt, key)];
@@ -501,9 +508,9 @@ __global__ void __launch_bounds__(kThreads, 4)
   int sx, sy, sz;
   sub_origin(I, (uint32_t)(key - I.key_off), bt.brick, bt.lsub, sb, sx, sy, sz);
   const int xend = g.lo[0] + g.dim[0], yend = g.lo[1] + g.dim[1], zend = g.lo[2] + g.dim[2];
-  if (sx >= xend || sy >= yend || sz >= zend) return;  // sub-brick outside the region
+  if (sx >= xend || sy >= yend || sz + k_lo >= zend) return;  // outside the region
   if (r.x == r.y) {
-    if (!COUNT) zero_brick(g, vol + I.vol_off, sx, sy, sz);
+    if (!COUNT) zero_brick(g, vol + I.vol_off, sx, sy, sz + k_lo, 2 * NP);
     return;
   }
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -514,9 +521,9 @@ __global__ void __launch_bounds__(kThreads, 4)
   const float xc = g.o[0] + ((float)x + 0.5f) * g.h[0];
   const float yc = g.o[1] + ((float)y + 0.5f) * g.h[1];
   const float zc0 = g.o[2] + ((float)sz + 0.5f) * hz;
-  float2 acc[kS / 2];
+  float2 acc[NP];
 #pragma unroll
-  for (int p = 0; p < kS / 2; ++p) acc[p] = make_float2(0.f, 0.f);
+  for (int p = 0; p < NP; ++p) acc[p] = make_float2(0.f, 0.f);
   for (uint32_t base = r.x; base < r.y; base += kThreads) {
     const int m = (int)min((uint32_t)kThreads, r.y - base);
     __syncthreads();  // the warps are done with the previous batch
@@ -531,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       s_vc[tid] = visit_coef(c0, c1);
     }
     __syncthreads();
-    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, s_zr);
+    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr);
     __syncthreads();
     const uint8_t* zrw = s_zr + w * kThreads;
     for (int j0 = 0; j0 < m; j0 += 32) {
@@ -555,12 +562,12 @@ __global__ void __launch_bounds__(kThreads, 4)
         // interleaves them.  dz of both voxels in one packed FMA (each component rounds like
         // the scalar fmaf); the cut is a predicate on the accumulating FMA (sums unchanged).
         auto pair = [&](int p) {
-          const float2 dz =
-              __ffma2_rn(make_float2((float)(2 * p), (float)(2 * p + 1)), hz2, dz02);
+          const float2 dz = __ffma2_rn(
+              make_float2((float)(k_lo + 2 * p), (float)(k_lo + 2 * p + 1)), hz2, dz02);
           const float2 e = __ffma2_rn(__ffma2_rn(c22, dz, l2), dz, q2);
           if (COUNT) {
-            cnt += (e.x > c1.z && sz + 2 * p < zend) ? 1u : 0u;
-            cnt += (e.y > c1.z && sz + 2 * p + 1 < zend) ? 1u : 0u;
+            cnt += (e.x > c1.z && sz + k_lo + 2 * p < zend) ? 1u : 0u;
+            cnt += (e.y > c1.z && sz + k_lo + 2 * p + 1 < zend) ? 1u : 0u;
           } else {
             const float vx = ex2(e.x), vy = ex2(e.y);
             if (e.x > c1.z) acc[p].x = fmaf(G.w, vx, acc[p].x);
@@ -575,7 +582,9 @@ __global__ void __launch_bounds__(kThreads, 4)
         using std::integral_constant;
 #define GS_WALK(F, N) \
   case (F / 2) * 4 + N / 2 - 1: walk(integral_constant<int, F>(), integral_constant<int, N>()); break;
-        switch (walk_window(code & 15, code >> 4)) {  // warp-uniform
+        if constexpr (NP < 8) {
+          walk(integral_constant<int, 0>(), integral_constant<int, NP>());
+        } else switch (walk_window(code & 15, code >> 4)) {  // warp-uniform
           GS_WALK(0, 2) GS_WALK(0, 4) GS_WALK(0, 6)
           GS_WALK(2, 2) GS_WALK(2, 4) GS_WALK(2, 6)
           GS_WALK(4, 2) GS_WALK(4, 4) GS_WALK(6, 2)
@@ -598,8 +607,8 @@ __global__ void __launch_bounds__(kThreads, 4)
   const size_t sxy = (size_t)g.dim[0] * g.dim[1];
   float* vo = vol + I.vol_off + (size_t)(y - g.lo[1]) * g.dim[0] + (x - g.lo[0]);
 #pragma unroll
-  for (int p = 0; p < kS / 2; ++p) {
-    const int z = sz + 2 * p;
+  for (int p = 0; p < NP; ++p) {
+    const int z = sz + k_lo + 2 * p;
     if (z < zend) vo[(size_t)(z - g.lo[2]) * sxy] = acc[p].x;
     if (z + 1 < zend) vo[(size_t)(z + 1 - g.lo[2]) * sxy] = acc[p].y;
   }
@@ -653,6 +662,7 @@ __device__ __forceinline__ int moment_index(int lane) {
 
 constexpr int kMoments = 10;
 
+template <int NP>  // z pairs per column and CTA, as in the forward
 __global__ void __launch_bounds__(kThreads, 4)
     k_vox_bwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
               const float4* __restrict__ geo, const float4* __restrict__ cov0,
@@ -668,9 +678,12 @@ __global__ void __launch_bounds__(kThreads, 4)
   __shared__ VisitCoef s_vc[kThreads];
   __shared__ uint8_t s_zr[kWarps * kThreads];
   __shared__ float s_mom[kThreads * kMoments];
-  // one CTA per (brick, sub-brick)
-  const int key = (int)(blockIdx.x >> (3 * bt.lsub));
-  const int sb = (int)(blockIdx.x & ((1u << (3 * bt.lsub)) - 1u));
+  // one CTA per (brick, sub-brick, run of NP z pairs)
+  constexpr uint32_t PARTS = kS / 2 / NP;
+  const uint32_t cta = blockIdx.x / PARTS;
+  const int k_lo = (int)(blockIdx.x % PARTS) * 2 * NP;  // first layer in the sub-brick
+  const int key = (int)(cta >> (3 * bt.lsub));
+  const int sb = (int)(cta & ((1u << (3 * bt.lsub)) - 1u));
   const uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
   if (r.x == r.y) return;
@@ -679,7 +692,7 @@ __global__ void __launch_bounds__(kThreads, 4)
   int sx, sy, sz;
   sub_origin(I, (uint32_t)(key - I.key_off), bt.brick, bt.lsub, sb, sx, sy, sz);
   const int xend = g.lo[0] + g.dim[0], yend = g.lo[1] + g.dim[1], zend = g.lo[2] + g.dim[2];
-  if (sx >= xend || sy >= yend || sz >= zend) return;  // sub-brick outside the region
+  if (sx >= xend || sy >= yend || sz + k_lo >= zend) return;  // outside the region
   const float* dvol = dvol_all + I.vol_off;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const float hz = g.h[2];
@@ -687,13 +700,13 @@ __global__ void __launch_bounds__(kThreads, 4)
   const int x = sx + (w & 1) * 8 + (lane & 7), y = sy + (w >> 1) * 4 + (lane >> 3);
   const bool in_xy = x < xend && y < yend;
   // dL/dV of this lane's column (0 outside the region)
-  float2 gv[kS / 2];
+  float2 gv[NP];
   {
     const size_t sxy = (size_t)g.dim[0] * g.dim[1];
     const float* gc = dvol + (in_xy ? (size_t)(y - g.lo[1]) * g.dim[0] + (x - g.lo[0]) : 0);
 #pragma unroll
-    for (int p = 0; p < kS / 2; ++p) {
-      const int z = sz + 2 * p;
+    for (int p = 0; p < NP; ++p) {
+      const int z = sz + k_lo + 2 * p;
       gv[p].x = in_xy && z < zend ? __ldg(gc + (size_t)(z - g.lo[2]) * sxy) : 0.f;
       gv[p].y = in_xy && z + 1 < zend ? __ldg(gc + (size_t)(z + 1 - g.lo[2]) * sxy) : 0.f;
     }
@@ -718,7 +731,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       for (int k = 0; k < kMoments; ++k) s_mom[tid * kMoments + k] = 0.f;
     }
     __syncthreads();
-    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, s_zr);
+    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr);
     __syncthreads();
     const uint8_t* zrw = s_zr + w * kThreads;
     for (int j0 = 0; j0 < m; j0 += 32) {
@@ -743,10 +756,10 @@ __global__ void __launch_bounds__(kThreads, 4)
         // pays for the uniform branches (dz of both voxels in one packed FMA, as the forward)
         const int p0 = code & 15, p1 = code >> 4;  // warp-uniform
 #pragma unroll
-        for (int p = 0; p < kS / 2; ++p) {
+        for (int p = 0; p < NP; ++p) {
           if (p < p0 || p > p1) continue;
-          const float2 dz =
-              __ffma2_rn(make_float2((float)(2 * p), (float)(2 * p + 1)), hz2, dz02);
+          const float2 dz = __ffma2_rn(
+              make_float2((float)(k_lo + 2 * p), (float)(k_lo + 2 * p + 1)), hz2, dz02);
           const float2 e = __ffma2_rn(__ffma2_rn(c22, dz, l2), dz, q2);
           const float2 val = make_float2(e.x > c1.z ? ex2(e.x) : 0.f,
                                          e.y > c1.z ? ex2(e.y) : 0.f);
@@ -906,16 +919,37 @@ int bin_bricks(const Plan& p, const Layout& L, const float* mr, const float* sc,
   return GS_OK;
 }
 
+// Whether the walking kernels split each sub-brick into four runs of two z pairs: while the
+// sub-bricks make less than eight CTAs per SM, two waves of the four that are resident.  Below it
+// the longest lists decide and idle SMs take the quarters (whole -> quartered, forward / backward:
+// 38^3, 57k Gaussians of 7 voxels, 27 sub-bricks 915 / 1730 -> 374 / 707 us; 96^3, 5k of 2 voxels,
+// 216 sub-bricks 24.8 / 43.1 -> 17.2 / 28.5; 128^3, 20k, 512 sub-bricks 41.1 / 70.0 -> 34.3 /
+// 58.6; 160^3, 30k, 1000 sub-bricks 47.8 / 80.7 -> 43.8 / 74.5).  Above it the SMs are busy anyway
+// and each list would be staged four times for nothing (2704 sub-bricks: 81.3 / 137 -> 80.9 / 136).
+bool quarters(const Plan& p) { return p.n_ctas < 8 * (int64_t)num_sms(); }
+
+template <bool COUNT, int NP>
+int vox_fwd_np(const Plan& p, const Layout& L, const uint32_t* vals, float* vol, cudaStream_t s) {
+  return launch(COUNT ? "vox_count" : "vox_fwd", k_vox_fwd<COUNT, NP>,
+                dim3((unsigned)(p.n_ctas * (kS / 2 / NP))), dim3(kThreads), 0, s,
+                (const uint2*)L.ranges, vals, (const float4*)L.geo, (const float4*)L.cov0,
+                (const float4*)L.cov1, (const short4*)L.lo, (const short4*)L.hi, p.b, vol, L.st);
+}
+
 int vox_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* vol, bool count,
             cudaStream_t s) {
-  dim3 grid((unsigned)p.n_ctas), block(kThreads);
-  if (count)
-    return launch("vox_count", k_vox_fwd<true>, grid, block, 0, s, (const uint2*)L.ranges, vals,
-                  (const float4*)L.geo, (const float4*)L.cov0, (const float4*)L.cov1,
-                  (const short4*)L.lo, (const short4*)L.hi, p.b, vol, L.st);
-  return launch("vox_fwd", k_vox_fwd<false>, grid, block, 0, s, (const uint2*)L.ranges, vals,
-                (const float4*)L.geo, (const float4*)L.cov0, (const float4*)L.cov1,
-                (const short4*)L.lo, (const short4*)L.hi, p.b, vol, L.st);
+  if (count) return vox_fwd_np<true, 8>(p, L, vals, vol, s);
+  return quarters(p) ? vox_fwd_np<false, 2>(p, L, vals, vol, s)
+                     : vox_fwd_np<false, 8>(p, L, vals, vol, s);
+}
+
+template <int NP>
+int vox_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float* dvol,
+            cudaStream_t s) {
+  return launch("vox_bwd", k_vox_bwd<NP>, dim3((unsigned)(p.n_ctas * (kS / 2 / NP))),
+                dim3(kThreads), 0, s, (const uint2*)L.ranges, vals, (const float4*)L.geo,
+                (const float4*)L.cov0, (const float4*)L.cov1, (const short4*)L.lo,
+                (const short4*)L.hi, p.b, dvol, L.vgrad, (const gs_status*)L.st);
 }
 
 gs_voxel_instance one(int n, const gs_grid* grid, const int32_t* lo, const int32_t* dim) {
@@ -1012,10 +1046,7 @@ int gs_voxelize_batch_backward(const float* d_mean_rho, const float* d_scale,
     GS_TRY(bin_bricks(p, L, d_mean_rho, d_scale, d_quat, s, d_ws, &k, &v));
   }
   GS_CUDA(cudaMemsetAsync(L.vgrad, 0, (size_t)p.n * 3 * sizeof(float4), s));
-  GS_TRY(launch("vox_bwd", k_vox_bwd, dim3((unsigned)p.n_ctas), dim3(kThreads), 0, s,
-                (const uint2*)L.ranges, (const uint32_t*)v, (const float4*)L.geo,
-                (const float4*)L.cov0, (const float4*)L.cov1, (const short4*)L.lo,
-                (const short4*)L.hi, p.b, d_dvol, L.vgrad, (const gs_status*)L.st));
+  GS_TRY(quarters(p) ? vox_bwd<2>(p, L, v, d_dvol, s) : vox_bwd<8>(p, L, v, d_dvol, s));
   return launch_after("vox_chain", k_vox_chain, dim3(p.nblocks), dim3(kThreads), 0, s,
                 (const float4*)d_mean_rho, (const float4*)d_scale, (const float4*)d_quat, p.n,
                 (const float4*)L.vgrad, (float4*)d_g_mean_rho, (float4*)d_g_scale,

@@ -265,3 +265,28 @@ def test_empty_bricks_are_zeroed(orc, gsct, lo, dim, brick, shift):
     got = out.cpu().numpy().astype(np.float64)
     assert (np.abs(got - want) <= IMG_TOL * np.abs(want).max() + allow).all()
     assert np.all(got[(want == 0) & (allow == 0)] == 0)
+
+
+@pytest.mark.parametrize("brick", [16, 32, 64])
+@pytest.mark.parametrize("lo,dim", [((32, 16, 48), (40, 33, 61)), ((160, 160, 160), (16, 16, 16)),
+                                    ((0, 0, 16), (1, 17, 9))])
+def test_small_regions_equal_the_whole_volume(gsct, brick, lo, dim):
+    """A region of few bricks (whose bricks are split over several CTAs) equals its part of the
+    whole 176^3 volume (whose bricks are not) bit for bit; with a gradient that is zero outside
+    the region so do the gradients, up to the order in which the parts' FP32 sums meet (at most 100
+    parts of one Gaussian, each rounded to 6e-8)."""
+    import torch
+
+    mr, sc, qt = synth.gaussians(6, 400, radius=1.0, scale_median=0.05)
+    grid = synth.cube_grid(176)
+    p = to_dev(mr, sc, qt)
+    part = tuple(slice(lo[k], lo[k] + dim[k]) for k in (2, 1, 0))
+    whole, small = (gsct.Voxelizer(grid, a, b, brick=brick)
+                    for a, b in (((0, 0, 0), (176, 176, 176)), (lo, dim)))
+    vw, vs = whole.forward(*p), small.forward(*p)
+    assert torch.equal(vs, vw[part])
+    dv = torch.randn(vs.shape, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    dw = torch.zeros_like(vw)
+    dw[part] = dv
+    for a, b in zip(whole.backward(*p, dw), small.backward(*p, dv.contiguous())):
+        assert torch.all((a - b).abs() <= 6e-6 * a.abs().max())
