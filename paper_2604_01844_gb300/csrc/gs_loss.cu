@@ -27,8 +27,17 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// two set-on-compare instructions and a subtraction (no integer conversion)
+// sign(x): two set-on-compare instructions and a subtraction (no integer conversion)
 __device__ __forceinline__ float sgnf(float x) { return (x > 0.f ? 1.f : 0.f) - (x < 0.f ? 1.f : 0.f); }
+
+// 1 / x: the hardware approximation and one Newton step (within an ulp), without the branch and
+// the call that a correctly rounded division brings; 0 and infinity keep their reciprocals.
+__device__ __forceinline__ float rcp_newton(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  const float e = fmaf(-x, r, 1.f);
+  return fabsf(e) < 1.f ? fmaf(r, e, r) : r;
+}
 
 template <typename T>
 __device__ __forceinline__ void block_add(T v, T* target) {
@@ -223,7 +232,7 @@ __device__ __forceinline__ float2 pair_at(const float* base, int64_t n, int m, i
 template <int NIN>  // 2: (X, Y) -> 5 moments; 3: maps (pair layout) -> 3 filtered maps
 __global__ void __launch_bounds__(kThreads)
     k_ssim3d_z(const __grid_constant__ Win W, const float* __restrict__ A0,
-               const float* __restrict__ A1, int nx, int ny, int nz, int64_t plane,
+               const float* __restrict__ A1, int nx, int ny, int nz, int zc, int64_t plane,
                float* __restrict__ out, float l1_scale, float* __restrict__ loss) {
   constexpr int NOUT = NIN == 2 ? 5 : 3;
   const int64_t sxy = (int64_t)nx * ny;
@@ -247,26 +256,30 @@ __global__ void __launch_bounds__(kThreads)
   for (int k = 0; k <= 2 * kR; ++k)
 #pragma unroll
     for (int i = 0; i < NIN; ++i) ring[k][i] = 0.f;
+  // this chunk's outputs z0 .. z1 - 1; plane zi = z0 - kR + p enters ring slot p % 11, and output
+  // z = zi - kR is complete once it is in
+  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
   float nxt[NIN];
-  load(col, nxt);
-  // plane zi enters ring slot zi % 11; output z = zi - kR is complete once plane zi is in
-  for (int zb = 0; zb < nz + kR; zb += 2 * kR + 1) {
+  auto next_plane = [&](int zn) {
+    if (zn >= 0 && zn < nz) {
+      load((int64_t)zn * sxy + col, nxt);
+    } else {
+#pragma unroll
+      for (int i = 0; i < NIN; ++i) nxt[i] = 0.f;
+    }
+  };
+  next_plane(z0 - kR);
+  for (int zb = z0 - kR; zb < z1 + kR; zb += 2 * kR + 1) {
 #pragma unroll
     for (int k = 0; k <= 2 * kR; ++k) {
       const int zi = zb + k;
 #pragma unroll
       for (int i = 0; i < NIN; ++i) ring[k][i] = nxt[i];
-      if (NIN == 2 && l1_scale != 0.f) l1 += fabsf(nxt[0] - nxt[1]);  // 0 beyond the volume
-      const int zn = zi + 1;
-      if (zn < nz) {
-        load((int64_t)zn * sxy + col, nxt);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NIN; ++i) nxt[i] = 0.f;
-      }
+      if (NIN == 2 && l1_scale != 0.f && zi >= z0 && zi < z1) l1 += fabsf(nxt[0] - nxt[1]);
+      next_plane(zi + 1);
       // the column's element 4 planes ahead is requested into L2 now, so that the load of the
       // next plane rarely waits for DRAM
-      if (zi + 4 < nz) {
+      if (zi + 4 >= 0 && zi + 4 < min(nz, z1 + kR)) {
         const int64_t o4 = (int64_t)(zi + 4) * sxy + col;
         if (NIN == 2) {
           asm volatile("prefetch.global.L2 [%0];" ::"l"(A0 + o4));
@@ -277,7 +290,7 @@ __global__ void __launch_bounds__(kThreads)
         }
       }
       const int z = zi - kR;
-      if (z < 0 || z >= nz) continue;
+      if (z < z0 || z >= z1) continue;
       float acc[NOUT];
 #pragma unroll
       for (int m = 0; m < NOUT; ++m) acc[m] = 0.f;
@@ -406,7 +419,8 @@ __global__ void __launch_bounds__(kSsimThreads)
   }
   float2 w2[2 * kR + 1];
 #pragma unroll
-  for (int k = 0; k <= 2 * kR; ++k) w2[k] = make_float2(W.w[k], W.w[k]);
+  for (int k = 0; k <= 2 * kR; ++k)  // symmetric: six values
+    w2[k] = make_float2(W.w[k < kR ? k : 2 * kR - k], W.w[k < kR ? k : 2 * kR - k]);
   __syncthreads();
   // ---- horizontal pass: item p = (row r, columns c0 .. c0 + 3); lanes take consecutive rows
   for (int p = tid; p < kIn2 * (kT2 / kG); p += kSsimThreads) {
@@ -513,7 +527,7 @@ __global__ void __launch_bounds__(kSsimThreads)
       }
       const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
       const float C = mx * mx + my * my + C1;
-      const float inv = 1.f / (C * D);  // 1/C = D inv, 1/D = C inv
+      const float inv = rcp_newton(C * D);  // 1/C = D inv, 1/D = C inv
       const float Sv = (Am * Bn) * inv;
       const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
       const float dsxx = -Sv * (C * inv);
@@ -549,10 +563,10 @@ int ssim_xy_attributes() {
 //      (zero fill outside the volume; the box starts 8 columns left of the tile, so that its x
 //      coordinate stays 16-byte aligned, and 5 rows above it),
 //   2. filters the box along y: items of one halo column and four output rows share the 14
-//      inputs they need (register blocking), results in shared memory (forward one float4
-//      of channels per column, backward a float2 and a float),
-//   3. filters along x for its own column, which leaves the thread the plane's xy-filtered
-//      channels of its column,
+//      inputs they need (register blocking), results in shared memory (one float4 of channels
+//      per column),
+//   3. filters along x: a warp per row, items of four columns share the 14 inputs they need,
+//      results in place of the row; each thread then takes its own column,
 //   4. keeps them in a register ring of the last 12 planes and, once 11 planes are in,
 //      filters along z for the plane 5 behind and completes that voxel: SSIM, the loss term
 //      and the maps in the forward, the gradient in the backward.
@@ -567,6 +581,10 @@ int ssim_xy_attributes() {
 // directions, as in the separable kernels above (the y, x, z
 // order and the summed channel only change FP32 rounding).  Traffic: forward X, Y in and three
 // maps out (20 bytes per voxel); backward the maps, X and Y in and the gradient out (24).
+// Bound by instruction issue and shared memory (64 % of the issue slots, 16 warps per SM; the
+// backward 76 % of the shared-memory wavefronts).  With an own column per thread in the x filter
+// (11 float4 a voxel instead of 3.5, and one back and forth) and the items of the y pass laid over
+// 42-column rows (two-way bank conflicts) 384^3 took 674 + 518 us; now 559 + 443.
 // ------------------------------------------------------------------------------------------
 constexpr int kFX = 32, kFY = 8;                       // output tile (x, y)
 constexpr int kFThreads = kFX * kFY;                   // a thread per column
@@ -574,13 +592,18 @@ constexpr int kBoxX = kFX + 16, kBoxY = kFY + 2 * kR;  // staged box 48 x 18
 constexpr int kHaloX = kFX + 2 * kR;                   // 42 y-filtered columns
 constexpr int kPP = 3;                                 // planes per iteration
 constexpr int kFStages = 2 * kPP;                      // planes in flight (2 iterations)
-constexpr int kYItems = kPP * kHaloX * (kFY / 4);      // 252 y-pass items (3 planes)
+constexpr int kYRuns = kPP * (kFY / 4);                // runs of four output rows (3 planes): 6
 constexpr uint32_t kBox4 = kBoxX * kBoxY * 4;          // bytes of a 4-byte channel box (3456)
 constexpr uint32_t kBox8 = 2 * kBox4;                  // of an 8-byte (pair) box
 constexpr uint32_t kTile4 = kFX * kFY * 4;             // of a 4-byte output tile (1024)
 static_assert(kBox4 % 128 == 0 && kTile4 % 128 == 0, "TMA destinations stay 128-byte aligned");
-static_assert(kFY % 4 == 0 && kFThreads % 32 == 0 && kYItems <= kFThreads,
-              "y items take four rows; whole warps");
+static_assert(kFY % 4 == 0 && kYRuns + 2 == kFThreads / 32 && kYRuns * (kHaloX - 32) <= 2 * 30,
+              "y items take four rows: a warp per run, two warps for the last ten columns");
+static_assert(kPP * (kFX / 4) <= 32, "x items of a warp's row: one per lane");
+// Place of y-filtered column c in its row of float4: the gaps put four-column steps (the x items'
+// reads and writes) as well as consecutive columns into eight different 16-byte bank groups.
+__device__ __forceinline__ int h_slot(int c) { return c + (c >> 3) + 4 * (c >> 5); }
+constexpr int kHPitch = 52;                            // > h_slot(kHaloX - 1) = 50
 
 // Stage layout and filtered channels of the two directions.
 //   forward (BWD = false): X box | Y box; NP = 2 filtered pairs (x, y), (x^2 + y^2, x y)
@@ -592,9 +615,7 @@ struct FusedShape {
   static constexpr uint32_t offX = kBox8 + kBox4, offY = offX + kTile4;  // backward only
   static constexpr uint32_t stage = BWD ? offY + kTile4 : 2 * kBox4;
   static constexpr uint32_t txbytes = BWD ? kBox8 + kBox4 + 2 * kTile4 : 2 * kBox4;
-  // y-filtered channels of one plane: forward one float4 per column, backward a float2 plane
-  // (m1, m2) and a float plane (m3)
-  static constexpr uint32_t hbuf = (BWD ? 12 : 16) * kFY * kHaloX;
+  static constexpr uint32_t hbuf = 16 * kFY * kHPitch;  // y-filtered channels of one plane
   static constexpr size_t smem = 128 + kFStages * stage + 2 * kPP * hbuf;  // h: 2 x kPP
 };
 
@@ -605,23 +626,20 @@ constexpr int kRing = 12;
 static_assert(kRing % kPP == 0 && kRing >= 2 * kR + 1, "ring holds every window");
 template <int K, int NP, int NS>
 __device__ __forceinline__ void ring_zp(float2 (&rp)[NP][kRing], float (&rs)[NS ? NS : 1][kRing],
-                                        const float2 (&vp)[kPP][NP],
-                                        const float (&vs)[kPP][NS ? NS : 1],
+                                        const float4* col,
                                         const float2 (&w2)[2 * kR + 1], float2 (&fp)[kPP][NP],
                                         float (&fs)[kPP][NS ? NS : 1]) {
   // plane by plane: each insert overwrites the plane 12 behind, which no later window needs
 #pragma unroll
   for (int h = 0; h < kPP; ++h) {
+    const float4 q = col[h * kFY * kHPitch];
+    rp[0][kPP * K + h] = make_float2(q.x, q.y);
+    if constexpr (NP == 2) rp[NP - 1][kPP * K + h] = make_float2(q.z, q.w);
+    else rs[0][kPP * K + h] = q.z;
 #pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      rp[m][kPP * K + h] = vp[h][m];
-      fp[h][m] = make_float2(0.f, 0.f);
-    }
+    for (int m = 0; m < NP; ++m) fp[h][m] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 0; m < NS; ++m) {
-      rs[m][kPP * K + h] = vs[h][m];
-      fs[h][m] = 0.f;
-    }
+    for (int m = 0; m < NS; ++m) fs[h][m] = 0.f;
 #pragma unroll
     for (int t = 0; t <= 2 * kR; ++t) {
       const int sl = (kPP * K + h + kRing - 2 * kR + t) % kRing;
@@ -636,16 +654,15 @@ __device__ __forceinline__ void ring_zp(float2 (&rp)[NP][kRing], float (&rs)[NS 
 template <int NP, int NS>
 __device__ __forceinline__ void ring_push(int k, float2 (&rp)[NP][kRing],
                                           float (&rs)[NS ? NS : 1][kRing],
-                                          const float2 (&vp)[kPP][NP],
-                                          const float (&vs)[kPP][NS ? NS : 1],
+                                          const float4* col,
                                           const float2 (&w2)[2 * kR + 1], float2 (&fp)[kPP][NP],
                                           float (&fs)[kPP][NS ? NS : 1]) {
   static_assert(kRing / kPP == 4, "one case per ring position");
   switch (k) {
-    case 0: ring_zp<0, NP, NS>(rp, rs, vp, vs, w2, fp, fs); break;
-    case 1: ring_zp<1, NP, NS>(rp, rs, vp, vs, w2, fp, fs); break;
-    case 2: ring_zp<2, NP, NS>(rp, rs, vp, vs, w2, fp, fs); break;
-    default: ring_zp<3, NP, NS>(rp, rs, vp, vs, w2, fp, fs); break;
+    case 0: ring_zp<0, NP, NS>(rp, rs, col, w2, fp, fs); break;
+    case 1: ring_zp<1, NP, NS>(rp, rs, col, w2, fp, fs); break;
+    case 2: ring_zp<2, NP, NS>(rp, rs, col, w2, fp, fs); break;
+    default: ring_zp<3, NP, NS>(rp, rs, col, w2, fp, fs); break;
   }
 }
 
@@ -665,20 +682,16 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
   extern __shared__ __align__(16) unsigned char dyn_raw[];
   // 128-byte aligned start, derived from the shared array itself (shared-space addressing)
   unsigned char* base = dyn_raw + ((128u - (smem_u32(dyn_raw) & 127u)) & 127u);
-  // y-filtered planes [2 buffers][2 planes][kFY][kHaloX]: forward float4; backward float2
-  // (m1, m2), then float m3
+  // y-filtered planes [2 buffers][kPP planes][kFY][kHPitch], the channels of a column together
+  // (backward: m1, m2, m3 and a zero)
   float4* h4 = reinterpret_cast<float4*>(base + kFStages * S::stage);
-  float2* h2 = reinterpret_cast<float2*>(base + kFStages * S::stage);
-  float* h1 = reinterpret_cast<float*>(h2 + 2 * kPP * kFY * kHaloX);
   __shared__ __align__(8) uint64_t bar[kFStages];
   __shared__ int abort_flag;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const int bx0 = blockIdx.x * kFX, by0 = blockIdx.y * kFY;
   // planes p = 0 .. kPP iters - 1 enter at z = z0 - kR + p (up to kPP - 1 past the range)
   const int planes = (z1 - z0) + 2 * kR, iters = (planes + kPP - 1) / kPP, total = kPP * iters;
-  int issued = 0;
-  auto issue = [&](int p) {
-    const int st = p % kFStages;
+  auto issue = [&](int p, int st) {  // st = p % kFStages
     unsigned char* dst = base + st * S::stage;
     const int zi = z0 - kR + p;
     mbar_expect_tx(&bar[st], S::txbytes);
@@ -693,12 +706,25 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
     abort_flag = 0;
     for (int st = 0; st < kFStages; ++st) mbar_init(&bar[st], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (; issued < kFStages && issued < total; ++issued) issue(issued);
+    for (int p = 0; p < kFStages && p < total; ++p) issue(p, p);
   }
   __syncthreads();
+  // the thread's y item: output rows 4 yq .. of plane yh at halo column yc.  A warp per run takes
+  // its first 32 columns (consecutive banks); two warps take the last ten columns of three each.
+  const bool tail = ty >= kYRuns;
+  const int yrun = tail ? (ty - kYRuns) * 3 + tx / (kHaloX - 32) : ty;
+  const int yc = tail ? 32 + tx % (kHaloX - 32) : tx;
+  const bool yitem = !tail || tx < 3 * (kHaloX - 32);
+  const int yh = yrun / (kFY / 4), yq = yrun % (kFY / 4);
+  // the lane's x item: columns 4 xq .. 4 xq + 3 of the warp's row in plane xh
+  const int xh = tx >> 3, xq = tx & 7;
+  const int xrow = (xh * kFY + ty) * kHPitch;
+  const int xs0 = xrow + h_slot(4 * xq), xs1 = xrow + h_slot(4 * xq + 4),
+            xs2 = xrow + h_slot(4 * xq + 8), xs3 = xrow + h_slot(4 * xq + 12);
   float2 w2[2 * kR + 1];
 #pragma unroll
-  for (int t = 0; t <= 2 * kR; ++t) w2[t] = make_float2(W.w[t], W.w[t]);
+  for (int t = 0; t <= 2 * kR; ++t)  // symmetric: six values
+    w2[t] = make_float2(W.w[t < kR ? t : 2 * kR - t], W.w[t < kR ? t : 2 * kR - t]);
   float2 rp[NP][kRing];
   float rs[NSA][kRing];
 #pragma unroll
@@ -710,20 +736,20 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
   }
   int k = 0;  // ring position of iteration i: i % (kRing / kPP)
   bool failed = false;
+  int failed_at = 0;  // the first plane of the iteration that gave up
   for (int i = 0; i < iters; ++i) {
     const int p0 = kPP * i;
+    const int st0 = (i & 1) * kPP;  // stages st0 .. st0 + kPP - 1: (p0 + h) % kFStages
     // a wait that gives up raises the flag; the planes are still walked (on whatever the
     // buffers hold) so that every thread reaches the barrier, after which all leave together
 #pragma unroll
     for (int h = 0; h < kPP; ++h)
-      if (!mbar_wait(&bar[(p0 + h) % kFStages], (uint32_t)((p0 + h) / kFStages) & 1u))
-        abort_flag = 1;
-    const int hoff = (i & 1) * kPP * kFY * kHaloX;  // this iteration's buffer
-    // ---- y pass of the iteration's planes: item (plane h, halo column c, output rows 4q ..
-    // 4q + 3), the 14 box rows from 4q on at box column c + 3
-    if (tid < kYItems) {
-      const int c = tid % kHaloX, hq = tid / kHaloX, h = hq / (kFY / 4), q = hq % (kFY / 4);
-      const unsigned char* sb = base + ((p0 + h) % kFStages) * S::stage;
+      if (!mbar_wait(&bar[st0 + h], (uint32_t)(i >> 1) & 1u)) abort_flag = 1;
+    float4* hb = h4 + (i & 1) * kPP * kFY * kHPitch;  // this iteration's buffer
+    // ---- y pass of the iteration's planes: the item's 14 box rows from 4 yq on, at box column
+    // yc + 3
+    if (yitem) {
+      const unsigned char* sb = base + (st0 + yh) * S::stage;
       float2 a[4][NP];
       float cs[4];
 #pragma unroll
@@ -734,7 +760,7 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
       }
 #pragma unroll
       for (int r = 0; r < 4 + 2 * kR; ++r) {
-        const int e = (4 * q + r) * kBoxX + c + 3;
+        const int e = (4 * yq + r) * kBoxX + yc + 3;
         float2 u[NP];
         float us = 0.f;
         if constexpr (!BWD) {  // X, Y -> (x, y), (x^2 + y^2, x y)
@@ -757,53 +783,63 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
       }
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
-        const int oo = hoff + (h * kFY + 4 * q + o) * kHaloX + c;
-        if constexpr (NP == 2) {  // (x, y, x^2 + y^2, x y) of a column as one float4
-          h4[oo] = make_float4(a[o][0].x, a[o][0].y, a[o][1].x, a[o][1].y);
+        const int oo = (yh * kFY + 4 * yq + o) * kHPitch + h_slot(yc);
+        if constexpr (NP == 2) {  // (x, y, x^2 + y^2, x y)
+          hb[oo] = make_float4(a[o][0].x, a[o][0].y, a[o][1].x, a[o][1].y);
         } else {
-          h2[oo] = a[o][0];
-          h1[oo] = cs[o];
+          hb[oo] = make_float4(a[o][0].x, a[o][0].y, cs[o], 0.f);
         }
       }
     }
 #pragma unroll
-    for (int h = 0; h < kPP; ++h) on_stage(base + ((p0 + h) % kFStages) * S::stage, p0 + h, h);
+    for (int h = 0; h < kPP; ++h) on_stage(base + (st0 + h) * S::stage, p0 + h, h);
     __syncthreads();
     if (abort_flag) {
       failed = true;
+      failed_at = p0;
       break;
     }
-    if (tid == 0)  // refill the stages just read
-      for (int n = 0; n < kPP && issued < total; ++n) issue(issued++);
-    // ---- x pass of the iteration's planes for the thread's column
-    float2 vp[kPP][NP];
-    float vs[kPP][NSA];
+    // refill the stages just read, a warp each
+    if (tx == 0 && ty < kPP && p0 + kFStages + ty < total) issue(p0 + kFStages + ty, st0 + ty);
+    // ---- x pass of the iteration's planes.  Every row belongs to one warp: its lanes filter four
+    // columns each from 14 inputs and put them back in place, then every thread takes its column
+    if (xh < kPP) {
+      float2 a[4][NP];
+      float cs[4];
 #pragma unroll
-    for (int h = 0; h < kPP; ++h) {
+      for (int o = 0; o < 4; ++o) {
 #pragma unroll
-      for (int m = 0; m < NP; ++m) vp[h][m] = make_float2(0.f, 0.f);
+        for (int m = 0; m < NP; ++m) a[o][m] = make_float2(0.f, 0.f);
+        cs[o] = 0.f;
+      }
 #pragma unroll
-      for (int m = 0; m < NSA; ++m) vs[h][m] = 0.f;
-    }
+      for (int r = 0; r < 4 + 2 * kR; ++r) {
+        const float4 q = hb[(r < 4 ? xs0 : r < 8 ? xs1 : r < 12 ? xs2 : xs3) + (r & 3)];
 #pragma unroll
-    for (int t = 0; t <= 2 * kR; ++t) {
-#pragma unroll
-      for (int h = 0; h < kPP; ++h) {
-        const int o = hoff + (h * kFY + ty) * kHaloX + tx + t;
-        if constexpr (NP == 2) {
-          const float4 q = h4[o];
-          vp[h][0] = __ffma2_rn(w2[t], make_float2(q.x, q.y), vp[h][0]);
-          vp[h][NP - 1] = __ffma2_rn(w2[t], make_float2(q.z, q.w), vp[h][NP - 1]);
-        } else {
-          vp[h][0] = __ffma2_rn(w2[t], h2[o], vp[h][0]);
-          vs[h][0] = fmaf(w2[t].x, h1[o], vs[h][0]);
+        for (int o = 0; o < 4; ++o) {
+          const int k = r - o;
+          if (k < 0 || k > 2 * kR) continue;
+          a[o][0] = __ffma2_rn(w2[k], make_float2(q.x, q.y), a[o][0]);
+          if constexpr (NP == 2)
+            a[o][NP - 1] = __ffma2_rn(w2[k], make_float2(q.z, q.w), a[o][NP - 1]);
+          else
+            cs[o] = fmaf(w2[k].x, q.z, cs[o]);
         }
       }
+      __syncwarp((1u << (8 * kPP)) - 1u);  // the row's reads are done
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        if constexpr (NP == 2)
+          hb[xs0 + o] = make_float4(a[o][0].x, a[o][0].y, a[o][NP - 1].x, a[o][NP - 1].y);
+        else
+          hb[xs0 + o] = make_float4(a[o][0].x, a[o][0].y, cs[o], 0.f);
+      }
     }
+    __syncwarp();
     // ---- ring, z filter, completion of output planes z0 + p0 - 2 kR and the next ones
     float2 fp[kPP][NP];
     float fs[kPP][NSA];
-    ring_push<NP, NS>(k, rp, rs, vp, vs, w2, fp, fs);
+    ring_push<NP, NS>(k, rp, rs, hb + ty * kHPitch + h_slot(tx), w2, fp, fs);
     k = k == kRing / kPP - 1 ? 0 : k + 1;
 #pragma unroll
     for (int h = 0; h < kPP; ++h) {
@@ -813,8 +849,8 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
   }
   if (failed && tid == 0) {
     // wait (bounded) for the copies still in flight before the CTA's shared memory goes away
-    for (int j = issued - kFStages; j < issued; ++j)
-      if (j >= 0) mbar_wait(&bar[j % kFStages], (uint32_t)(j / kFStages) & 1u);
+    for (int j = failed_at; j < min(failed_at + kFStages, total); ++j)
+      mbar_wait(&bar[j % kFStages], (uint32_t)(j / kFStages) & 1u);
   }
   return !failed;
 }
@@ -831,21 +867,25 @@ __global__ void __launch_bounds__(kFThreads, 2)
   const int x = blockIdx.x * kFX + tx, y = blockIdx.y * kFY + ty;
   const bool own = x < nx && y < ny;
   float contrib = 0.f, l1 = 0.f;
-  auto finish = [&](int z, int, const float2 (&fp)[2], const float (&)[1]) {
+  // the voxel the thread finishes next: planes come in order, one call per plane
+  const int64_t sxy = (int64_t)nx * ny;
+  int64_t next = (int64_t)z0 * sxy + (int64_t)y * nx + x;
+  auto finish = [&](int, int, const float2 (&fp)[2], const float (&)[1]) {
+    const int64_t o = next;
+    next += sxy;
     if (!own) return;
     const float mx = fp[0].x, my = fp[0].y;
     const float sxy = fp[1].y - mx * my;
     const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
     const float C = mx * mx + my * my + C1;
     const float D = (fp[1].x - mx * mx - my * my) + C2;  // sigma_x^2 + sigma_y^2 + C2
-    const float inv = 1.f / (C * D);
+    const float inv = rcp_newton(C * D);
     const float Sv = (Am * Bn) * inv;
     contrib += 1.f - Sv;
     if (MAPS) {
       const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
       const float dsxx = -Sv * (C * inv);
       const float dsxy = 2.f * Am * inv;
-      const size_t o = ((size_t)z * ny + y) * nx + x;
       m12[o] = make_float2(gscale * (dmu - 2.f * mx * dsxx - my * dsxy), gscale * dsxx);
       m3[o] = gscale * dsxy;
     }
@@ -888,9 +928,12 @@ __global__ void __launch_bounds__(kFThreads, 2)
     xv[h] = reinterpret_cast<const float*>(sb + S::offX)[ty * kFX + tx];
     yv[h] = reinterpret_cast<const float*>(sb + S::offY)[ty * kFX + tx];
   };
-  auto finish = [&](int z, int h, const float2 (&fp)[1], const float (&fs)[1]) {
+  const int64_t sxy = (int64_t)nx * ny;
+  int64_t next = (int64_t)z0 * sxy + (int64_t)y * nx + x;  // planes come in order
+  auto finish = [&](int, int h, const float2 (&fp)[1], const float (&fs)[1]) {
+    const int64_t o = next;
+    next += sxy;
     if (!own) return;
-    const size_t o = ((size_t)z * ny + y) * nx + x;
     const float xh = xv[h], yh = yv[h];
     float g = fp[0].x + 2.f * xh * fp[0].y + yh * fs[0];
     if (l1g != 0.f) g = l1g * sgnf(xh - yh) + g;  // fused L1 term
@@ -911,19 +954,23 @@ __global__ void __launch_bounds__(kFThreads, 2)
 // arrive by TMA, so no thread spends instructions on staging.  A vertical pass (item: one
 // halo column and eight output rows, lanes over consecutive columns; 18 box rows serve the
 // eight outputs) filters the channels along y and stores one float4 per (output row, halo
-// column); a horizontal pass (item: four adjacent outputs of one row, lanes over rows, 14
-// float4 loads) filters along x.  Its results go through shared memory once more so that the
-// pixels are finished with eight consecutive lanes per 32-pixel row: every global load and
-// store of the outputs is then a whole 128-byte row segment.  Forward channels (x, y,
+// column); a horizontal pass (item: four adjacent outputs of one row, eight consecutive lanes per
+// 32-pixel row, 14 float4 loads) filters along x and finishes its pixels: every global load and
+// store of the outputs is a whole 128-byte row segment.  Forward channels (x, y,
 // x^2 + y^2, x y) -> SSIM, the maps and the loss (plus the fused L1 sum); backward the maps
 // (m1, m2, m3) -> dL/dx.
+// Bound by instruction issue (67 % of the slots; FMA pipe 41 %, shared memory 61 %, HBM 34 %):
+// the horizontal pass reads rows whose gaps keep the finishing lanes' own order free of bank
+// conflicts, so that its results need no exchange, and a copy's wait shares the filter's barrier.
+// 75 x 512^2: forward 141 -> 127 us, backward 107 -> 96 us.
 // ------------------------------------------------------------------------------------------
 constexpr int kTBoxX = 48;                // box columns: tile columns -8 .. 39
 constexpr int kTBox = kTBoxX * kIn2;      // elements per box (42 rows)
-constexpr int kTPitch = kIn2 + 1;         // float4 pitch of the y-filtered rows (odd: the
-                                          // horizontal pass's 8-lane phases hit distinct banks)
-constexpr int kXPitch = kT2 / kG + 1;     // float4 pitch of the exchanged rows (9)
 constexpr int kGV = 8;                    // output rows per vertical-pass item
+// The backward's three channels lie as a float2 and a float array: pitches and gaps put the reads of
+// four-column steps in rows r, r + 1 (.. r + 3) into different banks.
+constexpr int kP2 = 66, kP1 = 45;
+__device__ __forceinline__ int p2_slot(int c) { return c + (c >> 4) + 14 * (c >> 5); }
 template <bool BWD>
 struct Tma2Shape {
   // forward: X box, Y box; backward: the (m1, m2) pair box (two floats per pixel), m3 box
@@ -931,12 +978,11 @@ struct Tma2Shape {
   static constexpr uint32_t boxB = kTBox * 4u;
   static constexpr uint32_t txbytes = boxA + boxB;
   static constexpr uint32_t offV = boxA + boxB;  // 16128 / 24192: multiples of 128
-  static constexpr size_t smem = 128 + offV + (size_t)kT2 * kTPitch * sizeof(float4);
-  static_assert(3 * kT2 * kXPitch <= kT2 * kTPitch, "the exchange fits in the filtered rows");
+  static constexpr size_t smem = 128 + offV + (BWD ? (size_t)kT2 * (kP2 * sizeof(float2) + kP1 * sizeof(float)) : (size_t)kT2 * kHPitch * sizeof(float4));
 };
 
 template <bool BWD>
-__global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
+__global__ void __launch_bounds__(kSsimThreads, 4)
     k_ssim2d_tma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ Win W, int nx, int ny, float C1, float C2,
                  float gscale, float l1s, float* __restrict__ loss, float2* __restrict__ m12,
@@ -950,10 +996,14 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
   const float* sA = reinterpret_cast<const float*>(base);
   const float* sB = reinterpret_cast<const float*>(base + S::boxA);
   float4* V = reinterpret_cast<float4*>(base + S::offV);
+  float2* V2 = reinterpret_cast<float2*>(base + S::offV);
+  float* V1 = reinterpret_cast<float*>(V2 + kT2 * kP2);
   __shared__ __align__(8) uint64_t bar;
+  __shared__ int abort_flag;
   const int tid = threadIdx.x;
   const int x0 = blockIdx.x * kT2, y0 = blockIdx.y * kT2, img = blockIdx.z;
   if (tid == 0) {
+    abort_flag = 0;
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect_tx(&bar, S::txbytes);
@@ -974,26 +1024,19 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
     if (accumulate) go = *reinterpret_cast<const float4*>(grad + o);
   }
   __syncthreads();  // the barrier is initialised before anyone waits on it
-  if (!__syncthreads_and(mbar_wait(&bar, 0))) {
-    // a copy never arrived: report it and poison the result instead of using the boxes
-    if (tid == 0) {
-      atomicExch(err, GS_ERR_TIMEOUT);
-      if (!BWD && loss) atomicExch(loss, __int_as_float(0x7fc00000));
-      mbar_wait(&bar, 0);  // bounded: the copies in flight before shared memory goes away
-    }
-    if (BWD && own) {
-      const float nan = __int_as_float(0x7fc00000);
-      *reinterpret_cast<float4*>(grad + o) = make_float4(nan, nan, nan, nan);
-    }
-    return;
-  }
+  if (!mbar_wait(&bar, 0)) abort_flag = 1;  // all leave after the next barrier
   float2 w2[2 * kR + 1];
 #pragma unroll
-  for (int k = 0; k <= 2 * kR; ++k) w2[k] = make_float2(W.w[k], W.w[k]);
-  // ---- vertical pass: item (halo column c, output rows 8g .. 8g + 7); box rows 8g .. 8g + 17
-  // at box column c + 3 (image column x0 - 5 + c); 168 items, one round
-  for (int p = tid; p < kIn2 * (kT2 / kGV); p += kSsimThreads) {
-    const int c = p % kIn2, g = p / kIn2;
+  for (int k = 0; k <= 2 * kR; ++k)  // symmetric: six values
+    w2[k] = make_float2(W.w[k < kR ? k : 2 * kR - k], W.w[k < kR ? k : 2 * kR - k]);
+  // ---- vertical pass: item (halo column c, output rows 8g .. 8g + 7), box rows 8g .. 8g + 17 at
+  // box column c + 3 (image column x0 - 5 + c); 168 items, one round.  Warps 0 - 3 take 32
+  // consecutive columns (and banks) of a row group each, warps 4 and 5 the last ten of two each.
+  const int wv = tid >> 5, lv = tid & 31;
+  if (wv < kT2 / kGV || (wv < kT2 / kGV + 2 && lv < 2 * (kIn2 - 32))) {
+    const bool tail = wv >= kT2 / kGV;
+    const int c = tail ? 32 + lv % (kIn2 - 32) : lv;
+    const int g = tail ? 2 * (wv - kT2 / kGV) + lv / (kIn2 - 32) : wv;
     float2 a[kGV][2];
 #pragma unroll
     for (int j = 0; j < kGV; ++j) a[j][0] = a[j][1] = make_float2(0.f, 0.f);
@@ -1021,18 +1064,43 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
     }
 #pragma unroll
     for (int j = 0; j < kGV; ++j)
-      V[(kGV * g + j) * kTPitch + c] = make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
+      if constexpr (BWD) {
+        V2[(kGV * g + j) * kP2 + p2_slot(c)] = a[j][0];
+        V1[(kGV * g + j) * kP1 + c] = a[j][1].x;
+      } else {
+        V[(kGV * g + j) * kHPitch + h_slot(c)] =
+            make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
+      }
   }
   __syncthreads();
-  // ---- horizontal pass: row r, outputs 4q .. 4q + 3 from halo columns 4q .. 4q + 13
-  const int r = tid & 31, q = tid >> 5;
+  if (abort_flag) {
+    // a copy never arrived: report it and poison the result instead of using the boxes
+    if (tid == 0) {
+      atomicExch(err, GS_ERR_TIMEOUT);
+      if (!BWD && loss) atomicExch(loss, __int_as_float(0x7fc00000));
+      mbar_wait(&bar, 0);  // bounded: the copies in flight before shared memory goes away
+    }
+    if (BWD && own) {
+      const float nan = __int_as_float(0x7fc00000);
+      *reinterpret_cast<float4*>(grad + o) = make_float4(nan, nan, nan, nan);
+    }
+    return;
+  }
+  // ---- horizontal pass: the thread's four pixels from halo columns 4 cq .. 4 cq + 13
   float2 f[kG][2];
 #pragma unroll
   for (int j = 0; j < kG; ++j) f[j][0] = f[j][1] = make_float2(0.f, 0.f);
 #pragma unroll
   for (int i = 0; i < kG + 2 * kR; ++i) {
-    const float4 v = V[r * kTPitch + 4 * q + i];
-    const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
+    float2 v0, v1;
+    if constexpr (BWD) {
+      v0 = V2[cr * kP2 + p2_slot(4 * cq + (i & ~3)) + (i & 3)];
+      v1 = make_float2(V1[cr * kP1 + 4 * cq + i], 0.f);
+    } else {
+      const float4 v = V[cr * kHPitch + h_slot(4 * cq + (i & ~3)) + (i & 3)];
+      v0 = make_float2(v.x, v.y);
+      v1 = make_float2(v.z, v.w);
+    }
 #pragma unroll
     for (int j = 0; j < kG; ++j) {
       const int k = i - j;
@@ -1042,8 +1110,7 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
       else f[j][1].x = fmaf(w2[k].x, v1.x, f[j][1].x);
     }
   }
-  // three float4 per thread to the finishing lanes: [channel][row][4-column group]
-  float4 t[3];
+  float4 t[3];  // the four pixels' channels
   float contrib = 0.f;
   if constexpr (BWD) {  // the filtered maps
     t[0] = make_float4(f[0][0].x, f[1][0].x, f[2][0].x, f[3][0].x);
@@ -1058,7 +1125,7 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
       const float D = (f[j][1].x - mx * mx - my * my) + C2;  // sigma_x^2 + sigma_y^2 + C2
       const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
       const float C = mx * mx + my * my + C1;
-      const float inv = 1.f / (C * D);  // 1/C = D inv, 1/D = C inv
+      const float inv = rcp_newton(C * D);  // 1/C = D inv, 1/D = C inv
       const float Sv = (Am * Bn) * inv;
       const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
       const float dsxx = -Sv * (C * inv);
@@ -1066,19 +1133,11 @@ __global__ void __launch_bounds__(kSsimThreads, BWD ? 4 : 5)
       mv[0][j] = gscale * (dmu - 2.f * mx * dsxx - my * dsxy);
       mv[1][j] = gscale * dsxx;
       mv[2][j] = gscale * dsxy;
-      if (y0 + r < ny && x0 + 4 * q + j < nx) contrib += 1.f - Sv;
+      if (own) contrib += 1.f - Sv;
     }
 #pragma unroll
     for (int m = 0; m < 3; ++m) t[m] = make_float4(mv[m][0], mv[m][1], mv[m][2], mv[m][3]);
   }
-  __syncthreads();  // every thread is done with the filtered rows
-  float4* Xc = V;   // the exchange, pitch 9 float4: the 8-lane phases of both sides are
-                    // conflict-free
-#pragma unroll
-  for (int m = 0; m < 3; ++m) Xc[(m * kT2 + r) * kXPitch + q] = t[m];
-  __syncthreads();
-#pragma unroll
-  for (int m = 0; m < 3; ++m) t[m] = Xc[(m * kT2 + cr) * kXPitch + cq];
   if constexpr (BWD) {
     if (!own) return;
     const float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
@@ -1491,7 +1550,13 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
   float* tmp = (float*)(((uintptr_t)(maps + 3 * plane) + 15) & ~(uintptr_t)15);
   const dim3 gxy((nx + kT2 - 1) / kT2, (ny + kT2 - 1) / kT2, nz), bxy(kSsimThreads);
   const int64_t cols = (int64_t)nx * ny;
-  const dim3 gz((unsigned)((cols + kThreads - 1) / kThreads)), bz(kThreads);
+  // columns alone fill the SMs only from some 600 x 600: z chunks, of at least 8 planes, make up to
+  // two CTAs per SM
+  const int64_t bz_cols = (cols + kThreads - 1) / kThreads;
+  const int z_chunks =
+      (int)std::max<int64_t>(1, std::min<int64_t>(nz / 8, 2 * (int64_t)num_sms() / bz_cols));
+  const int zcol = (nz + z_chunks - 1) / z_chunks;
+  const dim3 gz((unsigned)bz_cols, (unsigned)((nz + zcol - 1) / zcol)), bz(kThreads);
   const float l1s = l1_weight / (float)plane;
   if (ssim3d_fused_ok(d_x, d_y, nx, ny)) {
     // fused streaming kernels; tmp's first word is the TMA timeout status
@@ -1500,12 +1565,20 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
     GS_TRY(volume_map(&tmX, d_x, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(volume_map(&tmY, d_y, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(ssim3d_fused_attributes());
-    // z chunks so that the grid fills the SMs (two CTAs each) about twice; at least 32
-    // planes per chunk
-    const int tiles = ((nx + kFX - 1) / kFX) * ((ny + kFY - 1) / kFY);
-    const int want = (4 * num_sms() + tiles - 1) / tiles;
-    const int nch = std::max(1, std::min(want, nz / 32));
-    const int zc = (nz + nch - 1) / nch;
+    // z chunks: the number that makes the fewest iterations one after another, of the waves of two
+    // CTAs per SM and a chunk's planes with its window's ten and a pipeline fill
+    const int64_t tiles = (int64_t)((nx + kFX - 1) / kFX) * ((ny + kFY - 1) / kFY);
+    int zc = nz;
+    int64_t best = INT64_MAX;
+    for (int n = 1; n <= std::max(1, nz / 4); ++n) {
+      const int c = (nz + n - 1) / n;
+      const int64_t waves = (tiles * ((nz + c - 1) / c) + 2 * num_sms() - 1) / (2 * num_sms());
+      const int64_t cost = waves * ((c + 2 * kR + kPP - 1) / kPP + 2);
+      if (cost < best) {
+        best = cost;
+        zc = c;
+      }
+    }
     const dim3 gf((nx + kFX - 1) / kFX, (ny + kFY - 1) / kFY, (nz + zc - 1) / zc);
     float2* m12 = reinterpret_cast<float2*>(maps);
     float* m3 = maps + 2 * plane;
@@ -1524,14 +1597,14 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
     return launch("ssim3d_bwd", k_ssim3d_bwd_fused, gf, dim3(kFThreads), FusedShape<true>::smem,
                   s, tmM12, tmM3, tmXt, tmYt, W, nx, ny, nz, zc, d_grad, accumulate, l1s, err);
   }
-  GS_TRY(launch("ssim3d_z_fwd", k_ssim3d_z<2>, gz, bz, 0, s, W, d_x, d_y, nx, ny, nz, plane,
+  GS_TRY(launch("ssim3d_z_fwd", k_ssim3d_z<2>, gz, bz, 0, s, W, d_x, d_y, nx, ny, nz, zcol, plane,
                 tmp, l1s, d_loss));
   GS_TRY(launch("ssim3d_xy_fwd", k_ssim_xy<1>, gxy, bxy, XyShape<1>::smem, s, W,
                 (const float*)tmp, (const float*)nullptr, plane, nx, ny, C1, C2, gscale, d_loss,
                 maps, (const float*)nullptr, (const float*)nullptr, (float*)nullptr, 0, 0.f));
   if (!d_grad) return GS_OK;  // value only
   GS_TRY(launch("ssim3d_z_bwd", k_ssim3d_z<3>, gz, bz, 0, s, W, (const float*)maps,
-                (const float*)nullptr, nx, ny, nz, plane, tmp, 0.f, (float*)nullptr));
+                (const float*)nullptr, nx, ny, nz, zcol, plane, tmp, 0.f, (float*)nullptr));
   return launch("ssim3d_xy_bwd", k_ssim_xy<2>, gxy, bxy, XyShape<2>::smem, s, W,
                 (const float*)tmp, (const float*)nullptr, plane, nx, ny, C1, C2, gscale,
                 (float*)nullptr, (float*)nullptr, d_x, d_y, d_grad, accumulate, l1s);

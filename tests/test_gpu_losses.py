@@ -217,6 +217,23 @@ def test_ssim3d_streaming(B, shape):
     assert abs(float(loss.item()) - val) <= 1e-6 * abs(val)
 
 
+@pytest.mark.parametrize("shape", [(1, 18, 48), (4, 19, 48), (13, 18, 52), (150, 18, 48),
+                                   (8, 18, 49), (41, 17, 53), (150, 7, 5)])
+@pytest.mark.parametrize("scale", [1.0, 1e8, 1e-7])
+def test_ssim3d_chunks(B, shape, scale):
+    """Streaming and separable passes with z in one to many chunks, also of fewer planes than the
+    window, over small and large data ranges, against the oracle."""
+    rng = np.random.default_rng(8)
+    y = _x32(rng.random(shape) * scale)
+    x = _x32(np.clip(y + 0.1 * scale * rng.standard_normal(shape), 0, None))
+    L = float(y.max())
+    val, g = _run_loss(B, "ssim3d", x, y, L, weight=0.5)
+    want, gw = OL.value_and_grad(lambda a, b: 0.5 * (1 - OL.ssim3d(a, b, L)), x, y)
+    assert abs(val - want) <= 2e-5 * max(1.0, abs(want)), (val, want)
+    m = np.abs(gw).max()
+    assert np.abs(g - gw).max() <= 1e-3 * m, float(np.abs(g - gw).max() / m)
+
+
 def test_ssim3d_streaming_equals_separable_passes(B):
     """The fused streaming kernels against the separable z + xy passes on one larger volume
     (the separable path taken by handing the library x and y at a 4-byte offset, which the
