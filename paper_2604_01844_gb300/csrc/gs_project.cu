@@ -15,8 +15,9 @@
 //   sorted       (more tiles) block sums and their scan, emit of (key, record) pairs in record
 //                order, stable radix sort over the tile bits, ranges
 //   raster_fwd   one CTA per (instance, view, tile), records on lanes
-//   raster_bwd   the same shape; six moment sums of g * exp(-q/2) per record, then one pair of
-//                float4 atomics (per-Gaussian backward, Sec. 3.5)
+//   raster_bwd   one warp per (instance, view, tile), records on lanes; six moment sums of
+//                g * exp(-q/2) per record, then one pair of float4 atomics (per-Gaussian backward,
+//                Sec. 3.5)
 //   chain        a thread per (Gaussian, 8 views): moments -> footprint gradients ->
 //                d(mean, rho, scale, quaternion)
 // The instance table travels by value as a __grid_constant__ kernel parameter, so a call does
@@ -756,47 +757,35 @@ __device__ __forceinline__ void slab_rows(const float4 g, const float4 c, float 
   yhi = min(T - 1, (int)floorf(g.y + ymax + 0.01f) - ty0);
 }
 
-// Bit mask of the (4-row x BW-column) blocks of a (T x T) tile at (tx0, ty0) that a record's
-// cut ellipse reaches: per column slab of its box, the reached rows (slab_rows) turned into
-// row bands.
-template <int T, int BW, int LBW, int NBX, int NBY>
+// Bit mask of the (4-row x BW-column) blocks of a (T x T) tile at (tx0, ty0) that a record's cut
+// ellipse reaches, bit column * NBY + band: per column slab of its box the reached rows
+// (slab_rows) make a run of bands.
+template <int T, int BW>
 __device__ __forceinline__ uint32_t block_mask(const float4 g, const float4 c, const short4 bx,
                                                int tx0, int ty0) {
+  constexpr int LBW = BW == 16 ? 4 : 3, NBX = T / BW, NBY = T / 4;
   const float cm = g.w * 1.001f;
   const SlabExt X = make_slab(c, cm);
-  const int bx0 = max(0, (bx.x - tx0) >> LBW), bx1 = min(NBX - 1, (bx.z - tx0) >> LBW);
+  const int bx0 = (bx.x - tx0) >> LBW, bx1 = (bx.z - tx0) >> LBW;
   const int ry0 = max(0, bx.y - ty0), ry1 = min(T - 1, bx.w - ty0);
   uint32_t mask = 0u;
-  for (int bxi = bx0; bxi <= bx1; ++bxi) {
-    const float x0 = (float)(tx0 + bxi * BW);
+#pragma unroll
+  for (int k = 0; k < NBX; ++k) {
+    const float x0 = (float)(tx0 + k * BW);
     int ylo, yhi;
     slab_rows(g, c, cm, X, x0, x0 + (float)(BW - 1), ty0, T, ylo, yhi);
     ylo = max(ylo, ry0);
     yhi = min(yhi, ry1);
-    for (int by = ylo >> 2; by <= (yhi >> 2) && ylo <= yhi; ++by) mask |= 1u << (by * NBX + bxi);
+    if (k >= bx0 && k <= bx1 && ylo <= yhi)
+      mask |= ((2u << (yhi >> 2)) - (1u << (ylo >> 2))) << (k * NBY);
   }
   return mask;
 }
 
-// Backward CTA shape: warps own blocks of 4 rows x BW columns (records on lanes, one pixel
-// column per unrolled step).  16 columns measured faster than 8 (fewer record visits outweigh
-// the lower in-cut share of a wider block).
-template <int T, int BW_>
-struct BlockShape {
-  static constexpr int BW = BW_;
-  static constexpr int LBW = BW_ == 16 ? 4 : 3;
-  static constexpr int NBX = T / BW, NBY = T / 4, NB = NBX * NBY;
-  static constexpr int NW = NB < 8 ? NB : 8;
-  static constexpr int NT = 32 * NW;
-  static constexpr int BPW = NB / NW;
-};
-template <int T>
-using BwdBlocks = BlockShape<T, (T >= 16 ? 16 : 8)>;
-
 // Raster forward (and the in-cut evaluation counter) with records on lanes, LPB lanes per
 // 4 x BW block of the (view, tile), 32 / LPB vertically adjacent blocks per warp.  Per batch of
-// staged records each warp lists the records whose cut ellipse reaches each of its blocks (the
-// block masks of the backward); the LPB lanes of a block take its records one per lane, and every
+// staged records each warp lists the records whose cut ellipse reaches each of its blocks (block
+// masks); the LPB lanes of a block take its records one per lane, and every
 // lane walks the block's pixels in the same unrolled order (pixel pairs in packed FP32x2
 // arithmetic, the exponent and the cut exactly as the backward computes them) and adds A 2^e to
 // its own accumulator of each pixel.  The accumulators live through all batches; at the end one
@@ -813,12 +802,11 @@ using BwdBlocks = BlockShape<T, (T >= 16 ? 16 : 8)>;
 // would take 1.00 -> 0.88 ms at 75 x 512^2, but in another order of the sums, and the L1 term of
 // a reconstruction step turns last-bit differences into flipped signs of its gradient.
 // Staging (two dependent gathers per record and its block mask) is about 30 % of the kernel:
-// records as one 32-byte sector, two gathers in flight per thread and approximate roots in the
-// mask took tile 16 from 1.00 to 0.93 ms and tile 32 from 4.49 to 4.34.
+// records as one 32-byte sector, two gathers in flight per thread, approximate roots in the mask and
+// its bands set as runs of bits took tile 16 from 1.00 to 0.93 ms and tile 32 from 4.49 to 4.17.
 template <int T>
 struct FwdBlocks {
   static constexpr int BW = T >= 16 ? 16 : 8;  // block width; 4 rows
-  static constexpr int LBW = BW == 16 ? 4 : 3;
   static constexpr int NBX = T / BW, NBY = T / 4, NB = NBX * NBY;
   static constexpr int LPB = T == 32 ? 8 : T == 16 ? 32 : 16;  // lanes per block
   static constexpr int BPW = 32 / LPB;             // blocks per warp, one above the other
@@ -851,8 +839,7 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   constexpr int LPB = S::LPB, BPW = S::BPW;
   const int part = lane / LPB, lp = lane % LPB;
-  // the warp's blocks bit0 (half 0) and bit0 + NBX (half 1, the block below)
-  const int bit0 = (w / S::NBX) * BPW * S::NBX + w % S::NBX;
+  const int bit0 = (w % S::NBX) * S::NBY + (w / S::NBX) * BPW;  // the warp's blocks: bits bit0 ..
   const int bxl = (w % S::NBX) * BW, byl = ((w / S::NBX) * BPW + part) * 4;
   const float fx0 = (float)(tx0 + bxl), fy0 = (float)(ty0 + byl);
   const unsigned lt = gsd::lanemask_lt();
@@ -874,11 +861,11 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
       const short4 b0 = rect[rec0], b1 = rect[rec1];
       s_geo[q] = g0;
       s_con[q] = c0;
-      s_mask[q] = block_mask<T, BW, S::LBW, S::NBX, S::NBY>(g0, c0, b0, tx0, ty0);
+      s_mask[q] = block_mask<T, BW>(g0, c0, b0, tx0, ty0);
       if (two) {
         s_geo[q + S::NT] = g1;
         s_con[q + S::NT] = c1;
-        s_mask[q + S::NT] = block_mask<T, BW, S::LBW, S::NBX, S::NBY>(g1, c1, b1, tx0, ty0);
+        s_mask[q + S::NT] = block_mask<T, BW>(g1, c1, b1, tx0, ty0);
       }
     }
     __syncthreads();
@@ -890,7 +877,7 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
       const uint32_t mk = jl < m ? s_mask[jl] >> bit0 : 0u;
 #pragma unroll
       for (int k = 0; k < BPW; ++k) {
-        const bool hit = (mk >> (k * S::NBX)) & 1u;
+        const bool hit = (mk >> k) & 1u;
         const unsigned bits = __ballot_sync(0xffffffffu, hit);
         if (hit) s_list[BPW * w + k][cnts[k] + __popc(bits & lt)] = (uint16_t)jl;
         cnts[k] += __popc(bits);
@@ -977,36 +964,47 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 }
 
 // ------------------------------------------------------------------------------------------
-// raster backward, per Gaussian (Sec. 3.5), with records on lanes.  The CTA shape is the
-// forward's: warps own blocks of 4 rows x BW columns of the (view, tile).  Per batch of staged
-// records, each warp lists the records whose cut ellipse reaches its block (closed-form test
-// of the ellipse against the block's rectangle, a superset of the per-pixel test) and takes
-// them 32 at a time, one per lane.  Every lane walks the block's 4 x BW pixels in the same
-// fully unrolled order, so the warp never diverges: dL/dI comes from shared memory as a
-// broadcast, the cut is decided exactly as in the forward (same offsets, same expression), and
-// the six moments of g exp(-q/2) stay in the lane's registers (row sums folded with dy; the x
-// moments taken about the block's centre column, whose offsets are compile-time constants,
-// and moved to the record's centre once per visit).  A lane then adds its six sums to the
-// record's shared accumulators; after the batch one thread per record adds them to the
-// record's moments (two float4 atomics).
+// raster backward, per Gaussian (Sec. 3.5), with records on lanes: one warp per (view, tile), or
+// per part of its list.  A lane holds one record at a time, walks the 4 x 8 blocks of the tile that
+// the record's cut ellipse reaches (closed-form test of the ellipse against the block's columns, a
+// superset of the per-pixel test), one block per round, keeps the six moments of g exp(-q/2) in
+// registers over all of them, adds them to the record's moments with two float4 atomics and takes
+// the next record from a queue that the warp refills 32 records at a time.  So every lane has a
+// block in every round but the list's last ones, nothing is summed through shared memory, and no
+// warp waits for another.  A round is fully unrolled and the same for all lanes: dL/dI comes from
+// shared memory at the lane's own block (blocks lie in different bank groups), the cut is decided
+// exactly as in the forward (same offsets, same expression).
+// Bound by instruction issue (71 %; FMA pipe 59 % of its cycles): per pixel pair two FMAs for the
+// exponent, two ex2, the cut, one product and three moment sums, and as much again per block for the
+// record's row coefficients, the centre shift and the queue.  Against warps that own 4 x 16 blocks,
+// list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1040 us;
+// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; tile 8, 30 x 512^2, 270 -> 242; 16 small reconstructions
+// 391 -> 314.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
+// Blocks that start at the record's own box instead of the grid cost their gain in bank conflicts
+// (1211).  24, 28, 32 warps per SM: 1051, 1043, 1079 (tile 32: 5.81, 5.88, 6.41 ms).
 // ------------------------------------------------------------------------------------------
 template <int T>
-__global__ void __launch_bounds__(BwdBlocks<T>::NT, 1024 / BwdBlocks<T>::NT)
+struct BwdBlocks {
+  static constexpr int BW = 8;             // block of 4 rows x 8 columns
+  static constexpr int NBX = T / BW, NBY = T / 4, NB = NBX * NBY;
+  // dL/dI in shared memory, in float4: per block, per pair of mirrored columns (p, 7 - p), the
+  // pair's four rows; one more float4 puts the blocks' equal places in different bank groups
+  static constexpr int GS = 9;
+};
+
+template <int T>
+__global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
     k_raster_bwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
                  const uint32_t* __restrict__ vals, const float4* __restrict__ recs,
                  const short4* __restrict__ rect,
                  const float* __restrict__ dimg, float4* __restrict__ fpgrad,
                  const gs_status* st) {
-  using S = BwdBlocks<T>;  // blockIdx.y: the part of the list this CTA takes
-  constexpr int BW = S::BW;
-  __shared__ __align__(16) float s_g[T][T];
-  constexpr int SB = 2 * S::NT;  // records staged per batch (more costs occupancy here)
-  __shared__ float4 s_geo[SB];
-  __shared__ float4 s_con[SB];
-  __shared__ uint32_t s_rec[SB];
-  __shared__ uint32_t s_mask[SB];
-  __shared__ float s_acc[6][SB];
-  __shared__ uint16_t s_list[S::NW][SB];
+  using S = BwdBlocks<T>;  // blockIdx.y: the part of the list this warp takes
+  __shared__ float4 s_g[(S::NB + 1) * S::GS];  // one block more, of zeros, for lanes without a record
+  __shared__ float2 s_xy[S::NB + 1];           // a block's first pixel centre
+  __shared__ float4 q_geo[32];  // the queue: records of a staged run that reach the tile
+  __shared__ float4 q_con[32];
+  __shared__ uint2 q_rm[32];    // record and block mask
   const int64_t key = blockIdx.x;
   uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
@@ -1022,112 +1020,161 @@ __global__ void __launch_bounds__(BwdBlocks<T>::NT, 1024 / BwdBlocks<T>::NT)
   const int W = I.W, H = I.H;
   const int tx0 = (tile % I.TW) * T, ty0 = (tile / I.TW) * T;
   const float* dv = dimg + I.img_off + (int64_t)v * H * W;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  for (int p = t; p < T * T; p += S::NT) {
-    const int x = tx0 + p % T, y = ty0 + p / T;
-    s_g[p / T][p % T] = (x < W && y < H) ? dv[(size_t)y * W + x] : 0.f;
+  const int lane = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < T * T / 32; ++k) {
+    const int q = lane + 32 * k, px = q % T, py = q / T, x = tx0 + px, y = ty0 + py;
+    const int col = px & 7, pair = col < 4 ? col : 7 - col;
+    reinterpret_cast<float*>(s_g)[((px >> 3) * S::NBY + (py >> 2)) * 4 * S::GS + pair * 8 +
+                                  (py & 3) * 2 + (col >> 2)] =
+        (x < W && y < H) ? dv[(size_t)y * W + x] : 0.f;
   }
+  if (lane < S::GS) s_g[S::NB * S::GS + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (lane == 0) s_xy[S::NB] = make_float2((float)tx0, (float)ty0);
+  if (lane < S::NB)
+    s_xy[lane] = make_float2((float)(tx0 + (lane / S::NBY) * S::BW),
+                             (float)(ty0 + (lane % S::NBY) * 4));
   const unsigned lt = gsd::lanemask_lt();
-  for (uint32_t base = r.x; base < r.y; base += SB) {
-    const int m = (int)min((uint32_t)SB, r.y - base);
-    __syncthreads();
-    for (int q = t; q < m; q += S::NT) {
-      const uint32_t rec = vals[base + q];
-      const float4 g = recs[2 * (size_t)rec], c = recs[2 * (size_t)rec + 1];
-      const short4 bx = rect[rec];
-      s_rec[q] = rec;
-      s_geo[q] = g;
-      s_con[q] = c;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) s_acc[k][q] = 0.f;
-      s_mask[q] = block_mask<T, S::BW, S::LBW, S::NBX, S::NBY>(g, c, bx, tx0, ty0);
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int k = 0; k < S::BPW; ++k) {
-      const int wb = w + k * S::NW;
-      const int bxl = (wb % S::NBX) * BW, byl = (wb / S::NBX) * 4;  // block origin in the tile
-      // this warp's list of the records that reach its block
-      int cnt = 0;
-      for (int j0 = 0; j0 < m; j0 += 32) {
-        const int jl = j0 + lane;
-        const bool hit = jl < m && ((s_mask[jl] >> wb) & 1u);
-        const unsigned bits = __ballot_sync(0xffffffffu, hit);
-        if (hit) s_list[w][cnt + __popc(bits & lt)] = (uint16_t)jl;
-        cnt += __popc(bits);
-      }
-      __syncwarp();
-      for (int c0 = 0; c0 < cnt; c0 += 32) {
-        const int li = c0 + lane;
-        const bool active = li < cnt;
-        const int j = active ? s_list[w][li] : 0;
-        const float4 g = s_geo[j];
-        const float4 c = s_con[j];
-        const float cut = active ? g.w : 1.f;  // e <= 0 < 1: an idle lane never passes
-        // pixel pairs (q, q + 1) of a row in packed FP32x2 arithmetic: each component rounds
-        // like the scalar fmaf / add / mul, so e and the cut are exactly the forward's
-        float2 dx[BW / 2];
-#pragma unroll
-        for (int p = 0; p < BW / 2; ++p)
-          dx[p] = make_float2((float)(tx0 + bxl + 2 * p) - g.x, (float)(tx0 + bxl + 2 * p + 1) - g.x);
-        const float2 ca = make_float2(c.x, c.x);
-        float s0 = 0.f, sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f;
-#pragma unroll
-        for (int ry = 0; ry < 4; ++ry) {
-          const float dy = (float)(ty0 + byl + ry) - g.y;
-          const float B = row_b(c, dy), cdy2 = row_c(c, dy);
-          const float2 B2 = make_float2(B, B), C2 = make_float2(cdy2, cdy2);
-          const float4* grow = reinterpret_cast<const float4*>(&s_g[byl + ry][bxl]);
-          float2 r0 = make_float2(0.f, 0.f), rx = r0, rxx = r0;
-#pragma unroll
-          for (int p = 0; p < BW / 2; ++p) {
-            const float2 e = __ffma2_rn(__ffma2_rn(ca, dx[p], B2), dx[p], C2);
-            const float4 g4 = grow[p >> 1];
-            const float2 gg = (p & 1) ? make_float2(g4.z, g4.w) : make_float2(g4.x, g4.y);
-            const float2 val = make_float2(e.x > cut ? ex2(e.x) : 0.f, e.y > cut ? ex2(e.y) : 0.f);
-            const float2 G = __fmul2_rn(gg, val);
-            // x moments about the block's centre: X = x - (x_block + (BW - 1) / 2) is a
-            // compile-time half-integer, so G X and G X^2 cost one packed FMA each
-            const float Xa = (float)(2 * p) - 0.5f * (float)(BW - 1), Xb = Xa + 1.f;
-            r0 = __fadd2_rn(r0, G);
-            rx = __ffma2_rn(G, make_float2(Xa, Xb), rx);
-            rxx = __ffma2_rn(G, make_float2(Xa * Xa, Xb * Xb), rxx);
-          }
-          const float r0s = r0.x + r0.y, rxs = rx.x + rx.y;
-          s0 += r0s;
-          sx += rxs;
-          sxx += rxx.x + rxx.y;
-          sy = fmaf(dy, r0s, sy);
-          sxy = fmaf(dy, rxs, sxy);
-          syy = fmaf(dy * dy, r0s, syy);
+  uint32_t pos = r.x;    // next record of the list to stage
+  int qh = 0, qn = 0;    // the queue's next and its end
+  // the lane's record: the blocks still to walk, its coefficients and its six sums
+  uint32_t rec = 0u, mask = 0u;
+  float gx = 0.f, gy = 0.f, cut = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+  float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
+  for (;;) {
+    bool need = mask == 0u;
+    unsigned idle = __ballot_sync(0xffffffffu, need);
+    if (idle) {
+      // finished records leave, waiting ones come in
+      if (need) {
+        if ((__float_as_uint(m0) | __float_as_uint(mx) | __float_as_uint(my)) |
+            (__float_as_uint(mxx) | __float_as_uint(mxy) | __float_as_uint(myy))) {
+          atomicAdd(&fpgrad[2 * (size_t)rec], make_float4(m0, mx, my, mxx));
+          atomicAdd(&fpgrad[2 * (size_t)rec + 1], make_float4(mxy, myy, 0.f, 0.f));
         }
-        {  // back to moments about the record's centre: dx = X + o
-          const float o = ((float)(tx0 + bxl) + 0.5f * (float)(BW - 1)) - g.x;
-          sxx = fmaf(o, fmaf(2.f, sx, o * s0), sxx);
-          sxy = fmaf(o, sy, sxy);
-          sx = fmaf(o, s0, sx);
+        m0 = mx = my = mxx = mxy = myy = 0.f;
+        cut = 1.f;  // e <= 0 < 1: an idle lane never passes
+      }
+      for (;;) {
+        const int slot = qh + __popc(idle & lt);
+        if (need && slot < qn) {
+          const float4 g = q_geo[slot], c = q_con[slot];
+          const uint2 rm = q_rm[slot];
+          gx = g.x;
+          gy = g.y;
+          cut = g.w;
+          c0 = c.x;
+          c1 = c.y;
+          c2 = c.z;
+          rec = rm.x;
+          mask = rm.y;
+          need = false;
         }
-        if (s0 != 0.f || sx != 0.f || sy != 0.f || sxx != 0.f || sxy != 0.f || syy != 0.f) {
-          atomicAdd(&s_acc[0][j], s0);
-          atomicAdd(&s_acc[1][j], sx);
-          atomicAdd(&s_acc[2][j], sy);
-          atomicAdd(&s_acc[3][j], sxx);
-          atomicAdd(&s_acc[4][j], sxy);
-          atomicAdd(&s_acc[5][j], syy);
+        qh += __popc(idle);
+        if (qh <= qn) {  // every lane has one
+          idle = 0u;
+          break;
+        }
+        qh = qn;
+        idle = __ballot_sync(0xffffffffu, need);
+        if (pos >= r.y) break;
+        // the queue is empty: stage the next run of records
+        const bool in = pos + lane < r.y;
+        float4 g, c;
+        uint32_t nrec = 0, nmask = 0;
+        if (in) {
+          nrec = vals[pos + lane];
+          g = recs[2 * (size_t)nrec];
+          c = recs[2 * (size_t)nrec + 1];
+          nmask = block_mask<T, S::BW>(g, c, rect[nrec], tx0, ty0);
+        }
+        pos += 32;
+        __syncwarp();  // the queue's last reads are done
+        const unsigned keep = __ballot_sync(0xffffffffu, nmask != 0u);
+        if (nmask) {
+          const int q = __popc(keep & lt);
+          q_geo[q] = g;
+          q_con[q] = c;
+          q_rm[q] = make_uint2(nrec, nmask);
+        }
+        qh = 0;
+        qn = __popc(keep);
+        __syncwarp();
+      }
+      if (idle == 0xffffffffu) break;
+    }
+    // ---- every lane walks the next block of its record
+    const int blk = mask ? 31 - __clz(mask) : S::NB;
+    mask &= ~(1u << (blk & 31));
+    const float2 xy = s_xy[blk];
+    const float4* gp = s_g + blk * S::GS;
+    // pixel pairs of a row in packed FP32x2 arithmetic: each component rounds like the scalar
+    // fmaf / add / mul, so e and the cut are exactly the forward's
+    const float2 ca = make_float2(c0, c0);
+    float2 B2[4], C2[4];
+#pragma unroll
+    for (int ry = 0; ry < 4; ++ry) {
+      const float dy = (xy.y + (float)ry) - gy;
+      const float B = c1 * dy, cdy2 = (c2 * dy) * dy;
+      B2[ry] = make_float2(B, B);
+      C2[ry] = make_float2(cdy2, cdy2);
+    }
+    // Moments about the block's centre.  Per pair of mirrored columns the four rows fold into
+    // Q = sum G, D = 2 sum Y G and P0, the outer rows' part (sum Y^2 G = 2 P0 + Q / 4).  Along x the
+    // outermost pair comes first and running sums give the weights: with n = 3 - p, |X| = n + 1/2
+    // and X^2 = 2 (n (n + 1) / 2) + 1/4, where the sum of the running sums weighs pair p by n and
+    // the sum of those by n (n + 1) / 2.  (No constants, so every step is one packed addition.)
+    float2 a0, q0, q1, q2, d0, d1;
+    float2 xp = make_float2(xy.x, xy.x + 7.f);
+    const float2 ngx = make_float2(-gx, -gx), m1 = make_float2(-1.f, -1.f);
+    const float2 step = make_float2(1.f, -1.f), three = make_float2(3.f, 3.f);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const float2 dx = __fadd2_rn(xp, ngx);
+      xp = __fadd2_rn(xp, step);  // exact
+      const float4 ga = gp[2 * p], gb = gp[2 * p + 1];  // rows 0, 1 and 2, 3
+      float2 G[4];
+#pragma unroll
+      for (int ry = 0; ry < 4; ++ry) {
+        const float2 e = __ffma2_rn(__ffma2_rn(ca, dx, B2[ry]), dx, C2[ry]);
+        const float2 gg = ry == 0   ? make_float2(ga.x, ga.y)
+                          : ry == 1 ? make_float2(ga.z, ga.w)
+                          : ry == 2 ? make_float2(gb.x, gb.y)
+                                    : make_float2(gb.z, gb.w);
+        const float2 val = make_float2(ex2(e.x), ex2(e.y));
+        G[ry] = __fmul2_rn(gg, make_float2(e.x > cut ? val.x : 0.f, e.y > cut ? val.y : 0.f));
+      }
+      const float2 P0 = __fadd2_rn(G[0], G[3]), P1 = __fadd2_rn(G[1], G[2]);
+      const float2 M0 = __ffma2_rn(G[0], m1, G[3]), M1 = __ffma2_rn(G[1], m1, G[2]);
+      const float2 D = __ffma2_rn(M0, three, M1), Q = __fadd2_rn(P0, P1);
+      if (p == 0) {
+        a0 = P0;
+        q0 = q1 = q2 = Q;
+        d0 = d1 = D;
+      } else {
+        a0 = __fadd2_rn(a0, P0);
+        q0 = __fadd2_rn(q0, Q);
+        d0 = __fadd2_rn(d0, D);
+        if (p < 3) {
+          q1 = __fadd2_rn(q1, q0);
+          q2 = __fadd2_rn(q2, q1);
+          d1 = __fadd2_rn(d1, d0);
         }
       }
-      __syncwarp();
     }
-    __syncthreads();
-    for (int q = t; q < m; q += S::NT) {
-      const float a0 = s_acc[0][q], a1 = s_acc[1][q], a2 = s_acc[2][q];
-      const float a3 = s_acc[3][q], a4 = s_acc[4][q], a5 = s_acc[5][q];
-      if (a0 != 0.f || a1 != 0.f || a2 != 0.f || a3 != 0.f || a4 != 0.f || a5 != 0.f) {
-        const uint32_t rec = s_rec[q];
-        atomicAdd(&fpgrad[2 * (size_t)rec], make_float4(a0, a1, a2, a3));
-        atomicAdd(&fpgrad[2 * (size_t)rec + 1], make_float4(a4, a5, 0.f, 0.f));
-      }
-    }
+    const float t0 = q0.x + q0.y, tx = fmaf(0.5f, q0.y - q0.x, q1.y - q1.x);
+    const float txx = fmaf(2.f, q2.x + q2.y, 0.25f * t0);
+    const float ty = 0.5f * (d0.x + d0.y), txy = 0.5f * fmaf(0.5f, d0.y - d0.x, d1.y - d1.x);
+    const float tyy = fmaf(2.f, a0.x + a0.y, 0.25f * t0);
+    // to moments about the record's centre: dx = X + ox, dy = Y + oy
+    const float ox = (xy.x + 3.5f) - gx, oy = (xy.y + 1.5f) - gy;
+    const float ux = fmaf(ox, t0, tx);
+    m0 += t0;
+    mx += ux;
+    my += fmaf(oy, t0, ty);
+    mxx += fmaf(ox, tx + ux, txx);
+    mxy += fmaf(ox, ty, fmaf(oy, ux, txy));
+    myy += fmaf(oy, fmaf(2.f, ty, oy * t0), tyy);
   }
 }
 
@@ -1352,12 +1399,13 @@ int raster_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* img,
 template <int T>
 int raster_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float* dimg,
                cudaStream_t s) {
-  // few tiles: their lists are split over up to 8 CTAs (the records' sums meet in atomics anyway),
-  // while the grid holds less than four CTAs per SM.  8 views of 64^2, 2000 Gaussians (128 tiles):
-  // 19 -> 11 us
-  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(8, 4 * (int64_t)num_sms() / p.n_keys));
+  // few tiles: their lists are split over up to 16 warps (the records' sums meet in atomics anyway),
+  // while the grid holds less than 16 warps per SM.  8 views of 64^2, 2000 Gaussians (128 tiles),
+  // up to 8 parts and 4 warps per SM: 14.7 us, 16: 11.8, 32 and 24 per SM: 12.2
+  const int parts =
+      (int)std::max<int64_t>(1, std::min<int64_t>(16, 16 * (int64_t)num_sms() / p.n_keys));
   return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys, parts),
-                dim3(BwdBlocks<T>::NT), 0, s,
+                dim3(32), 0, s,
                 p.b, (const uint2*)L.ranges, vals, (const float4*)L.rec,
                 (const short4*)L.rect, dimg, L.fpgrad, (const gs_status*)L.st);
 }

@@ -338,3 +338,11 @@ def test_lists_of_both_routes(orc, gsct, W, H, n, median):
     keep = ~amb[v_g, rd % n]
     want = np.sort((ko % TWH * nv + ko // TWH) * n + vo)
     assert np.array_equal(want, ((t_g * nv + v_g) * n + rd % n)[keep])
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n,median", [(1, 0.3), (31, 0.05), (32, 0.2), (33, 0.01), (130, 0.1)])
+def test_backward_list_lengths(orc, gsct, tile, n, median):
+    """Backward lists of one record, of just under, at and over a warp's width, of tiny and of
+    tile-filling footprints, over a ragged detector, against the oracle's gradients."""
+    _grad_case(orc, gsct, 40 + n, n, 3, 45, 39, tile, median=median)
