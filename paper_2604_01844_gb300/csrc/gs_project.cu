@@ -978,10 +978,11 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 // exponent, two ex2, the cut, one product and three moment sums, and as much again per block for the
 // record's row coefficients, the centre shift and the queue.  Against warps that own 4 x 16 blocks,
 // list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1040 us;
-// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; tile 8, 30 x 512^2, 270 -> 242; 16 small reconstructions
-// 391 -> 314.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
+// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; 41 x 389 x 517 parallel, 270 -> 243; 16 small
+// reconstructions 391 -> 318.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
 // Blocks that start at the record's own box instead of the grid cost their gain in bank conflicts
-// (1211).  24, 28, 32 warps per SM: 1051, 1043, 1079 (tile 32: 5.81, 5.88, 6.41 ms).
+// (1211).  24, 28, 32 warps per SM: 1051, 1043, 1079 (tile 32: 5.81, 5.88, 6.41 ms).  The last rows
+// of the grid take the narrow records (below), which the tiles' warps leave out.
 // ------------------------------------------------------------------------------------------
 template <int T>
 struct BwdBlocks {
@@ -990,7 +991,88 @@ struct BwdBlocks {
   // dL/dI in shared memory, in float4: per block, per pair of mirrored columns (p, 7 - p), the
   // pair's four rows; one more float4 puts the blocks' equal places in different bank groups
   static constexpr int GS = 9;
+  static constexpr int CW = T >= 16 ? 16 : 8;  // columns about whose centre narrow records sum
 };
+
+// Narrow records: the footprint may have a variance below kNarrowVar square pixels in some direction
+// (the trace of the conic bounds its inverse), in a box of at most 32 x 32 pixels.  Moved from a
+// block's centre to such a record's, second moments lose the digits that the centres' distance squared
+// has over the variance (50 times the rounding at 0.16 and 16-column blocks), so the order of their
+// sums shows in the gradients: they keep the one about 16-column runs, row by row (8 at tile 8), and
+// one thread takes all pixels of a record.  Gradients then move by at most 5e-6 (2-norm) against
+// warps that walk those blocks, instead of up to 2e-5.
+template <int T>
+__device__ __forceinline__ bool is_narrow(const float4 c, const short4 bx) {
+  constexpr float kNarrowVar = T >= 16 ? 0.16f : 0.04f;
+  return -(c.x + c.z) * kNarrowVar > 0.72134752f /* log2(e) / 2 */ &&
+         bx.z - bx.x < 32 && bx.w - bx.y < 32;
+}
+
+// The moments of a narrow record, one thread for all its pixels: bands of four rows by runs of CW
+// columns, about each run's centre, or about the record's own where its variance may lie below 0.005
+// (the move would cost more than four digits there).
+template <int T>
+__device__ __forceinline__ void narrow_moments(const float4 g, const float4 c, const short4 bx,
+                                               const float* __restrict__ dv, int W, int H,
+                                               float4* __restrict__ out) {
+  constexpr int CW = BwdBlocks<T>::CW;
+  const float cm = g.w * 1.001f, ia = 0.5f * rcp_approx(c.x);  // < 0
+  const bool own = -(c.x + c.z) * 0.005f > 0.72134752f;
+  float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
+  for (int by = bx.y & ~3; by <= bx.w; by += 4)
+    for (int x0 = bx.x & ~(CW - 1); x0 <= bx.z; x0 += CW) {
+      const float xc = own ? g.x : (float)x0 + 0.5f * (float)(CW - 1);
+      float s0 = 0.f, sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f;
+      for (int y = by; y < min(by + 4, H); ++y) {
+        const float dy = (float)y - g.y;
+        const float B = row_b(c, dy), C = row_c(c, dy);
+        // the row's section of the widened cut ellipse, to 1/50 pixel
+        const float D = fmaf(B, B, -4.f * c.x * (C - cm));
+        if (!(D >= 0.f)) continue;
+        const float mid = g.x - B * ia, half = 0.02f - sqrt_approx(D) * ia;
+        const int xa = max(x0, (int)ceilf(mid - half));
+        const int xb = min(min(x0 + CW, W) - 1, (int)floorf(mid + half));
+        float2 r0 = make_float2(0.f, 0.f), rx = r0, rxx = r0;  // even and odd columns
+        const float* row = dv + (size_t)y * W;
+        for (int x = xa & ~1; x <= xb; x += 4) {  // four pixels' loads at once
+          float G[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float dx = (float)(x + k) - g.x;
+            const float e = fmaf(fmaf(c.x, dx, B), dx, C);
+            const bool in = x + k >= xa && x + k <= xb;
+            G[k] = in && e > g.w ? __ldg(row + x + k) * ex2(e) : 0.f;
+          }
+#pragma unroll
+          for (int k = 0; k < 4; k += 2) {
+            const float X = (float)(x + k) - xc, X1 = (float)(x + k + 1) - xc;
+            r0.x += G[k];
+            r0.y += G[k + 1];
+            rx.x = fmaf(G[k], X, rx.x);
+            rx.y = fmaf(G[k + 1], X1, rx.y);
+            rxx.x = fmaf(G[k], X * X, rxx.x);
+            rxx.y = fmaf(G[k + 1], X1 * X1, rxx.y);
+          }
+        }
+        const float r0s = r0.x + r0.y, rxs = rx.x + rx.y;
+        s0 += r0s;
+        sx += rxs;
+        sxx += rxx.x + rxx.y;
+        sy = fmaf(dy, r0s, sy);
+        sxy = fmaf(dy, rxs, sxy);
+        syy = fmaf(dy * dy, r0s, syy);
+      }
+      const float o = xc - g.x;  // to moments about the record's centre: dx = X + o
+      m0 += s0;
+      mx += fmaf(o, s0, sx);
+      my += sy;
+      mxx += fmaf(o, fmaf(2.f, sx, o * s0), sxx);
+      mxy += fmaf(o, sy, sxy);
+      myy += syy;
+    }
+  out[0] = make_float4(m0, mx, my, mxx);
+  out[1] = make_float4(mxy, myy, 0.f, 0.f);
+}
 
 template <int T>
 __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
@@ -998,7 +1080,7 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
                  const uint32_t* __restrict__ vals, const float4* __restrict__ recs,
                  const short4* __restrict__ rect,
                  const float* __restrict__ dimg, float4* __restrict__ fpgrad,
-                 const gs_status* st) {
+                 const gs_status* st, int parts, int nblocks, int chunk) {
   using S = BwdBlocks<T>;  // blockIdx.y: the part of the list this warp takes
   __shared__ float4 s_g[(S::NB + 1) * S::GS];  // one block more, of zeros, for lanes without a record
   __shared__ float2 s_xy[S::NB + 1];           // a block's first pixel centre
@@ -1006,10 +1088,31 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
   __shared__ float4 q_con[32];
   __shared__ uint2 q_rm[32];    // record and block mask
   const int64_t key = blockIdx.x;
+  const int lane = threadIdx.x;
+  if (blockIdx.y >= parts) {  // the last rows of the grid: the narrow records, 32 chunk of them a warp
+    const int per = kThreads / 32 / chunk;  // warps per block of records
+    if (st->code != GS_OK) return;
+    const int64_t n = (int64_t)nblocks * per, step = (int64_t)(gridDim.y - parts) * gridDim.x;
+    for (int64_t w = (int64_t)(blockIdx.y - parts) * gridDim.x + blockIdx.x; w < n; w += step) {
+      const BlockItems bi = block_items(b, w / per);
+      const Inst& I = b.in[bi.inst];
+      const float* dv = dimg + I.img_off + (int64_t)bi.v * I.H * I.W;
+      const int64_t item0 = I.item_off + (int64_t)bi.v * I.n;
+      const int i0 = bi.i0 + (int)(w % per) * 32 * chunk + lane;
+#pragma unroll 4
+      for (int i = i0; i < min(I.n, i0 + 32 * chunk); i += 32) {
+        const float4 c = recs[2 * (item0 + i) + 1];
+        const short4 bx = rect[item0 + i];
+        if (is_narrow<T>(c, bx))
+          narrow_moments<T>(recs[2 * (item0 + i)], c, bx, dv, I.W, I.H, fpgrad + 2 * (item0 + i));
+      }
+    }
+    return;
+  }
   uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
-  if (gridDim.y > 1) {  // an equal part, in whole warps of records
-    const uint32_t part = ((r.y - r.x + gridDim.y - 1) / gridDim.y + 31u) & ~31u;
+  if (parts > 1) {  // an equal part, in whole warps of records
+    const uint32_t part = ((r.y - r.x + parts - 1) / parts + 31u) & ~31u;
     r.x = min(r.y, r.x + blockIdx.y * part);
     r.y = min(r.y, r.x + part);
   }
@@ -1020,7 +1123,6 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
   const int W = I.W, H = I.H;
   const int tx0 = (tile % I.TW) * T, ty0 = (tile / I.TW) * T;
   const float* dv = dimg + I.img_off + (int64_t)v * H * W;
-  const int lane = threadIdx.x;
 #pragma unroll
   for (int k = 0; k < T * T / 32; ++k) {
     const int q = lane + 32 * k, px = q % T, py = q / T, x = tx0 + px, y = ty0 + py;
@@ -1086,7 +1188,8 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
           nrec = vals[pos + lane];
           g = recs[2 * (size_t)nrec];
           c = recs[2 * (size_t)nrec + 1];
-          nmask = block_mask<T, S::BW>(g, c, rect[nrec], tx0, ty0);
+          const short4 bx = rect[nrec];
+          if (!is_narrow<T>(c, bx)) nmask = block_mask<T, S::BW>(g, c, bx, tx0, ty0);
         }
         pos += 32;
         __syncwarp();  // the queue's last reads are done
@@ -1404,10 +1507,15 @@ int raster_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float
   // up to 8 parts and 4 warps per SM: 14.7 us, 16: 11.8, 32 and 24 per SM: 12.2
   const int parts =
       (int)std::max<int64_t>(1, std::min<int64_t>(16, 16 * (int64_t)num_sms() / p.n_keys));
-  return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys, parts),
+  // warps for the narrow records: 32 records each while they are few, up to 256
+  int chunk = 1;
+  while (chunk < 8 && (int64_t)p.nblocks * (8 / chunk) > 16 * (int64_t)num_sms()) chunk *= 2;
+  const int64_t rows = std::min<int64_t>(
+      ((int64_t)p.nblocks * (8 / chunk) + p.n_keys - 1) / p.n_keys, 65535 - parts);
+  return launch("raster_bwd", k_raster_bwd<T>, dim3((unsigned)p.n_keys, (unsigned)(parts + rows)),
                 dim3(32), 0, s,
                 p.b, (const uint2*)L.ranges, vals, (const float4*)L.rec,
-                (const short4*)L.rect, dimg, L.fpgrad, (const gs_status*)L.st);
+                (const short4*)L.rect, dimg, L.fpgrad, (const gs_status*)L.st, parts, p.nblocks, chunk);
 }
 
 int dispatch_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* img, bool count,

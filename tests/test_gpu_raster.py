@@ -346,3 +346,12 @@ def test_backward_list_lengths(orc, gsct, tile, n, median):
     """Backward lists of one record, of just under, at and over a warp's width, of tiny and of
     tile-filling footprints, over a ragged detector, against the oracle's gradients."""
     _grad_case(orc, gsct, 40 + n, n, 3, 45, 39, tile, median=median)
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n,median,W,H", [(500, 0.004, 45, 39), (700, 0.008, 70, 33),
+                                          (2000, 0.02, 7, 5)])
+def test_backward_narrow_footprints(orc, gsct, tile, n, median, W, H):
+    """Footprints around and below a pixel (summed by one thread each), over several tiles and
+    inside one, against the oracle's gradients."""
+    _grad_case(orc, gsct, 50 + W, n, 4, W, H, tile, median=median)
