@@ -428,11 +428,11 @@ __device__ __forceinline__ uint8_t visit_code(const VGrid& g, const float4 G, co
 __device__ __forceinline__ void visit_codes(const VGrid& g, const float4* s_geo,
                                             const VisitCoef* s_vc, const short4* s_lo,
                                             const short4* s_hi, int m, int sx, int sy, int sz,
-                                            int k_lo, int depth, uint8_t* s_zr) {
+                                            int k_lo, int depth, uint8_t* s_zr, int pitch) {
   const float inv_hz = 1.f / g.h[2];
   for (int t = threadIdx.x; t < m * kWarps; t += kThreads) {
     const int j = t >> 3, w = t & 7;
-    s_zr[w * kThreads + j] = visit_code(g, s_geo[j], s_vc[j], s_lo[j], s_hi[j], sx, sy, sz,
+    s_zr[w * pitch + j] = visit_code(g, s_geo[j], s_vc[j], s_lo[j], s_hi[j], sx, sy, sz,
                                         k_lo, depth, w, inv_hz);
   }
 }
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       s_vc[tid] = visit_coef(c0, c1);
     }
     __syncthreads();
-    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr);
+    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr, kThreads);
     __syncthreads();
     const uint8_t* zrw = s_zr + w * kThreads;
     for (int j0 = 0; j0 < m; j0 += 32) {
@@ -614,53 +614,21 @@ __global__ void __launch_bounds__(kThreads, 4)
   }
 }
 
-// The ten moment sums of a warp patch from each column's three z moments q0, q1, qzz (of 1, dz,
-// dz^2), dx depending on the lane's position in its row of eight and dy on the row.  First along x:
-// the six sums of q0 {1, dx, dx^2}, q1 {1, dx} and qzz over a row's eight lanes, a reduce-scatter
-// in six shuffles that leaves lane x of the row with sum number x (0 .. 5, in the order (q0, q0
-// dx), (q1, q1 dx), (q0 dx^2, qzz)); then each lane's sum and its products with dy and dy^2 over
-// the four rows, six shuffles.  Lane x of row 0 holds sum x, of row 1 its dy moment, of row 2 its
-// dy^2 moment; moment_index gives the place among the ten, or -1.
-__device__ __forceinline__ float patch_moments(float q0, float q1, float qzz, float dx, float dy,
-                                               int lane) {
-  const float ex = q0 * dx;
-  // the lane's low bits choose: bit 0 the second of a pair, bits 1 and 2 the pair
-  const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
-  const float a0 = b0 ? ex : q0, s0 = b0 ? q0 : ex;
-  const float e1 = q1 * dx;
-  const float a1 = b0 ? e1 : q1, s1 = b0 ? q1 : e1;
-  const float e2 = ex * dx;
-  const float a2 = b0 ? qzz : e2, s2 = b0 ? e2 : qzz;
-  const float r0 = a0 + __shfl_xor_sync(0xffffffffu, s0, 1);  // pairs summed over bit 0
-  const float r1 = a1 + __shfl_xor_sync(0xffffffffu, s1, 1);
-  float r2 = a2 + __shfl_xor_sync(0xffffffffu, s2, 1);
-  // bit 1: lanes keep pair 0 or 1; the third pair is summed over bit 1 by both
-  const float k = (b1 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, b1 ? r0 : r1, 2);
-  r2 += __shfl_xor_sync(0xffffffffu, r2, 2);
-  // bit 2: lanes 0 - 3 keep pairs 0 and 1, lanes 4 - 7 the third pair
-  const float v = (b2 ? r2 : k) + __shfl_xor_sync(0xffffffffu, b2 ? k : r2, 4);
-  float m0 = v, m1 = v * dy, m2 = m1 * dy;
-#pragma unroll
-  for (int o = 8; o <= 16; o <<= 1) {
-    m0 += __shfl_xor_sync(0xffffffffu, m0, o);
-    m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-    m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-  }
-  const int row = lane >> 3;
-  return row == 0 ? m0 : row == 1 ? m1 : m2;
-}
-// Ten moments {1, dx, dy, dz, dx dx, dx dy, dx dz, dy dy, dy dz, dz dz}; the lane's one, or -1.
-__device__ __forceinline__ int moment_index(int lane) {
-  // by row (power of dy) and lane in the row: q0, q0 dx, q1, q1 dx, q0 dx^2, qzz
-  const uint32_t row0 = 0x946310u;  // 0, 1, 3, 6, 4, 9
-  const uint32_t row1 = 0x852u;      // dy times: 2, 5, 8
-  const int x = lane & 7, row = lane >> 3;
-  if (row == 0) return x < 6 ? (int)((row0 >> (4 * x)) & 15u) : -1;
-  if (row == 1) return x < 3 ? (int)((row1 >> (4 * x)) & 15u) : -1;
-  return row == 2 && x == 0 ? 7 : -1;
-}
+// A warp's visits leave each column's three z moments q0, q1, qzz (of 1, dz, dz^2) in shared memory;
+// after kVisits of them (or the batch's last) four lanes per visit, one per row of its patch, sum
+// the columns' ten moments {1, dx, dy, dz, dx dx, dx dy, dx dz, dy dy, dy dz, dz dz}.  A reduction
+// over the warp for each visit (12 shuffles, and atomics by ten lanes) took a third of the kernel's
+// instructions, which are what bounds it: 256^3, 50k Gaussians 138 -> 122 us, 1024^3, 500k 2107 ->
+// 1906 us, with the switch into the pairs' walk.  Batches of 216 records instead of 256 pay for the
+// buffer: long lists of Gaussians below a voxel gain nothing (92 x 75 x 83, 30k 111 -> 118 us).
+constexpr int kVisits = 8;
+constexpr int kVPitch = 36;  // floats per visit: rows of two neighbours in different bank groups
+struct VisitBuf {
+  float q[3][kVisits][kVPitch];
+};
 
 constexpr int kMoments = 10;
+constexpr int kRB = 216;  // records per batch of the backward: its shared memory stays below 48 KB
 
 template <int NP>  // z pairs per column and CTA, as in the forward
 __global__ void __launch_bounds__(kThreads, 4)
@@ -670,14 +638,17 @@ __global__ void __launch_bounds__(kThreads, 4)
               const short4* __restrict__ hi_in, const __grid_constant__ VBatch bt,
               const float* __restrict__ dvol_all, float4* __restrict__ vgrad,
               const gs_status* st) {
-  __shared__ float4 s_geo[kThreads];
-  __shared__ float4 s_c0[kThreads];
-  __shared__ float4 s_c1[kThreads];
-  __shared__ short4 s_lo[kThreads];
-  __shared__ short4 s_hi[kThreads];
-  __shared__ VisitCoef s_vc[kThreads];
-  __shared__ uint8_t s_zr[kWarps * kThreads];
-  __shared__ float s_mom[kThreads * kMoments];
+  __shared__ float4 s_geo[kRB];
+  __shared__ float4 s_c0[kRB];
+  __shared__ float4 s_c1[kRB];
+  __shared__ uint8_t s_zr[kWarps * kRB];
+  __shared__ float s_mom[kRB * kMoments];
+  // the visits' moments; while a batch is staged, what its visit codes are made from
+  __shared__ __align__(16) VisitBuf s_buf[kWarps];
+  short4* s_lo = reinterpret_cast<short4*>(s_buf);
+  short4* s_hi = s_lo + kRB;
+  VisitCoef* s_vc = reinterpret_cast<VisitCoef*>(s_hi + kRB);
+  static_assert(kRB * (2 * sizeof(short4) + sizeof(VisitCoef)) <= sizeof(s_buf), "fits");
   // one CTA per (brick, sub-brick, run of NP z pairs)
   constexpr uint32_t PARTS = kS / 2 / NP;
   const uint32_t cta = blockIdx.x / PARTS;
@@ -696,7 +667,6 @@ __global__ void __launch_bounds__(kThreads, 4)
   const float* dvol = dvol_all + I.vol_off;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const float hz = g.h[2];
-  const int mom_index = moment_index(lane);
   const int x = sx + (w & 1) * 8 + (lane & 7), y = sy + (w >> 1) * 4 + (lane >> 3);
   const bool in_xy = x < xend && y < yend;
   // dL/dV of this lane's column (0 outside the region)
@@ -714,8 +684,8 @@ __global__ void __launch_bounds__(kThreads, 4)
   const float xc = g.o[0] + ((float)x + 0.5f) * g.h[0];
   const float yc = g.o[1] + ((float)y + 0.5f) * g.h[1];
   const float zc0 = g.o[2] + ((float)sz + 0.5f) * hz;
-  for (uint32_t base = r.x; base < r.y; base += kThreads) {
-    const int m = (int)min((uint32_t)kThreads, r.y - base);
+  for (uint32_t base = r.x; base < r.y; base += kRB) {
+    const int m = (int)min((uint32_t)kRB, r.y - base);
     __syncthreads();  // the previous batch's accumulators are flushed
     uint32_t myI = 0;
     if (tid < m) {
@@ -731,9 +701,72 @@ __global__ void __launch_bounds__(kThreads, 4)
       for (int k = 0; k < kMoments; ++k) s_mom[tid * kMoments + k] = 0.f;
     }
     __syncthreads();
-    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr);
+    visit_codes(g, s_geo, s_vc, s_lo, s_hi, m, sx, sy, sz, k_lo, 2 * NP, s_zr, kRB);
     __syncthreads();
-    const uint8_t* zrw = s_zr + w * kThreads;
+    const uint8_t* zrw = s_zr + w * kRB;
+    VisitBuf& vb = s_buf[w];
+    int nv = 0, vj = 0;  // buffered visits; the record of the lane's one
+    // the buffered visits' moments, added to their records
+    auto flush = [&] {
+      __syncwarp();
+      const int vi = lane >> 2, row = lane & 3;
+      const bool in = vi < nv;
+      float M[kMoments];
+      {
+        const float4 G = s_geo[vj];
+        const float x0 = (float)(sx + (w & 1) * 8) + 0.5f;
+        const float dy = g.o[1] + ((float)(sy + (w >> 1) * 4 + row) + 0.5f) * g.h[1] - G.y;
+        float q[3][8];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float4 f = *reinterpret_cast<const float4*>(&vb.q[c][vi][8 * row + 4 * h]);
+            q[c][4 * h] = f.x;
+            q[c][4 * h + 1] = f.y;
+            q[c][4 * h + 2] = f.z;
+            q[c][4 * h + 3] = f.w;
+          }
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, t0 = 0.f, t1 = 0.f, u0 = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          // the column's centre rounded as the walk has it
+          const float xc = g.o[0] + (x0 + (float)i) * g.h[0], dx = xc - G.x, e = q[0][i] * dx;
+          s0 += q[0][i];
+          s1 += e;
+          s2 = fmaf(e, dx, s2);
+          t0 += q[1][i];
+          t1 = fmaf(q[1][i], dx, t1);
+          u0 += q[2][i];
+        }
+        M[0] = s0;
+        M[1] = s1;
+        M[2] = dy * s0;
+        M[3] = t0;
+        M[4] = s2;
+        M[5] = dy * s1;
+        M[6] = t1;
+        M[7] = dy * M[2];
+        M[8] = dy * t0;
+        M[9] = u0;
+      }
+#pragma unroll
+      for (int c = 0; c < kMoments; ++c) {
+        M[c] += __shfl_xor_sync(0xffffffffu, M[c], 1);
+        M[c] += __shfl_xor_sync(0xffffffffu, M[c], 2);
+      }
+      if (in) {  // the four lanes share the ten sums
+        float* mm = s_mom + vj * kMoments;
+        const float a = row == 0 ? M[0] : row == 1 ? M[1] : row == 2 ? M[2] : M[3];
+        const float b = row == 0 ? M[4] : row == 1 ? M[5] : row == 2 ? M[6] : M[7];
+        atomicAdd(mm + row, a);
+        atomicAdd(mm + 4 + row, b);
+        if (row < 2) atomicAdd(mm + 8 + row, row ? M[9] : M[8]);
+      }
+      __syncwarp();
+      nv = 0;
+    };
+
     for (int j0 = 0; j0 < m; j0 += 32) {
       const uint8_t mine = j0 + lane < m ? zrw[j0 + lane] : kNoVisit;
       unsigned todo = __ballot_sync(0xffffffffu, mine != kNoVisit);
@@ -751,13 +784,10 @@ __global__ void __launch_bounds__(kThreads, 4)
         const float2 c22 = make_float2(c1.y, c1.y), hz2 = make_float2(hz, hz);
         const float2 dz02 = make_float2(dz0, dz0);
         float2 s0 = make_float2(0.f, 0.f), s1 = s0, s2 = s0;
-        // the forward's closed-form exponent over the record's exact pair range: the
-        // backward's per-pair work is long enough that skipping the pairs outside the range
-        // pays for the uniform branches (dz of both voxels in one packed FMA, as the forward)
-        const int p0 = code & 15, p1 = code >> 4;  // warp-uniform
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          if (p < p0 || p > p1) continue;
+        // the forward's closed-form exponent over the record's exact pair range, entered at its
+        // first pair and left after its last (dz of both voxels in one packed FMA, as the forward)
+        const int p1 = code >> 4;  // warp-uniform
+        auto pair = [&](int p) {
           const float2 dz = __ffma2_rn(
               make_float2((float)(k_lo + 2 * p), (float)(k_lo + 2 * p + 1)), hz2, dz02);
           const float2 e = __ffma2_rn(__ffma2_rn(c22, dz, l2), dz, q2);
@@ -768,12 +798,27 @@ __global__ void __launch_bounds__(kThreads, 4)
           s0 = __fadd2_rn(s0, q);
           s1 = __fadd2_rn(s1, qd);
           s2 = __ffma2_rn(qd, dz, s2);
+        };
+#define GS_PAIR(P)                          \
+  case P:                                   \
+    if constexpr (P < NP) {                 \
+      pair(P);                              \
+      if (P == NP - 1 || p1 == P) break;    \
+    }                                       \
+    [[fallthrough]];
+        switch (code & 15) {
+          GS_PAIR(0) GS_PAIR(1) GS_PAIR(2) GS_PAIR(3) GS_PAIR(4) GS_PAIR(5) GS_PAIR(6) GS_PAIR(7)
+          default: break;
         }
-        const float q0 = s0.x + s0.y, q1 = s1.x + s1.y, qzz = s2.x + s2.y;
-        const float mv = patch_moments(q0, q1, qzz, dx, dy, lane);
-        if (mom_index >= 0) atomicAdd(&s_mom[j * kMoments + mom_index], mv);
+#undef GS_PAIR
+        vb.q[0][nv][lane] = s0.x + s0.y;
+        vb.q[1][nv][lane] = s1.x + s1.y;
+        vb.q[2][nv][lane] = s2.x + s2.y;
+        if (lane >> 2 == nv) vj = j;
+        if (++nv == kVisits) flush();
       }
     }
+    if (nv) flush();
     __syncthreads();
     if (tid < m) {
       const float* mm = s_mom + tid * kMoments;
