@@ -19,10 +19,10 @@
 //               before) and the grid divisions by multiplication
 //   vox_bwd     the same visits, over each record's exact pair range, with dL/dV of the lane's
 //               column in registers; per visited record each lane forms its column's three z
-//               moments of g exp(-q/2), which the warp sums along x, then along y (12 shuffles),
-//               leaving each of the ten moments in one lane, which adds it to the record's
+//               moments of g exp(-q/2) and leaves them in shared memory, and after eight visits
+//               four lanes per visit sum the columns' ten moments and add them to the record's
 //               shared accumulators; after the sub-brick, three float4 atomics per record
-//               (1024^3: 2.30 -> 2.11 ms; forming all ten products per lane first cost more)
+//               (1024^3: 2.30 -> 1.91 ms)
 //   vox_chain   one thread per Gaussian: moments -> d(mean, rho, scale, quaternion)
 //
 // Visit test of a record against a warp patch.  In the pre-scaled base-2 exponent

@@ -355,3 +355,23 @@ def test_backward_narrow_footprints(orc, gsct, tile, n, median, W, H):
     """Footprints around and below a pixel (summed by one thread each), over several tiles and
     inside one, against the oracle's gradients."""
     _grad_case(orc, gsct, 50 + W, n, 4, W, H, tile, median=median)
+
+
+def test_stream_handle_follows_the_current_stream(gsct):
+    """The handle is the calling thread's current stream, inside and outside a stream context."""
+    import threading
+
+    import torch
+
+    from paper_2604_01844_gb300 import binding as B
+
+    side, seen = torch.cuda.Stream(), []
+    want = torch.cuda.current_stream().cuda_stream
+    assert B.stream_handle() == want
+    with torch.cuda.stream(side):
+        assert B.stream_handle() == side.cuda_stream != want
+        t = threading.Thread(target=lambda: seen.append(B.stream_handle()))
+        t.start()
+        t.join()
+    assert seen == [want] and B.stream_handle() == want
+    assert B.stream_handle(side) == side.cuda_stream
