@@ -208,7 +208,8 @@ Layout carve(void* ws, const Plan& p) {
     L.gsum = c.take<unsigned long long>(groups);
     L.ticket = c.take<uint32_t>(1);
     L.vkeys = c.take<long long>(p.total_v + 1);
-    L.vals = c.take<uint32_t>(p.cap);
+    // the lists; 16 bytes per pair as on the other route, so that both hold the same capacity
+    L.vals = c.take<uint32_t>(4 * p.cap);
   } else {
     L.keys = c.take<uint32_t>(p.cap);
     L.vals = c.take<uint32_t>(p.cap);
@@ -1392,9 +1393,8 @@ int cap_from_ws(const gs_instance* inst, int n_inst, const gs_opts* o, size_t ws
   GS_TRY(make_plan(inst, n_inst, o, 0, p0));
   const size_t base = carve(nullptr, p0).bytes;
   if (ws_bytes < base) return GS_ERR_CAPACITY;
-  // each unit of capacity costs 4 bytes (direct: the lists) or 16 (sorted: keys, vals and their
-  // alternates) plus alignment
-  int64_t c = (int64_t)((ws_bytes - base) / (p0.direct ? 4 : 16));
+  // each unit of capacity costs 16 bytes (keys, vals and their alternates) plus alignment
+  int64_t c = (int64_t)((ws_bytes - base) / 16);
   while (c > 0) {
     Plan p;
     GS_TRY(make_plan(inst, n_inst, o, c, p));
