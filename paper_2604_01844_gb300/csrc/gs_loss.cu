@@ -39,8 +39,8 @@ __device__ __forceinline__ float rcp_newton(float x) {
   return fabsf(e) < 1.f ? fmaf(r, e, r) : r;
 }
 
-template <typename T>
-__device__ __forceinline__ void block_add(T v, T* target) {
+template <typename T, typename U>
+__device__ __forceinline__ void block_add(T v, U* target) {
   __shared__ T part[32];
   v = gsd::warp_sum(v);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -55,7 +55,7 @@ __device__ __forceinline__ void block_add(T v, T* target) {
   if (tid == 0) {
     T s = 0;
     for (int i = 0; i < (nthreads + 31) / 32; ++i) s += part[i];
-    if (s != (T)0) atomicAdd(target, s);
+    if (s != (T)0) atomicAdd(target, (U)s);
   }
   __syncthreads();
 }
@@ -256,30 +256,28 @@ __global__ void __launch_bounds__(kThreads)
   for (int k = 0; k <= 2 * kR; ++k)
 #pragma unroll
     for (int i = 0; i < NIN; ++i) ring[k][i] = 0.f;
-  // this chunk's outputs z0 .. z1 - 1; plane zi = z0 - kR + p enters ring slot p % 11, and output
-  // z = zi - kR is complete once it is in
-  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  // this chunk's outputs z0 .. z1 - 1 from planes zb .. zend - 1 (zeros beyond the volume); the
+  // k-th plane enters ring slot k % 11, output z = zi - kR is complete once plane zi is in
+  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc), zend = min(nz, z1 + kR);
   float nxt[NIN];
-  auto next_plane = [&](int zn) {
-    if (zn >= 0 && zn < nz) {
-      load((int64_t)zn * sxy + col, nxt);
-    } else {
-#pragma unroll
-      for (int i = 0; i < NIN; ++i) nxt[i] = 0.f;
-    }
-  };
-  next_plane(z0 - kR);
-  for (int zb = z0 - kR; zb < z1 + kR; zb += 2 * kR + 1) {
+  load((int64_t)max(0, z0 - kR) * sxy + col, nxt);
+  for (int zb = max(0, z0 - kR); zb < z1 + kR; zb += 2 * kR + 1) {
 #pragma unroll
     for (int k = 0; k <= 2 * kR; ++k) {
       const int zi = zb + k;
 #pragma unroll
       for (int i = 0; i < NIN; ++i) ring[k][i] = nxt[i];
       if (NIN == 2 && l1_scale != 0.f && zi >= z0 && zi < z1) l1 += fabsf(nxt[0] - nxt[1]);
-      next_plane(zi + 1);
+      const int zn = zi + 1;
+      if (zn < zend) {
+        load((int64_t)zn * sxy + col, nxt);
+      } else {
+#pragma unroll
+        for (int i = 0; i < NIN; ++i) nxt[i] = 0.f;
+      }
       // the column's element 4 planes ahead is requested into L2 now, so that the load of the
       // next plane rarely waits for DRAM
-      if (zi + 4 >= 0 && zi + 4 < min(nz, z1 + kR)) {
+      if (zi + 4 < zend) {
         const int64_t o4 = (int64_t)(zi + 4) * sxy + col;
         if (NIN == 2) {
           asm volatile("prefetch.global.L2 [%0];" ::"l"(A0 + o4));
@@ -419,8 +417,7 @@ __global__ void __launch_bounds__(kSsimThreads)
   }
   float2 w2[2 * kR + 1];
 #pragma unroll
-  for (int k = 0; k <= 2 * kR; ++k)  // symmetric: six values
-    w2[k] = make_float2(W.w[k < kR ? k : 2 * kR - k], W.w[k < kR ? k : 2 * kR - k]);
+  for (int k = 0; k <= 2 * kR; ++k) w2[k] = make_float2(W.w[k], W.w[k]);
   __syncthreads();
   // ---- horizontal pass: item p = (row r, columns c0 .. c0 + 3); lanes take consecutive rows
   for (int p = tid; p < kIn2 * (kT2 / kG); p += kSsimThreads) {
@@ -527,7 +524,7 @@ __global__ void __launch_bounds__(kSsimThreads)
       }
       const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
       const float C = mx * mx + my * my + C1;
-      const float inv = rcp_newton(C * D);  // 1/C = D inv, 1/D = C inv
+      const float inv = 1.f / (C * D);  // 1/C = D inv, 1/D = C inv
       const float Sv = (Am * Bn) * inv;
       const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
       const float dsxx = -Sv * (C * inv);
@@ -959,14 +956,16 @@ __global__ void __launch_bounds__(kFThreads, 2)
 // store of the outputs is a whole 128-byte row segment.  Forward channels (x, y,
 // x^2 + y^2, x y) -> SSIM, the maps and the loss (plus the fused L1 sum); backward the maps
 // (m1, m2, m3) -> dL/dx.
+// A CTA takes its tile of up to four images: the next image's copies start once the boxes are read.
 // Bound by instruction issue (67 % of the slots; FMA pipe 41 %, shared memory 61 %, HBM 34 %):
 // the horizontal pass reads rows whose gaps keep the finishing lanes' own order free of bank
 // conflicts, so that its results need no exchange, and a copy's wait shares the filter's barrier.
-// 75 x 512^2: forward 141 -> 127 us, backward 107 -> 96 us.
+// 75 x 512^2: forward 141 -> 118 us, backward 107 -> 92 us.
 // ------------------------------------------------------------------------------------------
 constexpr int kTBoxX = 48;                // box columns: tile columns -8 .. 39
 constexpr int kTBox = kTBoxX * kIn2;      // elements per box (42 rows)
 constexpr int kGV = 8;                    // output rows per vertical-pass item
+constexpr int kLossSlots = 16;            // double sums of many CTAs' losses
 // The backward's three channels lie as a float2 and a float array: pitches and gaps put the reads of
 // four-column steps in rows r, r + 1 (.. r + 3) into different banks.
 constexpr int kP2 = 66, kP1 = 45;
@@ -988,7 +987,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
                  float gscale, float l1s, float* __restrict__ loss, float2* __restrict__ m12,
                  float* __restrict__ m3, const float* __restrict__ X,
                  const float* __restrict__ Y, float* __restrict__ grad, int accumulate,
-                 int* __restrict__ err) {
+                 int* __restrict__ err, int n, int per, double* __restrict__ slots) {
   using S = Tma2Shape<BWD>;
   extern __shared__ __align__(16) unsigned char dyn_raw[];
   // 128-byte aligned start, derived from the shared array itself (shared-space addressing)
@@ -1001,19 +1000,35 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
   const int tid = threadIdx.x;
-  const int x0 = blockIdx.x * kT2, y0 = blockIdx.y * kT2, img = blockIdx.z;
+  const int x0 = blockIdx.x * kT2, y0 = blockIdx.y * kT2;
+  const int img0 = blockIdx.z * per, img1 = min(n, img0 + per);  // the CTA's images
+  auto fetch = [&](int img) {
+    mbar_expect_tx(&bar, S::txbytes);
+    tma_load_3d(&tmA, &bar, base, (BWD ? 2 : 1) * (x0 - 8), y0 - kR, img);
+    tma_load_3d(&tmB, &bar, base + S::boxA, x0 - 8, y0 - kR, img);
+  };
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(&bar, S::txbytes);
-    tma_load_3d(&tmA, &bar, base, (BWD ? 2 : 1) * (x0 - 8), y0 - kR, img);
-    tma_load_3d(&tmB, &bar, base + S::boxA, x0 - 8, y0 - kR, img);
+    fetch(img0);
   }
   // the pixels a thread finishes: row cr, columns 4 cq .. 4 cq + 3 (eight lanes per row)
   const int cq = tid & 7, cr = tid >> 3;
   const int y = y0 + cr, xb = x0 + 4 * cq;
   const bool own = y < ny && xb < nx;  // nx % 4 == 0: the four columns are all inside or out
+  __syncthreads();  // the barrier is initialised before anyone waits on it
+  float2 w2[2 * kR + 1];
+#pragma unroll
+  for (int k = 0; k <= 2 * kR; ++k)  // symmetric: six values
+    w2[k] = make_float2(W.w[k < kR ? k : 2 * kR - k], W.w[k < kR ? k : 2 * kR - k]);
+  if (BWD && slots && tid == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) {
+    double t = 0.0;  // the forward's loss sums
+    for (int k = 0; k < kLossSlots; ++k) t += slots[k];
+    atomicAdd(loss, (float)t);
+  }
+  float contrib = 0.f, l1 = 0.f;
+  for (int img = img0; img < img1; ++img) {
   const size_t o = ((size_t)img * ny + y) * nx + xb;
   // backward: the pixels' x, y (and the gradient to add to) are requested now, so that their
   // latency overlaps the copies and the filter passes
@@ -1023,12 +1038,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
     yo = *reinterpret_cast<const float4*>(Y + o);
     if (accumulate) go = *reinterpret_cast<const float4*>(grad + o);
   }
-  __syncthreads();  // the barrier is initialised before anyone waits on it
-  if (!mbar_wait(&bar, 0)) abort_flag = 1;  // all leave after the next barrier
-  float2 w2[2 * kR + 1];
-#pragma unroll
-  for (int k = 0; k <= 2 * kR; ++k)  // symmetric: six values
-    w2[k] = make_float2(W.w[k < kR ? k : 2 * kR - k], W.w[k < kR ? k : 2 * kR - k]);
+  if (!mbar_wait(&bar, (uint32_t)(img - img0) & 1u)) abort_flag = 1;  // all leave at the barrier
   // ---- vertical pass: item (halo column c, output rows 8g .. 8g + 7), box rows 8g .. 8g + 17 at
   // box column c + 3 (image column x0 - 5 + c); 168 items, one round.  Warps 0 - 3 take 32
   // consecutive columns (and banks) of a row group each, warps 4 and 5 the last ten of two each.
@@ -1072,20 +1082,29 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
             make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
       }
   }
+  if (!BWD && own && l1s != 0.f) {  // the pixels' own x, y from the boxes (box row cr + 5)
+    const int e = (cr + kR) * kTBoxX + 4 * cq + 8;
+    const float4 xv = *reinterpret_cast<const float4*>(sA + e);
+    const float4 yv = *reinterpret_cast<const float4*>(sB + e);
+    l1 += fabsf(xv.x - yv.x) + fabsf(xv.y - yv.y) + fabsf(xv.z - yv.z) + fabsf(xv.w - yv.w);
+  }
   __syncthreads();
   if (abort_flag) {
     // a copy never arrived: report it and poison the result instead of using the boxes
     if (tid == 0) {
       atomicExch(err, GS_ERR_TIMEOUT);
       if (!BWD && loss) atomicExch(loss, __int_as_float(0x7fc00000));
-      mbar_wait(&bar, 0);  // bounded: the copies in flight before shared memory goes away
+      mbar_wait(&bar, (uint32_t)(img - img0) & 1u);  // bounded: the copies in flight before shared memory goes away
     }
     if (BWD && own) {
       const float nan = __int_as_float(0x7fc00000);
-      *reinterpret_cast<float4*>(grad + o) = make_float4(nan, nan, nan, nan);
+      for (int rest = img; rest < img1; ++rest)
+        *reinterpret_cast<float4*>(grad + ((size_t)rest * ny + y) * nx + xb) =
+            make_float4(nan, nan, nan, nan);
     }
     return;
   }
+  if (tid == 0 && img + 1 < img1) fetch(img + 1);  // the boxes are free: while the rest is filtered
   // ---- horizontal pass: the thread's four pixels from halo columns 4 cq .. 4 cq + 13
   float2 f[kG][2];
 #pragma unroll
@@ -1111,7 +1130,6 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
     }
   }
   float4 t[3];  // the four pixels' channels
-  float contrib = 0.f;
   if constexpr (BWD) {  // the filtered maps
     t[0] = make_float4(f[0][0].x, f[1][0].x, f[2][0].x, f[3][0].x);
     t[1] = make_float4(f[0][0].y, f[1][0].y, f[2][0].y, f[3][0].y);
@@ -1139,34 +1157,34 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
     for (int m = 0; m < 3; ++m) t[m] = make_float4(mv[m][0], mv[m][1], mv[m][2], mv[m][3]);
   }
   if constexpr (BWD) {
-    if (!own) return;
-    const float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
-    const float gs[4] = {go.x, go.y, go.z, go.w};
-    const float a1[4] = {t[0].x, t[0].y, t[0].z, t[0].w}, a2[4] = {t[1].x, t[1].y, t[1].z, t[1].w};
-    const float a3[4] = {t[2].x, t[2].y, t[2].z, t[2].w};
-    float gv[4];
-#pragma unroll
-    for (int j = 0; j < kG; ++j) {
-      float g = a1[j] + 2.f * xs[j] * a2[j] + ys[j] * a3[j];
-      if (l1s != 0.f) g = l1s * sgnf(xs[j] - ys[j]) + g;  // fused L1 term
-      gv[j] = accumulate ? gs[j] + g : g;
-    }
-    *reinterpret_cast<float4*>(grad + o) = make_float4(gv[0], gv[1], gv[2], gv[3]);
-  } else {
-    float l1 = 0.f;
     if (own) {
-      float4* m12o = reinterpret_cast<float4*>(m12 + o);  // o % 4 == 0: 32-byte aligned
-      m12o[0] = make_float4(t[0].x, t[1].x, t[0].y, t[1].y);
-      m12o[1] = make_float4(t[0].z, t[1].z, t[0].w, t[1].w);
-      *reinterpret_cast<float4*>(m3 + o) = t[2];
-      if (l1s != 0.f) {  // the pixels' own x, y from the staged boxes (box row cr + 5)
-        const int e = (cr + kR) * kTBoxX + 4 * cq + 8;
-        const float4 xv = *reinterpret_cast<const float4*>(sA + e);
-        const float4 yv = *reinterpret_cast<const float4*>(sB + e);
-        l1 = fabsf(xv.x - yv.x) + fabsf(xv.y - yv.y) + fabsf(xv.z - yv.z) + fabsf(xv.w - yv.w);
+      const float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
+      const float gs[4] = {go.x, go.y, go.z, go.w};
+      const float a1[4] = {t[0].x, t[0].y, t[0].z, t[0].w}, a2[4] = {t[1].x, t[1].y, t[1].z, t[1].w};
+      const float a3[4] = {t[2].x, t[2].y, t[2].z, t[2].w};
+      float gv[4];
+#pragma unroll
+      for (int j = 0; j < kG; ++j) {
+        float g = a1[j] + 2.f * xs[j] * a2[j] + ys[j] * a3[j];
+        if (l1s != 0.f) g = l1s * sgnf(xs[j] - ys[j]) + g;  // fused L1 term
+        gv[j] = accumulate ? gs[j] + g : g;
       }
+      *reinterpret_cast<float4*>(grad + o) = make_float4(gv[0], gv[1], gv[2], gv[3]);
     }
-    if (loss) block_add(contrib * (-gscale) + l1 * l1s, loss);
+  } else if (own) {
+    float4* m12o = reinterpret_cast<float4*>(m12 + o);  // o % 4 == 0: 32-byte aligned
+    m12o[0] = make_float4(t[0].x, t[1].x, t[0].y, t[1].y);
+    m12o[1] = make_float4(t[0].z, t[1].z, t[0].w, t[1].w);
+    *reinterpret_cast<float4*>(m3 + o) = t[2];
+  }
+  if (img + 1 < img1) __syncthreads();  // the filtered rows are free
+  }
+  if (!BWD && loss) {
+    if (slots)
+      block_add(contrib * (-gscale) + l1 * l1s,
+                slots + (blockIdx.x + blockIdx.y + blockIdx.z) % kLossSlots);
+    else
+      block_add(contrib * (-gscale) + l1 * l1s, loss);
   }
 }
 
@@ -1353,12 +1371,25 @@ int ssim2d(const float* d_x, const float* d_y, int H, int W, dim3 grid, float C1
     GS_TRY(volume_map(&tmY, d_y, W, H, n, 4, kTBoxX, kIn2));
     GS_TRY(volume_map(&tmP, maps, 2 * W, H, n, 4, 2 * kTBoxX, kIn2));
     GS_TRY(volume_map(&tmS, m3, W, H, n, 4, kTBoxX, kIn2));
+    // a CTA takes its tile of up to four images, whose copies then run under the filters, while the
+    // grid holds four waves (75 x 512^2: 129 + 97 -> 118 + 92 us; two images 118 + 92, eight 121 + 92)
+    const int64_t tiles = (int64_t)grid.x * grid.y * n;
+    const int per =
+        (int)std::max<int64_t>(1, std::min<int64_t>(4, tiles / (16 * (int64_t)num_sms())));
+    grid.z = (n + per - 1) / per;
+    // The loss of many tiles is summed in double next to the status word, by the backward's first
+    // CTA: thousands of float atomics on one sum leave errors of 1e-6 to 3e-6 of it.
+    double* slots = nullptr;
+    if (d_loss && tiles > 512) {
+      slots = reinterpret_cast<double*>(err + 4);
+      GS_CUDA(cudaMemsetAsync(slots, 0, kLossSlots * sizeof(double), s));
+    }
     GS_TRY(launch("ssim2d_fwd", k_ssim2d_tma<false>, grid, block, Tma2Shape<false>::smem, s,
                   tmX, tmY, Wn, W, H, C1, C2, gscale, l1s, d_loss, m12, m3,
-                  (const float*)nullptr, (const float*)nullptr, (float*)nullptr, 0, err));
+                  (const float*)nullptr, (const float*)nullptr, (float*)nullptr, 0, err, n, per, slots));
     return launch("ssim2d_bwd", k_ssim2d_tma<true>, grid, block, Tma2Shape<true>::smem, s, tmP,
-                  tmS, Wn, W, H, C1, C2, gscale, l1s, (float*)nullptr, m12, m3, d_x, d_y,
-                  d_grad, accumulate, err);
+                  tmS, Wn, W, H, C1, C2, gscale, l1s, d_loss, m12, m3, d_x, d_y, d_grad,
+                  accumulate, err, n, per, slots);
   }
   GS_TRY(launch("ssim2d_fwd", k_ssim_xy<0>, grid, block, XyShape<0>::smem, s, Wn, d_x, d_y,
                 plane, W, H, C1, C2, gscale, d_loss, maps, (const float*)nullptr,

@@ -355,3 +355,23 @@ def test_pipelined_step_equals_serial_step(B, chunks):
         la = float(recs[0].step().item())
         lb = float(recs[1].step(serial=True).item())
     assert abs(la - lb) <= 1e-3 * abs(lb), (la, lb)
+
+
+@pytest.mark.parametrize("n", [1, 3, 40, 43])
+def test_l1_ssim2d_many_images(B, n):
+    """Stacks of few and of many images (whose CTAs take several images each, the last group fewer,
+    and whose losses are summed in double): every image's gradient equals the one that a stack of
+    one gives, scaled by the pixel count, and the loss the mean of the images' own.  Gradients differ
+    by the rounding of that scale only, losses by that of float sums over 256 tiles (1e-6)."""
+    rng = np.random.default_rng(12)
+    H, W = 256, 264
+    y = _x32(rng.random((n, H, W)))
+    x = _x32(np.clip(y + 0.1 * rng.standard_normal((n, H, W)), 0, None))
+    val, g = _run_loss(B, "l1ssim2d", x, y, 1.0, 0.6, weight=0.25)
+    vals = []
+    for k in sorted({0, n // 2, n - 1}):
+        v1, g1 = _run_loss(B, "l1ssim2d", x[k:k + 1], y[k:k + 1], 1.0, 0.6, weight=0.25)
+        assert np.abs(g[k] * n - g1[0]).max() <= 1e-6 * np.abs(g1).max()
+    for k in range(n):
+        vals.append(_run_loss(B, "l1ssim2d", x[k:k + 1], y[k:k + 1], 1.0, 0.6, weight=0.25)[0])
+    assert abs(val - np.mean(vals)) <= 3e-6 * abs(val)
