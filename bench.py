@@ -417,16 +417,10 @@ def run_ours(args, ws, rank, local):
                                "frac_folded_count": round(kach / kpeak_f, 4),
                                "evals_per_launch": units}
 
-    # HBM rooflines of the step's memory-heavy kernels from algorithmic bytes: a radix pass
-    # reads and writes every (key, value) pair (16 B), the 2D SSIM passes read and write each
-    # image or map pixel once.  The pairs sort over the tile bits of their keys in passes of
-    # at most 8 bits (two passes of 5 bits for the 1024 tiles of 512^2 at tile 16).
-    tiles = ((WORKLOAD["W"] + WORKLOAD["tile"] - 1) // WORKLOAD["tile"]) * \
-        ((WORKLOAD["H"] + WORKLOAD["tile"] - 1) // WORKLOAD["tile"])
-    passes = ((tiles - 1).bit_length() + 7) // 8
+    # HBM rooflines of the step's memory-heavy kernels from algorithmic bytes: the 2D SSIM passes
+    # read and write each image or map pixel once.
     px = int(WORKLOAD["views"]) * WORKLOAD["W"] * WORKLOAD["H"]
-    step_bytes = {"radix_scatter": 16 * pairs * passes, "ssim2d_fwd": 20 * px,
-                  "ssim2d_bwd": 24 * px}
+    step_bytes = {"ssim2d_fwd": 20 * px, "ssim2d_bwd": 24 * px}
     hbm_roofs = {}
     for k, nb in step_bytes.items():
         if k in per_kernel and mp.get("hbm_gbs"):
