@@ -978,9 +978,9 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 // Bound by instruction issue (71 %; FMA pipe 59 % of its cycles): per pixel pair two FMAs for the
 // exponent, two ex2, the cut, one product and three moment sums, and as much again per block for the
 // record's row coefficients, the centre shift and the queue.  Against warps that own 4 x 16 blocks,
-// list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1040 us;
-// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; 41 x 389 x 517 parallel, 270 -> 243; 16 small
-// reconstructions 391 -> 318.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
+// list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1032 us;
+// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; 41 x 389 x 517 parallel, 270 -> 238; 16 small
+// reconstructions 391 -> 311.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
 // Blocks that start at the record's own box instead of the grid cost their gain in bank conflicts
 // (1211).  24, 28, 32 warps per SM: 1051, 1043, 1079 (tile 32: 5.81, 5.88, 6.41 ms).  The last rows
 // of the grid take the narrow records (below), which the tiles' warps leave out.
@@ -1139,6 +1139,10 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
                              (float)(ty0 + (lane % S::NBY) * 4));
   const unsigned lt = gsd::lanemask_lt();
   uint32_t pos = r.x;    // next record of the list to stage
+  // the next run's records are requested one run ahead, so that staging waits for one gather, not
+  // two (75 x 512^2: 1059 -> 1032 us; at tile 32 the register costs more, 5.82 -> 5.94 ms)
+  constexpr bool AHEAD = T < 32;
+  uint32_t ahead = AHEAD && pos + lane < r.y ? vals[pos + lane] : 0u;
   int qh = 0, qn = 0;    // the queue's next and its end
   // the lane's record: the blocks still to walk, its coefficients and its six sums
   uint32_t rec = 0u, mask = 0u;
@@ -1186,13 +1190,14 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
         float4 g, c;
         uint32_t nrec = 0, nmask = 0;
         if (in) {
-          nrec = vals[pos + lane];
+          nrec = AHEAD ? ahead : vals[pos + lane];
           g = recs[2 * (size_t)nrec];
           c = recs[2 * (size_t)nrec + 1];
           const short4 bx = rect[nrec];
           if (!is_narrow<T>(c, bx)) nmask = block_mask<T, S::BW>(g, c, bx, tx0, ty0);
         }
         pos += 32;
+        if (AHEAD) ahead = pos + lane < r.y ? vals[pos + lane] : 0u;
         __syncwarp();  // the queue's last reads are done
         const unsigned keep = __ballot_sync(0xffffffffu, nmask != 0u);
         if (nmask) {
