@@ -229,7 +229,9 @@ __device__ __forceinline__ float2 pair_at(const float* base, int64_t n, int m, i
 
 // With l1_scale != 0 the forward also adds l1_scale * sum |X - Y| over its columns to *loss
 // (the L1 term of a fused L1 + SSIM loss).
-template <int NIN>  // 2: (X, Y) -> 5 moments; 3: maps (pair layout) -> 3 filtered maps
+// NIN 2: (X, Y) -> 5 moments; 3: maps (pair layout) -> 3 filtered maps.  CHUNK: z in several chunks
+// (one chunk by the same code cost 2 %, for the ranges' limits).
+template <int NIN, bool CHUNK>
 __global__ void __launch_bounds__(kThreads)
     k_ssim3d_z(const __grid_constant__ Win W, const float* __restrict__ A0,
                const float* __restrict__ A1, int nx, int ny, int nz, int zc, int64_t plane,
@@ -258,7 +260,8 @@ __global__ void __launch_bounds__(kThreads)
     for (int i = 0; i < NIN; ++i) ring[k][i] = 0.f;
   // this chunk's outputs z0 .. z1 - 1 from planes zb .. zend - 1 (zeros beyond the volume); the
   // k-th plane enters ring slot k % 11, output z = zi - kR is complete once plane zi is in
-  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc), zend = min(nz, z1 + kR);
+  const int z0 = CHUNK ? blockIdx.y * zc : 0, z1 = CHUNK ? min(nz, z0 + zc) : nz;
+  const int zend = CHUNK ? min(nz, z1 + kR) : nz;
   float nxt[NIN];
   load((int64_t)max(0, z0 - kR) * sxy + col, nxt);
   for (int zb = max(0, z0 - kR); zb < z1 + kR; zb += 2 * kR + 1) {
@@ -267,7 +270,8 @@ __global__ void __launch_bounds__(kThreads)
       const int zi = zb + k;
 #pragma unroll
       for (int i = 0; i < NIN; ++i) ring[k][i] = nxt[i];
-      if (NIN == 2 && l1_scale != 0.f && zi >= z0 && zi < z1) l1 += fabsf(nxt[0] - nxt[1]);
+      if (NIN == 2 && l1_scale != 0.f && (!CHUNK || (zi >= z0 && zi < z1)))
+        l1 += fabsf(nxt[0] - nxt[1]);  // 0 beyond the volume
       const int zn = zi + 1;
       if (zn < zend) {
         load((int64_t)zn * sxy + col, nxt);
@@ -977,7 +981,9 @@ struct Tma2Shape {
   static constexpr uint32_t boxB = kTBox * 4u;
   static constexpr uint32_t txbytes = boxA + boxB;
   static constexpr uint32_t offV = boxA + boxB;  // 16128 / 24192: multiples of 128
-  static constexpr size_t smem = 128 + offV + (BWD ? (size_t)kT2 * (kP2 * sizeof(float2) + kP1 * sizeof(float)) : (size_t)kT2 * kHPitch * sizeof(float4));
+  static constexpr size_t rows = BWD ? kP2 * sizeof(float2) + kP1 * sizeof(float)
+                                     : kHPitch * sizeof(float4);  // a filtered row
+  static constexpr size_t smem = 128 + offV + kT2 * rows;
 };
 
 template <bool BWD>
@@ -1029,155 +1035,156 @@ __global__ void __launch_bounds__(kSsimThreads, 4)
   }
   float contrib = 0.f, l1 = 0.f;
   for (int img = img0; img < img1; ++img) {
-  const size_t o = ((size_t)img * ny + y) * nx + xb;
-  // backward: the pixels' x, y (and the gradient to add to) are requested now, so that their
-  // latency overlaps the copies and the filter passes
-  float4 xo = make_float4(0.f, 0.f, 0.f, 0.f), yo = xo, go = xo;
-  if (BWD && own) {
-    xo = *reinterpret_cast<const float4*>(X + o);
-    yo = *reinterpret_cast<const float4*>(Y + o);
-    if (accumulate) go = *reinterpret_cast<const float4*>(grad + o);
-  }
-  if (!mbar_wait(&bar, (uint32_t)(img - img0) & 1u)) abort_flag = 1;  // all leave at the barrier
-  // ---- vertical pass: item (halo column c, output rows 8g .. 8g + 7), box rows 8g .. 8g + 17 at
-  // box column c + 3 (image column x0 - 5 + c); 168 items, one round.  Warps 0 - 3 take 32
-  // consecutive columns (and banks) of a row group each, warps 4 and 5 the last ten of two each.
-  const int wv = tid >> 5, lv = tid & 31;
-  if (wv < kT2 / kGV || (wv < kT2 / kGV + 2 && lv < 2 * (kIn2 - 32))) {
-    const bool tail = wv >= kT2 / kGV;
-    const int c = tail ? 32 + lv % (kIn2 - 32) : lv;
-    const int g = tail ? 2 * (wv - kT2 / kGV) + lv / (kIn2 - 32) : wv;
-    float2 a[kGV][2];
-#pragma unroll
-    for (int j = 0; j < kGV; ++j) a[j][0] = a[j][1] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < kGV + 2 * kR; ++i) {
-      const int e = (kGV * g + i) * kTBoxX + c + 3;
-      float2 u0, u1;
-      if constexpr (!BWD) {
-        const float xv = sA[e], yv = sB[e];
-        u0 = make_float2(xv, yv);
-        // second moments as (x^2 + y^2, x y): SSIM needs sigma_x^2 + sigma_y^2 only
-        u1 = make_float2(fmaf(xv, xv, yv * yv), xv * yv);
-      } else {
-        u0 = reinterpret_cast<const float2*>(sA)[e];
-        u1 = make_float2(sB[e], 0.f);
-      }
-#pragma unroll
-      for (int j = 0; j < kGV; ++j) {
-        const int k = i - j;
-        if (k < 0 || k > 2 * kR) continue;
-        a[j][0] = __ffma2_rn(w2[k], u0, a[j][0]);
-        if constexpr (!BWD) a[j][1] = __ffma2_rn(w2[k], u1, a[j][1]);
-        else a[j][1].x = fmaf(w2[k].x, u1.x, a[j][1].x);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kGV; ++j)
-      if constexpr (BWD) {
-        V2[(kGV * g + j) * kP2 + p2_slot(c)] = a[j][0];
-        V1[(kGV * g + j) * kP1 + c] = a[j][1].x;
-      } else {
-        V[(kGV * g + j) * kHPitch + h_slot(c)] =
-            make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
-      }
-  }
-  if (!BWD && own && l1s != 0.f) {  // the pixels' own x, y from the boxes (box row cr + 5)
-    const int e = (cr + kR) * kTBoxX + 4 * cq + 8;
-    const float4 xv = *reinterpret_cast<const float4*>(sA + e);
-    const float4 yv = *reinterpret_cast<const float4*>(sB + e);
-    l1 += fabsf(xv.x - yv.x) + fabsf(xv.y - yv.y) + fabsf(xv.z - yv.z) + fabsf(xv.w - yv.w);
-  }
-  __syncthreads();
-  if (abort_flag) {
-    // a copy never arrived: report it and poison the result instead of using the boxes
-    if (tid == 0) {
-      atomicExch(err, GS_ERR_TIMEOUT);
-      if (!BWD && loss) atomicExch(loss, __int_as_float(0x7fc00000));
-      mbar_wait(&bar, (uint32_t)(img - img0) & 1u);  // bounded: the copies in flight before shared memory goes away
-    }
+    const size_t o = ((size_t)img * ny + y) * nx + xb;
+    // backward: the pixels' x, y (and the gradient to add to) are requested now, so that their
+    // latency overlaps the copies and the filter passes
+    float4 xo = make_float4(0.f, 0.f, 0.f, 0.f), yo = xo, go = xo;
     if (BWD && own) {
-      const float nan = __int_as_float(0x7fc00000);
-      for (int rest = img; rest < img1; ++rest)
-        *reinterpret_cast<float4*>(grad + ((size_t)rest * ny + y) * nx + xb) =
-            make_float4(nan, nan, nan, nan);
+      xo = *reinterpret_cast<const float4*>(X + o);
+      yo = *reinterpret_cast<const float4*>(Y + o);
+      if (accumulate) go = *reinterpret_cast<const float4*>(grad + o);
     }
-    return;
-  }
-  if (tid == 0 && img + 1 < img1) fetch(img + 1);  // the boxes are free: while the rest is filtered
-  // ---- horizontal pass: the thread's four pixels from halo columns 4 cq .. 4 cq + 13
-  float2 f[kG][2];
+    if (!mbar_wait(&bar, (uint32_t)(img - img0) & 1u)) abort_flag = 1;  // all leave at the barrier
+    // ---- vertical pass: item (halo column c, output rows 8g .. 8g + 7), box rows 8g .. 8g + 17 at
+    // box column c + 3 (image column x0 - 5 + c); 168 items, one round.  Warps 0 - 3 take 32
+    // consecutive columns (and banks) of a row group each, warps 4 and 5 the last ten of two each.
+    const int wv = tid >> 5, lv = tid & 31;
+    if (wv < kT2 / kGV || (wv < kT2 / kGV + 2 && lv < 2 * (kIn2 - 32))) {
+      const bool tail = wv >= kT2 / kGV;
+      const int c = tail ? 32 + lv % (kIn2 - 32) : lv;
+      const int g = tail ? 2 * (wv - kT2 / kGV) + lv / (kIn2 - 32) : wv;
+      float2 a[kGV][2];
 #pragma unroll
-  for (int j = 0; j < kG; ++j) f[j][0] = f[j][1] = make_float2(0.f, 0.f);
+      for (int j = 0; j < kGV; ++j) a[j][0] = a[j][1] = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < kG + 2 * kR; ++i) {
-    float2 v0, v1;
-    if constexpr (BWD) {
-      v0 = V2[cr * kP2 + p2_slot(4 * cq + (i & ~3)) + (i & 3)];
-      v1 = make_float2(V1[cr * kP1 + 4 * cq + i], 0.f);
-    } else {
-      const float4 v = V[cr * kHPitch + h_slot(4 * cq + (i & ~3)) + (i & 3)];
-      v0 = make_float2(v.x, v.y);
-      v1 = make_float2(v.z, v.w);
+      for (int i = 0; i < kGV + 2 * kR; ++i) {
+        const int e = (kGV * g + i) * kTBoxX + c + 3;
+        float2 u0, u1;
+        if constexpr (!BWD) {
+          const float xv = sA[e], yv = sB[e];
+          u0 = make_float2(xv, yv);
+          // second moments as (x^2 + y^2, x y): SSIM needs sigma_x^2 + sigma_y^2 only
+          u1 = make_float2(fmaf(xv, xv, yv * yv), xv * yv);
+        } else {
+          u0 = reinterpret_cast<const float2*>(sA)[e];
+          u1 = make_float2(sB[e], 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < kGV; ++j) {
+          const int k = i - j;
+          if (k < 0 || k > 2 * kR) continue;
+          a[j][0] = __ffma2_rn(w2[k], u0, a[j][0]);
+          if constexpr (!BWD) a[j][1] = __ffma2_rn(w2[k], u1, a[j][1]);
+          else a[j][1].x = fmaf(w2[k].x, u1.x, a[j][1].x);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kGV; ++j)
+        if constexpr (BWD) {
+          V2[(kGV * g + j) * kP2 + p2_slot(c)] = a[j][0];
+          V1[(kGV * g + j) * kP1 + c] = a[j][1].x;
+        } else {
+          V[(kGV * g + j) * kHPitch + h_slot(c)] =
+              make_float4(a[j][0].x, a[j][0].y, a[j][1].x, a[j][1].y);
+        }
     }
-#pragma unroll
-    for (int j = 0; j < kG; ++j) {
-      const int k = i - j;
-      if (k < 0 || k > 2 * kR) continue;
-      f[j][0] = __ffma2_rn(w2[k], v0, f[j][0]);
-      if constexpr (!BWD) f[j][1] = __ffma2_rn(w2[k], v1, f[j][1]);
-      else f[j][1].x = fmaf(w2[k].x, v1.x, f[j][1].x);
+    if (!BWD && own && l1s != 0.f) {  // the pixels' own x, y from the boxes (box row cr + 5)
+      const int e = (cr + kR) * kTBoxX + 4 * cq + 8;
+      const float4 xv = *reinterpret_cast<const float4*>(sA + e);
+      const float4 yv = *reinterpret_cast<const float4*>(sB + e);
+      l1 += fabsf(xv.x - yv.x) + fabsf(xv.y - yv.y) + fabsf(xv.z - yv.z) + fabsf(xv.w - yv.w);
     }
-  }
-  float4 t[3];  // the four pixels' channels
-  if constexpr (BWD) {  // the filtered maps
-    t[0] = make_float4(f[0][0].x, f[1][0].x, f[2][0].x, f[3][0].x);
-    t[1] = make_float4(f[0][0].y, f[1][0].y, f[2][0].y, f[3][0].y);
-    t[2] = make_float4(f[0][1].x, f[1][1].x, f[2][1].x, f[3][1].x);
-  } else {  // SSIM and its maps (rows and columns past the image are never stored)
-    float mv[3][kG];
-#pragma unroll
-    for (int j = 0; j < kG; ++j) {
-      const float mx = f[j][0].x, my = f[j][0].y;
-      const float sxy = f[j][1].y - mx * my;
-      const float D = (f[j][1].x - mx * mx - my * my) + C2;  // sigma_x^2 + sigma_y^2 + C2
-      const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
-      const float C = mx * mx + my * my + C1;
-      const float inv = rcp_newton(C * D);  // 1/C = D inv, 1/D = C inv
-      const float Sv = (Am * Bn) * inv;
-      const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
-      const float dsxx = -Sv * (C * inv);
-      const float dsxy = 2.f * Am * inv;
-      mv[0][j] = gscale * (dmu - 2.f * mx * dsxx - my * dsxy);
-      mv[1][j] = gscale * dsxx;
-      mv[2][j] = gscale * dsxy;
-      if (own) contrib += 1.f - Sv;
+    __syncthreads();
+    if (abort_flag) {
+      // a copy never arrived: report it and poison the result instead of using the boxes
+      if (tid == 0) {
+        atomicExch(err, GS_ERR_TIMEOUT);
+        if (!BWD && loss) atomicExch(loss, __int_as_float(0x7fc00000));
+        // bounded: the copies in flight, before shared memory goes away
+        mbar_wait(&bar, (uint32_t)(img - img0) & 1u);
+      }
+      if (BWD && own) {
+        const float nan = __int_as_float(0x7fc00000);
+        for (int rest = img; rest < img1; ++rest)
+          *reinterpret_cast<float4*>(grad + ((size_t)rest * ny + y) * nx + xb) =
+              make_float4(nan, nan, nan, nan);
+      }
+      return;
     }
+    if (tid == 0 && img + 1 < img1) fetch(img + 1);  // the boxes are free: while the rest is filtered
+    // ---- horizontal pass: the thread's four pixels from halo columns 4 cq .. 4 cq + 13
+    float2 f[kG][2];
 #pragma unroll
-    for (int m = 0; m < 3; ++m) t[m] = make_float4(mv[m][0], mv[m][1], mv[m][2], mv[m][3]);
-  }
-  if constexpr (BWD) {
-    if (own) {
-      const float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
-      const float gs[4] = {go.x, go.y, go.z, go.w};
-      const float a1[4] = {t[0].x, t[0].y, t[0].z, t[0].w}, a2[4] = {t[1].x, t[1].y, t[1].z, t[1].w};
-      const float a3[4] = {t[2].x, t[2].y, t[2].z, t[2].w};
-      float gv[4];
+    for (int j = 0; j < kG; ++j) f[j][0] = f[j][1] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kG + 2 * kR; ++i) {
+      float2 v0, v1;
+      if constexpr (BWD) {
+        v0 = V2[cr * kP2 + p2_slot(4 * cq + (i & ~3)) + (i & 3)];
+        v1 = make_float2(V1[cr * kP1 + 4 * cq + i], 0.f);
+      } else {
+        const float4 v = V[cr * kHPitch + h_slot(4 * cq + (i & ~3)) + (i & 3)];
+        v0 = make_float2(v.x, v.y);
+        v1 = make_float2(v.z, v.w);
+      }
 #pragma unroll
       for (int j = 0; j < kG; ++j) {
-        float g = a1[j] + 2.f * xs[j] * a2[j] + ys[j] * a3[j];
-        if (l1s != 0.f) g = l1s * sgnf(xs[j] - ys[j]) + g;  // fused L1 term
-        gv[j] = accumulate ? gs[j] + g : g;
+        const int k = i - j;
+        if (k < 0 || k > 2 * kR) continue;
+        f[j][0] = __ffma2_rn(w2[k], v0, f[j][0]);
+        if constexpr (!BWD) f[j][1] = __ffma2_rn(w2[k], v1, f[j][1]);
+        else f[j][1].x = fmaf(w2[k].x, v1.x, f[j][1].x);
       }
-      *reinterpret_cast<float4*>(grad + o) = make_float4(gv[0], gv[1], gv[2], gv[3]);
     }
-  } else if (own) {
-    float4* m12o = reinterpret_cast<float4*>(m12 + o);  // o % 4 == 0: 32-byte aligned
-    m12o[0] = make_float4(t[0].x, t[1].x, t[0].y, t[1].y);
-    m12o[1] = make_float4(t[0].z, t[1].z, t[0].w, t[1].w);
-    *reinterpret_cast<float4*>(m3 + o) = t[2];
-  }
-  if (img + 1 < img1) __syncthreads();  // the filtered rows are free
+    float4 t[3];  // the four pixels' channels
+    if constexpr (BWD) {  // the filtered maps
+      t[0] = make_float4(f[0][0].x, f[1][0].x, f[2][0].x, f[3][0].x);
+      t[1] = make_float4(f[0][0].y, f[1][0].y, f[2][0].y, f[3][0].y);
+      t[2] = make_float4(f[0][1].x, f[1][1].x, f[2][1].x, f[3][1].x);
+    } else {  // SSIM and its maps (rows and columns past the image are never stored)
+      float mv[3][kG];
+#pragma unroll
+      for (int j = 0; j < kG; ++j) {
+        const float mx = f[j][0].x, my = f[j][0].y;
+        const float sxy = f[j][1].y - mx * my;
+        const float D = (f[j][1].x - mx * mx - my * my) + C2;  // sigma_x^2 + sigma_y^2 + C2
+        const float Am = 2.f * mx * my + C1, Bn = 2.f * sxy + C2;
+        const float C = mx * mx + my * my + C1;
+        const float inv = rcp_newton(C * D);  // 1/C = D inv, 1/D = C inv
+        const float Sv = (Am * Bn) * inv;
+        const float dmu = (2.f * my * Bn) * inv - Sv * (2.f * mx) * (D * inv);
+        const float dsxx = -Sv * (C * inv);
+        const float dsxy = 2.f * Am * inv;
+        mv[0][j] = gscale * (dmu - 2.f * mx * dsxx - my * dsxy);
+        mv[1][j] = gscale * dsxx;
+        mv[2][j] = gscale * dsxy;
+        if (own) contrib += 1.f - Sv;
+      }
+#pragma unroll
+      for (int m = 0; m < 3; ++m) t[m] = make_float4(mv[m][0], mv[m][1], mv[m][2], mv[m][3]);
+    }
+    if constexpr (BWD) {
+      if (own) {
+        const float xs[4] = {xo.x, xo.y, xo.z, xo.w}, ys[4] = {yo.x, yo.y, yo.z, yo.w};
+        const float gs[4] = {go.x, go.y, go.z, go.w};
+        const float a1[4] = {t[0].x, t[0].y, t[0].z, t[0].w}, a2[4] = {t[1].x, t[1].y, t[1].z, t[1].w};
+        const float a3[4] = {t[2].x, t[2].y, t[2].z, t[2].w};
+        float gv[4];
+#pragma unroll
+        for (int j = 0; j < kG; ++j) {
+          float g = a1[j] + 2.f * xs[j] * a2[j] + ys[j] * a3[j];
+          if (l1s != 0.f) g = l1s * sgnf(xs[j] - ys[j]) + g;  // fused L1 term
+          gv[j] = accumulate ? gs[j] + g : g;
+        }
+        *reinterpret_cast<float4*>(grad + o) = make_float4(gv[0], gv[1], gv[2], gv[3]);
+      }
+    } else if (own) {
+      float4* m12o = reinterpret_cast<float4*>(m12 + o);  // o % 4 == 0: 32-byte aligned
+      m12o[0] = make_float4(t[0].x, t[1].x, t[0].y, t[1].y);
+      m12o[1] = make_float4(t[0].z, t[1].z, t[0].w, t[1].w);
+      *reinterpret_cast<float4*>(m3 + o) = t[2];
+    }
+    if (img + 1 < img1) __syncthreads();  // the filtered rows are free
   }
   if (!BWD && loss) {
     if (slots)
@@ -1372,7 +1379,8 @@ int ssim2d(const float* d_x, const float* d_y, int H, int W, dim3 grid, float C1
     GS_TRY(volume_map(&tmP, maps, 2 * W, H, n, 4, 2 * kTBoxX, kIn2));
     GS_TRY(volume_map(&tmS, m3, W, H, n, 4, kTBoxX, kIn2));
     // a CTA takes its tile of up to four images, whose copies then run under the filters, while the
-    // grid holds four waves (75 x 512^2: 129 + 97 -> 118 + 92 us; two images 118 + 92, eight 121 + 92)
+    // grid holds four waves (75 x 512^2: 129 + 97 -> 118 + 92 us; two images 118 + 92, eight 121 +
+    // 92)
     const int64_t tiles = (int64_t)grid.x * grid.y * n;
     const int per =
         (int)std::max<int64_t>(1, std::min<int64_t>(4, tiles / (16 * (int64_t)num_sms())));
@@ -1628,14 +1636,15 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
     return launch("ssim3d_bwd", k_ssim3d_bwd_fused, gf, dim3(kFThreads), FusedShape<true>::smem,
                   s, tmM12, tmM3, tmXt, tmYt, W, nx, ny, nz, zc, d_grad, accumulate, l1s, err);
   }
-  GS_TRY(launch("ssim3d_z_fwd", k_ssim3d_z<2>, gz, bz, 0, s, W, d_x, d_y, nx, ny, nz, zcol, plane,
-                tmp, l1s, d_loss));
+  GS_TRY(launch("ssim3d_z_fwd", gz.y > 1 ? k_ssim3d_z<2, true> : k_ssim3d_z<2, false>, gz, bz, 0,
+                s, W, d_x, d_y, nx, ny, nz, zcol, plane, tmp, l1s, d_loss));
   GS_TRY(launch("ssim3d_xy_fwd", k_ssim_xy<1>, gxy, bxy, XyShape<1>::smem, s, W,
                 (const float*)tmp, (const float*)nullptr, plane, nx, ny, C1, C2, gscale, d_loss,
                 maps, (const float*)nullptr, (const float*)nullptr, (float*)nullptr, 0, 0.f));
   if (!d_grad) return GS_OK;  // value only
-  GS_TRY(launch("ssim3d_z_bwd", k_ssim3d_z<3>, gz, bz, 0, s, W, (const float*)maps,
-                (const float*)nullptr, nx, ny, nz, zcol, plane, tmp, 0.f, (float*)nullptr));
+  GS_TRY(launch("ssim3d_z_bwd", gz.y > 1 ? k_ssim3d_z<3, true> : k_ssim3d_z<3, false>, gz, bz, 0,
+                s, W, (const float*)maps, (const float*)nullptr, nx, ny, nz, zcol, plane, tmp, 0.f,
+                (float*)nullptr));
   return launch("ssim3d_xy_bwd", k_ssim_xy<2>, gxy, bxy, XyShape<2>::smem, s, W,
                 (const float*)tmp, (const float*)nullptr, plane, nx, ny, C1, C2, gscale,
                 (float*)nullptr, (float*)nullptr, d_x, d_y, d_grad, accumulate, l1s);

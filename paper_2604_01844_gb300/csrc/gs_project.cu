@@ -980,7 +980,8 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 // record's row coefficients, the centre shift and the queue.  Against warps that own 4 x 16 blocks,
 // list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1032 us;
 // tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; 41 x 389 x 517 parallel, 270 -> 238; 16 small
-// reconstructions 391 -> 311.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at the same stage.
+// reconstructions 391 -> 311.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at
+// the same stage.
 // Blocks that start at the record's own box instead of the grid cost their gain in bank conflicts
 // (1211).  24, 28, 32 warps per SM: 1051, 1043, 1079 (tile 32: 5.81, 5.88, 6.41 ms).  The last rows
 // of the grid take the narrow records (below), which the tiles' warps leave out.
@@ -997,10 +998,10 @@ struct BwdBlocks {
 
 // Narrow records: the footprint may have a variance below kNarrowVar square pixels in some direction
 // (the trace of the conic bounds its inverse), in a box of at most 32 x 32 pixels.  Moved from a
-// block's centre to such a record's, second moments lose the digits that the centres' distance squared
-// has over the variance (50 times the rounding at 0.16 and 16-column blocks), so the order of their
-// sums shows in the gradients: they keep the one about 16-column runs, row by row (8 at tile 8), and
-// one thread takes all pixels of a record.  Gradients then move by at most 5e-6 (2-norm) against
+// block's centre to such a record's, second moments lose the digits that the centres' distance
+// squared has over the variance (50 times the rounding at 0.16 and 16-column blocks), so the order
+// of their sums shows in the gradients: they keep the one about 16-column runs, row by row (8 at
+// tile 8), and one thread takes all pixels of a record.  Gradients then move by at most 5e-6 (2-norm) against
 // warps that walk those blocks, instead of up to 2e-5.
 template <int T>
 __device__ __forceinline__ bool is_narrow(const float4 c, const short4 bx) {
@@ -1090,7 +1091,7 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
   __shared__ uint2 q_rm[32];    // record and block mask
   const int64_t key = blockIdx.x;
   const int lane = threadIdx.x;
-  if (blockIdx.y >= parts) {  // the last rows of the grid: the narrow records, 32 chunk of them a warp
+  if (blockIdx.y >= parts) {  // the last rows of the grid: narrow records, 32 chunk of them a warp
     const int per = kThreads / 32 / chunk;  // warps per block of records
     if (st->code != GS_OK) return;
     const int64_t n = (int64_t)nblocks * per, step = (int64_t)(gridDim.y - parts) * gridDim.x;
