@@ -94,7 +94,7 @@ struct Layout {
   gs_status* st = nullptr;
   ViewFrame* frames = nullptr;
   // two float4 per record, one 32-byte sector: (px, py, A, e_cut), e_cut = -1/2 log2(e) * Q, and
-  // -1/2 log2(e) * (a, 2b, c, 0): exponent = a'dx^2 + b'dx dy + c'dy^2
+  // -1/2 log2(e) * (a, 2b, c) with the widened cut: exponent = a'dx^2 + b'dx dy + c'dy^2
   float4* rec = nullptr;
   short4* rect = nullptr;   // clipped inclusive pixel box (x0, y0, x1, y1); x0 > x1 if culled
   uint32_t* tmask = nullptr;  // tight tile rule answers for the box's first 32 tiles
@@ -220,22 +220,9 @@ Layout carve(void* ws, const Plan& p) {
   return L;
 }
 
-// Tight tile rule: a tile is listed for a record if its cut ellipse, enlarged by a relative
-// margin of 1e-3 of the cut (e > 1.001 e_cut, e the exponent), meets the rectangle of pixel
-// centres the tile shares with the record's clipped box.  The margin makes the lists a superset
-// of the per-pixel FP32 test, so a tile left out never held a contribution.  Per tile row the
-// enlarged ellipse's section by the row's slab of pixel centres is convex, so the tiles it meets
-// are those whose pixel columns meet its x extent [xa, xb]: the left (right) end lies at the
-// ellipse's own leftmost (rightmost) point when that is inside the slab, else on the slab's
-// nearer edge.  The ends become pixel columns through the centre's integer and fractional parts,
-// where FP32 resolves far more than the margin.
-struct Ell {
-  float py, fx, ia, hb, kap, vr, cm;  // 1/a, -b/(2a), c - b^2/(4a), v of the rightmost point
-  int ix;                             // centre column px = ix + fx
-};
-// Every operation below is one fixed instruction: preprocess counts the tiles and emit places
-// them, so both must get the same answers.  The approximate reciprocals and roots are within two
-// ulp, far inside the margin.
+// Every operation of the tile rule is one fixed instruction: preprocess counts the tiles and emit
+// places them, so both must get the same answers.  The approximate reciprocals and roots are within
+// two ulp.
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -246,20 +233,59 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+
+// What the closed forms below (tiles of a row, rows of a column slab, columns of a row) need of a
+// record's cut ellipse e = a x^2 + b x y + c y^2 > e_cut, so that each keeps every pixel of the box
+// that the per-pixel FP32 test accepts.
+// D = 4ac - b^2 is a small difference for thin ellipses: Kahan's difference of products gives it
+// to two ulp of the stored conic, and every extent comes from D instead of from another difference.
+// The per-pixel test itself is off by at most 15 u k |e_cut| inside the box (u = 2^-24, k = 4ac / D;
+// at the tips a x^2, b x y / 2 and c y^2 all reach k e_cut), so the cut is widened by 32 u k, twice
+// that, and by the 1e-3 that covers the closed forms' own rounding.  From k = 2^21 (an aspect ratio
+// of 2900 at 45 degrees) the stored conic no longer fixes the ellipse, and beyond 2^22 pixels FP32
+// no longer resolves them: there the whole box counts, by a cut of -infinity.
+// (c - b^2 / (4a) and a fixed margin of 1e-3 lost in-cut pixels from aspect ratios of 300 on:
+// 0.01 % of them at 1000, 4 % at 5000, sigma 60 pixels.)
+__device__ __forceinline__ float conic_det(const float4 c) {
+  const float bb = __fmul_rn(c.y, c.y), rest = __fmaf_rn(c.y, c.y, -bb);
+  return __fsub_rn(__fmaf_rn(__fmul_rn(4.f, c.x), c.z, -bb), rest);
+}
+// The widened cut of a record centred at column px; preprocess keeps it in c.w.
+__device__ __forceinline__ float wide_cut(float cut, float px, const float4 c) {
+  constexpr float kFar = 4194304.f, kThin = 2097152.f;  // 2^22, 2^21
+  const float iD = rcp_approx(conic_det(c));
+  const float k = __fmaf_rn(__fmul_rn(c.y, c.y), iD, 1.f);
+  const float cm = __fmul_rn(cut, __fmaf_rn(k, 1.f / 524288.f, 1.001f));
+  const float ext2 = __fmul_rn(__fmul_rn(4.f * fminf(c.x, c.z), cm), iD);  // the longer half extent
+  return k >= 1.f && k < kThin && fabsf(px) < kFar && ext2 < kFar * kFar ? cm : -INFINITY;
+}
+
+// Tight tile rule: a tile is listed for a record if its cut ellipse, widened as above, meets the
+// rectangle of pixel centres the tile shares with the record's clipped box; a tile left out never
+// held a contribution.  Per tile row the ellipse's section by the row's slab of pixel centres is
+// convex, so the tiles it meets are those whose pixel columns meet its x extent [xa, xb]: the left
+// (right) end lies at the ellipse's own leftmost (rightmost) point when that is inside the slab,
+// else on the slab's nearer edge.  The ends become pixel columns through the centre's integer and
+// fractional parts, where FP32 resolves far more than the margin.
+struct Ell {
+  float py, fx, ia, hb, kap, vr, cm;  // 1/a, -b/(2a), c - b^2/(4a), v of the rightmost point
+  int ix;                             // centre column px = ix + fx
+};
 __device__ __forceinline__ Ell make_ell(const float4 g, const float4 c) {
   Ell E;
-  const float fl = floorf(g.x);  // |px| stays far below 2^24 where a box meets the detector
+  const float D = conic_det(c);
+  const float fl = floorf(g.x);
   E.ix = (int)fl;
   E.fx = __fsub_rn(g.x, fl);
   E.py = g.y;
   E.ia = rcp_approx(c.x);
   const float hb = __fmul_rn(-0.5f, c.y);
   E.hb = __fmul_rn(hb, E.ia);
-  E.kap = __fmaf_rn(-hb, E.hb, c.z);
-  E.cm = __fmul_rn(g.w, 1.001f);
-  const float ih = __fmul_rn(hb, rcp_approx(c.z));  // v = ih u where u is extreme on the ellipse
-  const float u2 = __fmul_rn(E.cm, rcp_approx(__fmaf_rn(-hb, ih, c.x)));
-  E.vr = __fmul_rn(ih, sqrt_approx(fmaxf(u2, 0.f)));
+  E.kap = __fmul_rn(__fmul_rn(0.25f, D), E.ia);
+  E.cm = c.w;
+  // the rightmost point: u = sqrt(4 c e / D), v = -b / (2c) u
+  const float u2 = __fmul_rn(__fmul_rn(__fmul_rn(4.f, c.z), c.w), rcp_approx(D));
+  E.vr = __fmul_rn(__fmul_rn(hb, rcp_approx(c.z)), sqrt_approx(fmaxf(u2, 0.f)));
   return E;
 }
 __device__ __forceinline__ float half_width(const Ell& E, float v) {
@@ -275,7 +301,9 @@ __device__ __forceinline__ void row_tiles(const Ell& E, int lT, int ty, int x0, 
   const float xb = __fmaf_rn(E.hb, vb, half_width(E, vb));
   const float xa = __fmaf_rn(E.hb, va, -half_width(E, va));
   // first pixel column >= xa and last <= xb, from the centre's integer and fractional column
-  const int fa = E.ix + (int)ceilf(__fadd_rn(xa, E.fx)), fb = E.ix + (int)floorf(__fadd_rn(xb, E.fx));
+  const int ca = E.ix + (int)ceilf(__fadd_rn(xa, E.fx)), cb = E.ix + (int)floorf(__fadd_rn(xb, E.fx));
+  const bool whole = E.cm == -INFINITY;
+  const int fa = whole ? x0 : ca, fb = whole ? x1 : cb;
   // an extent between two neighbouring columns (fa = fb + 1) meets their tile if both are the
   // box's and in one tile; one left or right of the box meets none
   const bool none = fb < x0 || fa > x1;
@@ -358,7 +386,8 @@ __global__ void __launch_bounds__(kThreads)
     if (live) {
       const float k = gsd::kNegHalfLog2e;
       const float4 gg = make_float4(o.px, o.py, o.A, k * o.Q);
-      const float4 cc = make_float4(k * o.ca, 2.f * k * o.cb, k * o.cc, 0.f);
+      float4 cc = make_float4(k * o.ca, 2.f * k * o.cb, k * o.cc, 0.f);
+      cc.w = wide_cut(gg.w, o.px, cc);
       const Ell E = make_ell(gg, cc);
       const int lT = b.lT, tx0 = x0 >> lT, ty0 = y0 >> lT;
       const int ntx = (x1 >> lT) - tx0 + 1, ty1 = y1 >> lT;
@@ -728,34 +757,38 @@ __global__ void __launch_bounds__(kThreads)
 __device__ __forceinline__ float row_b(const float4 c, float dy) { return c.y * dy; }
 __device__ __forceinline__ float row_c(const float4 c, float dy) { return (c.z * dy) * dy; }
 
-// Rows [ylo, yhi] (tile-local, clamped to [0, T-1]; ylo > yhi if none) that a record's cut
-// ellipse, enlarged like the tight tile rule (e > 1.001 e_cut), reaches inside the column
-// slab of pixel centres [x0, x1].  The ellipse's section by the slab is convex, so its rows
-// form an interval: its top (bottom) is the ellipse's own top (bottom) point when that lies in
-// the slab, else the boundary at the slab's nearer edge (the upper boundary is concave).
-// Widened by 1/100 pixel: a superset of the rows the per-pixel test accepts.
+// Rows [ylo, yhi] (tile-local, not clamped to it; ylo > yhi if none) that a record's widened cut
+// ellipse reaches inside the column slab of pixel centres [x0, x1].  The ellipse's
+// section by the slab is convex, so its rows form an interval: its top (bottom) is the ellipse's own
+// top (bottom) point when that lies in the slab, else the boundary at the slab's nearer edge (the
+// upper boundary is concave).  Widened by 1/100 pixel and 16 u of the ellipse's half height, for the
+// rounding of rows far from the centre: a superset of the rows the per-pixel test accepts.
 struct SlabExt {
-  float dyt, dxt;  // the ellipse's top point relative to its centre (bottom = -top)
+  float D, c4, inv2c;   // 4ac - b^2, 4 c e (> 0), 1 / (2c) (< 0)
+  float dxt;            // the ellipse's top point left or right of its centre
+  float ylo, yhi;       // the centre's row in the tile, less and plus the rows' margin
 };
-// (Approximate reciprocals and roots, within two ulp: far inside the 1/100 pixel.)
-__device__ __forceinline__ SlabExt make_slab(const float4 c, float cm) {
-  const float ia = rcp_approx(c.x);
-  const float kz = fmaf(-0.25f * c.y * c.y, ia, c.z);  // < 0
-  const float dyt = sqrt_approx(fmaxf(cm * rcp_approx(kz), 0.f));
-  return SlabExt{dyt, -0.5f * c.y * dyt * ia};
+__device__ __forceinline__ SlabExt make_slab(const float4 g, const float4 c, int ty0) {
+  SlabExt X;
+  const float D = conic_det(c);
+  const float dyt = sqrt_approx(fmaxf(4.f * c.x * c.w * rcp_approx(D), 0.f));  // the top's height
+  X.dxt = -0.5f * c.y * dyt * rcp_approx(c.x);
+  X.D = c.w == -INFINITY ? 0.f : D;  // the whole box: rows without bound
+  X.c4 = 4.f * c.z * c.w;
+  X.inv2c = 0.5f * rcp_approx(c.z);
+  const float my = fmaf(dyt, 1.f / 1048576.f, 0.01f), gy = g.y - (float)ty0;
+  X.ylo = gy - my;
+  X.yhi = gy + my;
+  return X;
 }
-__device__ __forceinline__ void slab_rows(const float4 g, const float4 c, float cm,
-                                          const SlabExt& X, float x0, float x1, int ty0, int T,
-                                          int& ylo, int& yhi) {
+__device__ __forceinline__ void slab_rows(const float4 g, const float4 c, const SlabExt& X,
+                                          float x0, float x1, int& ylo, int& yhi) {
   const float u0 = x0 - g.x, u1 = x1 - g.x;
-  const float inv2c = 0.5f * rcp_approx(c.z);  // < 0
   const float xu = fminf(fmaxf(X.dxt, u0), u1), xl = fminf(fmaxf(-X.dxt, u0), u1);
-  const float Du = fmaxf(fmaf(c.y * xu, c.y * xu, -4.f * c.z * fmaf(c.x * xu, xu, -cm)), 0.f);
-  const float Dl = fmaxf(fmaf(c.y * xl, c.y * xl, -4.f * c.z * fmaf(c.x * xl, xl, -cm)), 0.f);
-  const float ymax = (-c.y * xu - sqrt_approx(Du)) * inv2c;
-  const float ymin = (-c.y * xl + sqrt_approx(Dl)) * inv2c;
-  ylo = max(0, (int)ceilf(g.y + ymin - 0.01f) - ty0);
-  yhi = min(T - 1, (int)floorf(g.y + ymax + 0.01f) - ty0);
+  const float Du = fmaxf(fmaf(-X.D * xu, xu, X.c4), 0.f);  // (b x)^2 - 4 c (a x^2 - e)
+  const float Dl = fmaxf(fmaf(-X.D * xl, xl, X.c4), 0.f);
+  ylo = (int)ceilf(fmaf(-c.y * xl + sqrt_approx(Dl), X.inv2c, X.ylo));
+  yhi = (int)floorf(fmaf(-c.y * xu - sqrt_approx(Du), X.inv2c, X.yhi));
 }
 
 // Bit mask of the (4-row x BW-column) blocks of a (T x T) tile at (tx0, ty0) that a record's cut
@@ -765,8 +798,7 @@ template <int T, int BW>
 __device__ __forceinline__ uint32_t block_mask(const float4 g, const float4 c, const short4 bx,
                                                int tx0, int ty0) {
   constexpr int LBW = BW == 16 ? 4 : 3, NBX = T / BW, NBY = T / 4;
-  const float cm = g.w * 1.001f;
-  const SlabExt X = make_slab(c, cm);
+  const SlabExt X = make_slab(g, c, ty0);
   const int bx0 = (bx.x - tx0) >> LBW, bx1 = (bx.z - tx0) >> LBW;
   const int ry0 = max(0, bx.y - ty0), ry1 = min(T - 1, bx.w - ty0);
   uint32_t mask = 0u;
@@ -774,7 +806,7 @@ __device__ __forceinline__ uint32_t block_mask(const float4 g, const float4 c, c
   for (int k = 0; k < NBX; ++k) {
     const float x0 = (float)(tx0 + k * BW);
     int ylo, yhi;
-    slab_rows(g, c, cm, X, x0, x0 + (float)(BW - 1), ty0, T, ylo, yhi);
+    slab_rows(g, c, X, x0, x0 + (float)(BW - 1), ylo, yhi);
     ylo = max(ylo, ry0);
     yhi = min(yhi, ry1);
     if (k >= bx0 && k <= bx1 && ylo <= yhi)
@@ -1018,7 +1050,9 @@ __device__ __forceinline__ void narrow_moments(const float4 g, const float4 c, c
                                                const float* __restrict__ dv, int W, int H,
                                                float4* __restrict__ out) {
   constexpr int CW = BwdBlocks<T>::CW;
-  const float cm = g.w * 1.001f, ia = 0.5f * rcp_approx(c.x);  // < 0
+  const bool whole = c.w == -INFINITY;
+  const float ia = 0.5f * rcp_approx(c.x);  // < 0
+  const float D4 = conic_det(c), a4 = 4.f * c.x * c.w;
   const bool own = -(c.x + c.z) * 0.005f > 0.72134752f;
   float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
   for (int by = bx.y & ~3; by <= bx.w; by += 4)
@@ -1029,11 +1063,11 @@ __device__ __forceinline__ void narrow_moments(const float4 g, const float4 c, c
         const float dy = (float)y - g.y;
         const float B = row_b(c, dy), C = row_c(c, dy);
         // the row's section of the widened cut ellipse, to 1/50 pixel
-        const float D = fmaf(B, B, -4.f * c.x * (C - cm));
-        if (!(D >= 0.f)) continue;
+        const float D = fmaf(-D4 * dy, dy, a4);  // (b y)^2 - 4 a (c y^2 - e)
+        if (!whole && !(D >= 0.f)) continue;
         const float mid = g.x - B * ia, half = 0.02f - sqrt_approx(D) * ia;
-        const int xa = max(x0, (int)ceilf(mid - half));
-        const int xb = min(min(x0 + CW, W) - 1, (int)floorf(mid + half));
+        const int xa = max(x0, whole ? x0 : (int)ceilf(mid - half));
+        const int xb = min(min(x0 + CW, W) - 1, whole ? W : (int)floorf(mid + half));
         float2 r0 = make_float2(0.f, 0.f), rx = r0, rxx = r0;  // even and odd columns
         const float* row = dv + (size_t)y * W;
         for (int x = xa & ~1; x <= xb; x += 4) {  // four pixels' loads at once
