@@ -930,7 +930,7 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
       const int j = active ? list[li] : 0;
       const float4 g = s_geo[j];
       const float4 c = s_con[j];
-      const float cut = active ? g.w : 1.f;  // e <= 0 < 1: an idle lane never passes
+      const float cut = active ? g.w : INFINITY;  // an idle lane never passes
       float2 dx[HP];
 #pragma unroll
       for (int p = 0; p < HP; ++p)
@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
   int qh = 0, qn = 0;    // the queue's next and its end
   // the lane's record: the blocks still to walk, its coefficients and its six sums
   uint32_t rec = 0u, mask = 0u;
-  float gx = 0.f, gy = 0.f, cut = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+  float gx = 0.f, gy = 0.f, cut = INFINITY, c0 = 0.f, c1 = 0.f, c2 = 0.f;
   float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
   for (;;) {
     bool need = mask == 0u;
@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
           atomicAdd(&fpgrad[2 * (size_t)rec + 1], make_float4(mxy, myy, 0.f, 0.f));
         }
         m0 = mx = my = mxx = mxy = myy = 0.f;
-        cut = 1.f;  // e <= 0 < 1: an idle lane never passes
+        cut = INFINITY;  // an idle lane never passes, whatever a thin ellipse's e rounds to
       }
       for (;;) {
         const int slot = qh + __popc(idle & lt);

@@ -377,8 +377,7 @@ def test_stream_handle_follows_the_current_stream(gsct):
     assert B.stream_handle(side) == side.cuda_stream
 
 
-@pytest.mark.parametrize("ratio", [300, 1000, 2500])
-def test_thin_ellipses_lose_no_pixel(orc, gsct, ratio):
+def _thin_case(orc, gsct, ratio):
     """Long thin footprints (sigma 60 pixels by 60 / ratio), one Gaussian per view: tiles of 8, 16
     and 32 pixels, whose lists and blocks lie differently, draw the same bits inside the Gaussian's
     box, and the backward sums the same pixels (less than 400 terms of one sign: 400 x 2^-24 of the
@@ -409,3 +408,15 @@ def test_thin_ellipses_lose_no_pixel(orc, gsct, ratio):
             same = (imgs[k] == imgs[0]) | ~inside
             assert bool(same.all()), (seed, k, int((~same).sum()))
             assert abs(grads[k] - grads[0]) <= 800 * 2.0 ** -24 * abs(grads[0]), (seed, grads)
+
+
+@pytest.mark.parametrize("ratio", [300, 1000, 2500])
+def test_thin_ellipses_lose_no_pixel(orc, gsct, ratio):
+    """Lists and block masks hold every in-cut pixel of ellipses whose conic nearly cancels."""
+    _thin_case(orc, gsct, ratio)
+
+
+def test_idle_lanes_add_nothing(orc, gsct):
+    """Where the exponent of a degenerate ellipse rounds above zero, lanes without a record of their
+    own leave the sums alone."""
+    _thin_case(orc, gsct, 10000)
