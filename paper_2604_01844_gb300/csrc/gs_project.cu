@@ -491,10 +491,17 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
     run += tcount[e];
   }
   if (seg == 0) {  // the first two warps hold the group's keys
-    const uint32_t incl = gsd::warp_inclusive_scan(total);
+    // (in 64 bits: 2^27 records that each cover 32 neighbouring tiles pass 2^32; where a 32-bit
+    // place would wrap, the pair total is above any capacity and nothing is placed)
+    unsigned long long incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
     if (lane == 31) wtot[t >> 5] = incl;
     asm volatile("bar.sync 1, %0;" ::"n"(kScanKeys) : "memory");
-    const uint32_t first = incl - total + (t >= 32 ? (uint32_t)wtot[0] : 0u);
+    const uint32_t first = (uint32_t)(incl - total + (t >= 32 ? wtot[0] : 0ull));
     if (key < n_keys) {
       klocal[key] = first;
       ranges[key] = make_uint2(first, total);
@@ -1152,7 +1159,7 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
     r.x = min(r.y, r.x + blockIdx.y * part);
     r.y = min(r.y, r.x + part);
   }
-  if (r.x == r.y) return;
+  if (r.x >= r.y) return;  // (>: lists of an instance without Gaussians, which no emit completes)
   const Inst& I = b.in[inst_of_key(b, key)];
   const int64_t lk = key - I.key_off;
   const int v = (int)(lk / (I.TW * I.TH)), tile = (int)(lk - (int64_t)v * I.TW * I.TH);

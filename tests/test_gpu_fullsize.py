@@ -341,3 +341,23 @@ def test_voxelize_backward_1024_sampled(orc, gsct):
         want[k] = orc.voxelize_grad(P[i:i + 1], grid, crop, roi_lo=tuple(int(a) for a in lo),
                                     roi_dim=tuple(int(a) for a in dim))[0]
     assert_grads_close(got[sel], want, np.ones(len(sel), dtype=bool))
+
+
+def test_pair_total_beyond_32_bits(gsct):
+    """2^27 Gaussians that all cover the 32 tiles of one small view: 2^32 pairs, counted in 64 bits
+    and refused as more than the workspace holds, with the image left as it was."""
+    n, W, H = 1 << 27, 64, 32
+    views = synth.cone_views(1, W, H)
+    mr = torch.zeros((n, 4), device="cuda")
+    mr[:, 3] = 1.0
+    sc = torch.ones((n, 4), device="cuda")
+    qt = torch.zeros((n, 4), device="cuda")
+    qt[:, 0] = 1.0
+    proj = gsct.Projector(views, W, H, tile=8)
+    assert proj.count_pairs(mr, sc, qt) == 1 << 32
+    proj._alloc(n, 1 << 16)
+    img = torch.full((1, H, W), 7.0, device="cuda")
+    proj.forward(mr, sc, qt, out=img)
+    st = proj.status()
+    assert st.code != 0 and st.pairs == 1 << 32
+    assert bool((img == 7.0).all())
