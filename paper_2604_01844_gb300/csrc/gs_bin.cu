@@ -25,7 +25,7 @@ __global__ void k_scan_block_sums(const uint32_t* __restrict__ sums, uint32_t* _
   const int per = (nb + blockDim.x - 1) / blockDim.x;
   const int b0 = min(nb, t * per), b1 = min(nb, b0 + per);
   unsigned long long local = 0;
-  for (int b = b0; b < b1; ++b) local += sums[b];
+  for (int b = b0; b < b1; ++b) local += __ldcg(sums + b);
   // block-wide exclusive scan of `local`
   unsigned long long incl = local;
 #pragma unroll
@@ -49,7 +49,7 @@ __global__ void k_scan_block_sums(const uint32_t* __restrict__ sums, uint32_t* _
   unsigned long long run = incl - local + (w > 0 ? warp_tot[w - 1] : 0ull);
   for (int b = b0; b < b1; ++b) {
     offs[b] = (uint32_t)run;
-    run += sums[b];
+    run += __ldcg(sums + b);
   }
   if (t == blockDim.x - 1) {
     unsigned long long total = warp_tot[(blockDim.x >> 5) - 1];
@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(kSortThreads)
     for (int h = 0; h < 2; ++h) {
       const int64_t ih = i + h * kStep;
       if (ih + 4 <= hi) {
-        const uint4 q = *reinterpret_cast<const uint4*>(keys + ih);
+        const uint4 q = __ldcg(reinterpret_cast<const uint4*>(keys + ih));
         k[4 * h] = q.x, k[4 * h + 1] = q.y, k[4 * h + 2] = q.z, k[4 * h + 3] = q.w;
       } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) k[4 * h + j] = ih + j < hi ? keys[ih + j] : 0u;
+        for (int j = 0; j < 4; ++j) k[4 * h + j] = ih + j < hi ? __ldcg(keys + ih + j) : 0u;
       }
     }
 #pragma unroll
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kSortThreads)
   const int per = (D + kSortThreads - 1) / kSortThreads;
   {
     uint32_t s0 = 0;
-    for (int d = t * per; d < min(D, t * per + per); ++d) s0 += totals[d];
+    for (int d = t * per; d < min(D, t * per + per); ++d) s0 += __ldcg(totals + d);
     const uint32_t incl = gsd::warp_inclusive_scan(s0);
     if (lane == 31) wtot[w] = incl;
     __syncthreads();
@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(kSortThreads)
 #pragma unroll
     for (int ww = 0; ww < NW; ++ww) acc += ww < w ? wtot[ww] : 0u;
     for (int d = t * per; d < min(D, t * per + per); ++d) {
-      run[d] = acc + hist[(size_t)d * G + blockIdx.x];
-      acc += totals[d];
+      run[d] = acc + __ldcg(hist + (size_t)d * G + blockIdx.x);
+      acc += __ldcg(totals + d);
     }
   }
   for (int i = t; i < NW * D; i += kSortThreads) wcnt[i] = 0;
@@ -295,9 +295,9 @@ __global__ void k_ranges(const uint32_t* __restrict__ keys, uint2* __restrict__ 
   const int64_t n = st->pairs;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const uint32_t k = keys[i];
-    if (i == 0 || keys[i - 1] != k) ranges[k].x = (uint32_t)i;
-    if (i == n - 1 || keys[i + 1] != k) ranges[k].y = (uint32_t)(i + 1);
+    const uint32_t k = __ldcg(keys + i);
+    if (i == 0 || __ldcg(keys + i - 1) != k) ranges[k].x = (uint32_t)i;
+    if (i == n - 1 || __ldcg(keys + i + 1) != k) ranges[k].y = (uint32_t)(i + 1);
   }
 }
 

@@ -35,13 +35,18 @@ int launch(const char* name, void (*kernel)(KArgs...), dim3 grid, dim3 block, si
   return GS_OK;
 }
 
-// The same for a kernel that begins with gsd::pdl_begin() and directly follows another kernel of
-// the same library call on the same stream (no event wait or copy can lie between): a
-// programmatic launch, scheduled while its predecessor drains.  It takes the launch latency out
-// of the short kernels' chains (gradient of 1024 bricks, 17 launches: 276 -> 248 us; the
-// 256^3 voxelizer pass, 14: 320 -> 296 us).  Not for a call's first kernel: in tests a
-// programmatic launch behind a cross-stream event wait did not keep the wait.  Not for the
-// kernels of very many short CTAs either: the wait at the start of each CTA of the raster
+// The same for a kernel that calls gsd::pdl_begin() and directly follows another kernel of the
+// same library call on the same stream: a programmatic launch, scheduled while its predecessor
+// drains.  It takes the launch latency out of the short kernels' chains (gradient of 1024 bricks,
+// 17 launches: 276 -> 248 us; the 256^3 voxelizer pass, 14: 320 -> 296 us).
+// What such a kernel waits for is that one predecessor.  So it is never a call's first kernel, which
+// may follow an event wait, a copy or a memset, and the launch before it in the call always takes
+// place (a call without Gaussians returns first).  All other kernels of the call are complete by
+// then: the predecessor was launched behind them, or itself waited for them before it let this one
+// be scheduled.  What the predecessor wrote is read with __ldcg (or TMA): a read-only load is for
+// data that nothing writes while the kernel lives, and this one's life begins before the
+// predecessor's end.
+// Not for the kernels of very many short CTAs: the wait at the start of each CTA of the raster
 // kernels cost 7 %.
 template <typename... KArgs, typename... Args>
 int launch_after(const char* name, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
@@ -175,8 +180,8 @@ namespace gsd {
 
 // Waits until the kernels before this one in the stream are complete and their writes visible
 // (a kernel launched the ordinary way passes at once), then lets the next kernel be scheduled.
-// First statement of every kernel that launch_after() launches: it waits before it touches
-// global memory, and it cannot complete before its predecessor has.
+// Every thread of every kernel that launch_after() launches calls it before it touches global
+// memory, so that the kernel cannot complete before its predecessor has.
 __device__ __forceinline__ void pdl_begin() {
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();

@@ -336,7 +336,7 @@ __global__ void __cluster_dims__(1, kColsumCtas, 1) __launch_bounds__(1024)
   float s = 0.f;
   if (c < cols) {
 #pragma unroll 8
-    for (int r = r0 + w; r < r1; r += 32) s += g[(size_t)r * cols + c];
+    for (int r = r0 + w; r < r1; r += 32) s += __ldcg(g + (size_t)r * cols + c);
   }
   part[w][lane] = s;
   __syncthreads();

@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
     at = I.mat_off + (int64_t)v * I.bpv * tp + tile;
     if (seg == 0 && tile == 0) vkeys[I.v_off + v] = key;
 #pragma unroll 8
-    for (int k = b0; k < b1; ++k) sum += tcount[at + (int64_t)k * tp];
+    for (int k = b0; k < b1; ++k) sum += __ldcg(tcount + at + (int64_t)k * tp);
   }
   if (blockIdx.x == 0 && t == 0) vkeys[total_v] = n_keys;
   part[seg][kl] = sum;
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
   for (int k = b0; k < b1; ++k) {
     const int64_t e = at + (int64_t)k * tp;
     toffset[e] = run;
-    run += tcount[e];
+    run += __ldcg(tcount + e);
   }
   if (seg == 0) {  // the first two warps hold the group's keys
     // (in 64 bits: 2^27 records that each cover 32 neighbouring tiles pass 2^32; where a 32-bit
@@ -1368,13 +1368,13 @@ __global__ void __launch_bounds__(kThreads, 2)
   float st_acc = 0.f;
   int vis_acc = 0;
   size_t rec = (size_t)(I.item_off + (int64_t)v0 * I.n + il);
-  float4 n0 = fpgrad[2 * rec], n1 = fpgrad[2 * rec + 1];  // the next view's moments, one ahead
+  float4 n0 = __ldcg(fpgrad + 2 * rec), n1 = __ldcg(fpgrad + 2 * rec + 1);  // the next view's moments, one ahead
   for (int v = v0; v < v1; ++v, rec += I.n) {
     if (stat && counts[rec] > 0u) ++vis_acc;
     const float4 m0 = n0, m1 = n1;
     if (v + 1 < v1) {
-      n0 = fpgrad[2 * (rec + I.n)];
-      n1 = fpgrad[2 * (rec + I.n) + 1];
+      n0 = __ldcg(fpgrad + 2 * (rec + I.n));
+      n1 = __ldcg(fpgrad + 2 * (rec + I.n) + 1);
     }
     if (m0.x == 0.f && m0.y == 0.f && m0.z == 0.f && m0.w == 0.f && m1.x == 0.f && m1.y == 0.f)
       continue;

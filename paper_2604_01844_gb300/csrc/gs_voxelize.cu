@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kThreads)
   const uint32_t cnt = in ? counts[i] : 0u;
   const short4 a = in ? lo_in[i] : make_short4(0, 0, 0, 0);
   const short4 b = in ? hi_in[i] : make_short4(0, 0, 0, 0);
-  const uint32_t boff = block_offs[blockIdx.x];
+  const uint32_t boff = __ldcg(block_offs + blockIdx.x);
   if (st->code != GS_OK) return;
   const uint32_t incl = gsd::warp_inclusive_scan(cnt);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -825,7 +825,7 @@ __global__ void __launch_bounds__(kThreads)
   gsd::pdl_begin();
   const int i = blockIdx.x * kThreads + threadIdx.x;
   if (i >= n) return;
-  const float4 a = vgrad[3 * i], b = vgrad[3 * i + 1], c = vgrad[3 * i + 2];
+  const float4 a = __ldcg(vgrad + 3 * i), b = __ldcg(vgrad + 3 * i + 1), c = __ldcg(vgrad + 3 * i + 2);
   float gp[3] = {0.f, 0.f, 0.f}, grho = 0.f, gs[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
   VFwd o;
   const float4 mr = mean_rho[i];
