@@ -59,6 +59,9 @@ __global__ void k_fdk_setup(const gs_view* __restrict__ views, int nv, FdkView* 
 // back-projection reads all four bilinear neighbours of a clamped position without a test.
 constexpr int kPadL = 4;
 int fdk_pitch(int W) { return (W + kPadL + 2 + 3) / 4 * 4; }  // rows stay 16-byte aligned
+size_t fdk_padded(int n_views, int W, int H) {
+  return (size_t)n_views * ((size_t)H + 4) * fdk_pitch(W);
+}
 
 // Weight and ramp-filter.  The Ram-Lak kernel vanishes at even distances, so the outputs of one
 // parity are a convolution of the inputs of the other parity with the weights h(2 d + 1): a
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(kFilterThreads)
   const float h0 = 0.25f / (tau * tau);
   const float hk = -1.f / (float)(kPi * kPi) / (tau * tau);
   const float* p = proj + (size_t)v * H * W;
-  float* ov = out + (size_t)v * (H + 4) * pitch;
+  float* ov = out + (size_t)v * ((size_t)H + 4) * pitch;
   // padding: the columns beside this CTA's rows, the rows above the first and below the last
   for (int r = 0; r < 2 * RP; ++r) {
     if (row0 + r >= H) break;
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(kThreads)
     if (!live) continue;
     for (int k = 0; k < m; ++k) {
       const FdkView& f = s_v[k];
-      const float* qv = q + (size_t)(base + k) * (H + 4) * pitch + kPadL;
+      const float* qv = q + (size_t)(base + k) * ((size_t)H + 4) * pitch + kPadL;
       const float rx = px - f.s[0], ry = py - f.s[1];
       const float Ub = rx * f.n[0] + ry * f.n[1];
       const float ub = rx * f.eu[0] + ry * f.eu[1], vb = rx * f.ev[0] + ry * f.ev[1];
@@ -659,8 +662,8 @@ extern "C" {
 
 size_t gs_fdk_workspace_size(int n_views, int W, int H) {
   if (n_views < 1 || W < 1 || H < 1) return 0;
-  return align_up((size_t)n_views * (H + 4) * fdk_pitch(W) * sizeof(float), 256) +
-         align_up((size_t)n_views * sizeof(FdkView), 256);
+  return align_up(fdk_padded(n_views, W, H) * sizeof(float), 256) +
+         align_up((size_t)n_views * sizeof(FdkView), 256) + 16;  // the workspace may start anywhere
 }
 
 }  // extern "C"
@@ -703,8 +706,8 @@ int gs_fdk(const float* d_proj, const gs_view* d_views, int n_views, int W, int 
     if (grid->dims[k] < 1 || !(grid->voxel[k] > 0.f)) return GS_ERR_ARG;
   if (ws_bytes < gs_fdk_workspace_size(n_views, W, H)) return GS_ERR_CAPACITY;
   cudaStream_t s = (cudaStream_t)stream;
-  Carve c(d_ws);
-  float* q = c.take<float>((size_t)n_views * (H + 4) * fdk_pitch(W));
+  Carve c((void*)(((uintptr_t)d_ws + 15) & ~(uintptr_t)15));
+  float* q = c.take<float>(fdk_padded(n_views, W, H));
   FdkView* fv = c.take<FdkView>(n_views);
   GS_TRY(launch("fdk_setup", k_fdk_setup, dim3((n_views + 63) / 64), dim3(64), 0, s, d_views,
                 n_views, fv));

@@ -145,3 +145,26 @@ def test_fdk_ragged_and_tilted(orc, gsct, nv, W, H, dims, tilt):
     assert np.abs(want).max() > 0
     tol = 1e-4 + 2.0 ** -21 * max(W, H)
     assert np.abs(vol.cpu().numpy() - want).max() <= tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("offset", [4, 8, 12])
+def test_fdk_workspace_at_any_address(orc, gsct, offset):
+    """A workspace that starts between 16-byte boundaries: the same volume, and not a byte written
+    outside the size asked for."""
+    B = gsct.binding
+    nv, W, H, dims = 3, 37, 21, (9, 10, 11)
+    grid = synth.cube_grid(16)
+    grid["dims"] = dims
+    d_views = gsct.views_to_device(synth.cone_views(nv, W, H), "cuda")
+    proj = torch.rand((nv, H, W), device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    size = B.lib().gs_fdk_workspace_size(nv, W, H)
+    vols = []
+    for off in (0, offset):
+        room = torch.full((size + 64,), 171, dtype=torch.uint8, device="cuda")
+        vol = torch.empty(tuple(reversed(dims)), device="cuda")
+        B.check(B.lib().gs_fdk(B.ptr(proj), B.ptr(d_views), nv, W, H,
+                               ctypes.byref(B.grid_struct(grid)), B.ptr(vol), B.ptr(room) + off, size,
+                               _s()), "gs_fdk")
+        assert bool((room[:off] == 171).all()) and bool((room[off + size:] == 171).all())
+        vols.append(vol)
+    assert torch.equal(vols[0], vols[1])
