@@ -331,12 +331,13 @@ __global__ void __cluster_dims__(1, kColsumCtas, 1) __launch_bounds__(1024)
   __shared__ float cta_sum[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  const int per = (rows + kColsumCtas - 1) / kColsumCtas;
-  const int r0 = min(rows, (int)blockIdx.y * per), r1 = min(rows, r0 + per);
+  // unsigned: rows up to 2^31 - 1 and a step beyond them
+  const uint32_t n = (uint32_t)rows, per = (n + kColsumCtas - 1) / kColsumCtas;
+  const uint32_t r0 = min(n, blockIdx.y * per), r1 = min(n, r0 + per);
   float s = 0.f;
   if (c < cols) {
 #pragma unroll 8
-    for (int r = r0 + w; r < r1; r += 32) s += __ldcg(g + (size_t)r * cols + c);
+    for (uint32_t r = r0 + w; r < r1; r += 32) s += __ldcg(g + (size_t)r * cols + c);
   }
   part[w][lane] = s;
   __syncthreads();

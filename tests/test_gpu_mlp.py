@@ -287,3 +287,14 @@ def test_infer_equals_forward_and_decode(gsct):
     torch.cuda.synchronize()
     for u, v in zip(got, want):
         assert torch.equal(u, v)
+
+
+def test_colsum_of_the_longest_column(gsct):
+    """2^31 - 1 rows, the most an int holds: every row is read, and none beyond the last."""
+    B = gsct.binding
+    x = torch.zeros((2 ** 31 - 1, 1), device="cuda")
+    x[0], x[2 ** 30], x[2 ** 31 - 9:] = 1.0, 2.0, 4.0
+    out = torch.full((1,), -1.0, device="cuda")
+    B.check(B.lib().gs_colsum(B.ptr(x), x.shape[0], 1, B.ptr(out),
+                              torch.cuda.current_stream().cuda_stream), "colsum")
+    assert float(out) == 1.0 + 2.0 + 4.0 * 8
