@@ -243,11 +243,11 @@ constexpr int kPatchX = 8, kPatchY = 4;                   // and of a warp
 template <int ZT>
 __global__ void __launch_bounds__(kThreads)
     k_fdk_backproject(const float* __restrict__ q, const FdkView* __restrict__ fv, int nv, int W,
-                      int H, int pitch, int nx, int ny, int nz, float ox, float oy, float oz,
-                      float hx, float hy, float hz, float* __restrict__ vol) {
+                      int H, int pitch, int64_t view, int nx, int ny, int nz, float ox, float oy,
+                      float oz, float hx, float hy, float hz, float* __restrict__ vol) {
   __shared__ FdkView s_v[64];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int bx = (nx + kBackX - 1) / kBackX, by = (ny + kBackY - 1) / kBackY;
+  const int bx = (nx - 1) / kBackX + 1, by = (ny - 1) / kBackY + 1;  // up to 2^31 - 1 voxels a side
   const int x = (int)(blockIdx.x % bx) * kBackX + w % (kBackX / kPatchX) * kPatchX + lane % kPatchX;
   const int y = (int)(blockIdx.x / bx % by) * kBackY + w / (kBackX / kPatchX) * kPatchY + lane / kPatchX;
   const int z0 = (int)(blockIdx.x / bx / by) * ZT;
@@ -266,9 +266,9 @@ __global__ void __launch_bounds__(kThreads)
     for (int k = threadIdx.x; k < m; k += kThreads) s_v[k] = fv[base + k];
     __syncthreads();
     if (!live) continue;
-    for (int k = 0; k < m; ++k) {
+    const float* qv = q + base * view + kPadL;
+    for (int k = 0; k < m; ++k, qv += view) {
       const FdkView& f = s_v[k];
-      const float* qv = q + (size_t)(base + k) * ((size_t)H + 4) * pitch + kPadL;
       const float rx = px - f.s[0], ry = py - f.s[1];
       const float Ub = rx * f.n[0] + ry * f.n[1];
       const float ub = rx * f.eu[0] + ry * f.eu[1], vb = rx * f.ev[0] + ry * f.ev[1];
@@ -681,16 +681,21 @@ int fdk_filter(const float* proj, const FdkView* fv, int nv, int W, int H, float
                 dim3(kFilterThreads), smem, s, proj, fv, W, H, fdk_pitch(W), q);
 }
 
+// 16 x 16 blocks of columns of the back-projection.
+int64_t fdk_columns(const gs_grid* g) {
+  return (((int64_t)g->dims[0] + kBackX - 1) / kBackX) * (((int64_t)g->dims[1] + kBackY - 1) / kBackY);
+}
+
 template <int ZT>
 int fdk_backproject(const float* q, const FdkView* fv, int nv, int W, int H, const gs_grid* g,
                     float* vol, cudaStream_t s) {
   const int nx = g->dims[0], ny = g->dims[1], nz = g->dims[2];
-  const int64_t blocks = (int64_t)((nx + kBackX - 1) / kBackX) * ((ny + kBackY - 1) / kBackY) *
-                         ((nz + ZT - 1) / ZT);
+  const int64_t blocks = fdk_columns(g) * (((int64_t)nz + ZT - 1) / ZT);
   if (blocks > ((int64_t)1 << 31) - 1) return GS_ERR_ARG;
   return launch("fdk_backproject", k_fdk_backproject<ZT>, dim3((unsigned)blocks), dim3(kThreads),
-                0, s, q, fv, nv, W, H, fdk_pitch(W), nx, ny, nz, g->origin[0], g->origin[1],
-                g->origin[2], g->voxel[0], g->voxel[1], g->voxel[2], vol);
+                0, s, q, fv, nv, W, H, fdk_pitch(W), (int64_t)fdk_padded(1, W, H), nx, ny, nz,
+                g->origin[0], g->origin[1], g->origin[2], g->voxel[0], g->voxel[1], g->voxel[2],
+                vol);
 }
 }  // namespace
 }  // namespace gs
@@ -718,12 +723,11 @@ int gs_fdk(const float* d_proj, const gs_view* d_views, int n_views, int W, int 
   // more voxels per thread share more of a column's geometry; fewer while the grid would leave
   // SMs idle (four CTAs each).  256^3 from 75 x 512^2: 1.56 ms with 16, 1.83 with 8, 2.1 with 4;
   // 32 spills the block's rows out of L1 (2.9 ms)
-  const int64_t cols = (int64_t)((grid->dims[0] + kBackX - 1) / kBackX) *
-                       ((grid->dims[1] + kBackY - 1) / kBackY);
+  const int64_t cols = fdk_columns(grid), nz = grid->dims[2];
   const int64_t want = 4 * (int64_t)num_sms();
-  if (cols * ((grid->dims[2] + 15) / 16) >= want)
+  if (cols * ((nz + 15) / 16) >= want)
     return fdk_backproject<16>(q, fv, n_views, W, H, grid, d_vol, s);
-  if (cols * ((grid->dims[2] + 3) / 4) >= want)
+  if (cols * ((nz + 3) / 4) >= want)
     return fdk_backproject<4>(q, fv, n_views, W, H, grid, d_vol, s);
   return fdk_backproject<1>(q, fv, n_views, W, H, grid, d_vol, s);
 }

@@ -168,3 +168,32 @@ def test_fdk_workspace_at_any_address(orc, gsct, offset):
         assert bool((room[:off] == 171).all()) and bool((room[off + size:] == 171).all())
         vols.append(vol)
     assert torch.equal(vols[0], vols[1])
+
+
+@pytest.mark.parametrize("axis", [0, 2])
+def test_fdk_of_the_longest_line(orc, gsct, axis):
+    """2^31 - 1 voxels in one line, the most an int holds: every voxel is written, and the last one
+    holds what a single voxel there holds (1e-4 of it, as for volumes)."""
+    B = gsct.binding
+    nv, W, H = 2, 16, 16
+    d_views = gsct.views_to_device(synth.cone_views(nv, W, H), "cuda")
+    proj = torch.ones((nv, H, W), device="cuda")
+    ws = torch.empty(B.lib().gs_fdk_workspace_size(nv, W, H), dtype=torch.uint8, device="cuda")
+
+    def run(dims, origin, voxel):
+        grid = synth.cube_grid(8)
+        grid["dims"], grid["origin"], grid["voxel"] = dims, origin, voxel
+        vol = torch.full((int(np.prod(dims, dtype=np.int64)),), float("nan"), device="cuda")
+        B.check(B.lib().gs_fdk(B.ptr(proj), B.ptr(d_views), nv, W, H,
+                               ctypes.byref(B.grid_struct(grid)), B.ptr(vol), B.ptr(ws), ws.numel(),
+                               _s()), "gs_fdk")
+        return vol
+
+    n, origin, voxel = 2 ** 31 - 1, [0.0, 0.0, 0.0], [1e-3] * 3
+    dims = [1, 1, 1]
+    dims[axis], voxel[axis] = n, 0.5 / n
+    line = run(dims, origin, voxel)
+    origin[axis], voxel[axis] = 0.5 - 1e-6, 2e-6
+    one = run([1, 1, 1], origin, voxel)
+    assert not bool(torch.isnan(line).any())
+    assert float(one) != 0 and abs(float(line[-1]) - float(one)) <= 1e-4 * abs(float(one))
