@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kThreads)
   const int y = cols >> 32 ? (int)(p / nxv) : (int)((uint32_t)p / (uint32_t)nxv);
   const int x = (int)(p - (int64_t)y * nxv) * VW;
   const int lane = threadIdx.x & 31;
-  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  const int z0 = blockIdx.y * zc, z1 = (int)min((uint32_t)nz, (uint32_t)z0 + zc);
   const bool xl = x > 0, xr = x + VW < nx, yl = y > 0, yr = y + 1 < ny;
   using V = typename std::conditional<VW == 4, float4, float>::type;
   auto load = [&](int64_t i, float (&f)[VW]) {
@@ -1456,8 +1456,8 @@ int gs_tv3d_loss(const float* d_vol, int nx, int ny, int nz, float weight, float
   // than eight CTAs per SM
   const int64_t want = std::max<int64_t>(1, 8 * (int64_t)num_sms() / bx);
   int zc = (int)std::max<int64_t>(1, std::min<int64_t>(16, nz / want));
-  zc = std::max(zc, (nz + 65534) / 65535);
-  const dim3 grid((unsigned)bx, (unsigned)((nz + zc - 1) / zc));
+  zc = std::max(zc, (nz - 1) / 65535 + 1);
+  const dim3 grid((unsigned)bx, (unsigned)((nz - 1) / zc + 1));
   return launch("tv3d_loss", vec ? k_tv3d<4> : k_tv3d<1>, grid, dim3(kThreads), 0,
                 (cudaStream_t)stream, d_vol, nx, ny, nz, zc, weight / (float)total, d_loss, d_grad,
                 accumulate);

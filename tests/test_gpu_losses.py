@@ -375,3 +375,18 @@ def test_l1_ssim2d_many_images(B, n):
     for k in range(n):
         vals.append(_run_loss(B, "l1ssim2d", x[k:k + 1], y[k:k + 1], 1.0, 0.6, weight=0.25)[0])
     assert abs(val - np.mean(vals)) <= 3e-6 * abs(val)
+
+
+def test_tv3d_of_the_longest_line(B):
+    """2^31 - 1 planes of one voxel, the most an int holds: a step near the end is one difference of
+    the loss and a pair of signs in the gradient, every other voxel of which is written as zero."""
+    n = 2 ** 31 - 1
+    vol = torch.zeros(n, device="cuda")
+    vol[-5:] = 1.0
+    grad, loss = torch.full((n,), float("nan"), device="cuda"), torch.zeros(1, device="cuda")
+    B.check(B.lib().gs_tv3d_loss(B.ptr(vol), 1, 1, n, float(n), B.ptr(loss), B.ptr(grad), 0, _s()),
+            "tv3d_loss")
+    assert float(loss) == 1.0
+    assert float(grad[-6]) == -1.0 and float(grad[-5]) == 1.0
+    grad[-6:-4] = 0.0
+    assert bool((grad == 0.0).all())
