@@ -39,15 +39,13 @@ __device__ __forceinline__ float rcp_newton(float x) {
   return fabsf(e) < 1.f ? fmaf(r, e, r) : r;
 }
 
-template <typename T, typename U>
+// Adds the block's sum of v to *target, or (STORE) puts it there.
+template <bool STORE = false, typename T, typename U>
 __device__ __forceinline__ void block_add(T v, U* target) {
   __shared__ T part[32];
   v = gsd::warp_sum(v);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nthreads = blockDim.x * blockDim.y * blockDim.z;
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  (void)lane;
-  (void)w;
   // linear thread id for multi-dimensional blocks
   const int l2 = tid & 31, w2 = tid >> 5;
   if (l2 == 0) part[w2] = v;
@@ -55,7 +53,10 @@ __device__ __forceinline__ void block_add(T v, U* target) {
   if (tid == 0) {
     T s = 0;
     for (int i = 0; i < (nthreads + 31) / 32; ++i) s += part[i];
-    if (s != (T)0) atomicAdd(target, (U)s);
+    if (STORE)
+      *target = (U)s;
+    else if (s != (T)0)
+      atomicAdd(target, (U)s);
   }
   __syncthreads();
 }
@@ -856,12 +857,22 @@ __device__ __forceinline__ bool fused_stream(const CUtensorMap* tmA, const CUten
   return !failed;
 }
 
+// Index of the CTA in its grid, read where it is used: taken from blockIdx it is kept through the
+// streaming loop, whose registers then change places (384^3 forward 554 -> 570 us).
+__device__ __forceinline__ uint32_t late_cta() {
+  uint32_t x, y, z;
+  asm volatile("mov.u32 %0, %ctaid.x;" : "=r"(x));
+  asm volatile("mov.u32 %0, %ctaid.y;" : "=r"(y));
+  asm volatile("mov.u32 %0, %ctaid.z;" : "=r"(z));
+  return x + gridDim.x * (y + gridDim.y * z);
+}
+
 template <bool MAPS>
 __global__ void __launch_bounds__(kFThreads, 2)
     k_ssim3d_fwd_fused(const __grid_constant__ CUtensorMap tmX,
                        const __grid_constant__ CUtensorMap tmY, const __grid_constant__ Win W,
                        int nx, int ny, int nz, int zc, float C1, float C2, float gscale,
-                       float l1s, float* __restrict__ loss, float2* __restrict__ m12,
+                       float l1s, float* __restrict__ parts, float2* __restrict__ m12,
                        float* __restrict__ m3, int* __restrict__ err) {
   const int z0 = blockIdx.z * zc, z1 = min(nz, z0 + zc);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -905,11 +916,25 @@ __global__ void __launch_bounds__(kFThreads, 2)
   if (!ok) {  // a tile copy never arrived: report it and poison the loss
     if (threadIdx.x == 0) {
       atomicExch(err, GS_ERR_TIMEOUT);
-      if (loss) atomicExch(loss, __int_as_float(0x7fc00000));
+      if (parts) parts[late_cta()] = __int_as_float(0x7fc00000);
     }
     return;
   }
-  if (loss) block_add(contrib * (-gscale) + l1 * l1s, loss);
+  if (parts) block_add<true>(contrib * (-gscale) + l1 * l1s, parts + late_cta());
+}
+
+// The forward's loss: its CTAs' n sums added up in double by one CTA, always in the same order,
+// and then added to *loss.  (As float atomics on one word, a few hundred CTAs' sums left an error of
+// up to 1e-6 of the loss that depended on their order.)
+__device__ __forceinline__ void add_loss_parts(const float* parts, int n, float* loss) {
+  double t = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) t += (double)__ldcg(parts + i);
+  block_add(t, loss);
+}
+__global__ void __launch_bounds__(kThreads)
+    k_loss_parts(const float* __restrict__ parts, int n, float* __restrict__ loss) {
+  gsd::pdl_begin();
+  add_loss_parts(parts, n, loss);
 }
 
 __global__ void __launch_bounds__(kFThreads, 2)
@@ -918,7 +943,8 @@ __global__ void __launch_bounds__(kFThreads, 2)
                        const __grid_constant__ CUtensorMap tmXt,
                        const __grid_constant__ CUtensorMap tmYt, const __grid_constant__ Win W,
                        int nx, int ny, int nz, int zc, float* __restrict__ grad, int accumulate,
-                       float l1g, int* __restrict__ err) {
+                       float l1g, const float* __restrict__ parts, float* __restrict__ loss,
+                       int* __restrict__ err) {
   using S = FusedShape<true>;
   const int z0 = blockIdx.z * zc, z1 = min(nz, z0 + zc);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -946,6 +972,8 @@ __global__ void __launch_bounds__(kFThreads, 2)
     if (own)
       for (int z = z0; z < z1; ++z) grad[((size_t)z * ny + y) * nx + x] = __int_as_float(0x7fc00000);
   }
+  if (loss && blockIdx.x + blockIdx.y + blockIdx.z == 0)
+    add_loss_parts(parts, gridDim.x * gridDim.y * gridDim.z, loss);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1598,8 +1626,10 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
   const dim3 gz((unsigned)bz_cols, (unsigned)((nz + zcol - 1) / zcol)), bz(kThreads);
   const float l1s = l1_weight / (float)plane;
   if (ssim3d_fused_ok(d_x, d_y, nx, ny)) {
-    // fused streaming kernels; tmp's first word is the TMA timeout status
+    // fused streaming kernels; tmp holds the TMA timeout status and, from its fifth word on, the
+    // forward CTAs' shares of the loss
     int* err = (int*)tmp;
+    float* parts = d_loss ? tmp + 4 : nullptr;
     CUtensorMap tmX, tmY;
     GS_TRY(volume_map(&tmX, d_x, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(volume_map(&tmY, d_y, nx, ny, nz, 4, kBoxX, kBoxY));
@@ -1621,20 +1651,24 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
     const dim3 gf((nx + kFX - 1) / kFX, (ny + kFY - 1) / kFY, (nz + zc - 1) / zc);
     float2* m12 = reinterpret_cast<float2*>(maps);
     float* m3 = maps + 2 * plane;
-    if (!d_grad)
-      return launch("ssim3d_fwd", k_ssim3d_fwd_fused<false>, gf, dim3(kFThreads),
+    if (!d_grad) {
+      GS_TRY(launch("ssim3d_fwd", k_ssim3d_fwd_fused<false>, gf, dim3(kFThreads),
                     FusedShape<false>::smem, s, tmX, tmY, W, nx, ny, nz, zc, C1, C2, gscale,
-                    l1s, d_loss, m12, m3, err);
+                    l1s, parts, m12, m3, err));
+      return launch_after("ssim3d_loss", k_loss_parts, dim3(1), dim3(kThreads), 0, s,
+                          (const float*)parts, (int)(gf.x * gf.y * gf.z), d_loss);
+    }
     GS_TRY(launch("ssim3d_fwd", k_ssim3d_fwd_fused<true>, gf, dim3(kFThreads),
                   FusedShape<false>::smem, s, tmX, tmY, W, nx, ny, nz, zc, C1, C2, gscale, l1s,
-                  d_loss, m12, m3, err));
+                  parts, m12, m3, err));
     CUtensorMap tmM12, tmM3, tmXt, tmYt;
     GS_TRY(volume_map(&tmM12, m12, nx, ny, nz, 8, kBoxX, kBoxY));
     GS_TRY(volume_map(&tmM3, m3, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(volume_map(&tmXt, d_x, nx, ny, nz, 4, kFX, kFY));
     GS_TRY(volume_map(&tmYt, d_y, nx, ny, nz, 4, kFX, kFY));
     return launch("ssim3d_bwd", k_ssim3d_bwd_fused, gf, dim3(kFThreads), FusedShape<true>::smem,
-                  s, tmM12, tmM3, tmXt, tmYt, W, nx, ny, nz, zc, d_grad, accumulate, l1s, err);
+                  s, tmM12, tmM3, tmXt, tmYt, W, nx, ny, nz, zc, d_grad, accumulate, l1s,
+                  (const float*)parts, d_loss, err);
   }
   GS_TRY(launch("ssim3d_z_fwd", gz.y > 1 ? k_ssim3d_z<2, true> : k_ssim3d_z<2, false>, gz, bz, 0,
                 s, W, d_x, d_y, nx, ny, nz, zcol, plane, tmp, l1s, d_loss));

@@ -390,3 +390,22 @@ def test_tv3d_of_the_longest_line(B):
     assert float(grad[-6]) == -1.0 and float(grad[-5]) == 1.0
     grad[-6:-4] = 0.0
     assert bool((grad == 0.0).all())
+
+
+@pytest.mark.parametrize("shape", [(97, 160, 200), (40, 18, 48), (16, 300, 400)])
+@pytest.mark.parametrize("with_grad", [True, False])
+def test_ssim3d_loss_does_not_depend_on_order(B, shape, with_grad):
+    """The streaming kernels' loss is the same bits on every call, and adds to what was there."""
+    g = torch.Generator(device="cuda").manual_seed(sum(shape))
+    y = torch.rand(shape, device="cuda", generator=g)
+    x = y + 0.05 * torch.randn(shape, device="cuda", generator=g)
+    nz, ny, nx = shape
+    grad = torch.empty_like(x) if with_grad else None
+    ws = torch.empty(B.lib().gs_ssim3d_workspace_size(x.numel()), dtype=torch.uint8, device="cuda")
+    first = None
+    for start in [0.0] * 6 + [2.0]:
+        loss = torch.full((1,), start, device="cuda")
+        B.check(B.lib().gs_ssim3d_loss(B.ptr(x), B.ptr(y), nx, ny, nz, 1.0, 1.0, B.ptr(loss),
+                                       B.ptr(grad), 0, B.ptr(ws), ws.numel(), _s()), "ssim3d")
+        first = loss if first is None else first
+        assert torch.equal(loss, first + start) and 0.0 < float(first) < 1.0
