@@ -43,9 +43,10 @@ int launch(const char* name, void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 // may follow an event wait, a copy or a memset, and the launch before it in the call always takes
 // place (a call without Gaussians returns first).  All other kernels of the call are complete by
 // then: the predecessor was launched behind them, or itself waited for them before it let this one
-// be scheduled.  What the predecessor wrote is read with __ldcg (or TMA): a read-only load is for
-// data that nothing writes while the kernel lives, and this one's life begins before the
-// predecessor's end.
+// be scheduled.  What the predecessor wrote is read through TMA, __ldcg or a pointer without __restrict__
+// (where __ldcg would keep the loads of a loop from overlapping): the read-only loads of a const
+// __restrict__ pointer are for data that nothing writes while the kernel lives, and this one's life
+// begins before the predecessor's end.
 // Not for the kernels of very many short CTAs: the wait at the start of each CTA of the raster
 // kernels cost 7 %.
 template <typename... KArgs, typename... Args>

@@ -445,8 +445,8 @@ __global__ void __launch_bounds__(kThreads)
 // second read hits L2).  ranges[key] gets (offset in the group, count), completed by emit.  The
 // last CTA to finish turns the groups' sums into offsets and records the pair total and whether
 // it fits.  Bound by memory: 2 + 2 + 4 bytes per (block, tile).
-__global__ void __launch_bounds__(kScanKeys * kScanSegs)
-    k_key_scan(const __grid_constant__ Batch b, int64_t n_keys, const uint16_t* __restrict__ tcount,
+__global__ void __launch_bounds__(kScanKeys * kScanSegs, 4)
+    k_key_scan(const __grid_constant__ Batch b, int64_t n_keys, const uint16_t* tcount,
                uint32_t* __restrict__ toffset, uint32_t* __restrict__ klocal,
                uint2* __restrict__ ranges, unsigned long long* __restrict__ gsum, uint32_t* ticket,
                long long* __restrict__ vkeys, int total_v, gs_status* st, int64_t cap,
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
     at = I.mat_off + (int64_t)v * I.bpv * tp + tile;
     if (seg == 0 && tile == 0) vkeys[I.v_off + v] = key;
 #pragma unroll 8
-    for (int k = b0; k < b1; ++k) sum += __ldcg(tcount + at + (int64_t)k * tp);
+    for (int k = b0; k < b1; ++k) sum += tcount[at + (int64_t)k * tp];
   }
   if (blockIdx.x == 0 && t == 0) vkeys[total_v] = n_keys;
   part[seg][kl] = sum;
@@ -484,11 +484,22 @@ __global__ void __launch_bounds__(kScanKeys * kScanSegs)
     run += q < seg ? x : 0u;
     total += x;
   }
-#pragma unroll 8
-  for (int k = b0; k < b1; ++k) {
-    const int64_t e = at + (int64_t)k * tp;
-    toffset[e] = run;
-    run += __ldcg(tcount + e);
+  const uint16_t* q = tcount + at + (int64_t)b0 * tp;
+  uint32_t* o = toffset + at + (int64_t)b0 * tp;
+  int left = b1 - b0;
+  for (; left >= 8; left -= 8, q += 8 * tp, o += 8 * tp) {  // eight loads ahead of the stores
+    uint32_t x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = q[j * tp];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      o[j * tp] = run;
+      run += x[j];
+    }
+  }
+  for (; left > 0; --left, q += tp, o += tp) {
+    *o = run;
+    run += *q;
   }
   if (seg == 0) {  // the first two warps hold the group's keys
     // (in 64 bits: 2^27 records that each cover 32 neighbouring tiles pass 2^32; where a 32-bit
@@ -1346,7 +1357,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_project_chain(const __grid_constant__ Batch b, const float4* __restrict__ mean_rho,
                     const float4* __restrict__ scale, const float4* __restrict__ quat,
                     int total_n, int vchunks, int cv, const ViewFrame* __restrict__ frames,
-                    const float4* __restrict__ fpgrad, float4* __restrict__ g_mr,
+                    const float4* fpgrad, float4* __restrict__ g_mr,
                     float4* __restrict__ g_sc, float4* __restrict__ g_q,
                     const uint32_t* __restrict__ counts, float* __restrict__ stat,
                     int* __restrict__ vis) {
@@ -1368,13 +1379,13 @@ __global__ void __launch_bounds__(kThreads, 2)
   float st_acc = 0.f;
   int vis_acc = 0;
   size_t rec = (size_t)(I.item_off + (int64_t)v0 * I.n + il);
-  float4 n0 = __ldcg(fpgrad + 2 * rec), n1 = __ldcg(fpgrad + 2 * rec + 1);  // the next view's moments, one ahead
+  float4 n0 = fpgrad[2 * rec], n1 = fpgrad[2 * rec + 1];  // the next view's moments, one ahead
   for (int v = v0; v < v1; ++v, rec += I.n) {
     if (stat && counts[rec] > 0u) ++vis_acc;
     const float4 m0 = n0, m1 = n1;
     if (v + 1 < v1) {
-      n0 = __ldcg(fpgrad + 2 * (rec + I.n));
-      n1 = __ldcg(fpgrad + 2 * (rec + I.n) + 1);
+      n0 = fpgrad[2 * (rec + I.n)];
+      n1 = fpgrad[2 * (rec + I.n) + 1];
     }
     if (m0.x == 0.f && m0.y == 0.f && m0.z == 0.f && m0.w == 0.f && m1.x == 0.f && m1.y == 0.f)
       continue;
