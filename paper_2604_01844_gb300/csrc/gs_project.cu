@@ -222,15 +222,21 @@ Layout carve(void* ws, const Plan& p) {
 
 // Every operation of the tile rule is one fixed instruction: preprocess counts the tiles and emit
 // places them, so both must get the same answers.  The approximate reciprocals and roots are within
-// two ulp.
+// two ulp; without subnormals, which only footprints beyond 10^15 pixels reach, each is one
+// instruction.
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ float sqrt_approx(float x) {
   float y;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
@@ -788,13 +794,14 @@ struct SlabExt {
 };
 __device__ __forceinline__ SlabExt make_slab(const float4 g, const float4 c, int ty0) {
   SlabExt X;
-  const float D = conic_det(c);
-  const float dyt = sqrt_approx(fmaxf(4.f * c.x * c.w * rcp_approx(D), 0.f));  // the top's height
-  X.dxt = -0.5f * c.y * dyt * rcp_approx(c.x);
-  X.D = c.w == -INFINITY ? 0.f : D;  // the whole box: rows without bound
+  X.D = conic_det(c);
+  // the top point: its height is sqrt(a t), its column -b / (2a) times that
+  const float t = 4.f * c.w * rcp_approx(X.D), at = c.x * t, r = rsqrt_approx(at);
+  X.dxt = -0.5f * c.y * t * r;
   X.c4 = 4.f * c.z * c.w;
   X.inv2c = 0.5f * rcp_approx(c.z);
-  const float my = fmaf(dyt, 1.f / 1048576.f, 0.01f), gy = g.y - (float)ty0;
+  const float my = c.w == -INFINITY ? 1e9f : fmaf(at * r, 1.f / 1048576.f, 0.01f);
+  const float gy = g.y - (float)ty0;
   X.ylo = gy - my;
   X.yhi = gy + my;
   return X;
