@@ -104,3 +104,24 @@ def test_gemm_row_stride(B, ldc):
     assert bool(((got - want).abs() <= bound).all())
     assert torch.allclose(c16[:, :N].cpu().double(), got, rtol=1e-2, atol=1e-2)
     assert bool((c32[:, N:] == 7.0).all()) and bool((c16[:, N:] == 7.0).all())
+
+
+# both sides of every border of the tile rule on 152 SMs: 32 and 64 columns (2304 and 2432 rows of
+# 256 outputs), 64 and 128 (4736 and 4864), 128 and 256 (19328 and 19456); 384 outputs, which no
+# tile of 256 divides
+@pytest.mark.parametrize("M,N,K", [(2304, 256, 128), (2432, 256, 512), (4736, 256, 448),
+                                   (4864, 256, 384), (3328, 384, 64), (19328, 256, 64),
+                                   (19456, 256, 512)])
+def test_gemm_tile_borders_match_float64(B, M, N, K):
+    """K FP32 additions of exact products: K 2^-24 of the sum of magnitudes, and the bias's."""
+    rng = np.random.default_rng(M + N + K)
+    a, b = _bf16(rng.standard_normal((M, K))).cuda(), _bf16(rng.standard_normal((N, K))).cuda()
+    bias = torch.from_numpy(rng.standard_normal(N).astype(np.float32)).cuda()
+    c32 = torch.full((M, N), float("nan"), device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.check(B.lib().gs_gemm_bf16(B.ptr(a), B.ptr(b), M, N, K, B.ptr(bias), 0, B.ptr(c32), None, N,
+                                 B.ptr(err), torch.cuda.current_stream().cuda_stream), "gemm")
+    assert int(err.item()) == 0
+    want = a.double() @ b.double().T + bias.double()
+    bound = (K + 1) * 2.0 ** -24 * (a.double().abs() @ b.double().abs().T + bias.double().abs())
+    assert bool(((c32.double() - want).abs() <= bound).all())

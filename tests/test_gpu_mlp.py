@@ -298,3 +298,23 @@ def test_colsum_of_the_longest_column(gsct):
     B.check(B.lib().gs_colsum(B.ptr(x), x.shape[0], 1, B.ptr(out),
                               torch.cuda.current_stream().cuda_stream), "colsum")
     assert float(out) == 1.0 + 2.0 + 4.0 * 8
+
+
+# the input gradient's tiles of 64 columns (2432 and 4736 bricks), 128 (4864) and 256 (19456); the
+# weight gradients, of at most 32 x 2 or 3 tiles of 128, take 64 whatever the batch
+@pytest.mark.parametrize("M", [2432, 4736, 4864, 19456])
+def test_train_step_tiles_equal_primitive_sequence(gsct, M):
+    """Every tile of the stored-operand GEMMs against the primitive calls on transposed copies: the
+    same products in the same order, so the gradients are equal bit for bit."""
+    from paper_2604_01844_gb300.mlp import BrickMLP
+
+    B = gsct.binding
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x16 = torch.rand(M, 4096, device="cuda", generator=g).to(torch.bfloat16)
+    t = 0.4 * torch.rand(M, 4096, device="cuda", generator=g)
+    a, b = BrickMLP(seed=5), BrickMLP(seed=5)
+    la, lb = torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda")
+    a.train_step(x16, t, la, lr=1e-3)
+    _primitive_train_step(B, b, x16, t, lb, 1e-3, M)
+    assert int(a.err.item()) == 0 and int(b.err.item()) == 0
+    assert torch.equal(a.flat_grad, b.flat_grad) and bool((a.flat_grad != 0).any())
