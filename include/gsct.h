@@ -642,7 +642,8 @@ int gs_gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, const fl
 
 /* y = bf16(x), n elements. */
 int gs_f32_to_bf16(const float* d_x, void* d_y, int64_t n, void* stream);
-/* out[cols][rows] = in[rows][cols] (bf16). */
+/* out[cols][rows] = in[rows][cols] (bf16).  This call and the next serve passes composed by the
+ * caller; gs_mlp_* reads its operands as they are stored and masks in the GEMM. */
 int gs_transpose_bf16(const void* d_in, int rows, int cols, void* d_out, void* stream);
 /* ReLU backward: g *= [act > 0] in place, and out = bf16(g). */
 int gs_relu_mask_bf16(float* d_g, const void* d_act, int64_t n, void* d_out, void* stream);

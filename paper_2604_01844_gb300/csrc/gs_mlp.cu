@@ -283,7 +283,8 @@ int make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_row
 }
 
 // ------------------------------------------------------------------------------------------
-// small helpers of the MLP: conversions, transposes, bias gradients, ReLU masks
+// small helpers of the MLP: conversions and bias gradients; transposes and ReLU masks as entry
+// points of their own, which the network's own passes no longer need
 // ------------------------------------------------------------------------------------------
 __global__ void k_f32_to_bf16(const float* __restrict__ x, __nv_bfloat16* __restrict__ y,
                               int64_t n) {
@@ -394,10 +395,11 @@ int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm fo
   // adds the same products in the same order).  A training batch of 1024 bricks, whose layers
   // make 16 to 64 tiles of 128 columns: forward and backward of the four layers 235 -> 145 us
   // with the transposed copies gone.  MN-major operands come in 64-wide boxes, which
-  // also keeps their TMA coordinates 16-byte aligned.
+  // also keeps their TMA coordinates 16-byte aligned.  The form with both operands MN-major is the
+  // weight gradient's, at most 64 tiles of 128 whatever the batch: it always takes 64.
   const int rows = M / kBM, sms = num_sms();
   int bn = N % 256 == 0 && (int64_t)(N / 256) * rows >= sms ? 256 : 128;
-  if (bn == 128 && 2 * (int64_t)(N / 128) * rows < sms) bn = 64;
+  if (form == GEMM_MN || (bn == 128 && 2 * (int64_t)(N / 128) * rows < sms)) bn = 64;
   if (bn == 64 && form == GEMM_TN && 2 * (int64_t)(N / 64) * rows < sms) bn = 32;
   GemmOut o{d_bias, (const __nv_bfloat16*)d_mask, d_c32, (__nv_bfloat16*)d_c16, ldc, relu, 0};
   o.vec = ldc % 8 == 0 && ((uintptr_t)d_c32 & 15u) == 0 && ((uintptr_t)d_c16 & 15u) == 0 &&
@@ -416,8 +418,6 @@ int gemm_bf16(const void* d_a, const void* d_b, int M, int N, int K, GemmForm fo
       if (bn == 128) return launch_gemm<128, false, true>(ma, mb, M, N, K, o, d_err, after, s);
       return launch_gemm<64, false, true>(ma, mb, M, N, K, o, d_err, after, s);
     default:
-      if (bn == 256) return launch_gemm<256, true, true>(ma, mb, M, N, K, o, d_err, after, s);
-      if (bn == 128) return launch_gemm<128, true, true>(ma, mb, M, N, K, o, d_err, after, s);
       return launch_gemm<64, true, true>(ma, mb, M, N, K, o, d_err, after, s);
   }
 }
