@@ -1384,6 +1384,27 @@ bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 namespace gs {
 namespace {
+// Planes per z chunk of the fused 3D SSIM: the chunks that make the fewest iterations one after
+// another, of the waves of `resident` CTAs and a chunk's planes with its window's ten and a pipeline
+// fill.  Every length that up to nz / 4 chunks can have is tried once, about 2 sqrt(nz) of them
+// (the call's host time at 48 x 18 x 65535: 20 us, where trying every number of chunks took 667).
+int fused_chunk(int64_t tiles, int nz, int resident) {
+  int best = nz;
+  int64_t least = INT64_MAX;
+  for (int n = 1; n <= std::max(1, nz / 4);) {
+    const int c = (nz + n - 1) / n;
+    const int64_t waves = (tiles * ((nz + c - 1) / c) + resident - 1) / resident;
+    const int64_t cost = waves * ((c + 2 * kR + kPP - 1) / kPP + 2);
+    if (cost < least) {
+      least = cost;
+      best = c;
+    }
+    if (c == 1) break;
+    n = (nz + c - 2) / (c - 1);  // the fewest chunks of at most c - 1 planes
+  }
+  return best;
+}
+
 // The two 2D SSIM launches: moments, SSIM and maps; then the gradient from the maps.  l1s
 // (the L1 weight over the pixel count, 0 for none) fuses an L1 term: its sum in the first
 // launch, its sign gradient in the second.
@@ -1634,20 +1655,8 @@ int ssim3d(const float* d_x, const float* d_y, int nx, int ny, int nz, float dat
     GS_TRY(volume_map(&tmX, d_x, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(volume_map(&tmY, d_y, nx, ny, nz, 4, kBoxX, kBoxY));
     GS_TRY(ssim3d_fused_attributes());
-    // z chunks: the number that makes the fewest iterations one after another, of the waves of two
-    // CTAs per SM and a chunk's planes with its window's ten and a pipeline fill
     const int64_t tiles = (int64_t)((nx + kFX - 1) / kFX) * ((ny + kFY - 1) / kFY);
-    int zc = nz;
-    int64_t best = INT64_MAX;
-    for (int n = 1; n <= std::max(1, nz / 4); ++n) {
-      const int c = (nz + n - 1) / n;
-      const int64_t waves = (tiles * ((nz + c - 1) / c) + 2 * num_sms() - 1) / (2 * num_sms());
-      const int64_t cost = waves * ((c + 2 * kR + kPP - 1) / kPP + 2);
-      if (cost < best) {
-        best = cost;
-        zc = c;
-      }
-    }
+    const int zc = fused_chunk(tiles, nz, 2 * num_sms());
     const dim3 gf((nx + kFX - 1) / kFX, (ny + kFY - 1) / kFY, (nz + zc - 1) / zc);
     float2* m12 = reinterpret_cast<float2*>(maps);
     float* m3 = maps + 2 * plane;
