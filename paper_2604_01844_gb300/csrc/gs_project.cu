@@ -9,9 +9,10 @@
 //                tiles that the cut ellipse actually meets (tight tile rule, a range of tiles
 //                per tile row)
 //   then the (view, tile) lists, by one of two routes with the same lists:
-//   direct       (up to kDirectTiles tiles per view) preprocess also counts each block's records
-//                per tile; key_scan turns the counts into each block's offset in every list, the
-//                ranges and the pair total; emit writes each record to its place in the lists
+//   direct       (up to 1600 tiles per view, 2048 in small calls) preprocess also counts each
+//                block's records per tile; key_scan turns the counts into each block's offset in
+//                every list, the ranges and the pair total; emit writes each record to its place
+//                in the lists
 //   sorted       (more tiles) block sums and their scan, emit of (key, record) pairs in record
 //                order, stable radix sort over the tile bits, ranges
 //   raster_fwd   one CTA per (instance, view, tile), records on lanes
@@ -38,11 +39,22 @@ constexpr int kMaxInst = GS_MAX_INSTANCES;
 constexpr int kTileDigitBits = 8;
 
 // The direct route keeps a counter per (block of 256 records, tile) and, in emit, a 32-bit lane
-// mask per (warp, tile) in shared memory: 88 KB at 2048 tiles, two CTAs per SM.  Its cost per
-// block grows with the tiles (10 bytes of counts and offsets each), the sort's with the pairs
-// (about 60 bytes each, some 1300 pairs per block): up to 2048 tiles the direct route is the
-// cheaper one (project 75 x 512^2, 1024 tiles: lists from the counts in 172 instead of 390 us).
-constexpr int kDirectTiles = 2048;
+// mask per (warp, tile) in shared memory: 44 bytes a tile, 88 KB at 2048.  Its cost grows with the
+// blocks times the tiles (10 bytes of counts and offsets each; two CTAs of emit per SM from 1764
+// tiles on), the sort's with the pairs (about 60 bytes each) and its launches.  Forward, sorted
+// against direct, us, from 4.6 pairs a record (scale 0.005) to 14 (0.02):
+//   75 views, 50k or 200k: 1024 tiles 894 / 824 (50k, 0.006) to 4926 / 4331 (200k, 0.012), 1296:
+//     2745 / 2676 to 3036 / 2655, 1600: 3006 / 3158 to 3563 / 3215, 1764: 3141 / 3659 to 3832 / 3652,
+//     2025: 3359 / 3982 to 4269 / 4047
+//   30 views, 20k: 2025 tiles 343 / 328, 522 / 493; 8 views, 5k: 124 / 101
+//   40, 60 and 75 views of 20k at 2025 tiles (6, 10 and 12 million counters) 434 / 436, 630 / 650, 780 /
+//     812; at 1600 tiles 373 / 348, 543 / 522, 668 / 650
+//   one view of 500k (key_scan walks 244 blocks in a row): 1024 tiles 133 / 130, 1296: 132 / 135, 2025:
+//     146 / 160
+// So the lists are direct up to 1600 tiles a view, and up to 2048 while the counters (6 bytes each)
+// take less than half of L2 and no view has more than 512 blocks.
+constexpr int kDirectTiles = 1600, kDirectTilesSmall = 2048, kDirectViewBlocks = 512;
+constexpr int64_t kDirectSmall = 8 << 20;
 
 struct Inst {
   int n, nv, W, H, TW, TH, g_off, v_off;
@@ -137,7 +149,7 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
   b.cut2 = o->cut * o->cut;
   b.eps = o->eps;
   b.znear = o->znear;
-  int64_t items = 0, keys = 0, img = 0, gsum = 0, vsum = 0, blocks = 0, mat = 0, max_tiles = 1;
+  int64_t items = 0, keys = 0, img = 0, gsum = 0, vsum = 0, blocks = 0, mat = 0, max_tiles = 1, max_bpv = 0;
   for (int k = 0; k < n_inst; ++k) {
     const gs_instance& s = inst[k];
     if (s.n < 0 || s.n_views < 1 || s.W < 1 || s.H < 1 || s.W > 32767 || s.H > 32767)
@@ -156,6 +168,7 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
     d.img_off = img;
     d.bpv = (s.n + kThreads - 1) / kThreads;
     d.tp = (d.TW * d.TH + 7) / 8 * 8;
+    max_bpv = std::max<int64_t>(max_bpv, d.bpv);
     d.blk_off = blocks;
     d.mat_off = mat;
     blocks += (int64_t)s.n_views * d.bpv;
@@ -179,7 +192,8 @@ int make_plan(const gs_instance* inst, int n_inst, const gs_opts* o, int64_t cap
   p.cap = std::min<int64_t>(cap, ((int64_t)1 << 31) - 1);
   p.nblocks = (int)blocks;
   p.max_tp = (int)((max_tiles + 7) / 8 * 8);
-  p.direct = max_tiles <= kDirectTiles;
+  p.direct = max_tiles <= kDirectTiles || (max_tiles <= kDirectTilesSmall && mat <= kDirectSmall &&
+                                           max_bpv <= kDirectViewBlocks);
   p.mat = p.direct ? mat : 0;
   p.key_bits = b.tbits;
   p.sort = make_sort_plan(p.key_bits, kTileDigitBits);

@@ -420,3 +420,36 @@ def test_idle_lanes_add_nothing(orc, gsct):
     """Where the exponent of a degenerate ellipse rounds above zero, lanes without a record of their
     own leave the sums alone."""
     _thin_case(orc, gsct, 10000)
+
+
+# beyond 1600 tiles a view the route depends on the counters (views x blocks x tiles against 8 Mi:
+# 60 views of 20,000 Gaussians at 2025 tiles are above, 30 below) ...
+def test_views_of_a_large_call_keep_their_lists(gsct):
+    """Images of the whole call (sorted lists) and of its halves (direct) are the same bits, and the
+    pairs add up."""
+    import torch
+
+    views = synth.cone_views(60, 712, 720)
+    d = to_dev(*synth.gaussians(3, 20000, scale_median=0.01))
+    proj = gsct.Projector(views, 712, 720, tile=16)
+    img, pairs = proj.forward(*d), 0
+    for a in (0, 30):
+        half = gsct.Projector(views[a:a + 30], 712, 720, tile=16)
+        assert torch.equal(half.forward(*d), img[a:a + 30]) and half.status().code == 0
+        pairs += half.count_pairs(*d)
+    assert proj.status().code == 0 and proj.count_pairs(*d) == pairs
+
+
+# ... and on the blocks of a view: at 1640 tiles 131,072 Gaussians are direct and one more is sorted;
+# 1600 tiles are direct with more
+@pytest.mark.parametrize("W,H,n", [(650, 640, 131072), (640, 640, 140000), (650, 640, 140000)])
+def test_one_more_gaussian_keeps_the_image(gsct, W, H, n):
+    """A last Gaussian of zero density is listed behind the others and adds nothing: same bits."""
+    import torch
+
+    mr, sc, qt = synth.gaussians(5, n + 1, scale_median=0.008)
+    mr[n, 3] = 0.0
+    views = synth.cone_views(2, W, H)
+    imgs = [gsct.Projector(views, W, H, tile=16).forward(*to_dev(mr[:k], sc[:k], qt[:k]))
+            for k in (n, n + 1)]
+    assert torch.equal(imgs[0], imgs[1]) and float(imgs[0].max()) > 0
