@@ -123,6 +123,7 @@ struct Plan {
   int n = 0;  // Gaussians over all instances
   int64_t n_keys = 0, cap = 0;
   int64_t n_ctas = 0;  // CTAs of the walking kernels: one per (brick, 16^3 sub-brick)
+  int64_t vox = 0;     // voxels over all regions
   int nblocks = 0, key_bits = 0;
   SortPlan sort;
 };
@@ -168,6 +169,7 @@ int make_plan(const gs_voxel_instance* inst, int n_inst, const gs_opts* o, int64
   if (n > ((int64_t)1 << 31) - kThreads || keys > ((int64_t)1 << 31) - 1) return GS_ERR_ARG;
   p.n = (int)n;
   p.n_keys = keys;
+  p.vox = vox;
   p.n_ctas = keys << (3 * p.b.lsub);
   if (p.n_ctas > ((int64_t)1 << 31) - 1) return GS_ERR_ARG;
   p.cap = std::min<int64_t>(cap, ((int64_t)1 << 31) - 1);
@@ -954,7 +956,16 @@ int bin_bricks(const Plan& p, const Layout& L, const float* mr, const float* sc,
 // 216 sub-bricks 24.8 / 43.1 -> 17.2 / 28.5; 128^3, 20k, 512 sub-bricks 41.1 / 70.0 -> 34.3 /
 // 58.6; 160^3, 30k, 1000 sub-bricks 47.8 / 80.7 -> 43.8 / 74.5).  Above it the SMs are busy anyway
 // and each list would be staged four times for nothing (2704 sub-bricks: 81.3 / 137 -> 80.9 / 136).
-bool quarters(const Plan& p) { return p.n_ctas < 8 * (int64_t)num_sms(); }
+// Bricks of 32 and 64 share a list of 8 or 64 sub-bricks, so staging is most of a CTA's work and four
+// times as much of it pays only while SMs would have no CTA at all: below 7/4 sub-bricks' worth of
+// voxels per SM (forward and backward together, whole -> quartered, brick 32: 96^3, 100k 1513 -> 1156,
+// 100^3, 200k 1510 -> 1263, 96 x 96 x 128, 200k 927 -> 960, 128 x 112 x 112 963 -> 1053, 132 x 163 x
+// 142, 251k 1826 -> 2289; brick 64: 2564 -> 2212, 3094 -> 2980, 2172 -> 2786, 1834 -> 3014, 3332 ->
+// 6255).
+bool quarters(const Plan& p) {
+  const int64_t sms = num_sms();
+  return p.b.lsub == 0 ? p.n_ctas < 8 * sms : 4 * p.vox < 7 * sms * kS * kS * kS;
+}
 
 template <bool COUNT, int NP>
 int vox_fwd_np(const Plan& p, const Layout& L, const uint32_t* vals, float* vol, cudaStream_t s) {

@@ -290,3 +290,20 @@ def test_small_regions_equal_the_whole_volume(gsct, brick, lo, dim):
     dw[part] = dv
     for a, b in zip(whole.backward(*p, dw), small.backward(*p, dv.contiguous())):
         assert torch.all((a - b).abs() <= 6e-6 * a.abs().max())
+
+
+@pytest.mark.parametrize("brick", [32, 64])
+@pytest.mark.parametrize("side", [100, 104])
+def test_split_border_of_large_bricks(gsct, brick, side):
+    """Regions on both sides of the border at which bricks of 32 and 64 stop being split (272 sub-bricks'
+    worth of voxels on 152 SMs: 100^3 is below, 104^3 above) equal their part of a 160^3 volume."""
+    import torch
+
+    p = to_dev(*synth.gaussians(8, 3000, radius=1.0, scale_median=0.03))
+    grid = synth.cube_grid(160)
+    lo, dim = (16, 32, 48), (side,) * 3  # sub-bricks at the same places: the same roundings
+    part = tuple(slice(lo[k], lo[k] + dim[k]) for k in (2, 1, 0))
+    whole = gsct.Voxelizer(grid, brick=16).forward(*p)
+    region = gsct.Voxelizer(grid, lo, dim, brick=brick)
+    got = region.forward(*p)
+    assert torch.equal(got, whole[part]) and region.status().code == 0
