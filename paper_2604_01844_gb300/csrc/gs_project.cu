@@ -1086,27 +1086,27 @@ __device__ __forceinline__ bool is_narrow(const float4 c, const short4 bx) {
 // (the move would cost more than four digits there).
 template <int T>
 __device__ __forceinline__ void narrow_moments(const float4 g, const float4 c, const short4 bx,
-                                               const float* __restrict__ dv, int W, int H,
+                                               const float* __restrict__ dv, int W,
                                                float4* __restrict__ out) {
   constexpr int CW = BwdBlocks<T>::CW;
   const bool whole = c.w == -INFINITY;
   const float ia = 0.5f * rcp_approx(c.x);  // < 0
-  const float D4 = conic_det(c), a4 = 4.f * c.x * c.w;
+  const float D4 = whole ? 0.f : conic_det(c), a4 = 4.f * c.x * c.w;  // whole: rows without end
   const bool own = -(c.x + c.z) * 0.005f > 0.72134752f;
   float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
   for (int by = bx.y & ~3; by <= bx.w; by += 4)
     for (int x0 = bx.x & ~(CW - 1); x0 <= bx.z; x0 += CW) {
       const float xc = own ? g.x : (float)x0 + 0.5f * (float)(CW - 1);
       float s0 = 0.f, sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f;
-      for (int y = by; y < min(by + 4, H); ++y) {
+      for (int y = max(by, (int)bx.y); y <= min(by + 3, (int)bx.w); ++y) {
         const float dy = (float)y - g.y;
         const float B = row_b(c, dy), C = row_c(c, dy);
         // the row's section of the widened cut ellipse, to 1/50 pixel
         const float D = fmaf(-D4 * dy, dy, a4);  // (b y)^2 - 4 a (c y^2 - e)
-        if (!whole && !(D >= 0.f)) continue;
+        if (!(D >= 0.f)) continue;
         const float mid = g.x - B * ia, half = 0.02f - sqrt_approx(D) * ia;
-        const int xa = max(x0, whole ? x0 : (int)ceilf(mid - half));
-        const int xb = min(min(x0 + CW, W) - 1, whole ? W : (int)floorf(mid + half));
+        const int xa = max(x0, (int)ceilf(mid - half));
+        const int xb = min(min(x0 + CW, W) - 1, (int)floorf(mid + half));
         float2 r0 = make_float2(0.f, 0.f), rx = r0, rxx = r0;  // even and odd columns
         const float* row = dv + (size_t)y * W;
         for (int x = xa & ~1; x <= xb; x += 4) {  // four pixels' loads at once
@@ -1149,6 +1149,16 @@ __device__ __forceinline__ void narrow_moments(const float4 g, const float4 c, c
   out[1] = make_float4(mxy, myy, 0.f, 0.f);
 }
 
+// The same out of line, for tiles of 16: inlined there, the rows of narrow records take longer (75 x
+// 512^2, 50k Gaussians of half a pixel: raster_bwd 422 instead of 398 us); tiles of 8 and 32 are better
+// off inlined (75 x 1024^2, 100k at 32: 3064 instead of 3110).
+template <int T>
+__device__ __noinline__ void narrow_moments_call(const float4 g, const float4 c, const short4 bx,
+                                                 const float* __restrict__ dv, int W,
+                                                 float4* __restrict__ out) {
+  narrow_moments<T>(g, c, bx, dv, W, out);
+}
+
 template <int T>
 __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
     k_raster_bwd(const __grid_constant__ Batch b, const uint2* __restrict__ ranges,
@@ -1178,8 +1188,13 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
       for (int i = i0; i < min(I.n, i0 + 32 * chunk); i += 32) {
         const float4 c = recs[2 * (item0 + i) + 1];
         const short4 bx = rect[item0 + i];
-        if (is_narrow<T>(c, bx))
-          narrow_moments<T>(recs[2 * (item0 + i)], c, bx, dv, I.W, I.H, fpgrad + 2 * (item0 + i));
+        if (is_narrow<T>(c, bx)) {
+          float4* out = fpgrad + 2 * (item0 + i);
+          if constexpr (T == 16)
+            narrow_moments_call<T>(recs[2 * (item0 + i)], c, bx, dv, I.W, out);
+          else
+            narrow_moments<T>(recs[2 * (item0 + i)], c, bx, dv, I.W, out);
+        }
       }
     }
     return;
