@@ -1066,6 +1066,7 @@ struct BwdBlocks {
   static constexpr int GS = 9;
   static constexpr int CW = T >= 16 ? 16 : 8;  // columns about whose centre narrow records sum
 };
+constexpr uint32_t kMinPart = 128;  // records of a list's part (64: one view of 1024^2, 20k, 29 instead of 25 us)
 
 // Narrow records: the footprint may have a variance below kNarrowVar square pixels in some direction
 // (the trace of the conic bounds its inverse), in a box of at most 32 x 32 pixels.  Moved from a
@@ -1201,8 +1202,8 @@ __global__ void __launch_bounds__(32, T == 32 ? 24 : 28)
   }
   uint2 r = ranges[key];  // requested together with the status word, not after it
   if (st->code != GS_OK) return;
-  if (parts > 1) {  // an equal part, in whole warps of records
-    const uint32_t part = ((r.y - r.x + parts - 1) / parts + 31u) & ~31u;
+  if (parts > 1) {  // an equal part, in whole warps of records, none of less than kMinPart
+    const uint32_t part = max(kMinPart, ((r.y - r.x + parts - 1) / parts + 31u) & ~31u);
     r.x = min(r.y, r.x + blockIdx.y * part);
     r.y = min(r.y, r.x + part);
   }
@@ -1597,10 +1598,15 @@ template <int T>
 int raster_bwd(const Plan& p, const Layout& L, const uint32_t* vals, const float* dimg,
                cudaStream_t s) {
   // few tiles: their lists are split over up to 16 warps (the records' sums meet in atomics anyway),
-  // while the grid holds less than 16 warps per SM.  8 views of 64^2, 2000 Gaussians (128 tiles),
-  // up to 8 parts and 4 warps per SM: 14.7 us, 16: 11.8, 32 and 24 per SM: 12.2
-  const int parts =
-      (int)std::max<int64_t>(1, std::min<int64_t>(16, 16 * (int64_t)num_sms() / p.n_keys));
+  // while the grid holds less than 64 warps per SM, two waves; a part that a short list does not
+  // need leaves before it reads dL/dI.  raster_bwd, us, unsplit below 16 warps per SM (as before) and now,
+  // against CTAs of a whole tile's warps: 8 views of 512^2, 2k large Gaussians, tile 16 257 -> 215 (184),
+  // tile 32 356 -> 246 (204); 50k, tile 32 208 -> 139 (154); 20 views of 256^2, 20k, tile 32 222 -> 137
+  // (178); 8 views of 64^2, 2k 10.8 -> 9.2 (15); short lists pay for the idle warps: one view of
+  // 1024^2, 20k, tile 32 44 -> 50 (27), tile 16 24.3 -> 24.6 (22).  Two waves' worth of parts for more
+  // tiles cost more than they bring (one view of 2048^2, 16,384 tiles: 63 -> 68).
+  const int64_t slots = 64 * (int64_t)num_sms();
+  const int parts = p.n_keys > slots ? 1 : (int)std::max<int64_t>(2, std::min<int64_t>(16, slots / p.n_keys));
   // warps for the narrow records: 32 records each while they are few, up to 256
   int chunk = 1;
   while (chunk < 8 && (int64_t)p.nblocks * (8 / chunk) > 16 * (int64_t)num_sms()) chunk *= 2;

@@ -453,3 +453,11 @@ def test_one_more_gaussian_keeps_the_image(gsct, W, H, n):
     imgs = [gsct.Projector(views, W, H, tile=16).forward(*to_dev(mr[:k], sc[:k], qt[:k]))
             for k in (n, n + 1)]
     assert torch.equal(imgs[0], imgs[1]) and float(imgs[0].max()) > 0
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n", [127, 129, 700])
+def test_backward_parts_of_long_lists(orc, gsct, tile, n):
+    """Lists just under and over the smallest part of 128 records, and of several parts, over few
+    tiles, against the oracle's gradients."""
+    _grad_case(orc, gsct, 60 + n, n, 2, 45, 39, tile, median=0.2)
