@@ -962,9 +962,14 @@ int bin_bricks(const Plan& p, const Layout& L, const float* mr, const float* sc,
 // 100^3, 200k 1510 -> 1263, 96 x 96 x 128, 200k 927 -> 960, 128 x 112 x 112 963 -> 1053, 132 x 163 x
 // 142, 251k 1826 -> 2289; brick 64: 2564 -> 2212, 3094 -> 2980, 2172 -> 2786, 1834 -> 3014, 3332 ->
 // 6255).
-bool quarters(const Plan& p) {
+// The backward moves a visit's moments once per quarter too, so it is split only up to four CTAs per SM
+// (backward alone, whole -> quartered: 128^3, 200k Gaussians below a voxel 223 -> 192, 20k of one voxel
+// 76 -> 72; 132 x 163 x 142, 251k 742 -> 767, 160^3, 30k 81 -> 84, 10k of four voxels 271 -> 297, 500 of
+// 24 voxels 507 -> 811).
+bool quarters(const Plan& p, bool backward) {
   const int64_t sms = num_sms();
-  return p.b.lsub == 0 ? p.n_ctas < 8 * sms : 4 * p.vox < 7 * sms * kS * kS * kS;
+  return p.b.lsub == 0 ? p.n_ctas < (backward ? 4 : 8) * sms
+                       : 4 * p.vox < 7 * sms * kS * kS * kS;
 }
 
 template <bool COUNT, int NP>
@@ -978,8 +983,8 @@ int vox_fwd_np(const Plan& p, const Layout& L, const uint32_t* vals, float* vol,
 int vox_fwd(const Plan& p, const Layout& L, const uint32_t* vals, float* vol, bool count,
             cudaStream_t s) {
   if (count) return vox_fwd_np<true, 8>(p, L, vals, vol, s);
-  return quarters(p) ? vox_fwd_np<false, 2>(p, L, vals, vol, s)
-                     : vox_fwd_np<false, 8>(p, L, vals, vol, s);
+  return quarters(p, false) ? vox_fwd_np<false, 2>(p, L, vals, vol, s)
+                            : vox_fwd_np<false, 8>(p, L, vals, vol, s);
 }
 
 template <int NP>
@@ -1085,7 +1090,7 @@ int gs_voxelize_batch_backward(const float* d_mean_rho, const float* d_scale,
     GS_TRY(bin_bricks(p, L, d_mean_rho, d_scale, d_quat, s, d_ws, &k, &v));
   }
   GS_CUDA(cudaMemsetAsync(L.vgrad, 0, (size_t)p.n * 3 * sizeof(float4), s));
-  GS_TRY(quarters(p) ? vox_bwd<2>(p, L, v, d_dvol, s) : vox_bwd<8>(p, L, v, d_dvol, s));
+  GS_TRY(quarters(p, true) ? vox_bwd<2>(p, L, v, d_dvol, s) : vox_bwd<8>(p, L, v, d_dvol, s));
   return launch_after("vox_chain", k_vox_chain, dim3(p.nblocks), dim3(kThreads), 0, s,
                 (const float4*)d_mean_rho, (const float4*)d_scale, (const float4*)d_quat, p.n,
                 (const float4*)L.vgrad, (float4*)d_g_mean_rho, (float4*)d_g_scale,
