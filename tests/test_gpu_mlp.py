@@ -318,3 +318,22 @@ def test_train_step_tiles_equal_primitive_sequence(gsct, M):
     _primitive_train_step(B, b, x16, t, lb, 1e-3, M)
     assert int(a.err.item()) == 0 and int(b.err.item()) == 0
     assert torch.equal(a.flat_grad, b.flat_grad) and bool((a.flat_grad != 0).any())
+
+
+# the narrowest matrix that takes a thread per column (128 columns an SM) and one column less
+@pytest.mark.parametrize("less", [0, 1])
+@pytest.mark.parametrize("rows", [1, 9, 500])
+def test_colsum_of_wide_matrices(gsct, rows, less):
+    """Kahan's sum is within 2 x 2^-24 of the sum of magnitudes (and 500 additions' second order), the
+    tree of the other route within (rows / 256 + 17) x 2^-24."""
+    B = gsct.binding
+    cols = 128 * torch.cuda.get_device_properties(0).multi_processor_count - less
+    x = torch.randn(rows, cols, device="cuda", generator=torch.Generator("cuda").manual_seed(rows))
+    x[0, 7] = float("inf")
+    out = torch.full((cols,), float("nan"), device="cuda")
+    B.check(B.lib().gs_colsum(B.ptr(x), rows, cols, B.ptr(out),
+                              torch.cuda.current_stream().cuda_stream), "colsum")
+    tol = (3 if less == 0 else rows / 256 + 17) * 2.0 ** -24 * x.double().abs().sum(0) + 1e-30
+    assert float(out[7]) == float("inf")
+    out[7], x[0, 7], tol[7] = 0.0, 0.0, float("inf")
+    assert bool(((out.double() - x.double().sum(0)).abs() <= tol).all())
