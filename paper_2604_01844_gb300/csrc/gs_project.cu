@@ -875,7 +875,7 @@ __device__ __forceinline__ uint32_t block_mask(const float4 g, const float4 c, c
 // a reconstruction step turns last-bit differences into flipped signs of its gradient.
 // Staging (two dependent gathers per record and its block mask) is about 30 % of the kernel:
 // records as one 32-byte sector, two gathers in flight per thread, approximate roots in the mask and
-// its bands set as runs of bits took tile 16 from 1.00 to 0.93 ms and tile 32 from 4.49 to 4.17.
+// its bands set as runs of bits took tile 16 from 1.00 to 0.93 ms and tile 32 from 4.49 to 4.11.
 template <int T>
 struct FwdBlocks {
   static constexpr int BW = T >= 16 ? 16 : 8;  // block width; 4 rows
@@ -1006,9 +1006,9 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
     __syncthreads();
     if (t == 0 && s_cnt) atomicAdd((unsigned long long*)&st->evals, s_cnt);
   } else {
-    // butterfly reduce-scatter of the half's 4 x BW pixel sums: at each stage a lane keeps the
-    // half of its pairs on its side of the partner bit and adds the partner's copy of that half;
-    // after four stages lane l holds the sums of pairs l NPR / 16 and up
+    // butterfly reduce-scatter of the block's 4 x BW pixel sums over its LPB lanes: at each stage a
+    // lane keeps the half of its pairs on its side of the partner bit and adds the partner's copy of
+    // that half; after log2 LPB stages lane l of them holds the sums of pairs l NPR / LPB and up
     constexpr int KEEP = NPR / LPB;
 #pragma unroll
     for (int bit = LPB / 2, n = NPR / 2; bit >= 1; bit >>= 1, n >>= 1) {
@@ -1049,8 +1049,8 @@ __global__ void __launch_bounds__(FwdBlocks<T>::NT, 512 / FwdBlocks<T>::NT)
 // Bound by instruction issue (71 %; FMA pipe 59 % of its cycles): per pixel pair two FMAs for the
 // exponent, two ex2, the cut, one product and three moment sums, and as much again per block for the
 // record's row coefficients, the centre shift and the queue.  Against warps that own 4 x 16 blocks,
-// list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1032 us;
-// tile 32, 75 x 1024^2, 7.33 -> 5.81 ms; 41 x 389 x 517 parallel, 270 -> 238; 16 small
+// list their records per batch and meet in shared atomics: tile 16, 75 x 512^2, 1228 -> 1020 us;
+// tile 32, 75 x 1024^2, 7.33 -> 5.80 ms; 41 x 389 x 517 parallel, 270 -> 238; 16 small
 // reconstructions 391 -> 311.  4 x 16 blocks here: 1172 instead of 1132, 6.38 instead of 6.41 ms at
 // the same stage.
 // Blocks that start at the record's own box instead of the grid cost their gain in bank conflicts
